@@ -124,7 +124,11 @@ void free_gp(gpmppi_gp h) {
     cudaFree(g.mma_xa);
     cudaFree(g.Wt);
     cudaFree(g.ubar);
+    cudaFree(g.xq[0]);
+    cudaFree(g.Wb[0]);
     if (!g.shared) {
+        cudaFree(g.xq[1]);
+        cudaFree(g.Wb[1]);
         cudaFree(g.Xs[1]);
         cudaFree(g.W[1]);
         cudaFree(g.Linv64[1]);
@@ -152,6 +156,7 @@ void free_ctrl(gpmppi_ctrl c) {
     cudaFree(c->gcell);
     cudaFree(c->gidx);
     cudaFree(c->err);
+    cudaFree(c->ws_buf);
     cudaFree(c->grad_scr);
     for (cudaEvent_t e : c->ev)
         if (e) cudaEventDestroy(e);
@@ -275,7 +280,53 @@ RolloutArgs gpm::make_rollout_args(gpmppi_ctrl c, const float* state, const floa
     return a;
 }
 
+QueryWs gpm::make_query_ws(gpmppi_ctrl c, int s0, int Ks) {
+    const size_t T = (size_t)c->p.T, n = (size_t)c->ws_Ks;
+    QueryWs ws;
+    ws.zq = static_cast<float4*>(c->ws_buf);
+    ws.st = ws.zq + (T + 1) * n;
+    ws.q = reinterpret_cast<float*>(ws.st + T * n);
+    ws.s0 = s0;
+    ws.Ks = Ks;
+    return ws;
+}
+
 namespace {
+
+// The workspace of the query rollout: the records of ws_Ks samples, all of
+// them up to 2^23 queries (36 bytes each for a single GP), beyond which a
+// rollout goes through its samples in pieces.
+int alloc_query_ws(gpmppi_ctrl c) {
+    const size_t T = (size_t)c->p.T, M = (size_t)c->gset.M;
+    size_t n = ((size_t)1 << 23) / T;
+    if (n > (size_t)c->p.K) n = (size_t)c->p.K;
+    c->ws_Ks = (int)n;
+    cudaFree(c->ws_buf);
+    c->ws_buf = nullptr;
+    cudaError_t e = cudaMalloc(&c->ws_buf, n * (16 * (2 * T + 1) + 4 * M * T));
+    if (e != cudaSuccess) return cuda_fail(e, "mppi_create: rollout workspace");
+    return GPMPPI_OK;
+}
+
+// Alg. 1 Step 1 as the query rollout (query.cuh).
+int launch_query_rollout(gpmppi_ctrl c, const RolloutArgs& a, cudaStream_t st) {
+    int rc;
+    for (int s0 = 0; s0 < c->p.K; s0 += c->ws_Ks) {
+        const int Ks = c->p.K - s0 < c->ws_Ks ? c->p.K - s0 : c->ws_Ks;
+        const QueryWs ws = make_query_ws(c, s0, Ks);
+        if ((rc = launch_chain(a, c->gset, ws, st))) return rc;
+        VarJob j = {};
+        j.z = reinterpret_cast<const float*>(ws.zq);
+        j.Q = c->p.T * Ks;
+        j.q = ws.q;
+        j.err = c->err;
+        j.wait_ns = c->wait_ns;
+        j.expire_first = c->expire_first;
+        if ((rc = launch_var_fp32(c->gset, j, true, st))) return rc;
+        if ((rc = launch_stage_cost(a, c->gset, ws, st))) return rc;
+    }
+    return GPMPPI_OK;
+}
 
 // Launch arguments of the ensemble rollout: the single-GP arguments plus the
 // per-terrain factors and weights.
@@ -528,6 +579,11 @@ int mppi_create(const gpmppi_params* p, const float* obstacles, int32_t O, const
             free_ctrl(c);
             return rc;
         }
+        c->gset = single_gp_set(gp->g, 0);
+        if (p->precision == GPMPPI_FP32 && (rc = alloc_query_ws(c))) {
+            free_ctrl(c);
+            return rc;
+        }
         if (p->precision != GPMPPI_FP32) {
             c->fmt = (p->precision == GPMPPI_FP16_SPLIT) ? 0 : (p->precision == GPMPPI_BF16_SPLIT ? 1 : 2);
             if ((rc = build_mma_tiles(gp->g, c->fmt))) {
@@ -633,8 +689,7 @@ int mppi_step(gpmppi_ctrl c, const float state[5], const float* U_nom, float* U_
     else if (c->cl)
         rc = launch_rollout_cl(a, c->cla, c->fmt, false, st);
     else
-        rc = (c->fmt < 0) ? launch_rollout_fp32(a, &c->tmW, false, st)
-                          : launch_rollout_mma(a, c->mm, c->fmt, false, st);
+        rc = (c->fmt < 0) ? launch_query_rollout(c, a, st) : launch_rollout_mma(a, c->mm, c->fmt, false, st);
     if (rc) return rc;
     if (c->profiling) GPM_CUDA(cudaEventRecord(c->ev[1], st));
     UpdateArgs u;
@@ -714,7 +769,7 @@ int mppi_rollout_trace(gpmppi_ctrl c, const float state[5], const float* U_nom, 
     if (c->ens && c->fmt < 0) return launch_rollout_ens(make_ens_args(c, a), true, (cudaStream_t)stream);
     if (c->cl) return launch_rollout_cl(a, c->cla, c->fmt, true, (cudaStream_t)stream);
     if (c->fmt >= 0) return launch_rollout_mma(a, c->mm, c->fmt, true, (cudaStream_t)stream);
-    return launch_rollout_fp32(a, &c->tmW, true, (cudaStream_t)stream);
+    return launch_query_rollout(c, a, (cudaStream_t)stream);
 }
 
 int mppi_create_ensemble(const gpmppi_params* p, const float* obstacles, int32_t O, const float* path,

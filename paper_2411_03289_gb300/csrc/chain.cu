@@ -1,0 +1,247 @@
+// The mean chain of the query rollout (Alg. 1 Step 1: noise, clamp, Eq. 1-3,
+// 6): all samples' means through the horizon, and the GP query of every step.
+//
+// A warp carries SG samples; its lanes share the training points, so that every
+// point read from shared memory serves SG samples.  A step is the samples'
+// kernel rows and their two mean sums (two points per packed instruction), a
+// reduction that scatters the 2 SG sums over the lanes, and the unicycle.  The
+// perturbed controls do not depend on the state, so the CTA draws those of all
+// its samples and steps first.
+// What bounds it: the latency of a step's serial chain (row -> reduction ->
+// dynamics -> next row) while K leaves few warps per scheduler, the issue slots
+// of the kernel rows (about 10 instructions for two points) once it does not.
+// With one sample per 16 lanes the shared-memory reads of the points bounded it
+// (12 KB per sample and step at N = 500): 112 us at K = 4096, T = 50, N = 500
+// against 87 us now.
+#include "query.cuh"
+
+namespace gpm {
+namespace {
+
+using namespace qr;
+
+constexpr int CT = 128;          // threads
+constexpr int CW = CT / 32;
+constexpr int GRP = 8;           // pairs of points summed plainly between compensated additions
+
+// Compensated sums over the warp's lanes of the NV values (v[i], c[i]): on
+// return v[0] holds the total of one of them, the one sum_lane maps to this
+// lane (the exchange halves the values a lane holds while it has several).
+template <int NV>
+__device__ __forceinline__ void scatter_sum(float (&v)[NV], float (&c)[NV]) {
+    const int lane = threadIdx.x & 31;
+    int n = NV;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        if (n > 1) {
+            n /= 2;
+            const bool up = lane & o;
+#pragma unroll
+            for (int i = 0; i < NV / 2; ++i) {
+                if (i >= n) break;
+                const float sv = up ? v[i] : v[i + n], sc = up ? c[i] : c[i + n];
+                float kv = up ? v[i + n] : v[i], kc = up ? c[i + n] : c[i];
+                const float ov = __shfl_xor_sync(0xffffffffu, sv, o), oc = __shfl_xor_sync(0xffffffffu, sc, o);
+                kahan_add(kv, kc, ov);
+                v[i] = kv;
+                c[i] = kc + oc;
+            }
+        } else {
+            const float ov = __shfl_xor_sync(0xffffffffu, v[0], o), oc = __shfl_xor_sync(0xffffffffu, c[0], o);
+            kahan_add(v[0], c[0], ov);
+            c[0] += oc;
+        }
+    }
+    v[0] += c[0];
+}
+
+// the lane that holds value i of scatter_sum<NV>
+template <int NV>
+__device__ __forceinline__ int sum_lane(int i) {
+    int lane = 0;
+#pragma unroll
+    for (int o = 16, n = NV; n > 1; o >>= 1) {
+        n /= 2;
+        if (i & n) lane |= o;
+    }
+    return lane;
+}
+
+// SMEM: the training sets of all GPs staged in shared memory (x in two arrays
+// of 16-byte halves, so that neighbouring lanes read neighbouring lines).
+template <int SG, bool SMEM>
+__global__ void __launch_bounds__(CT) k_chain(const RolloutArgs a, const GpSet gs, const QueryWs ws) {
+    extern __shared__ __align__(16) unsigned char csm[];
+    constexpr int SPC = CW * SG;               // samples per CTA
+    constexpr int NV = 2 * SG;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    float4* zs = reinterpret_cast<float4*>(csm) + warp * SG;            // the warp's queries
+    ulonglong2* xs = reinterpret_cast<ulonglong2*>(csm + CW * SG * 16);
+    const int l0 = blockIdx.x * SPC;
+    const int j = lane % SG;                                            // the sample whose state this lane carries
+    const int l = min(l0 + warp * SG + j, ws.Ks - 1);                   // spare ones repeat the last sample
+    const bool writer = lane < SG && l0 + warp * SG + j < ws.Ks;
+    const int s = ws.s0 + l;
+    const int K = a.K, T = a.T, Ks = ws.Ks;
+
+    float mu0 = a.x0[0], mu1 = a.x0[1], mu2 = a.x0[2], mu3 = a.x0[3], mu4 = a.x0[4];
+    uint32_t it0 = a.it0, it1 = a.it1;
+    if (a.x0_dev) {
+        mu0 = a.x0_dev[0]; mu1 = a.x0_dev[1]; mu2 = a.x0_dev[2]; mu3 = a.x0_dev[3]; mu4 = a.x0_dev[4];
+    }
+    if (a.it_dev) {
+        const unsigned long long v = *a.it_dev;
+        it0 = (uint32_t)v;
+        it1 = (uint32_t)(v >> 32);
+    }
+    if (SMEM) {
+        ulonglong2* dst = xs;
+        for (int t = 0; t < gs.M; ++t) {
+            const int np = gs.gp[t].npad / 2;           // pairs
+            const ulonglong2* src = reinterpret_cast<const ulonglong2*>(gs.gp[t].xq);
+            for (int i = tid; i < np; i += CT) {
+                dst[i] = __ldg(src + 2 * i);
+                dst[np + i] = __ldg(src + 2 * i + 1);
+                dst[2 * np + i] = __ldg(src + 2 * np + i);
+            }
+            dst += 3 * np;
+        }
+    }
+    // clamped perturbed controls (Eq. 8) of this CTA's samples, every step
+    if (a.u_tilde) {
+        const int n = min(SPC, Ks - l0);
+        for (int i = tid; i < SPC * T; i += CT) {
+            const int k = i / SPC, q = i % SPC;
+            if (q >= n) continue;
+            const float2 e = control_eps((uint32_t)k, (uint32_t)(ws.s0 + l0 + q), it0, it1, a.key0, a.key1, a.sig_v,
+                                         a.sig_w);
+            float2 u;
+            u.x = fminf(fmaxf(__ldg(a.U + 2 * k) + e.x, a.umin0), a.umax0);
+            u.y = fminf(fmaxf(__ldg(a.U + 2 * k + 1) + e.y, a.umin1), a.umax1);
+            a.u_tilde[(size_t)k * K + ws.s0 + l0 + q] = u;
+        }
+    }
+    __syncthreads();
+    // the control of step k (no sampled controls: the nominal trajectory)
+    auto control = [&](int k) {
+        if (a.u_tilde) return a.u_tilde[(size_t)k * K + s];
+        return make_float2(fminf(fmaxf(__ldg(a.U + 2 * k), a.umin0), a.umax0),
+                           fminf(fmaxf(__ldg(a.U + 2 * k + 1), a.umin1), a.umax1));
+    };
+    float2 un = control(0);
+    for (int k = 0; k < T; ++k) {
+        const float2 ut = un;
+        if (k + 1 < T) un = control(k + 1);
+        if (lane < SG) zs[lane] = make_float4(mu3, mu4, ut.x, ut.y);
+        __syncwarp();
+        float mean_v = 0.0f, mean_w = 0.0f;
+        const ulonglong2* base = xs;
+        for (int t = 0; t < gs.M; ++t) {
+            const GpSet::One& G = gs.gp[t];
+            const int np = G.npad / 2, pairs = (G.N + 1) / 2;
+            const ulonglong2* xg = reinterpret_cast<const ulonglong2*>(G.xq);
+            uint64_t zz[SG][4];
+#pragma unroll
+            for (int q = 0; q < SG; ++q) {
+                const float4 z = zs[q];
+                const float z0 = z.x * G.zscale[0], z1 = z.y * G.zscale[1];
+                const float z2 = z.z * G.zscale[2], z3 = z.w * G.zscale[3];
+                zz[q][0] = tc::f2pack(z0, z0);
+                zz[q][1] = tc::f2pack(z1, z1);
+                zz[q][2] = tc::f2pack(z2, z2);
+                zz[q][3] = tc::f2pack(z3, z3);
+            }
+            float v[NV], c[NV];
+#pragma unroll
+            for (int i = 0; i < NV; ++i) {
+                v[i] = 0.0f;
+                c[i] = 0.0f;
+            }
+            for (int p0 = 0; p0 < pairs; p0 += 32 * GRP) {
+                uint64_t pv[SG], pw[SG];
+#pragma unroll
+                for (int q = 0; q < SG; ++q) {
+                    pv[q] = 0ull;
+                    pw[q] = 0ull;
+                }
+                const int pe = min(pairs, p0 + 32 * GRP);
+#pragma unroll 2
+                for (int p = p0 + lane; p < pe; p += 32) {
+                    const ulonglong2 xa = SMEM ? base[p] : __ldg(xg + 2 * p);
+                    const ulonglong2 xb = SMEM ? base[np + p] : __ldg(xg + 2 * p + 1);
+                    const ulonglong2 al = SMEM ? base[2 * np + p] : __ldg(xg + 2 * np + p);
+#pragma unroll
+                    for (int q = 0; q < SG; ++q) {
+                        float k0, k1;
+                        kernel_pair(zz[q], xa, xb, k0, k1);
+                        const uint64_t kk = tc::f2pack(k0, k1);
+                        pv[q] = tc::f2fma(kk, al.x, pv[q]);
+                        pw[q] = tc::f2fma(kk, al.y, pw[q]);
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < SG; ++q) {
+                    float x, y;
+                    tc::f2unpack(pv[q], x, y);
+                    kahan_add(v[2 * q], c[2 * q], x + y);
+                    tc::f2unpack(pw[q], x, y);
+                    kahan_add(v[2 * q + 1], c[2 * q + 1], x + y);
+                }
+            }
+            scatter_sum<NV>(v, c);
+            const float wsf = G.w * G.sf2;
+            mean_v += wsf * __shfl_sync(0xffffffffu, v[0], sum_lane<NV>(2 * j));
+            mean_w += wsf * __shfl_sync(0xffffffffu, v[0], sum_lane<NV>(2 * j + 1));
+            base += 3 * np;
+        }
+        float sn, cs;
+        sincosf(mu2, &sn, &cs);
+        const float nX = mu0 + a.dt * mu3 * cs;
+        const float nY = mu1 + a.dt * mu3 * sn;
+        const float nT = mu2 + a.dt * mu4;
+        const float nV = mu3 + a.kv * (ut.x - mu3) + mean_v;
+        const float nW = mu4 + a.kw * (ut.y - mu4) + mean_w;
+        if (writer) {
+            ws.zq[(size_t)k * Ks + l] = make_float4(mu3, mu4, ut.x, ut.y);
+            ws.st[(size_t)k * Ks + l] = make_float4(nX, nY, nT, nV);
+        }
+        mu0 = nX; mu1 = nY; mu2 = nT; mu3 = nV; mu4 = nW;
+        __syncwarp();                          // every lane has read zs
+    }
+    if (writer) ws.zq[(size_t)T * Ks + l] = make_float4(mu3, mu4, 0.0f, 0.0f);
+}
+
+}  // namespace
+
+int launch_chain(const RolloutArgs& a, const GpSet& gs, const QueryWs& ws, cudaStream_t st) {
+    size_t points = 0;
+    for (int t = 0; t < gs.M; ++t) points += (size_t)gs.gp[t].npad;
+    // two CTAs per SM keep their training sets in shared memory up to 4096 points
+    const bool sm = points * 24 <= 100 * 1024;
+    // samples per warp: as many as leave every scheduler a warp and a half.
+    // Measured (us, 1 / 2 / 4 / 8 samples): K = 256 T = 20 N = 50: 14 / 16 / 16 /
+    // 20; K = 1000 T = 40 N = 300: 34 / 36 / 40 / 54; K = 4096 T = 50 N = 500:
+    // 114 / 98 / 87 / 87; K = 16384 T = 100 N = 2048: 2379 / 1683 / 1414 / 1509.
+    int sg = 1;
+    while (sg < 4 && ws.Ks / (2 * sg) >= 900) sg *= 2;
+#define GPM_CHAIN(L)                                                                                            \
+    do {                                                                                                        \
+        const dim3 grid((unsigned)((ws.Ks + CW * L - 1) / (CW * L)));                                           \
+        const size_t smem = CW * L * 16 + (sm ? points * 24 : 0);                                               \
+        if (sm) {                                                                                               \
+            GPM_CUDA(cudaFuncSetAttribute(k_chain<L, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,        \
+                                          101 * 1024));                                                         \
+            k_chain<L, true><<<grid, CT, smem, st>>>(a, gs, ws);                                                \
+        } else {                                                                                                \
+            k_chain<L, false><<<grid, CT, smem, st>>>(a, gs, ws);                                               \
+        }                                                                                                       \
+    } while (0)
+    if (sg == 1) GPM_CHAIN(1);
+    else if (sg == 2) GPM_CHAIN(2);
+    else GPM_CHAIN(4);
+#undef GPM_CHAIN
+    GPM_CUDA(cudaGetLastError());
+    return GPMPPI_OK;
+}
+
+}  // namespace gpm

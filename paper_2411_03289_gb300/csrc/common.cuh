@@ -141,6 +141,14 @@ struct GpDevice {
     // the cluster rollout's training inputs and alpha in pair layout (NpC x 4
     // floats, then NpC x 2), copied into shared memory by one bulk copy
     float* cl_xa = nullptr;
+    // Layouts of the query rollout (query.cuh), built by the fit, per distinct
+    // output: npad = N rounded up to 128 points; xq[o] = the scaled inputs in
+    // pair layout (npad x 4 floats: two points per 32 bytes, far points past
+    // N) then alpha (npad x 2 floats, both outputs, 0 past N); Wb[o] = L^-T in
+    // 16 x 128 pieces, block column cb holding rows 0 .. 128 (cb + 1) - 1.
+    int npad = 0;
+    float* xq[2] = {nullptr, nullptr};
+    float* Wb[2] = {nullptr, nullptr};
     // adjoint rollout, built on first use: rows of L^-1 (Np x Np) and the
     // vectors (dK/dl_d) alpha_o (8 x Np)
     float* Wt = nullptr;
@@ -352,7 +360,45 @@ struct UpdateArgs {
     float inv_lambda;
 };
 
+// ---- query rollout (chain.cu, variance_fp32.cu, stage_cost.cu) -------------
+// The GPs of one rollout (Eq. 3; a single GP has M = 1 and w = 1).
+struct GpSet {
+    int M;
+    struct One {
+        const float* xq;        // GpDevice::xq (pair layout, npad points)
+        const float* Wb;        // GpDevice::Wb
+        int N, npad;
+        float sf2, w;
+        float qscale;           // variance = sf2 - qscale * (what the variance kernel stored)
+        float zscale[4];
+    } gp[kMaxTerrains];
+};
+
+// Per-query records of the samples [s0, s0 + Ks) of one rollout (row k, sample
+// s at [k Ks + s - s0]).
+struct QueryWs {
+    float4* zq;                 // (T + 1) x Ks: (v, omega, u~_v, u~_omega) before step k
+    float4* st;                 // T x Ks: (X, Y, theta, v) after step k
+    float* q;                   // M x T x Ks: |L_t^-1 k*|^2 over the variance kernel's scale
+    int s0, Ks;
+};
+
 // launchers (defined in the .cu files)
+int launch_chain(const RolloutArgs& a, const GpSet& gs, const QueryWs& ws, cudaStream_t st);
+struct VarJob {
+    const float* z;             // Q x 4 queries (any 4-byte alignment)
+    int Q;
+    float* q;                   // M x Q
+    float* mean;                // Q x 2 or null: column `out` of the posterior mean (gp_predict)
+    float* var;                 // with mean: Q x 2 posterior variance
+    int out;                    // with mean: the output, or -1 for both from one kernel row
+    unsigned int* err;
+    unsigned long long wait_ns;
+    int expire_first;
+};
+int launch_var_fp32(const GpSet& gs, const VarJob& j, bool dependent, cudaStream_t st);
+int launch_stage_cost(const RolloutArgs& a, const GpSet& gs, const QueryWs& ws, cudaStream_t st);
+GpSet single_gp_set(const GpDevice& g, int o);
 int launch_rollout_fp32(const RolloutArgs& a, const CUtensorMap* tmap_w, bool trace,
                         cudaStream_t st);
 // TMA tensor map over W (Np x Np floats) with the box the FP32 rollout reads

@@ -177,6 +177,16 @@ __global__ void k_pack_w(const double* __restrict__ Xm, int N, int Np, float* __
     W[(size_t)j * Np + i] = v;
 }
 
+// L^-T in the pieces of the query rollout's variance (GpDevice::Wb): block
+// column cb = blockIdx.y holds rows 0 .. 128 (cb + 1) - 1, 128 columns each.
+__global__ void k_pack_wb(const float* __restrict__ W, int Np, float* __restrict__ Wb) {
+    const int cb = blockIdx.y;
+    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= (cb + 1) * 128 * 128) return;
+    const int j = idx / 128, i = 128 * cb + idx % 128;
+    Wb[(size_t)cb * (cb + 1) / 2 * (128 * 128) + idx] = (j < Np && i < Np) ? W[(size_t)j * Np + i] : 0.0f;
+}
+
 __global__ void k_pack_x(const double* __restrict__ X, int N, double s0, double s1, double s2,
                          double s3, float* __restrict__ Xs) {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
@@ -560,6 +570,8 @@ int gp_fit_device(GpDevice& g, const double* X, const double* Y, int N, cudaStre
     // of the rollout fits inside the tensor; N = 0 has no W at all
     g.Np = (N > 0) ? ((N + 15) / 16) * 16 : 0;
     if (g.Np > 0 && g.Np < 64) g.Np = 64;
+    g.npad = ((N + 127) / 128) * 128;
+    const size_t nb = (size_t)g.npad / 128;
     const double log2e = 1.4426950408889634;
     for (int o = 0; o < 2; ++o) {
         g.sf2[o] = (float)g.hyper[o].signal_var;
@@ -575,11 +587,15 @@ int gp_fit_device(GpDevice& g, const double* X, const double* Y, int N, cudaStre
         GPM_CUDA(cudaMalloc(&g.W[o], sizeof(float) * (g.Np > 0 ? (size_t)g.Np * g.Np : 1)));
         GPM_CUDA(cudaMalloc(&g.Linv64[o], sizeof(double) * (nn > 0 ? nn : 1)));
         GPM_CUDA(cudaMalloc(&g.alpha64[o], sizeof(double) * (N > 0 ? N : 1)));
+        GPM_CUDA(cudaMalloc(&g.xq[o], sizeof(float) * 6 * (g.npad > 0 ? g.npad : 1)));
+        GPM_CUDA(cudaMalloc(&g.Wb[o], sizeof(float) * (nb > 0 ? nb * (nb + 1) / 2 * (128 * 128) : 1)));
     }
     if (g.shared) {
         g.Xs[1] = g.Xs[0];
         g.W[1] = g.W[0];
         g.Linv64[1] = g.Linv64[0];
+        g.xq[1] = g.xq[0];
+        g.Wb[1] = g.Wb[0];
         GPM_CUDA(cudaMalloc(&g.alpha64[1], sizeof(double) * (N > 0 ? N : 1)));
     }
     if (N == 0) return GPMPPI_OK;
@@ -657,6 +673,10 @@ int gp_fit_device(GpDevice& g, const double* X, const double* Y, int N, cudaStre
         if ((rc = check(cudaGetLastError(), "inverse kernels"))) return rc;
     }
     k_pack_alpha<<<(N + 127) / 128, 128, 0, st>>>(g.alpha64[0], g.alpha64[1], N, g.alpha);
+    for (int o = 0; o < nout; ++o) {
+        k_pack_xa<<<(g.npad + 127) / 128, 128, 0, st>>>(g.Xs[o], g.alpha, N, g.npad, 0, g.npad, g.xq[o]);
+        k_pack_wb<<<dim3((unsigned)(nb * 64), (unsigned)nb), 256, 0, st>>>(g.W[o], g.Np, g.Wb[o]);
+    }
     if ((rc = check(cudaGetLastError(), "pack alpha"))) return rc;
     if ((rc = check(cudaStreamSynchronize(st), "gp_fit sync"))) return rc;
     cleanup();

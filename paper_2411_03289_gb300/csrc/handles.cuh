@@ -44,6 +44,11 @@ struct gpmppi_ctrl_s {
     int* gidx = nullptr;
     float gx0 = 0, gy0 = 0, ginv = 0;
     int gnx = 0, gny = 0;
+    // query rollout: the GP (or terrain GPs) and the records of up to ws_Ks
+    // samples at a time (allocated with the controller)
+    gpm::GpSet gset{};
+    void* ws_buf = nullptr;
+    int ws_Ks = 0;
     unsigned int* err = nullptr;  // device status word written by the rollout
     int stages = 2;               // per-warp TMA pipeline depth
     CUtensorMap tmW;              // TMA map over the GP's W
@@ -70,4 +75,6 @@ namespace gpm {
 // Launch arguments of one rollout of controller c from state (host, 5) with
 // nominal controls U (device, T x 2).
 RolloutArgs make_rollout_args(gpmppi_ctrl c, const float* state, const float* U);
+// Records of the samples [s0, s0 + Ks) in the controller's workspace.
+QueryWs make_query_ws(gpmppi_ctrl c, int s0, int Ks);
 }  // namespace gpm
