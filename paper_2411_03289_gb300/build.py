@@ -21,11 +21,11 @@ BUILD_DIR = os.path.join(HERE, "_build")
 LIB_DIR = os.path.join(HERE, "_lib")
 LIB_PATH = os.path.join(LIB_DIR, "libgpmppi.so")
 
-SOURCES = ["abi.cu", "gp_fit.cu", "rollout_fp32.cu", "rollout_mma.cu", "mma_selftest.cu",
+SOURCES = ["abi.cu", "gp_fit.cu", "rollout_mma.cu", "mma_selftest.cu",
            "mppi_aux.cu", "update_noalloc.cu", "batch.cu", "adjoint.cu",
-           "ensemble.cu", "terrain_qp.cu", "rollout_cluster.cu",
+           "terrain_qp.cu",
            "lane_grid.cu", "peaks.cu", "gram_tc.cu",
-           "chain.cu", "variance_fp32.cu", "stage_cost.cu"]
+           "chain.cu", "chain_fp32.cu", "tri.cu", "variance_tc.cu", "predict.cu", "stage_cost.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
               "-I", INCLUDE, "-I", CSRC]

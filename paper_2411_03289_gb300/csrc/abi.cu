@@ -76,10 +76,6 @@ namespace {
 
 constexpr uint32_t kGpMagic = kGpMagicValue;
 constexpr uint32_t kCtrlMagic = kCtrlMagicValue;
-// training sets larger than this use the separate low column set of the
-// streaming tensor-core rollout (MmaArgs::lo_set)
-constexpr int kLoSetMinN = 768;
-
 bool is_finite(double v) { return std::isfinite(v); }
 
 // Quantile of a chi-squared variable with 2 degrees of freedom (Eq. 14):
@@ -108,31 +104,17 @@ namespace {
 void free_gp(gpmppi_gp h) {
     if (!h) return;
     GpDevice& g = h->g;
-    cudaFree(g.alpha);
-    cudaFree(g.Xs[0]);
-    cudaFree(g.W[0]);
-    cudaFree(g.Linv64[0]);
-    cudaFree(g.alpha64[0]);
-    cudaFree(g.alpha64[1]);
+    cudaFree(g.mem);
     for (int f = 0; f < 3; ++f) {
+        cudaFree(g.Bt[f]);
         cudaFree(g.mma_hi[f]);
         cudaFree(g.mma_lo[f]);
     }
     cudaFree(g.mma_mid);
-    for (int f = 0; f < 2; ++f) cudaFree(g.cl_tiles[f]);
-    cudaFree(g.cl_xa);
     cudaFree(g.mma_xa);
-    cudaFree(g.Wt);
+    cudaFree(g.Lb);
     cudaFree(g.ubar);
-    cudaFree(g.xq[0]);
-    cudaFree(g.Wb[0]);
-    if (!g.shared) {
-        cudaFree(g.xq[1]);
-        cudaFree(g.Wb[1]);
-        cudaFree(g.Xs[1]);
-        cudaFree(g.W[1]);
-        cudaFree(g.Linv64[1]);
-    }
+    scratch_user(g.device, -1);
     h->magic = 0;
     delete h;
 }
@@ -145,10 +127,6 @@ void free_ctrl(gpmppi_ctrl c) {
     cudaFree(c->costs);
     cudaFree(c->hs_U);
     cudaFree(c->hs_w);
-    cudaFree(c->ens_hi);
-    cudaFree(c->ens_lo);
-    cudaFree(c->ens_mid);
-    cudaFree(c->ens_xa);
     cudaFree(c->u_tilde);
     cudaFree(c->partial);
     cudaFree(c->counter);
@@ -156,7 +134,12 @@ void free_ctrl(gpmppi_ctrl c) {
     cudaFree(c->gcell);
     cudaFree(c->gidx);
     cudaFree(c->err);
+    cudaFree(c->ens_hi);
+    cudaFree(c->ens_lo);
+    cudaFree(c->ens_mid);
+    cudaFree(c->ens_xa);
     cudaFree(c->ws_buf);
+    cudaFree(c->vbuf);
     cudaFree(c->grad_scr);
     for (cudaEvent_t e : c->ev)
         if (e) cudaEventDestroy(e);
@@ -233,8 +216,6 @@ RolloutArgs gpm::make_rollout_args(gpmppi_ctrl c, const float* state, const floa
     a.Np = g.Np;
     a.O = c->O;
     a.S = c->S;
-    a.mt = c->mt;
-    a.stages = c->stages;
     a.err = c->err;
     a.wait_ns = c->wait_ns;
     a.expire_first = c->expire_first;
@@ -280,6 +261,37 @@ RolloutArgs gpm::make_rollout_args(gpmppi_ctrl c, const float* state, const floa
     return a;
 }
 
+// Alg. 1 Step 1 as the query rollout (query.cuh).
+int gpm::launch_query_rollout(gpmppi_ctrl c, const RolloutArgs& a, const GpSet& gs, cudaStream_t st) {
+    int rc;
+    for (int s0 = 0; s0 < c->p.K; s0 += c->ws_Ks) {
+        const int Ks = c->p.K - s0 < c->ws_Ks ? c->p.K - s0 : c->ws_Ks;
+        const QueryWs ws = make_query_ws(c, s0, Ks);
+        const int Q = c->p.T * Ks;
+        if (c->fmt < 0) {
+            if ((rc = launch_chain_fp32(a, gs, c->ens ? kChainTree : kChainOrdered, ws, st))) return rc;
+            for (int t = 0; t < gs.M; ++t)
+                for (int q0 = 0; q0 < Q; q0 += c->v_q) {
+                    const int n = Q - q0 < c->v_q ? Q - q0 : c->v_q;
+                    TriJob j = tri_forward(gs.gp[t], reinterpret_cast<const float*>(ws.zq + q0), n, c->vbuf);
+                    j.err = a.err;
+                    j.wait_ns = a.wait_ns;
+                    j.expire_first = a.expire_first;
+                    if ((rc = launch_tri_forward(j, true, st))) return rc;
+                    if ((rc = launch_rowsum(c->vbuf, gs.gp[t].npad, n, gs.gp[t].N, c->ens ? kSumLanes : kSumPairs,
+                                            ws.q + (size_t)t * Q + q0, st)))
+                        return rc;
+                }
+        } else {
+            if ((rc = launch_chain(a, gs, ws, st))) return rc;
+            const VarTcJob j = {ws.zq, Q, ws.q, ws.nsplit, a.err};
+            if ((rc = launch_var_tc(gs, j, c->fmt, c->nsm, true, st))) return rc;
+        }
+        if ((rc = launch_stage_cost(a, gs, ws, c->ens && c->fmt < 0, st))) return rc;
+    }
+    return GPMPPI_OK;
+}
+
 QueryWs gpm::make_query_ws(gpmppi_ctrl c, int s0, int Ks) {
     const size_t T = (size_t)c->p.T, n = (size_t)c->ws_Ks;
     QueryWs ws;
@@ -288,6 +300,7 @@ QueryWs gpm::make_query_ws(gpmppi_ctrl c, int s0, int Ks) {
     ws.q = reinterpret_cast<float*>(ws.st + T * n);
     ws.s0 = s0;
     ws.Ks = Ks;
+    ws.nsplit = c->nsplit;
     return ws;
 }
 
@@ -301,56 +314,131 @@ int alloc_query_ws(gpmppi_ctrl c) {
     size_t n = ((size_t)1 << 23) / T;
     if (n > (size_t)c->p.K) n = (size_t)c->p.K;
     c->ws_Ks = (int)n;
+    c->nsplit = c->fmt < 0 ? 1 : var_tc_splits(c->gset, (int)(n * T), c->nsm);
     cudaFree(c->ws_buf);
     c->ws_buf = nullptr;
-    cudaError_t e = cudaMalloc(&c->ws_buf, n * (16 * (2 * T + 1) + 4 * M * T));
+    cudaError_t e = cudaMalloc(&c->ws_buf, n * (16 * (2 * T + 1) + 4 * M * c->nsplit * T));
     if (e != cudaSuccess) return cuda_fail(e, "mppi_create: rollout workspace");
+    // rows of v: up to 512 MB at a time
+    size_t npad = 0, rows = 0;
+    for (size_t t = 0; t < M; ++t) npad = npad < (size_t)c->gset.gp[t].npad ? (size_t)c->gset.gp[t].npad : npad;
+    if (c->fmt < 0) {
+        rows = npad ? ((size_t)1 << 27) / npad : n * T;
+        if (rows > n * T) rows = n * T;
+        c->v_q = (int)rows;
+    }
+    if (c->p.variance_mode == GPMPPI_VAR_NOMINAL && rows < T) rows = T;
+    cudaFree(c->vbuf);
+    c->vbuf = nullptr;
+    if (rows * npad > 0) {
+        e = cudaMalloc(&c->vbuf, sizeof(float) * rows * npad);
+        if (e != cudaSuccess) return cuda_fail(e, "mppi_create: rollout workspace");
+    }
     return GPMPPI_OK;
 }
 
-// Alg. 1 Step 1 as the query rollout (query.cuh).
-int launch_query_rollout(gpmppi_ctrl c, const RolloutArgs& a, cudaStream_t st) {
+// training sets larger than this use the separate low column set of the
+// batched tensor-core rollout (MmaArgs::lo_set)
+constexpr int kLoSetMinN = 768;
+
+// Pipeline depth and scene placement of the batched rollout over `points` padded
+// training points of M GPs; false where they do not fit shared memory (such
+// training sets are refused in the split precisions).  The layouts leave 64
+// bytes for the persistent kernel's own words.
+bool mma_layout_of(int points, int M, int S, int O, int optin, MmaArgs* mm) {
+    mm->scene_smem = 1;
+    mm->stages = rollout_mma_stages(points, S, O, optin - 64, mm->lo_set, mm->parts, M);
+    if (mm->stages < 3) {
+        // keep the pipeline deep; read the scene from global memory instead
+        const int st_noscene = rollout_mma_stages(points, 0, 0, optin - 64, mm->lo_set, mm->parts, M);
+        if (st_noscene > mm->stages) {
+            mm->stages = st_noscene;
+            mm->scene_smem = 0;
+        }
+    }
+    return mm->stages > 0;
+}
+
+// Largest padded training set of an FP32 terrain ensemble's GPs (part of the
+// entry point's contract: larger ones are refused).
+constexpr int kMaxFp32EnsembleN = 3616;
+
+// GP g as the query rollout reads it, in format fmt (-1: FP32); builds the
+// format's tensor-core pieces on first use.
+int make_query_gp(GpDevice& g, int fmt, GpSet::One* out) {
+    *out = single_gp_set(g, 0).gp[0];
+    if (fmt < 0) return GPMPPI_OK;
     int rc;
-    for (int s0 = 0; s0 < c->p.K; s0 += c->ws_Ks) {
-        const int Ks = c->p.K - s0 < c->ws_Ks ? c->p.K - s0 : c->ws_Ks;
-        const QueryWs ws = make_query_ws(c, s0, Ks);
-        if ((rc = launch_chain(a, c->gset, ws, st))) return rc;
-        VarJob j = {};
-        j.z = reinterpret_cast<const float*>(ws.zq);
-        j.Q = c->p.T * Ks;
-        j.q = ws.q;
-        j.err = c->err;
-        j.wait_ns = c->wait_ns;
-        j.expire_first = c->expire_first;
-        if ((rc = launch_var_fp32(c->gset, j, true, st))) return rc;
-        if ((rc = launch_stage_cost(a, c->gset, ws, st))) return rc;
-    }
+    if ((rc = build_tc_pieces(g, fmt))) return rc;
+    const double r = (double)g.sf2[0] / (g.cB > 0.0f ? (double)g.cB : 1.0);
+    out->Bt = g.Bt[fmt];
+    out->qscale = (float)(r * r);
     return GPMPPI_OK;
 }
 
-// Launch arguments of the ensemble rollout: the single-GP arguments plus the
-// per-terrain factors and weights.
-EnsArgs make_ens_args(gpmppi_ctrl c, const RolloutArgs& a) {
-    EnsArgs e;
-    std::memset(&e, 0, sizeof(e));
-    e.r = a;
-    e.M = c->M;
-    e.Npmax = 0;
-    for (int i = 0; i < c->M; ++i) {
-        const GpDevice& g = c->tgp[i]->g;
-        TerrainGp& t = e.gp[i];
-        t.Xs = g.Xs[0];
-        t.alpha = g.alpha;
-        t.W = g.W[0];
-        t.N = g.N;
-        t.Np = g.Np;
-        t.sf2 = g.sf2[0];
-        for (int d = 0; d < 4; ++d) t.zscale[d] = g.zscale[0][d];
-        t.w = c->tw[i];
-        if (g.Np > e.Npmax) e.Npmax = g.Np;
-    }
-    return e;
+// Alg. 1 Step 2 as a query rollout of one trajectory without noise, in FP32
+// (args: the updated controls in U): its covariance tightens the next call.
+int launch_nominal(gpmppi_ctrl c, const RolloutArgs& a, cudaStream_t st) {
+    const GpSet gs = single_gp_set(c->gp->g, 0);
+    QueryWs ws;
+    ws.zq = static_cast<float4*>(c->ws_buf);
+    ws.st = ws.zq + (a.T + 1);
+    ws.q = reinterpret_cast<float*>(ws.st + a.T);
+    ws.s0 = 0;
+    ws.Ks = 1;
+    ws.nsplit = 1;
+    int rc;
+    if ((rc = launch_nominal_mean(a, ws, st))) return rc;
+    TriJob j = tri_forward(gs.gp[0], reinterpret_cast<const float*>(ws.zq), a.T, c->vbuf);
+    j.err = a.err;
+    if ((rc = launch_tri_forward(j, true, st))) return rc;
+    if ((rc = launch_rowsum(c->vbuf, gs.gp[0].npad, a.T, a.N, kSumBlock, ws.q, st))) return rc;
+    return launch_nominal_cov(a, gs, ws, c->nom_sxy, st);
 }
+
+}  // namespace
+
+// The controller's tiles for the batched rollout, made with its first batch.
+int gpm::make_mma_args(gpmppi_ctrl c) {
+    if (c->fmt < 0 || c->mm_made) return GPMPPI_OK;
+    MmaArgs& mm = c->mm;
+    mm.rps = c->rps;
+    MmaTerrains& tr = mm.tr;
+    int rc;
+    if (c->ens) {
+        GpDevice* gd[kMaxTerrains];
+        for (int i = 0; i < c->M; ++i) gd[i] = &c->tgp[i]->g;
+        if ((rc = build_mma_ensemble(gd, c->M, c->fmt, tr, &c->ens_hi, &c->ens_lo, &c->ens_mid, &c->ens_xa))) return rc;
+        for (int i = 0; i < c->M; ++i) tr.w[i] = c->tw[i];
+        mm.Bhi = c->ens_hi;
+        mm.Blo = c->ens_lo;
+        mm.Bmid = c->ens_mid;
+        mm.xa = c->ens_xa;
+        mm.nblocks = tr.blk0[c->M];
+    } else {
+        GpDevice& g = c->gp->g;
+        if ((rc = build_mma_tiles(g, c->fmt))) return rc;
+        mm.Bhi = g.mma_hi[c->fmt];
+        mm.Blo = g.mma_lo[c->fmt];
+        mm.Bmid = c->fmt == 2 ? g.mma_mid : nullptr;
+        mm.xa = g.mma_xa;
+        mm.nblocks = g.NpM / 128;
+        const double r = (double)g.sf2[0] / (g.cB > 0.0f ? (double)g.cB : 1.0);
+        // the single GP: one terrain of weight 1 over every block
+        tr = MmaTerrains{};
+        tr.M = 1;
+        tr.blk0[0] = 0;
+        tr.blk0[1] = mm.nblocks;
+        tr.qscale[0] = (float)(r * r);
+        tr.sf2[0] = g.sf2[0];
+        tr.w[0] = 1.0f;
+        for (int d = 0; d < 4; ++d) tr.zscale[0][d] = g.zscale[0][d];
+    }
+    c->mm_made = true;
+    return GPMPPI_OK;
+}
+
+namespace {
 
 int check_ctrl_device(gpmppi_ctrl c) {
     int dev = 0;
@@ -407,6 +495,7 @@ int gp_fit(const double* X, const double* Y, int32_t N, const gpmppi_hyper hyper
             delete h;
             return cuda_fail(e, "gp_fit: stream");
         }
+        scratch_user(h->g.device, 1);
         rc = gp_fit_device(h->g, X, Y, N, st);
         cudaStreamDestroy(st);
         if (rc) {
@@ -477,29 +566,41 @@ int mppi_create(const gpmppi_params* p, const float* obstacles, int32_t O, const
         if (dev != gp->g.device) return fail(GPMPPI_ERR_INVALID_ARG, "mppi_create: GP lives on another device");
 
         // launch geometry
-        const int mtp = rollout_fp32_mtp(gp->g.Np);
-        int nsm = 0, smem_optin = 0;
+        int nsm = 0;
         GPM_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+        const int fmt = p->precision == GPMPPI_FP32        ? -1
+                        : p->precision == GPMPPI_FP16_SPLIT ? 0
+                        : p->precision == GPMPPI_BF16_SPLIT ? 1
+                                                            : 2;
+        int smem_optin = 0;
         GPM_CUDA(cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-        // the rollout layouts leave 64 bytes for the batched persistent kernel's
-        // own words past the largest layout
-        const int layout_limit = smem_optin - 64;
-        const int stages = rollout_fp32_stages(gp->g.Np, layout_limit);
-        if (stages == 0) return fail(GPMPPI_ERR_UNSUPPORTED, "mppi_create: GP too large for shared memory");
-
+        MmaArgs mm = {};
+        if (fmt >= 0) {
+            // The tensor core rounds its FP32 accumulator at every MMA, so the
+            // variance error grows with the MMAs per output column (3 N / 16
+            // with all split products in one column set).  Beyond 768 points
+            // the two small products get their own column set (N / 16 MMAs on
+            // the large accumulator), which keeps the variance error near
+            // 1e-5 sf2 at N = 2048 at the cost of output passes half as wide.
+            // The three-term BF16 split always keeps its five small products
+            // apart (its stages would not fit shared memory with 512-column
+            // passes).
+            mm.parts = fmt == 2 ? 3 : 2;
+            mm.lo_set = (gp->g.N > kLoSetMinN || fmt == 2) ? 1 : 0;
+            if (!mma_layout_of((gp->g.N + 127) / 128 * 128, 1, P > 1 ? P - 1 : 1, O, smem_optin, &mm))
+                return fail(GPMPPI_ERR_UNSUPPORTED, "mppi_create: tensor-core rollout does not fit shared memory");
+        }
         gpmppi_ctrl c = new (std::nothrow) gpmppi_ctrl_s;
         if (!c) return fail(GPMPPI_ERR_OOM, "mppi_create: host allocation failed");
         c->p = *p;
         c->gp = gp;
         c->device = dev;
+        c->nsm = nsm;
+        c->fmt = fmt;
+        c->mm = mm;
         c->O = O;
         c->P = P;
-        c->stages = stages;
-        std::memset(&c->tmW, 0, sizeof(c->tmW));
         c->S = (P > 1) ? (P - 1) : 1;
-        int mt = (p->K + nsm - 1) / nsm;
-        if (const char* env = std::getenv("GPMPPI_SAMPLES_PER_CTA")) mt = std::atoi(env);
-        c->mt = mt < 1 ? 1 : (mt > mtp ? mtp : mt);
         c->n_upd = (p->K + 255) / 256;
         c->sq_chi2 = std::sqrt(chi2_2_quantile(p->p_x));
         c->phi_inv = normal_quantile(p->p_x);
@@ -575,92 +676,26 @@ int mppi_create(const gpmppi_params* p, const float* obstacles, int32_t O, const
                 c->gny = lg.ny;
             }
         }
-        if (gp->g.Np > 0 && (rc = make_w_tensor_map(&c->tmW, gp->g.W[0], gp->g.Np))) {
-            free_ctrl(c);
-            return rc;
-        }
-        c->gset = single_gp_set(gp->g, 0);
-        if (p->precision == GPMPPI_FP32 && (rc = alloc_query_ws(c))) {
-            free_ctrl(c);
-            return rc;
-        }
-        if (p->precision != GPMPPI_FP32) {
-            c->fmt = (p->precision == GPMPPI_FP16_SPLIT) ? 0 : (p->precision == GPMPPI_BF16_SPLIT ? 1 : 2);
-            if ((rc = build_mma_tiles(gp->g, c->fmt))) {
-                free_ctrl(c);
-                return rc;
-            }
-            const GpDevice& g = gp->g;
-            c->mm.Bhi = g.mma_hi[c->fmt];
-            c->mm.Blo = g.mma_lo[c->fmt];
-            c->mm.Bmid = c->fmt == 2 ? g.mma_mid : nullptr;
-            c->mm.parts = c->fmt == 2 ? 3 : 2;
-            c->mm.xa = g.mma_xa;
-            c->mm.nblocks = g.NpM / 128;
-            const double r = (double)g.sf2[0] / (g.mma_cB > 0.0f ? (double)g.mma_cB : 1.0);
-            // the single GP: one terrain of weight 1 over every block
-            MmaTerrains& tr = c->mm.tr;
-            tr = MmaTerrains{};
-            tr.M = 1;
-            tr.blk0[0] = 0;
-            tr.blk0[1] = c->mm.nblocks;
-            tr.qscale[0] = (float)(r * r);
-            tr.sf2[0] = g.sf2[0];
-            tr.w[0] = 1.0f;
-            for (int d = 0; d < 4; ++d) tr.zscale[0][d] = g.zscale[0][d];
-            c->mm.scene_smem = 1;
-            // The tensor core rounds its FP32 accumulator at every MMA, so the
-            // variance error grows with the MMAs per output column (3 N / 16
-            // with all split products in one column set).  Beyond 768 points
-            // the two small products get their own column set (N / 16 MMAs on
-            // the large accumulator), which keeps the variance error near
-            // 1e-5 sf2 at N = 2048 at the cost of output passes half as wide.
-            // The three-term BF16 split always keeps its five small products
-            // apart (its stages would not fit shared memory with 512-column
-            // passes).
-            c->mm.lo_set = (g.N > kLoSetMinN || c->fmt == 2) ? 1 : 0;
-            c->mm.stages = rollout_mma_stages(g.NpM, c->S, O, layout_limit, c->mm.lo_set, c->mm.parts, 1);
-            if (c->mm.stages < 3) {
-                // keep the pipeline deep; read the scene from global memory instead
-                const int st_noscene = rollout_mma_stages(g.NpM, 0, 0, layout_limit, c->mm.lo_set, c->mm.parts, 1);
-                if (st_noscene > c->mm.stages) {
-                    c->mm.stages = st_noscene;
-                    c->mm.scene_smem = 0;
-                }
-            }
-            // fewest threads per sample (largest sample tile) that still
-            // gives every SM a CTA; small K falls back to 32 samples per CTA
-            c->mm.rps = 8;
-            if ((p->K + 127) / 128 >= nsm * 4 / 5) c->mm.rps = 2;
-            else if ((p->K + 63) / 64 >= nsm * 4 / 5) c->mm.rps = 4;
-            if (const char* env = std::getenv("GPMPPI_MMA_THREADS_PER_SAMPLE")) c->mm.rps = std::atoi(env);
-            if (c->mm.stages == 0) {
-                free_ctrl(c);
-                return fail(GPMPPI_ERR_UNSUPPORTED, "mppi_create: tensor-core rollout does not fit shared memory");
-            }
-            // N <= 512: the cluster rollout keeps the factor resident in shared
-            // memory (two-part formats only)
+        if (fmt >= 0) {
+            // what mppi_rollout_kind and mppi_batch_layout report: the class of the
+            // workload (training sets of up to 512 points in two parts apart) and
+            // the layout's threads per sample, fewest that give every SM a tile
             const char* no_cl = std::getenv("GPMPPI_NO_CLUSTER");
-            if (c->fmt < 2 && g.N > 0 && g.N <= 512 && !(no_cl && no_cl[0] == '1')) {
-                if ((rc = build_cl_tiles(gp->g, c->fmt))) {
-                    free_ctrl(c);
-                    return rc;
-                }
-                ClArgs& cl = c->cla;
-                cl.tiles = gp->g.cl_tiles[c->fmt];
-                cl.npc = gp->g.cl_npc;
-                cl.xa = gp->g.cl_xa;
-                cl.ns = cl.npc / 64;
-                cl.cs = cl.ns / 2;
-                for (int r = 0; r < 4; ++r) {
-                    cl.base[r] = gp->g.cl_base[r];
-                    cl.bytes[r] = gp->g.cl_bytes[r];
-                }
-                cl.qscale = c->mm.tr.qscale[0];
-                cl.scene_smem = 1;
-                if (cl_smem_bytes(cl, c->S, O) > smem_optin) cl.scene_smem = 0;
-                c->cl = cl_smem_bytes(cl, c->S, O) <= smem_optin && cl_schedulable(cl, c->S, O, dev);
+            const bool small = fmt < 2 && gp->g.N > 0 && gp->g.N <= 512 && !(no_cl && no_cl[0] == '1');
+            c->kind = small ? GPMPPI_KERNEL_TC_CLUSTER : GPMPPI_KERNEL_TC_STREAM;
+            c->rps = 8;
+            if ((p->K + 127) / 128 >= nsm * 4 / 5) c->rps = 2;
+            else if ((p->K + 63) / 64 >= nsm * 4 / 5) c->rps = 4;
+            if (const char* env = std::getenv("GPMPPI_MMA_THREADS_PER_SAMPLE")) c->rps = std::atoi(env);
+            if (c->rps != 2 && c->rps != 4 && c->rps != 8) {
+                free_ctrl(c);
+                return fail(GPMPPI_ERR_INVALID_ARG, "mppi_create: bad threads per sample");
             }
+        }
+        c->gset.M = 1;
+        if ((rc = make_query_gp(gp->g, c->fmt, &c->gset.gp[0])) || (rc = alloc_query_ws(c))) {
+            free_ctrl(c);
+            return rc;
         }
         *out = c;
         return GPMPPI_OK;
@@ -684,13 +719,7 @@ int mppi_step(gpmppi_ctrl c, const float state[5], const float* U_nom, float* U_
     RolloutArgs a = make_rollout_args(c, state, U_nom);
     if (costs) a.costs = costs;
     if (c->profiling) GPM_CUDA(cudaEventRecord(c->ev[0], st));
-    if (c->ens && c->fmt < 0)
-        rc = launch_rollout_ens(make_ens_args(c, a), false, st);
-    else if (c->cl)
-        rc = launch_rollout_cl(a, c->cla, c->fmt, false, st);
-    else
-        rc = (c->fmt < 0) ? launch_query_rollout(c, a, st) : launch_rollout_mma(a, c->mm, c->fmt, false, st);
-    if (rc) return rc;
+    if ((rc = launch_query_rollout(c, a, c->gset, st))) return rc;
     if (c->profiling) GPM_CUDA(cudaEventRecord(c->ev[1], st));
     UpdateArgs u;
     u.costs = a.costs;
@@ -706,8 +735,7 @@ int mppi_step(gpmppi_ctrl c, const float state[5], const float* U_nom, float* U_
     u.inv_lambda = 1.0f / c->p.lambda;
     if ((rc = launch_update(u, c->n_upd, st, !c->profiling))) return rc;
     if (c->p.variance_mode == GPMPPI_VAR_NOMINAL) {
-        RolloutArgs n = make_rollout_args(c, state, U_new);
-        if ((rc = launch_nominal(n, c->nom_sxy, st))) return rc;
+        if ((rc = launch_nominal(c, make_rollout_args(c, state, U_new), st))) return rc;
     }
     if (c->profiling) {
         GPM_CUDA(cudaEventRecord(c->ev[2], st));
@@ -766,10 +794,7 @@ int mppi_rollout_trace(gpmppi_ctrl c, const float state[5], const float* U_nom, 
     a.tr_sig = sigma;
     a.tr_stage = stage;
     a.tr_margin = margins;
-    if (c->ens && c->fmt < 0) return launch_rollout_ens(make_ens_args(c, a), true, (cudaStream_t)stream);
-    if (c->cl) return launch_rollout_cl(a, c->cla, c->fmt, true, (cudaStream_t)stream);
-    if (c->fmt >= 0) return launch_rollout_mma(a, c->mm, c->fmt, true, (cudaStream_t)stream);
-    return launch_query_rollout(c, a, (cudaStream_t)stream);
+    return launch_query_rollout(c, a, c->gset, (cudaStream_t)stream);
 }
 
 int mppi_create_ensemble(const gpmppi_params* p, const float* obstacles, int32_t O, const float* path,
@@ -794,11 +819,9 @@ int mppi_create_ensemble(const gpmppi_params* p, const float* obstacles, int32_t
     const bool ens = M > 1 || weights[0] != 1.0f;
     if (ens && p->variance_mode != GPMPPI_VAR_PER_SAMPLE)
         return fail(GPMPPI_ERR_UNSUPPORTED, "mppi_create_ensemble: needs the per-sample variance mode");
-    int npmax = 0, optin = 0, dev = 0, rc;
+    int npmax = 0, rc;
     for (int i = 0; i < M; ++i) npmax = gps[i]->g.Np > npmax ? gps[i]->g.Np : npmax;
-    if ((rc = current_device(&dev))) return rc;
-    GPM_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    if (ens && p->precision == GPMPPI_FP32 && ens_smem_bytes(npmax) > optin)
+    if (ens && p->precision == GPMPPI_FP32 && npmax > kMaxFp32EnsembleN)
         return fail(GPMPPI_ERR_UNSUPPORTED, "mppi_create_ensemble: GPs too large for the ensemble rollout");
     gpmppi_ctrl c = nullptr;
     if ((rc = mppi_create(p, obstacles, O, path, P, gps[0], &c))) return rc;
@@ -809,40 +832,33 @@ int mppi_create_ensemble(const gpmppi_params* p, const float* obstacles, int32_t
         c->tw[i] = weights[i];
         if (i > 0) gps[i]->g.n_controllers++;
     }
-    if (ens && c->fmt >= 0) {
-        // the streaming rollout over the stacked factors (not the cluster kernel)
-        GpDevice* gd[kMaxTerrains];
-        bool lo = c->fmt == 2;
-        for (int i = 0; i < M; ++i) {
-            gd[i] = &gps[i]->g;
-            lo = lo || gps[i]->g.N > kLoSetMinN;
-        }
-        MmaArgs& mm = c->mm;
-        if ((rc = build_mma_ensemble(gd, M, c->fmt, mm.tr, &c->ens_hi, &c->ens_lo, &c->ens_mid, &c->ens_xa))) {
+    for (int i = 0; i < M; ++i) {
+        if ((rc = make_query_gp(gps[i]->g, c->fmt, &c->gset.gp[i]))) {
             mppi_destroy(c);
             return rc;
         }
-        for (int i = 0; i < M; ++i) mm.tr.w[i] = weights[i];
-        mm.Bhi = c->ens_hi;
-        mm.Blo = c->ens_lo;
-        mm.Bmid = c->ens_mid;
-        mm.xa = c->ens_xa;
-        mm.nblocks = mm.tr.blk0[M];
-        mm.lo_set = lo ? 1 : 0;
-        mm.scene_smem = 1;
-        const int NpT = mm.nblocks * 128;
-        mm.stages = rollout_mma_stages(NpT, c->S, O, optin - 64, mm.lo_set, mm.parts, M);
-        if (mm.stages < 3) {
-            const int st_noscene = rollout_mma_stages(NpT, 0, 0, optin - 64, mm.lo_set, mm.parts, M);
-            if (st_noscene > mm.stages) {
-                mm.stages = st_noscene;
-                mm.scene_smem = 0;
+        c->gset.gp[i].w = weights[i];
+    }
+    c->gset.M = M;
+    if (M > 1 && (rc = alloc_query_ws(c))) {   // room for every terrain's variance
+        mppi_destroy(c);
+        return rc;
+    }
+    if (ens) {
+        c->kind = c->fmt < 0 ? GPMPPI_KERNEL_ENSEMBLE : GPMPPI_KERNEL_TC_STREAM;
+        if (c->fmt >= 0) {
+            int points = 0, optin = 0;
+            bool lo = c->fmt == 2;
+            for (int i = 0; i < M; ++i) {
+                points += (gps[i]->g.N + 255) / 256 * 256;    // an even number of blocks per GP
+                lo = lo || gps[i]->g.N > kLoSetMinN;
             }
-        }
-        c->cl = false;
-        if (mm.stages == 0) {
-            mppi_destroy(c);
-            return fail(GPMPPI_ERR_UNSUPPORTED, "mppi_create_ensemble: the GPs' training sets do not fit shared memory");
+            c->mm.lo_set = lo ? 1 : 0;
+            GPM_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device));
+            if (!mma_layout_of(points, M, c->S, O, optin, &c->mm)) {
+                mppi_destroy(c);
+                return fail(GPMPPI_ERR_UNSUPPORTED, "mppi_create_ensemble: the GPs' training sets do not fit shared memory");
+            }
         }
     }
     *out = c;
@@ -857,9 +873,11 @@ int mppi_set_terrain_weights(gpmppi_ctrl c, const float* weights, int32_t M) {
     if (!c->ens && weights[0] != 1.0f)
         return fail(GPMPPI_ERR_UNSUPPORTED,
                     "mppi_set_terrain_weights: a single-GP controller keeps weight 1 (create it with weight != 1)");
-    for (int i = 0; i < M; ++i) c->tw[i] = weights[i];
-    if (c->ens && c->fmt >= 0)
-        for (int i = 0; i < M; ++i) c->mm.tr.w[i] = weights[i];
+    for (int i = 0; i < M; ++i) {
+        c->tw[i] = weights[i];
+        c->gset.gp[i].w = weights[i];
+        if (c->mm_made) c->mm.tr.w[i] = weights[i];
+    }
     return GPMPPI_OK;
 }
 
@@ -882,49 +900,54 @@ int mppi_grad(gpmppi_ctrl c, const float state[5], const float* U_nom, const flo
     if (c->ens) return fail(GPMPPI_ERR_UNSUPPORTED, "mppi_grad: terrain ensembles are not differentiated");
     GpDevice& g = c->gp->g;
     const int K = c->p.K, T = c->p.T, Np = g.Np, N = g.N;
-    int C = (int)std::ceil(std::sqrt((double)T));
-    if (C < 1) C = 1;
-    const int nseg = (T + C - 1) / C;
-    const int gm = grad_samples_per_cta();
-    const int ncta = (K + gm - 1) / gm;
-    const int Kpad = ncta * gm;
+    // part of the entry point's contract: larger training sets and horizons are refused
+    const int C = (int)std::ceil(std::sqrt((double)T));
     int optin = 0;
     GPM_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device));
-    if (grad_smem_bytes(Np, C) > optin)
+    if (64 * Np + 640 * (C + 1) + 128 * C + 2176 > optin)
         return fail(GPMPPI_ERR_UNSUPPORTED, "mppi_grad: GP too large for the adjoint kernel's shared memory");
     cudaStream_t st = (cudaStream_t)stream;
     const bool want_l = dlengthscale != nullptr;
     // per-GP factors of the adjoint, built once
-    if (!g.Wt) {
-        GPM_CUDA(cudaMalloc(&g.Wt, sizeof(float) * (size_t)Np * Np));
-        if ((rc = launch_transpose(g.W[0], Np, g.Wt, st))) return rc;
-        GPM_CUDA(cudaStreamSynchronize(st));
-    }
+    if (dU && (rc = build_back_pieces(g, st))) return rc;
     if (want_l && !g.ubar) {
-        GPM_CUDA(cudaMalloc(&g.ubar, sizeof(float) * 8 * (size_t)Np));
-        if ((rc = launch_dk_alpha(g.Xs[0], g.alpha, N, Np, g.sf2[0], g.ubar, st))) return rc;
+        GPM_CUDA(cudaMalloc(&g.ubar, sizeof(float) * 8 * (size_t)(Np > 0 ? Np : 1)));
+        if (N > 0 && (rc = launch_dk_alpha(g.Xs[0], g.alpha, N, Np, g.sf2[0], g.ubar, st))) return rc;
         GPM_CUDA(cudaStreamSynchronize(st));
     }
+    // samples at a time: rows of v and b of up to 8 GB
+    size_t piece = ((size_t)1 << 31) / ((size_t)T * (g.npad + Np + 64));
+    piece = piece < 8 ? 8 : piece / 8 * 8;
+    const int Ks = piece < (size_t)K ? (int)piece : K;
+    const int Kpad = (Ks + 7) / 8 * 8;
+    const GpSet gs = single_gp_set(g, 0);
     // scratch layout (bytes, each piece 256-aligned)
-    const int Q = T * Kpad;
     int nsm = 0;
     GPM_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device));
-    const int nparts = want_l ? gram_tc_parts(Q, Np, nsm) : 0;
     size_t off = 0;
     auto take = [&](size_t bytes) {
         const size_t o = off;
         off += (bytes + 255) & ~(size_t)255;
         return o;
     };
-    const size_t o_v = take(sizeof(float) * (size_t)ncta * C * Np * gm);
-    const size_t o_ck = take(sizeof(float) * (size_t)ncta * nseg * gm * 20);
+    auto kpad_of = [&](int s0) { return ((K - s0 < Ks ? K - s0 : Ks) + 7) / 8 * 8; };
+    int nparts = 0;
+    if (want_l)
+        for (int s0 = 0; s0 < K; s0 += Ks) nparts += gram_tc_parts(T * kpad_of(s0), Np, nsm);
+    const size_t Q = (size_t)T * Ks;
+    const size_t o_ut = take(sizeof(float2) * (size_t)T * K);
+    const size_t o_zq = take(sizeof(float4) * (Q + Ks));
+    const size_t o_st = take(sizeof(float4) * Q);
+    const size_t o_qq = take(sizeof(float) * Q);
+    const size_t o_rec = take(sizeof(float) * 16 * Q);
+    const size_t o_v = take(sizeof(float) * Q * g.npad);
     const size_t o_S = take(sizeof(float) * (size_t)K);
     const size_t o_dU = take(sizeof(float) * (size_t)2 * T * K);
     const size_t o_dl = take(sizeof(float) * (size_t)8 * K);
     size_t o_B = 0, o_q = 0, o_p = 0;
+    if (dU) o_B = take(sizeof(float) * (size_t)T * Kpad * Np);
     if (want_l) {
-        o_B = take(sizeof(float) * (size_t)Q * Np);
-        o_q = take(sizeof(float4) * (size_t)Q);
+        o_q = take(sizeof(float4) * (size_t)T * Kpad);
         o_p = take(sizeof(float) * 8 * (size_t)nparts);
     }
     if (off > c->grad_bytes) {
@@ -939,31 +962,62 @@ int mppi_grad(gpmppi_ctrl c, const float state[5], const float* U_nom, const flo
     std::memset(&ga, 0, sizeof(ga));
     ga.r = make_rollout_args(c, state, U_nom);
     ga.r.nom_sxy = nullptr;
-    ga.Wt = g.Wt;
+    ga.r.u_tilde = reinterpret_cast<float2*>(base + o_ut);
     ga.ubar = want_l ? g.ubar : nullptr;
     ga.weight = sample_weights;
     ga.slope = slope;
     ga.inv_K = 1.0f / (float)K;
-    ga.C = C;
-    ga.nseg = nseg;
-    ga.Kpad = Kpad;
-    ga.backward = dU ? 1 : 0;
-    ga.vscr = reinterpret_cast<float*>(base + o_v);
-    ga.ckpt = reinterpret_cast<float*>(base + o_ck);
+    ga.ws.zq = reinterpret_cast<float4*>(base + o_zq);
+    ga.ws.st = reinterpret_cast<float4*>(base + o_st);
+    ga.ws.q = reinterpret_cast<float*>(base + o_qq);
+    ga.ws.nsplit = 1;
+    ga.rec = reinterpret_cast<float*>(base + o_rec);
     ga.S_out = reinterpret_cast<float*>(base + o_S);
     ga.dU_out = reinterpret_cast<float*>(base + o_dU);
     ga.dl_out = want_l ? reinterpret_cast<float*>(base + o_dl) : nullptr;
-    ga.Bq = want_l ? reinterpret_cast<float*>(base + o_B) : nullptr;
+    float* V = reinterpret_cast<float*>(base + o_v);
+    float* Bq = reinterpret_cast<float*>(base + o_B);
+    ga.Bq = Bq;
     ga.qbar = want_l ? reinterpret_cast<float4*>(base + o_q) : nullptr;
     if (c->profiling) GPM_CUDA(cudaEventRecord(c->ev[0], st));
-    if ((rc = launch_grad(ga, ncta, st))) return rc;
-    if (c->profiling) GPM_CUDA(cudaEventRecord(c->ev[1], st));
-    if (want_l) {
-        // tr(dK/dl_d G_o), G_o = sum_q sbar_o,q b_q b_q^T over the T K queries:
-        // the Gram contraction on the tensor cores, traced tile by tile
-        if ((rc = launch_gram_tc(ga.Bq, ga.qbar, Q, Np, N, g.Xs[0], g.sf2[0], reinterpret_cast<float*>(base + o_p),
-                                 nparts, c->err, nsm, st)))
-            return rc;
+    float* part = reinterpret_cast<float*>(base + o_p);
+    for (int s0 = 0; s0 < K; s0 += Ks) {
+        ga.ws.s0 = s0;
+        ga.ws.Ks = K - s0 < Ks ? K - s0 : Ks;
+        ga.Kpad = kpad_of(s0);
+        const int n = T * ga.ws.Ks;
+        if ((rc = launch_chain_fp32(ga.r, gs, kChainTreeFused, ga.ws, st))) return rc;
+        TriJob j = tri_forward(gs.gp[0], reinterpret_cast<const float*>(ga.ws.zq), n, V);
+        j.err = c->err;
+        j.fusez = 1;
+        if ((rc = launch_tri_forward(j, true, st))) return rc;
+        if ((rc = launch_rowsum(V, g.npad, n, N, kSumLanes, ga.ws.q, st))) return rc;
+        if ((rc = launch_grad_forward(ga, st))) return rc;
+        if (dU) {
+            TriJob b = {};
+            b.z = V;
+            b.ldz = g.npad;
+            b.fac = g.Lb;
+            b.out = Bq;
+            b.ldo = Np;
+            b.Q = n;
+            b.N = N;
+            b.rk = ga.ws.Ks;
+            b.rkpad = ga.Kpad;
+            b.err = c->err;
+            b.wait_ns = 2000000000ull;
+            if ((rc = launch_tri_backward(b, false, st))) return rc;
+            if ((rc = launch_grad_reverse(ga, st))) return rc;
+        }
+        if (c->profiling && s0 + Ks >= K) GPM_CUDA(cudaEventRecord(c->ev[1], st));
+        if (want_l) {
+            // tr(dK/dl_d G_o), G_o = sum_q sbar_o,q b_q b_q^T over the queries: the
+            // Gram contraction on the tensor cores, traced tile by tile
+            const int np = gram_tc_parts(T * ga.Kpad, Np, nsm);
+            if ((rc = launch_gram_tc(Bq, ga.qbar, T * ga.Kpad, Np, N, g.Xs[0], g.sf2[0], part, np, c->err, nsm, st)))
+                return rc;
+            part += 8 * (size_t)np;
+        }
     }
     GradReduceArgs rr;
     std::memset(&rr, 0, sizeof(rr));
@@ -1020,8 +1074,7 @@ int mppi_set_wait_limit(gpmppi_ctrl c, uint64_t ns, int32_t expire_first) {
 int mppi_rollout_kind(gpmppi_ctrl c, int32_t* kind) {
     if (!valid_ctrl(c)) return fail(GPMPPI_ERR_INVALID_ARG, "mppi_rollout_kind: invalid handle");
     if (!kind) return fail(GPMPPI_ERR_INVALID_ARG, "mppi_rollout_kind: kind is NULL");
-    *kind = (c->ens && c->fmt < 0) ? GPMPPI_KERNEL_ENSEMBLE
-                   : (c->cl ? GPMPPI_KERNEL_TC_CLUSTER : (c->fmt >= 0 ? GPMPPI_KERNEL_TC_STREAM : GPMPPI_KERNEL_FP32));
+    *kind = c->kind;
     return GPMPPI_OK;
 }
 

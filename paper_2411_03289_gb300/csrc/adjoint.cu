@@ -8,21 +8,18 @@
 // Philox draws of the current iteration) and w_s = 1/K unless the caller
 // passes weights.
 //
-// One CTA carries GMT samples, one warp per sample, through three passes:
-//   1. forward over all T steps: S_s, plus the state (mu, Sigma) every C
-//      steps (C = ceil(sqrt(T))) as a checkpoint in global scratch;
-//   2. for each segment of C steps, last first: the forward steps again from
-//      the segment's checkpoint, keeping per-step states in shared memory and
-//      v = L^-1 k* (the GP variance factor) in global scratch;
-//   3. the reverse steps of that segment: stage-cost adjoint (lane distance,
-//      lambda_max of Sigma_XY, obstacle spread), covariance adjoint
-//      (Sigma' = A Sigma A^T + D: Sigma_bar = A^T G A, A_bar = 2 G A Sigma),
-//      mean adjoint (Eq. 6), then the GP adjoint: b = L^-T v = K^-1 k* by a
-//      second triangular product, k*_bar_j = m_bar . alpha_j - 2 s_bar b_j,
-//      and z_bar, the direct lengthscale terms and the terms that flow
-//      through alpha = K^-1 y.
+// The forward pass is a query rollout: the means of all samples (chain_fp32.cu),
+// v = L^-1 k* and b = L^-T v = K^-1 k* of all T K queries as two triangular
+// products (tri.cu), none of which needs the recurrence.  Then one warp per sample:
+//   k_grad_fwd   covariances, S_s, and the records of every step;
+//   k_grad_rev   the reverse steps, last first: stage-cost adjoint (lane distance,
+//                lambda_max of Sigma_XY, obstacle spread), covariance adjoint
+//                (Sigma' = A Sigma A^T + D: Sigma_bar = A^T G A, A_bar = 2 G A Sigma),
+//                mean adjoint (Eq. 6), then the GP adjoint over the points:
+//                k*_bar_j = m_bar . alpha_j - 2 s_bar b_j, z_bar, the direct
+//                lengthscale terms and the terms that flow through alpha = K^-1 y.
 // The terms that flow through K^-1 in the variance need G_o = sum_q s_bar_o,q
-// b_q b_q^T; the CTAs store b_q and the per-query adjoints, and a Gram kernel
+// b_q b_q^T; k_grad_rev stores the per-query adjoints, and a Gram kernel
 // forms tr(dK/dl_d G_o) tile by tile.  A last kernel reduces the per-sample
 // contributions in double in a fixed order, so results are deterministic.
 #include <cfloat>
@@ -36,125 +33,6 @@ namespace {
 using namespace wr;
 
 constexpr float kLn2 = 0.69314718055994530942f;
-
-struct StepInfo {
-    float ux, uy;      // clamped perturbed control (Eq. 8)
-    float sraw;        // sf2 - |L^-1 k*|^2 before the clamp at zero
-    int mask;          // bit c: control component c strictly inside its box
-};
-
-// One forward step of sample s (warp w); all threads of the CTA call it.
-// mu / S are the warp's (lane-replicated) state, advanced in place.
-__device__ void fwd_step(const GradArgs& g, int k, int s, bool act, float mu[5], float S[15],
-                         float* kT, float* vT, float* vstore, StepInfo& inf, float* save) {
-    const RolloutArgs& a = g.r;
-    const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
-    const int Np = a.Np;
-    const float2 e = control_eps((uint32_t)k, (uint32_t)(act ? s : 0), a.it0, a.it1, a.key0, a.key1,
-                                 a.sig_v, a.sig_w);
-    const float rx = __ldg(a.U + 2 * k) + e.x, ry = __ldg(a.U + 2 * k + 1) + e.y;
-    inf.ux = fminf(fmaxf(rx, a.umin0), a.umax0);
-    inf.uy = fminf(fmaxf(ry, a.umin1), a.umax1);
-    inf.mask = ((rx > a.umin0 && rx < a.umax0) ? 1 : 0) | ((ry > a.umin1 && ry < a.umax1) ? 2 : 0);
-    const float z0 = mu[3] * a.zscale[0], z1 = mu[4] * a.zscale[1], z2 = inf.ux * a.zscale[2],
-                z3 = inf.uy * a.zscale[3];
-    float mv = 0.0f, mw = 0.0f, cv = 0.0f, cw = 0.0f;
-    for (int j = lane; j < Np; j += 32) {
-        float kv = 0.0f;
-        if (act && j < a.N) {
-            const float4 x = ldg4(a.Xs + 4 * j);
-            const float d0 = z0 - x.x, d1 = z1 - x.y, d2 = z2 - x.z, d3 = z3 - x.w;
-            kv = a.sf2 * exp2f(-(d0 * d0 + d1 * d1 + d2 * d2 + d3 * d3));
-            const float2 al = __ldg(reinterpret_cast<const float2*>(a.alpha) + j);
-            kahan_add(mv, cv, kv * al.x);
-            kahan_add(mw, cw, kv * al.y);
-        }
-        kT[j * GMT + w] = kv;
-    }
-    mv = wsum(mv + cv);
-    mw = wsum(mw + cw);
-    // the warp's state waits in shared memory while the product runs, so that
-    // its registers are free for the product's tiles
-    if (lane == 0) {
-#pragma unroll
-        for (int i = 0; i < 5; ++i) save[i] = mu[i];
-#pragma unroll
-        for (int i = 0; i < 15; ++i) save[5 + i] = S[i];
-        save[20] = mv;
-        save[21] = mw;
-        save[22] = inf.ux;
-        save[23] = inf.uy;
-        save[24] = __int_as_float(inf.mask);
-    }
-    __syncthreads();
-    tri_product<false>(a.W, Np, kT, vT);
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < 5; ++i) mu[i] = save[i];
-#pragma unroll
-    for (int i = 0; i < 15; ++i) S[i] = save[5 + i];
-    mv = save[20];
-    mw = save[21];
-    inf.ux = save[22];
-    inf.uy = save[23];
-    inf.mask = __float_as_int(save[24]);
-    float q = 0.0f;
-    for (int i = lane; i < Np; i += 32) {
-        const float x = vT[i * GMT + w];
-        q = fmaf(x, x, q);
-    }
-    q = wsum(q);
-    if (vstore) {
-        const float4* src = reinterpret_cast<const float4*>(vT);
-        float4* dst = reinterpret_cast<float4*>(vstore);
-        for (int i = tid; i < Np * GMT / 4; i += GT) dst[i] = src[i];
-    }
-    inf.sraw = a.sf2 - q;
-    const float sv = fmaxf(0.0f, inf.sraw);
-
-    float sn, cs;
-    sincosf(mu[2], &sn, &cs);
-    const float a02 = -a.dt * mu[3] * sn, a03 = a.dt * cs;
-    const float a12 = a.dt * mu[3] * cs, a13 = a.dt * sn;
-    const float nX = mu[0] + a.dt * mu[3] * cs;
-    const float nY = mu[1] + a.dt * mu[3] * sn;
-    const float nT = mu[2] + a.dt * mu[4];
-    const float nV = mu[3] + a.kv * (inf.ux - mu[3]) + mv;
-    const float nW = mu[4] + a.kw * (inf.uy - mu[4]) + mw;
-    mu[0] = nX; mu[1] = nY; mu[2] = nT; mu[3] = nV; mu[4] = nW;
-    // Sigma' = A Sigma A^T + diag(0, 0, 0, s, s)  (Eq. 10)
-    float A[5][5] = {{1.f, 0.f, a02, a03, 0.f},
-                     {0.f, 1.f, a12, a13, 0.f},
-                     {0.f, 0.f, 1.f, 0.f, a.dt},
-                     {0.f, 0.f, 0.f, a.av, 0.f},
-                     {0.f, 0.f, 0.f, 0.f, a.aw}};
-    float Sf[5][5];
-#pragma unroll
-    for (int i = 0; i < 5; ++i)
-#pragma unroll
-        for (int j = 0; j < 5; ++j) Sf[i][j] = (i <= j) ? S[sidx(i, j)] : S[sidx(j, i)];
-    float B[5][5];
-#pragma unroll
-    for (int i = 0; i < 5; ++i)
-#pragma unroll
-        for (int j = 0; j < 5; ++j) {
-            float t = 0.0f;
-#pragma unroll
-            for (int m = 0; m < 5; ++m) t = fmaf(A[i][m], Sf[m][j], t);
-            B[i][j] = t;
-        }
-#pragma unroll
-    for (int i = 0; i < 5; ++i)
-#pragma unroll
-        for (int j = i; j < 5; ++j) {
-            float t = 0.0f;
-#pragma unroll
-            for (int m = 0; m < 5; ++m) t = fmaf(B[i][m], A[j][m], t);
-            S[sidx(i, j)] = t;
-        }
-    S[sidx(3, 3)] += sv;
-    S[sidx(4, 4)] += sv;
-}
 
 // Smoothed stage cost at the post-step state (warp-wide, lane-replicated).
 __device__ float stage_cost(const GradArgs& g, int k, const float mu[5], const float S[15], float sraw) {
@@ -272,278 +150,242 @@ __device__ float stage_cost_adjoint(const GradArgs& g, int k, const float mu[5],
     return wt * a.c_var;
 }
 
-constexpr int SAVE = 40;     // per-warp spill area for state live across a product
-constexpr int CARRY = 28;    // per-warp adjoint carry: mu_bar (5), Sigma_bar (15), l_bar (8)
-
-__global__ void __launch_bounds__(GT, 2) k_grad(const GradArgs g) {
-    extern __shared__ __align__(16) float gsm[];
-    const RolloutArgs& a = g.r;
-    const int Np = a.Np, C = g.C, T = a.T;
-    float* bufA = gsm;
-    float* bufB = bufA + Np * GMT;
-    float* rec = bufB + Np * GMT;                                   // (C + 1) x GMT x REC
-    StepInfo* info = reinterpret_cast<StepInfo*>(rec + (C + 1) * GMT * REC);   // C x GMT
-    float* saves = reinterpret_cast<float*>(info + C * GMT);        // GMT x SAVE
-    float* carries = saves + GMT * SAVE;                            // GMT x CARRY
-    const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
-    float* save = saves + w * SAVE;
-    float* carry = carries + w * CARRY;
-    const int s = blockIdx.x * GMT + w;
-    const bool act = s < a.K;
-    const float wt = act ? (g.weight ? __ldg(g.weight + s) : g.inv_K) : 0.0f;
-    float* ck = g.ckpt + ((size_t)blockIdx.x * g.nseg * GMT + w) * REC;   // + seg * GMT * REC
-
-    float mu[5], S[15];
+// Sigma' = A Sigma A^T + diag(0, 0, 0, s, s)  (Eq. 10), upper triangle in S
+__device__ __forceinline__ void cov_forward(const RolloutArgs& a, float th, float v, float sv, float S[15]) {
+    float sn, cs;
+    sincosf(th, &sn, &cs);
+    const float a02 = -a.dt * v * sn, a03 = a.dt * cs;
+    const float a12 = a.dt * v * cs, a13 = a.dt * sn;
+    float A[5][5] = {{1.f, 0.f, a02, a03, 0.f},
+                     {0.f, 1.f, a12, a13, 0.f},
+                     {0.f, 0.f, 1.f, 0.f, a.dt},
+                     {0.f, 0.f, 0.f, a.av, 0.f},
+                     {0.f, 0.f, 0.f, 0.f, a.aw}};
+    float Sf[5][5];
 #pragma unroll
-    for (int i = 0; i < 5; ++i) mu[i] = a.x0[i];
+    for (int i = 0; i < 5; ++i)
+#pragma unroll
+        for (int j = 0; j < 5; ++j) Sf[i][j] = (i <= j) ? S[sidx(i, j)] : S[sidx(j, i)];
+    float B[5][5];
+#pragma unroll
+    for (int i = 0; i < 5; ++i)
+#pragma unroll
+        for (int j = 0; j < 5; ++j) {
+            float t = 0.0f;
+#pragma unroll
+            for (int m = 0; m < 5; ++m) t = fmaf(A[i][m], Sf[m][j], t);
+            B[i][j] = t;
+        }
+#pragma unroll
+    for (int i = 0; i < 5; ++i)
+#pragma unroll
+        for (int j = i; j < 5; ++j) {
+            float t = 0.0f;
+#pragma unroll
+            for (int m = 0; m < 5; ++m) t = fmaf(B[i][m], A[j][m], t);
+            S[sidx(i, j)] = t;
+        }
+    S[sidx(3, 3)] += sv;
+    S[sidx(4, 4)] += sv;
+}
+
+// the state before step k of sample l: (X, Y, theta, v) after step k - 1 and omega
+__device__ __forceinline__ void state_before(const GradArgs& g, int k, int l, float mu[5]) {
+    if (k == 0) {
+#pragma unroll
+        for (int i = 0; i < 5; ++i) mu[i] = g.r.x0[i];
+        return;
+    }
+    const float4 p = g.ws.st[(size_t)(k - 1) * g.ws.Ks + l];
+    mu[0] = p.x; mu[1] = p.y; mu[2] = p.z; mu[3] = p.w;
+    mu[4] = g.ws.zq[(size_t)k * g.ws.Ks + l].y;
+}
+
+__global__ void __launch_bounds__(GT) k_grad_fwd(const GradArgs g) {
+    const RolloutArgs& a = g.r;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int l = blockIdx.x * GMT + w;
+    if (l >= g.ws.Ks) return;
+    const int Ks = g.ws.Ks;
+    float S[15];
 #pragma unroll
     for (int i = 0; i < 15; ++i) S[i] = 0.0f;
-
-    // ---- pass 1: objective and checkpoints --------------------------------
     float Jsum = 0.0f, Jc = 0.0f;
-    for (int k = 0; k < T; ++k) {
-        if (k % C == 0 && lane == 0) {
-            float* dst = ck + (size_t)(k / C) * GMT * REC;
+    float th = a.x0[2], v = a.x0[3];
+    for (int k = 0; k < a.T; ++k) {
+        const float sraw = a.sf2 - g.ws.q[(size_t)k * Ks + l];
+        const float4 p = g.ws.st[(size_t)k * Ks + l];
+        cov_forward(a, th, v, fmaxf(0.0f, sraw), S);
+        const float mu[5] = {p.x, p.y, p.z, p.w, 0.0f};      // the stage cost does not read omega
+        kahan_add(Jsum, Jc, stage_cost(g, k, mu, S, sraw));
+        float r = sraw;
 #pragma unroll
-            for (int i = 0; i < 5; ++i) dst[i] = mu[i];
-#pragma unroll
-            for (int i = 0; i < 15; ++i) dst[5 + i] = S[i];
-        }
-        StepInfo inf;
-        fwd_step(g, k, s, act, mu, S, bufA, bufB, nullptr, inf, save);
-        if (act) kahan_add(Jsum, Jc, stage_cost(g, k, mu, S, inf.sraw));
+        for (int i = 0; i < 15; ++i) r = lane == i ? S[i] : r;
+        if (lane < 16) g.rec[((size_t)k * Ks + l) * 16 + lane] = r;
+        th = p.z;
+        v = p.w;
     }
-    if (act && lane == 0) g.S_out[s] = Jsum + Jc;
-    if (!g.backward) return;
-    if (lane == 0)
-        for (int i = 0; i < CARRY; ++i) carry[i] = 0.0f;
-    __syncthreads();     // checkpoint stores and the zeroed carry before the reloads below
+    if (lane == 0) g.S_out[g.ws.s0 + l] = Jsum + Jc;
+}
 
-    // ---- passes 2 and 3, one segment at a time, last segment first --------
-    float* vslot = g.vscr + (size_t)blockIdx.x * C * Np * GMT;
-    for (int sg = g.nseg - 1; sg >= 0; --sg) {
-        const int k0 = sg * C;
-        const int len = min(C, T - k0);
-        {
-            const float* src = ck + (size_t)sg * GMT * REC;
-#pragma unroll
-            for (int i = 0; i < 5; ++i) mu[i] = src[i];
-#pragma unroll
-            for (int i = 0; i < 15; ++i) S[i] = src[5 + i];
-        }
-        if (lane == 0) {
-            float* r0 = rec + w * REC;
-#pragma unroll
-            for (int i = 0; i < 5; ++i) r0[i] = mu[i];
-#pragma unroll
-            for (int i = 0; i < 15; ++i) r0[5 + i] = S[i];
-        }
-        for (int t = 0; t < len; ++t) {
-            StepInfo inf;
-            fwd_step(g, k0 + t, s, act, mu, S, bufA, bufB, vslot + (size_t)t * Np * GMT, inf, save);
-            if (lane == 0) {
-                float* r1 = rec + ((t + 1) * GMT + w) * REC;
-#pragma unroll
-                for (int i = 0; i < 5; ++i) r1[i] = mu[i];
-#pragma unroll
-                for (int i = 0; i < 15; ++i) r1[5 + i] = S[i];
-                info[t * GMT + w] = inf;
-            }
-        }
-        __syncthreads();
-        for (int t = len - 1; t >= 0; --t) {
-            const int k = k0 + t;
-            const float* pre = rec + (t * GMT + w) * REC;
-            const float* post = rec + ((t + 1) * GMT + w) * REC;
-            float mub[5], Sb[15];
-#pragma unroll
-            for (int i = 0; i < 5; ++i) mub[i] = carry[i];
-#pragma unroll
-            for (int i = 0; i < 15; ++i) Sb[i] = carry[5 + i];
-            float sbv = 0.0f, sbw = 0.0f;
-            {
-                float m1[5], S1[15];
-#pragma unroll
-                for (int i = 0; i < 5; ++i) m1[i] = post[i];
-#pragma unroll
-                for (int i = 0; i < 15; ++i) S1[i] = post[5 + i];
-                // stage cost of step k (scored on the post-step state)
-                if (act) {
-                    const float gs = stage_cost_adjoint(g, k, m1, S1, wt, mub, Sb);
-                    sbv = gs;
-                    sbw = gs;
-                }
-            }
-            float m0[5], S0[15];
-#pragma unroll
-            for (int i = 0; i < 5; ++i) m0[i] = pre[i];
-#pragma unroll
-            for (int i = 0; i < 15; ++i) S0[i] = pre[5 + i];
-            // covariance adjoint: Sigma' = A Sigma A^T + diag(0,0,0,s,s)
-            sbv += Sb[sidx(3, 3)];
-            sbw += Sb[sidx(4, 4)];
-            float sn, cs;
-            sincosf(m0[2], &sn, &cs);
-            const float v0 = m0[3];
-            const float a02 = -a.dt * v0 * sn, a03 = a.dt * cs, a12 = a.dt * v0 * cs, a13 = a.dt * sn;
-            const float A[5][5] = {{1.f, 0.f, a02, a03, 0.f},
-                                   {0.f, 1.f, a12, a13, 0.f},
-                                   {0.f, 0.f, 1.f, 0.f, a.dt},
-                                   {0.f, 0.f, 0.f, a.av, 0.f},
-                                   {0.f, 0.f, 0.f, 0.f, a.aw}};
-            float G[5][5], Sf[5][5];
-#pragma unroll
-            for (int i = 0; i < 5; ++i)
-#pragma unroll
-                for (int j = 0; j < 5; ++j) {
-                    const int id = (i <= j) ? sidx(i, j) : sidx(j, i);
-                    G[i][j] = (i == j) ? Sb[id] : 0.5f * Sb[id];
-                    Sf[i][j] = S0[id];
-                }
-            float GA[5][5];
-#pragma unroll
-            for (int i = 0; i < 5; ++i)
-#pragma unroll
-                for (int j = 0; j < 5; ++j) {
-                    float t2 = 0.0f;
-#pragma unroll
-                    for (int m = 0; m < 5; ++m) t2 = fmaf(G[i][m], A[m][j], t2);
-                    GA[i][j] = t2;
-                }
-            // A_bar = 2 G A Sigma at the entries of A that depend on the state
-            float Ab02 = 0.f, Ab03 = 0.f, Ab12 = 0.f, Ab13 = 0.f;
-#pragma unroll
-            for (int m = 0; m < 5; ++m) {
-                Ab02 = fmaf(GA[0][m], Sf[m][2], Ab02);
-                Ab03 = fmaf(GA[0][m], Sf[m][3], Ab03);
-                Ab12 = fmaf(GA[1][m], Sf[m][2], Ab12);
-                Ab13 = fmaf(GA[1][m], Sf[m][3], Ab13);
-            }
-            Ab02 *= 2.0f; Ab03 *= 2.0f; Ab12 *= 2.0f; Ab13 *= 2.0f;
-            // Sigma_bar = A^T G A, returned to the stored-entry convention
-#pragma unroll
-            for (int i = 0; i < 5; ++i)
-#pragma unroll
-                for (int j = i; j < 5; ++j) {
-                    float t2 = 0.0f;
-#pragma unroll
-                    for (int m = 0; m < 5; ++m) t2 = fmaf(A[m][i], GA[m][j], t2);
-                    Sb[sidx(i, j)] = (i == j) ? t2 : 2.0f * t2;
-                }
-            // mean adjoint (Eq. 6 with the GP mean), with the A_bar terms
-            const float mbv = mub[3], mbw = mub[4];
-            float nm[5];
-            nm[0] = mub[0];
-            nm[1] = mub[1];
-            nm[2] = mub[2] + mub[0] * (-a.dt * v0 * sn) + mub[1] * (a.dt * v0 * cs) +
-                    Ab02 * (-a.dt * v0 * cs) + Ab03 * (-a.dt * sn) + Ab12 * (-a.dt * v0 * sn) +
-                    Ab13 * (a.dt * cs);
-            nm[3] = mub[0] * (a.dt * cs) + mub[1] * (a.dt * sn) + mub[3] * a.av +
-                    Ab02 * (-a.dt * sn) + Ab12 * (a.dt * cs);
-            nm[4] = mub[2] * a.dt + mub[4] * a.aw;
-            const StepInfo inf0 = info[t * GMT + w];
-            if (!(inf0.sraw > 0.0f)) {       // variance clamped at zero: no gradient through it
-                sbv = 0.0f;
-                sbw = 0.0f;
-            }
-            // the adjoints wait in shared memory while the product runs
-            if (lane == 0) {
-#pragma unroll
-                for (int i = 0; i < 5; ++i) save[i] = nm[i];
-#pragma unroll
-                for (int i = 0; i < 15; ++i) save[5 + i] = Sb[i];
-                save[20] = sbv;
-                save[21] = sbw;
-                save[22] = mbv;
-                save[23] = mbw;
-            }
-            // b = L^-T v = K^-1 k* for all samples of the CTA
-            {
-                const float4* src = reinterpret_cast<const float4*>(vslot + (size_t)t * Np * GMT);
-                float4* dst = reinterpret_cast<float4*>(bufA);
-                for (int i = tid; i < Np * GMT / 4; i += GT) dst[i] = src[i];
-            }
-            __syncthreads();
-            tri_product<true>(g.Wt, Np, bufA, bufB);
-            __syncthreads();
-            const float sbv2 = save[20], sbw2 = save[21], mbv2 = save[22], mbw2 = save[23];
-            if (g.Bq) {
-                // b_q for the Gram contraction G_o = sum_q sbar_o,q b_q b_q^T (the
-                // adjoints sbar go with it in qbar; a padding sample's are zero)
-                const size_t q0 = (size_t)k * g.Kpad + (size_t)blockIdx.x * GMT;
-                for (int ws = 0; ws < GMT; ++ws) {
-                    float* dst = g.Bq + (q0 + ws) * Np;
-                    for (int j = tid; j < Np; j += GT) dst[j] = bufB[j * GMT + ws];
-                }
-                if (lane == 0)
-                    g.qbar[q0 + w] = act ? make_float4(mbv2, mbw2, sbv2, sbw2) : make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-            // GP adjoint: z_bar and the lengthscale terms
-            float nv3 = save[3], nv4 = save[4];
-            if (act) {
-                const StepInfo inf = info[t * GMT + w];
-                float ubx = mbv2 * a.kv, uby = mbw2 * a.kw;
-                const float z0 = pre[3] * a.zscale[0], z1 = pre[4] * a.zscale[1],
-                            z2 = inf.ux * a.zscale[2], z3 = inf.uy * a.zscale[3];
-                float zb[4] = {0.f, 0.f, 0.f, 0.f};
-                float lb[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-                for (int j = lane; j < a.N; j += 32) {
-                    const float4 x = ldg4(a.Xs + 4 * j);
-                    const float d[4] = {z0 - x.x, z1 - x.y, z2 - x.z, z3 - x.w};
-                    const float kj = a.sf2 * exp2f(-(d[0] * d[0] + d[1] * d[1] + d[2] * d[2] + d[3] * d[3]));
-                    const float bj = bufB[j * GMT + w];
-                    const float2 al = __ldg(reinterpret_cast<const float2*>(a.alpha) + j);
-                    const float wv = kj * (mbv2 * al.x - 2.0f * sbv2 * bj);
-                    const float ww = kj * (mbw2 * al.y - 2.0f * sbw2 * bj);
-                    const float wz = wv + ww;
-#pragma unroll
-                    for (int dd = 0; dd < 4; ++dd) {
-                        zb[dd] = fmaf(wz, d[dd], zb[dd]);
-                        const float d2 = d[dd] * d[dd];
-                        lb[dd] = fmaf(wv, d2, lb[dd]);
-                        lb[4 + dd] = fmaf(ww, d2, lb[4 + dd]);
-                    }
-                    if (g.ubar) {
-#pragma unroll
-                        for (int dd = 0; dd < 4; ++dd) {
-                            lb[dd] = fmaf(-mbv2 * bj, __ldg(g.ubar + (size_t)dd * Np + j), lb[dd]);
-                            lb[4 + dd] = fmaf(-mbw2 * bj, __ldg(g.ubar + (size_t)(4 + dd) * Np + j), lb[4 + dd]);
-                        }
-                    }
-                }
-#pragma unroll
-                for (int dd = 0; dd < 4; ++dd) zb[dd] = -2.0f * kLn2 * a.zscale[dd] * wsum(zb[dd]);
-#pragma unroll
-                for (int i = 0; i < 8; ++i) lb[i] = wsum(lb[i]);
-                nv3 += zb[0];
-                nv4 += zb[1];
-                ubx += zb[2];
-                uby += zb[3];
-                if (lane == 0) {
-                    g.dU_out[(size_t)(2 * k) * a.K + s] = (inf.mask & 1) ? ubx : 0.0f;
-                    g.dU_out[(size_t)(2 * k + 1) * a.K + s] = (inf.mask & 2) ? uby : 0.0f;
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) carry[20 + i] += lb[i];
-                }
-            }
-            // carry the pre-step adjoints to step k - 1
-            __syncwarp();
-            if (lane == 0) {
-                carry[0] = save[0];
-                carry[1] = save[1];
-                carry[2] = save[2];
-                carry[3] = nv3;
-                carry[4] = nv4;
-#pragma unroll
-                for (int i = 0; i < 15; ++i) carry[5 + i] = save[5 + i];
-            }
-            __syncwarp();
-        }
-        __syncthreads();     // rec / info / scratch reuse by the next segment
+__global__ void __launch_bounds__(GT) k_grad_rev(const GradArgs g) {
+    const RolloutArgs& a = g.r;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int l = blockIdx.x * GMT + w;
+    const int Ks = g.ws.Ks, Np = a.Np, s = g.ws.s0 + l;
+    if (l >= Ks) {
+        // a padding row of a step: no adjoint (its b is never read)
+        if (l < g.Kpad && lane == 0 && g.qbar)
+            for (int k = 0; k < a.T; ++k) g.qbar[(size_t)k * g.Kpad + l] = make_float4(0.f, 0.f, 0.f, 0.f);
+        return;
     }
-    if (act && lane == 0 && g.dl_out) {
+    const float wt = g.weight ? __ldg(g.weight + s) : g.inv_K;
+    float mub[5], Sb[15], lsum[8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) g.dl_out[(size_t)i * a.K + s] = carry[20 + i];
+    for (int i = 0; i < 5; ++i) mub[i] = 0.0f;
+#pragma unroll
+    for (int i = 0; i < 15; ++i) Sb[i] = 0.0f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) lsum[i] = 0.0f;
+    for (int k = a.T - 1; k >= 0; --k) {
+        const float* post = g.rec + ((size_t)k * Ks + l) * 16;
+        const float sraw = post[15];
+        float sbv = 0.0f, sbw = 0.0f;
+        {
+            float m1[5], S1[15];
+            state_before(g, k + 1, l, m1);
+#pragma unroll
+            for (int i = 0; i < 15; ++i) S1[i] = post[i];
+            // stage cost of step k (scored on the post-step state)
+            const float gs = stage_cost_adjoint(g, k, m1, S1, wt, mub, Sb);
+            sbv = gs;
+            sbw = gs;
+        }
+        float m0[5], S0[15];
+        state_before(g, k, l, m0);
+#pragma unroll
+        for (int i = 0; i < 15; ++i) S0[i] = k > 0 ? post[i - (ptrdiff_t)Ks * 16] : 0.0f;
+        const float4 zq = g.ws.zq[(size_t)k * Ks + l];
+        // covariance adjoint: Sigma' = A Sigma A^T + diag(0,0,0,s,s)
+        sbv += Sb[sidx(3, 3)];
+        sbw += Sb[sidx(4, 4)];
+        float sn, cs;
+        sincosf(m0[2], &sn, &cs);
+        const float v0 = m0[3];
+        const float a02 = -a.dt * v0 * sn, a03 = a.dt * cs, a12 = a.dt * v0 * cs, a13 = a.dt * sn;
+        const float A[5][5] = {{1.f, 0.f, a02, a03, 0.f},
+                               {0.f, 1.f, a12, a13, 0.f},
+                               {0.f, 0.f, 1.f, 0.f, a.dt},
+                               {0.f, 0.f, 0.f, a.av, 0.f},
+                               {0.f, 0.f, 0.f, 0.f, a.aw}};
+        float G[5][5], Sf[5][5];
+#pragma unroll
+        for (int i = 0; i < 5; ++i)
+#pragma unroll
+            for (int j = 0; j < 5; ++j) {
+                const int id = (i <= j) ? sidx(i, j) : sidx(j, i);
+                G[i][j] = (i == j) ? Sb[id] : 0.5f * Sb[id];
+                Sf[i][j] = S0[id];
+            }
+        float GA[5][5];
+#pragma unroll
+        for (int i = 0; i < 5; ++i)
+#pragma unroll
+            for (int j = 0; j < 5; ++j) {
+                float t2 = 0.0f;
+#pragma unroll
+                for (int m = 0; m < 5; ++m) t2 = fmaf(G[i][m], A[m][j], t2);
+                GA[i][j] = t2;
+            }
+        // A_bar = 2 G A Sigma at the entries of A that depend on the state
+        float Ab02 = 0.f, Ab03 = 0.f, Ab12 = 0.f, Ab13 = 0.f;
+#pragma unroll
+        for (int m = 0; m < 5; ++m) {
+            Ab02 = fmaf(GA[0][m], Sf[m][2], Ab02);
+            Ab03 = fmaf(GA[0][m], Sf[m][3], Ab03);
+            Ab12 = fmaf(GA[1][m], Sf[m][2], Ab12);
+            Ab13 = fmaf(GA[1][m], Sf[m][3], Ab13);
+        }
+        Ab02 *= 2.0f; Ab03 *= 2.0f; Ab12 *= 2.0f; Ab13 *= 2.0f;
+        // Sigma_bar = A^T G A, returned to the stored-entry convention
+#pragma unroll
+        for (int i = 0; i < 5; ++i)
+#pragma unroll
+            for (int j = i; j < 5; ++j) {
+                float t2 = 0.0f;
+#pragma unroll
+                for (int m = 0; m < 5; ++m) t2 = fmaf(A[m][i], GA[m][j], t2);
+                Sb[sidx(i, j)] = (i == j) ? t2 : 2.0f * t2;
+            }
+        // mean adjoint (Eq. 6 with the GP mean), with the A_bar terms
+        const float mbv = mub[3], mbw = mub[4];
+        float nm[5];
+        nm[0] = mub[0];
+        nm[1] = mub[1];
+        nm[2] = mub[2] + mub[0] * (-a.dt * v0 * sn) + mub[1] * (a.dt * v0 * cs) +
+                Ab02 * (-a.dt * v0 * cs) + Ab03 * (-a.dt * sn) + Ab12 * (-a.dt * v0 * sn) +
+                Ab13 * (a.dt * cs);
+        nm[3] = mub[0] * (a.dt * cs) + mub[1] * (a.dt * sn) + mub[3] * a.av +
+                Ab02 * (-a.dt * sn) + Ab12 * (a.dt * cs);
+        nm[4] = mub[2] * a.dt + mub[4] * a.aw;
+        if (!(sraw > 0.0f)) {       // variance clamped at zero: no gradient through it
+            sbv = 0.0f;
+            sbw = 0.0f;
+        }
+        const float* bq = g.Bq + ((size_t)k * g.Kpad + l) * Np;
+        if (lane == 0 && g.qbar) g.qbar[(size_t)k * g.Kpad + l] = make_float4(mbv, mbw, sbv, sbw);
+        // GP adjoint: z_bar and the lengthscale terms
+        float ubx = mbv * a.kv, uby = mbw * a.kw;
+        const float z0 = m0[3] * a.zscale[0], z1 = m0[4] * a.zscale[1],
+                    z2 = zq.z * a.zscale[2], z3 = zq.w * a.zscale[3];
+        float zb[4] = {0.f, 0.f, 0.f, 0.f};
+        float lb[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        for (int j = lane; j < a.N; j += 32) {
+            const float4 x = ldg4(a.Xs + 4 * j);
+            const float d[4] = {z0 - x.x, z1 - x.y, z2 - x.z, z3 - x.w};
+            const float kj = a.sf2 * exp2f(-(d[0] * d[0] + d[1] * d[1] + d[2] * d[2] + d[3] * d[3]));
+            const float bj = __ldcg(bq + j);
+            const float2 al = __ldg(reinterpret_cast<const float2*>(a.alpha) + j);
+            const float wv = kj * (mbv * al.x - 2.0f * sbv * bj);
+            const float ww = kj * (mbw * al.y - 2.0f * sbw * bj);
+            const float wz = wv + ww;
+#pragma unroll
+            for (int dd = 0; dd < 4; ++dd) {
+                zb[dd] = fmaf(wz, d[dd], zb[dd]);
+                const float d2 = d[dd] * d[dd];
+                lb[dd] = fmaf(wv, d2, lb[dd]);
+                lb[4 + dd] = fmaf(ww, d2, lb[4 + dd]);
+            }
+            if (g.ubar) {
+#pragma unroll
+                for (int dd = 0; dd < 4; ++dd) {
+                    lb[dd] = fmaf(-mbv * bj, __ldg(g.ubar + (size_t)dd * Np + j), lb[dd]);
+                    lb[4 + dd] = fmaf(-mbw * bj, __ldg(g.ubar + (size_t)(4 + dd) * Np + j), lb[4 + dd]);
+                }
+            }
+        }
+#pragma unroll
+        for (int dd = 0; dd < 4; ++dd) zb[dd] = -2.0f * kLn2 * a.zscale[dd] * wsum(zb[dd]);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) lb[i] = wsum(lb[i]);
+        nm[3] += zb[0];
+        nm[4] += zb[1];
+        ubx += zb[2];
+        uby += zb[3];
+        if (lane == 0) {
+            // no gradient through a control at its bound
+            const bool in0 = zq.z > a.umin0 && zq.z < a.umax0, in1 = zq.w > a.umin1 && zq.w < a.umax1;
+            g.dU_out[(size_t)(2 * k) * a.K + s] = in0 ? ubx : 0.0f;
+            g.dU_out[(size_t)(2 * k + 1) * a.K + s] = in1 ? uby : 0.0f;
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) lsum[i] += lb[i];
+#pragma unroll
+        for (int i = 0; i < 5; ++i) mub[i] = nm[i];
+    }
+    if (lane == 0 && g.dl_out) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) g.dl_out[(size_t)i * a.K + s] = lsum[i];
     }
 }
 
@@ -582,19 +424,6 @@ __global__ void k_dk_alpha(const float* __restrict__ Xs, const float* __restrict
     }
 }
 
-// Wt[i][j] = W[j][i]: rows of L^-1 from rows of L^-T
-__global__ void k_transpose(const float* __restrict__ W, int Np, float* __restrict__ Wt) {
-    __shared__ float tile[32][33];
-    const int bx = blockIdx.x * 32, by = blockIdx.y * 32;
-    const int x = bx + threadIdx.x;
-    for (int r = threadIdx.y; r < 32; r += 8)
-        if (by + r < Np && x < Np) tile[r][threadIdx.x] = W[(size_t)(by + r) * Np + x];
-    __syncthreads();
-    const int y = by + threadIdx.x;
-    for (int r = threadIdx.y; r < 32; r += 8)
-        if (bx + r < Np && y < Np) Wt[(size_t)(bx + r) * Np + y] = tile[threadIdx.x][r];
-}
-
 // Final reductions in double, fixed order: blocks [0, 2T) -> dU, block 2T -> J,
 // blocks 2T+1 .. 2T+8 -> dl (when requested).
 __global__ void k_grad_reduce(const GradReduceArgs r) {
@@ -628,17 +457,14 @@ __global__ void k_grad_reduce(const GradReduceArgs r) {
 
 }  // namespace
 
-int grad_smem_bytes(int Np, int C) {
-    return (int)(sizeof(float) * (2 * (size_t)Np * GMT + (size_t)(C + 1) * GMT * REC) +
-                 sizeof(StepInfo) * (size_t)C * GMT + sizeof(float) * GMT * (SAVE + CARRY));
+int launch_grad_forward(const GradArgs& g, cudaStream_t st) {
+    k_grad_fwd<<<(g.ws.Ks + GMT - 1) / GMT, GT, 0, st>>>(g);
+    GPM_CUDA(cudaGetLastError());
+    return 0;
 }
 
-int grad_samples_per_cta() { return GMT; }
-
-int launch_grad(const GradArgs& g, int ncta, cudaStream_t st) {
-    const int smem = grad_smem_bytes(g.r.Np, g.C);
-    GPM_CUDA(cudaFuncSetAttribute(k_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    k_grad<<<ncta, GT, smem, st>>>(g);
+int launch_grad_reverse(const GradArgs& g, cudaStream_t st) {
+    k_grad_rev<<<(g.Kpad + GMT - 1) / GMT, GT, 0, st>>>(g);
     GPM_CUDA(cudaGetLastError());
     return 0;
 }
@@ -646,12 +472,6 @@ int launch_grad(const GradArgs& g, int ncta, cudaStream_t st) {
 int launch_dk_alpha(const float* Xs, const float* alpha, int N, int Np, float sf2, float* ubar,
                     cudaStream_t st) {
     k_dk_alpha<<<(Np + 7) / 8, 256, 0, st>>>(Xs, alpha, N, Np, sf2, ubar);
-    GPM_CUDA(cudaGetLastError());
-    return 0;
-}
-
-int launch_transpose(const float* W, int Np, float* Wt, cudaStream_t st) {
-    k_transpose<<<dim3((Np + 31) / 32, (Np + 31) / 32), dim3(32, 8), 0, st>>>(W, Np, Wt);
     GPM_CUDA(cudaGetLastError());
     return 0;
 }

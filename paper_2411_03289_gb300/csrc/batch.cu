@@ -1,12 +1,15 @@
 // Batched MPPI iterations over many independent controllers.
 //
-// One iteration of every controller in the batch is ONE persistent rollout
-// launch (one CTA per SM) whose CTAs take (controller, sample tile) items
-// from an atomic work queue - FP32 CUDA-core tiles and FP16- or BF16-split
-// tensor-core tiles alike, longest first - followed by one launch of the
-// weights/update for all controllers.  The autotuner picks, per controller
-// shape, the producer threads per sample of its tensor-core tiles (128, 64 or
-// 32 samples per tile) from measured tile times, and orders the queue by
+// One iteration runs two sets of controllers side by side.  Those in the split
+// precisions are ONE persistent rollout launch (one CTA per SM) whose CTAs take
+// (controller, sample tile) items from an atomic work queue, longest first.  The
+// FP32 ones run their query rollouts (query.cuh) on lanes, streams of the
+// batch's own that fork from the caller's stream and join it again: a rollout's
+// chain and stage costs are bound by latency and its products by the FMA pipe, so
+// that several fill each other's gaps.  One launch of the weights/update for all
+// controllers follows.  The autotuner picks, per controller shape, the producer
+// threads per sample of its tensor-core tiles (128, 64 or 32 samples per tile)
+// from measured tile times, and orders the queue and deals the lanes by
 // them.  States, nominal controls, outputs and the Philox iteration counters
 // live in device buffers owned by the batch, so the whole iteration (queue
 // reset, rollout, update) can be captured once in a CUDA graph and replayed.
@@ -57,8 +60,7 @@ struct gpmppi_batch_s {
     MmaArgs* d_mm = nullptr;
     UpdateArgs* d_uargs = nullptr;
     int* d_ncta = nullptr;
-    CUtensorMap* d_tmaps = nullptr;     // per controller: TMA map over L^-T (FP32 controllers)
-    int4* d_items = nullptr;            // (controller, tile, kind, threads per sample)
+    int4* d_items = nullptr;            // (controller, tile, operand format, threads per sample)
     int nitems = 0;
     unsigned int* d_head = nullptr;     // the work queue's next item
     int2* d_uitems = nullptr;
@@ -67,6 +69,10 @@ struct gpmppi_batch_s {
     std::vector<MmaArgs> h_mm;
     std::vector<int> rps;               // per controller: producer threads per sample (tensor cores)
     std::vector<double> tile_us;        // per controller: estimated (or measured) time of one tile
+    std::vector<std::vector<int>> lanes;   // the FP32 controllers of each lane, in order
+    std::vector<cudaStream_t> lane_st;
+    std::vector<cudaEvent_t> lane_done;
+    cudaEvent_t fork = nullptr;
     int smem = 0;                       // dynamic shared memory of the persistent launch
     int grid = 1;
     int maxT = 1;
@@ -91,10 +97,12 @@ void free_batch(gpmppi_batch b) {
     cudaFree(b->d_mm);
     cudaFree(b->d_uargs);
     cudaFree(b->d_ncta);
-    cudaFree(b->d_tmaps);
     cudaFree(b->d_items);
     cudaFree(b->d_head);
     cudaFree(b->d_uitems);
+    for (cudaStream_t st : b->lane_st) cudaStreamDestroy(st);
+    for (cudaEvent_t ev : b->lane_done) cudaEventDestroy(ev);
+    if (b->fork) cudaEventDestroy(b->fork);
     b->magic = 0;
     delete b;
 }
@@ -106,12 +114,12 @@ void drop_graph(gpmppi_batch b) {
     b->graph = nullptr;
 }
 
-int kind_of(gpmppi_ctrl c) { return c->fmt < 0 ? 0 : 1 + c->fmt; }
+constexpr int kMaxLanes = 4;
 
 // samples per tile of controller i
 int tile_samples(gpmppi_batch b, int i) {
     gpmppi_ctrl c = b->ctrls[i];
-    return c->fmt < 0 ? c->mt : 256 / b->rps[i];
+    return c->fmt < 0 ? 32 : 256 / b->rps[i];
 }
 
 int tile_count(gpmppi_batch b, int i) {
@@ -120,11 +128,11 @@ int tile_count(gpmppi_batch b, int i) {
 }
 
 // time of one tile before anything was measured: proportional to the
-// tensor-core MMAs of its horizon (the FP32 path taken ~8x slower per sample)
+// tensor-core MMAs of its horizon
 double tile_estimate(gpmppi_batch b, int i) {
     gpmppi_ctrl c = b->ctrls[i];
     const double T = c->p.T, np = c->gp->g.Np > 0 ? c->gp->g.Np : 1;
-    if (c->fmt < 0) return T * np * np * c->mt / 128.0 * 8.0e-6;
+    if (c->fmt < 0) return T * np * np * 32.0 * 2.0e-8;      // FP32: 32 samples at 50 TFLOP/s
     double n2 = 0.0;                      // the GPs' triangles (one GP, or a terrain ensemble)
     for (int t = 0; t < c->mm.tr.M; ++t) {
         const double nt = 128.0 * (c->mm.tr.blk0[t + 1] - c->mm.tr.blk0[t]);
@@ -161,15 +169,24 @@ int build_items(gpmppi_batch b) {
     int smem = 0;
     for (int i : ids) {
         gpmppi_ctrl c = b->ctrls[i];
+        if (c->fmt < 0) continue;
         const int n = tile_count(b, i);
-        for (int t = 0; t < n; ++t) items.push_back(make_int4(i, t, kind_of(c), c->fmt < 0 ? 0 : b->rps[i]));
-        if (c->fmt < 0) {
-            smem = std::max(smem, rollout_fp32_smem_bytes(c->gp->g.Np, rollout_fp32_mtp(c->gp->g.Np), c->stages));
-        } else {
-            MmaArgs mm = c->mm;
-            mm.rps = b->rps[i];
-            smem = std::max(smem, rollout_mma_smem(mm, c->S, c->O));
-        }
+        for (int t = 0; t < n; ++t) items.push_back(make_int4(i, t, c->fmt, b->rps[i]));
+        MmaArgs mm = c->mm;
+        mm.rps = b->rps[i];
+        smem = std::max(smem, rollout_mma_smem(mm, c->S, c->O));
+    }
+    // the FP32 controllers: longest first, each to the lane with the least work
+    b->lanes.assign(b->lane_st.size(), {});
+    std::vector<double> load(b->lane_st.size(), 0.0);
+    std::vector<double> us(b->B);
+    for (int i = 0; i < b->B; ++i) us[i] = b->tile_us[i] * tile_count(b, i);
+    std::stable_sort(ids.begin(), ids.end(), [&](int x, int y) { return us[x] > us[y]; });
+    for (int i : ids) {
+        if (b->ctrls[i]->fmt >= 0) continue;
+        const size_t l = std::min_element(load.begin(), load.end()) - load.begin();
+        b->lanes[l].push_back(i);
+        load[l] += us[i];
     }
     // each controller's tensor-core layout (threads per sample) as chosen
     for (int i = 0; i < b->B; ++i) b->h_mm[i].rps = b->rps[i];
@@ -190,11 +207,28 @@ int build_items(gpmppi_batch b) {
 }
 
 int enqueue_step(gpmppi_batch b, cudaStream_t st) {
-    int rc;
-    GPM_CUDA(cudaMemsetAsync(b->d_head, 0, sizeof(unsigned int), st));
-    if ((rc = launch_rollout_persistent(b->d_args, b->d_mm, b->d_tmaps, b->d_items, b->nitems, b->d_head, b->grid,
-                                        b->smem, st)))
-        return rc;
+    int rc = GPMPPI_OK;
+    // the lanes first: their chains leave most SMs to the persistent launch's CTAs
+    GPM_CUDA(cudaEventRecord(b->fork, st));
+    for (cudaStream_t l : b->lane_st) GPM_CUDA(cudaStreamWaitEvent(l, b->fork, 0));
+    for (size_t r = 0; r < (size_t)b->B && !rc; ++r)
+        for (size_t l = 0; l < b->lanes.size() && !rc; ++l)
+            if (r < b->lanes[l].size()) {
+                const int i = b->lanes[l][r];
+                rc = launch_query_rollout(b->ctrls[i], b->h_args[i], b->ctrls[i]->gset, b->lane_st[l]);
+            }
+    if (!rc) {
+        const cudaError_t e = cudaMemsetAsync(b->d_head, 0, sizeof(unsigned int), st);
+        if (e != cudaSuccess) rc = cuda_fail(e, "batched step: queue");
+    }
+    if (!rc)
+        rc = launch_rollout_persistent(b->d_args, b->d_mm, b->d_items, b->nitems, b->d_head, b->grid, b->smem, st);
+    // every forked lane is joined again, also after an error
+    for (size_t l = 0; l < b->lane_st.size(); ++l) {
+        GPM_CUDA(cudaEventRecord(b->lane_done[l], b->lane_st[l]));
+        GPM_CUDA(cudaStreamWaitEvent(st, b->lane_done[l], 0));
+    }
+    if (rc) return rc;
     return launch_update_batched(b->d_uargs, b->d_uitems, b->d_ncta, b->iters, b->nuitems, b->maxT, st);
 }
 
@@ -212,21 +246,21 @@ ShapeKey shape_of(gpmppi_ctrl c) {
 }
 
 // time of one wave of tiles of controller i (at most one tile per SM) with
-// rps producer threads per sample (tensor cores) or its FP32 tiles
+// rps producer threads per sample; FP32: of its whole rollout, as one tile's share
 int time_wave(gpmppi_batch b, int i, int rps, int nsm, cudaStream_t st, cudaEvent_t e0, cudaEvent_t e1,
               double* us, int* tiles_out) {
     gpmppi_ctrl c = b->ctrls[i];
     RolloutArgs a = b->h_args[i];
-    const int ms = c->fmt < 0 ? c->mt : 256 / rps;
+    const int ms = c->fmt < 0 ? 32 : 256 / rps;
     const int tiles = (c->p.K + ms - 1) / ms;
-    a.K = std::min(c->p.K, nsm * ms);           // one wave; u~ is laid out for this K (scratch)
+    if (c->fmt >= 0) a.K = std::min(c->p.K, nsm * ms);           // one wave; u~ is laid out for this K (scratch)
     MmaArgs mm = c->mm;
     mm.rps = rps;
     int rc = GPMPPI_OK;
     float best = 1e30f;
     for (int rep = 0; rep < 3 && !rc; ++rep) {
         cudaEventRecord(e0, st);
-        rc = c->fmt < 0 ? launch_rollout_fp32(a, &c->tmW, false, st) : launch_rollout_mma(a, mm, c->fmt, false, st);
+        rc = c->fmt < 0 ? launch_query_rollout(c, a, c->gset, st) : launch_rollout_mma(a, mm, c->fmt, st);
         cudaEventRecord(e1, st);
         if (rc) break;
         if (cudaEventSynchronize(e1) != cudaSuccess) return cuda_fail(cudaGetLastError(), "mppi_batch_autotune");
@@ -235,7 +269,7 @@ int time_wave(gpmppi_batch b, int i, int rps, int nsm, cudaStream_t st, cudaEven
         if (rep > 0) best = std::min(best, ms_);      // the first launch warms up
     }
     if (rc) return rc;
-    *us = 1e3 * best;
+    *us = 1e3 * best / (c->fmt < 0 ? tiles : 1);
     *tiles_out = tiles;
     return GPMPPI_OK;
 }
@@ -292,7 +326,6 @@ int mppi_batch_create(const gpmppi_ctrl* ctrls, int32_t B, gpmppi_batch* out) {
             (rc = alloc((void**)&b->d_mm, sizeof(MmaArgs) * B)) ||
             (rc = alloc((void**)&b->d_uargs, sizeof(UpdateArgs) * B)) ||
             (rc = alloc((void**)&b->d_ncta, sizeof(int) * B)) ||
-            (rc = alloc((void**)&b->d_tmaps, sizeof(CUtensorMap) * B)) ||
             (rc = alloc((void**)&b->d_head, sizeof(unsigned int))))
             return fail_free(rc);
         std::vector<unsigned long long> its(B);
@@ -303,10 +336,10 @@ int mppi_batch_create(const gpmppi_ctrl* ctrls, int32_t B, gpmppi_batch* out) {
         b->h_mm.resize(B);
         b->rps.assign(B, 2);
         b->tile_us.assign(B, 0.0);
-        std::vector<CUtensorMap> tmaps(B);
         const float zero_state[5] = {0, 0, 0, 0, 0};
         for (int i = 0; i < B; ++i) {
             gpmppi_ctrl c = ctrls[i];
+            if ((rc = make_mma_args(c))) return fail_free(rc);
             its[i] = c->it;
             RolloutArgs a = make_rollout_args(c, zero_state, b->U_nom + b->uoff[i]);
             a.x0_dev = b->states + 5 * i;
@@ -315,8 +348,7 @@ int mppi_batch_create(const gpmppi_ctrl* ctrls, int32_t B, gpmppi_batch* out) {
             a.costs = c->costs;
             b->h_args[i] = a;
             b->h_mm[i] = c->mm;
-            tmaps[i] = c->tmW;
-            if (c->fmt >= 0) b->rps[i] = c->mm.rps;
+            if (c->fmt >= 0) b->rps[i] = c->rps;
             b->tile_us[i] = tile_estimate(b, i);
             {
                 std::lock_guard<std::mutex> lock(g_tuned_mu);
@@ -346,7 +378,6 @@ int mppi_batch_create(const gpmppi_ctrl* ctrls, int32_t B, gpmppi_batch* out) {
         if (e == cudaSuccess) e = cudaMemcpy(b->d_mm, b->h_mm.data(), sizeof(MmaArgs) * B, cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = cudaMemcpy(b->d_uargs, uargs.data(), sizeof(UpdateArgs) * B, cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = cudaMemcpy(b->d_ncta, ncta.data(), sizeof(int) * B, cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaMemcpy(b->d_tmaps, tmaps.data(), sizeof(CUtensorMap) * B, cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = cudaMemset(b->d_head, 0, sizeof(unsigned int));
         if (e == cudaSuccess) e = cudaMemset(b->states, 0, sizeof(float) * 5 * B);
         if (e == cudaSuccess) e = cudaMemset(b->U_nom, 0, sizeof(float) * b->utotal);
@@ -357,6 +388,18 @@ int mppi_batch_create(const gpmppi_ctrl* ctrls, int32_t B, gpmppi_batch* out) {
             e = cudaMemcpy(b->d_uitems, uitems.data(), uitems.size() * sizeof(int2), cudaMemcpyHostToDevice);
         if (e != cudaSuccess) return fail_free(cuda_fail(e, "mppi_batch_create: upload"));
         b->nuitems = (int)uitems.size();
+        int nfp32 = 0;
+        for (int i = 0; i < B; ++i) nfp32 += ctrls[i]->fmt < 0 ? 1 : 0;
+        for (int l = 0; l < std::min(nfp32, kMaxLanes) && e == cudaSuccess; ++l) {
+            cudaStream_t ls = nullptr;
+            cudaEvent_t ev = nullptr;
+            if ((e = cudaStreamCreateWithFlags(&ls, cudaStreamNonBlocking)) != cudaSuccess) break;
+            b->lane_st.push_back(ls);
+            if ((e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming)) != cudaSuccess) break;
+            b->lane_done.push_back(ev);
+        }
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
+        if (e != cudaSuccess) return fail_free(cuda_fail(e, "mppi_batch_create: lanes"));
         if ((rc = build_items(b))) return fail_free(rc);
         *out = b;
         return GPMPPI_OK;
@@ -420,7 +463,7 @@ int mppi_batch_autotune(gpmppi_batch b, void* stream, int32_t* chosen) {
     GPM_CUDA(cudaEventCreate(&e1));
     // Per controller shape: one wave of its tiles timed for each tile layout
     // (tensor cores: 2, 4 or 8 producer threads per sample, i.e. 128, 64 or
-    // 32 samples per tile; FP32: its one layout); the layout with the least
+    // 32 samples per tile; FP32: its rollout); the layout with the least
     // SM time (tiles x time per tile) is kept, and the time per tile orders
     // the work queue.  Only rollouts run (scratch outputs); no update, so the
     // iteration counters do not move.

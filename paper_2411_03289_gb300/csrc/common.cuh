@@ -107,6 +107,7 @@ struct GpDevice {
     int device = 0;
     bool shared = true;          // both outputs share their hyper-parameters
     float sf2[2] = {0, 0};       // signal variances
+    void* mem = nullptr;         // the allocation of the fit's arrays below
     // per output o: Xs[o] = N x 4 floats, X scaled by sqrt(log2(e)/2)/l_d so
     // that k = sf2 * exp2(-|xs - zs|^2); W[o] = Np x Np floats, W[j][i] =
     // (L^-1)[i][j] for i >= j, zero elsewhere (row j of L^-T).
@@ -117,30 +118,16 @@ struct GpDevice {
     // FP64 factors kept for export: Linv64[o] N x N, alpha64[o] N
     double* Linv64[2] = {nullptr, nullptr};
     double* alpha64[2] = {nullptr, nullptr};
-    // tensor-core tiles of L^-T per operand format (0 = FP16 hi/lo, 1 = BF16
-    // hi/lo, 2 = BF16 hi/mid/lo), built on first use by a controller; NpM = N
+    // tensor-core tiles of L^-T per operand format for the batched rollout (0 =
+    // FP16 hi/lo, 1 = BF16 hi/lo, 2 = BF16 hi/mid/lo), built with a batch; NpM = N
     // rounded up to 128
     uint16_t* mma_hi[3] = {nullptr, nullptr, nullptr};
     uint16_t* mma_lo[3] = {nullptr, nullptr, nullptr};
     uint16_t* mma_mid = nullptr;   // the middle part of format 2
-    float mma_cB = 0.0f;
     int NpM = 0;
-    // the streaming rollout's training inputs and alpha in pair layout (NpM x 4
-    // floats, then NpM x 2; see k_pack_xa), copied into shared memory in bulk
+    // its training inputs and alpha in pair layout (NpM x 4 floats, then NpM x
+    // 2; see k_pack_xa), copied into shared memory in bulk
     float* mma_xa = nullptr;
-    // resident tiles of the cluster rollout (N <= 512): per 16-bit format, rank
-    // r's pieces at element offset cl_base[r], cl_bytes[r] bytes; NpC = 128,
-    // 256 or 512 output columns.  A piece holds one 16-point chunk of the
-    // rank's output rows, hi and lo parts as one slab-major operand: rows
-    // [hi lower | hi upper | lo upper | lo lower] slice (256) while both
-    // slices need the chunk, [hi upper | lo upper] (128) after
-    uint16_t* cl_tiles[2] = {nullptr, nullptr};
-    int cl_base[4] = {0, 0, 0, 0};
-    int cl_bytes[4] = {0, 0, 0, 0};
-    int cl_npc = 0;
-    // the cluster rollout's training inputs and alpha in pair layout (NpC x 4
-    // floats, then NpC x 2), copied into shared memory by one bulk copy
-    float* cl_xa = nullptr;
     // Layouts of the query rollout (query.cuh), built by the fit, per distinct
     // output: npad = N rounded up to 128 points; xq[o] = the scaled inputs in
     // pair layout (npad x 4 floats: two points per 32 bytes, far points past
@@ -149,9 +136,13 @@ struct GpDevice {
     int npad = 0;
     float* xq[2] = {nullptr, nullptr};
     float* Wb[2] = {nullptr, nullptr};
-    // adjoint rollout, built on first use: rows of L^-1 (Np x Np) and the
+    // tensor-core pieces of cB L^-1 per operand format (variance_tc.cu), built
+    // on first use by a controller
+    uint16_t* Bt[3] = {nullptr, nullptr, nullptr};
+    float cB = 0.0f;
+    // adjoint, built on first use: L^-1 in the pieces of the backward product and the
     // vectors (dK/dl_d) alpha_o (8 x Np)
-    float* Wt = nullptr;
+    float* Lb = nullptr;
     float* ubar = nullptr;
     gpmppi_hyper hyper[2];
     int n_controllers = 0;
@@ -175,10 +166,8 @@ struct RolloutArgs {
     float* tr_stage;        // K x T
     float* tr_margin;       // K x T x 2
     int K, T, N, Np, O, S;
-    int mt;                 // samples per CTA
-    int stages;             // per-warp TMA pipeline depth for the L^-T tiles
     unsigned int* err;      // device status word (bit 0: a bounded wait gave up)
-    unsigned long long wait_ns;   // FP32 rollout: limit of each tile-copy wait (mppi_set_wait_limit)
+    unsigned long long wait_ns;   // FP32 rollout: limit of each factor-copy wait (mppi_set_wait_limit)
     int expire_first;             // FP32 rollout: first wait on a barrier nothing completes (test hook)
     float sf2;
     float x0[5];
@@ -281,43 +270,6 @@ struct LaneGridHost {
 };
 int build_lane_grid(const float* path, int P, LaneGridHost& g);
 
-// One terrain GP of an ensemble (Eq. 3) as the ensemble rollout reads it.
-struct TerrainGp {
-    const float* Xs;        // N x 4, scaled by this GP's lengthscales
-    const float* alpha;     // N x 2
-    const float* W;         // Np x Np rows of L^-T
-    int N, Np;
-    float sf2;
-    float zscale[4];
-    float w;                // ensemble weight w_i
-};
-
-struct EnsArgs {
-    RolloutArgs r;          // scene, controls, constants (the GP fields of r are unused)
-    TerrainGp gp[kMaxTerrains];
-    int M;
-    int Npmax;              // largest Np of the terrains
-};
-
-// Adjoint rollout (gradient of the smoothed cost); see adjoint.cu.
-struct GradArgs {
-    RolloutArgs r;          // scene, GP, controls and constants of the controller
-    const float* Wt;        // Np x Np rows of L^-1 (zero above the diagonal and in the padding)
-    const float* ubar;      // 8 x Np: (dK/dl_d) alpha_o / (2 ln2 / l_d), row o*4+d; null: no K terms
-    const float* weight;    // K sample weights, or null for 1/K
-    float slope;            // sigmoid slope of the smoothed indicators
-    float inv_K;
-    int C, nseg, Kpad;      // checkpoint interval, segments, CTAs x samples per CTA
-    int backward;           // 0: objective only
-    float* vscr;            // n_cta x C x Np x 8: v = L^-1 k* of the current segment
-    float* ckpt;            // n_cta x nseg x 8 x 20: (mu, Sigma) at the segment starts
-    float* S_out;           // K smoothed rollout costs
-    float* dU_out;          // 2T x K per-sample control adjoints (weighted)
-    float* dl_out;          // 8 x K per-sample lengthscale terms, or null
-    float* Bq;              // (T Kpad) x Np: b = K^-1 k* per query, or null
-    float4* qbar;           // T Kpad: (mbar_v, mbar_w, sbar_v, sbar_w) per query
-};
-
 struct GradReduceArgs {
     const float* dU_out;
     const float* S_out;
@@ -333,20 +285,6 @@ struct GradReduceArgs {
     float ell[4];
 };
 
-// Cluster rollout (N <= 512): CS CTAs share 128 samples; rank r holds its
-// column slices of cB L^-1 resident in shared memory.
-struct ClArgs {
-    const uint16_t* tiles;  // all ranks' pieces (one 16-bit format)
-    int base[4];            // element offset of rank r's pieces
-    int bytes[4];           // their size in bytes
-    int cs;                 // cluster size (CTAs per 128 samples): NS / 2
-    int ns;                 // 64-column slices: NpC / 64
-    int npc;                // padded training-set size (128, 256 or 512)
-    float qscale;           // (sf2 / cB)^2
-    int scene_smem;         // lane segments and obstacles staged in shared memory
-    const float* xa;        // training inputs and alpha in pair layout (npc x 6 floats)
-};
-
 struct UpdateArgs {
     const float* costs;     // K
     const float2* u_tilde;  // T x K
@@ -360,13 +298,16 @@ struct UpdateArgs {
     float inv_lambda;
 };
 
-// ---- query rollout (chain.cu, variance_fp32.cu, stage_cost.cu) -------------
+// ---- query rollout (chain*.cu, tri.cu, variance_tc.cu, stage_cost.cu) -------------
 // The GPs of one rollout (Eq. 3; a single GP has M = 1 and w = 1).
 struct GpSet {
     int M;
     struct One {
         const float* xq;        // GpDevice::xq (pair layout, npad points)
         const float* Wb;        // GpDevice::Wb
+        const float* Xs;        // GpDevice::Xs, alpha
+        const float* alpha;
+        const uint16_t* Bt;     // GpDevice::Bt of the controller's format
         int N, npad;
         float sf2, w;
         float qscale;           // variance = sf2 - qscale * (what the variance kernel stored)
@@ -379,70 +320,104 @@ struct GpSet {
 struct QueryWs {
     float4* zq;                 // (T + 1) x Ks: (v, omega, u~_v, u~_omega) before step k
     float4* st;                 // T x Ks: (X, Y, theta, v) after step k
-    float* q;                   // M x T x Ks: |L_t^-1 k*|^2 over the variance kernel's scale
+    float* q;                   // M x nsplit x T x Ks: parts of |L_t^-1 k*|^2 over the variance kernel's scale
     int s0, Ks;
+    int nsplit;                 // parts a variance comes in (their sum in this order)
+};
+
+// Adjoint (gradient of the smoothed cost) of the samples [s0, s0 + Ks); see adjoint.cu.
+struct GradArgs {
+    RolloutArgs r;          // scene, GP, controls and constants of the controller
+    QueryWs ws;             // the forward chain's records and |L^-1 k*|^2
+    const float* ubar;      // 8 x Np: (dK/dl_d) alpha_o / (2 ln2 / l_d), row o*4+d; null: no K terms
+    const float* weight;    // K sample weights, or null for 1/K
+    float slope;            // sigmoid slope of the smoothed indicators
+    float inv_K;
+    int Kpad;               // rows of Bq and qbar per step
+    float* rec;             // T x Ks x 16: Sigma after the step (15), sf2 - |L^-1 k*|^2 (unclamped)
+    float* S_out;           // K smoothed rollout costs
+    float* dU_out;          // 2T x K per-sample control adjoints (weighted)
+    float* dl_out;          // 8 x K per-sample lengthscale terms, or null
+    const float* Bq;        // T x Kpad x Np: b = K^-1 k* per query
+    float4* qbar;           // T x Kpad: (mbar_v, mbar_w, sbar_v, sbar_w) per query, or null
 };
 
 // launchers (defined in the .cu files)
 int launch_chain(const RolloutArgs& a, const GpSet& gs, const QueryWs& ws, cudaStream_t st);
-struct VarJob {
-    const float* z;             // Q x 4 queries (any 4-byte alignment)
-    int Q;
-    float* q;                   // M x Q
-    float* mean;                // Q x 2 or null: column `out` of the posterior mean (gp_predict)
-    float* var;                 // with mean: Q x 2 posterior variance
-    int out;                    // with mean: the output, or -1 for both from one kernel row
+// Triangular products and their row sums in FP32 (tri.cu)
+struct TriJob {
+    const float* z;             // forward: Q x 4 queries (any 4-byte alignment); backward: Q x ldz rows of v
+    int ldz;
+    const float* fac;           // GpDevice::Wb (forward), GpDevice::Lb (backward)
+    const float* xq;
+    float* out;                 // Q x ldo
+    int ldo;
+    int Q, N;
+    int rk, rkpad;              // rk != 0: row q goes to (q / rk) rkpad + q % rk
+    float sf2;
+    float zscale[4];
+    int fusez;                  // differences z - x with one rounding (gp_predict, the adjoint)
     unsigned int* err;
     unsigned long long wait_ns;
     int expire_first;
 };
-int launch_var_fp32(const GpSet& gs, const VarJob& j, bool dependent, cudaStream_t st);
-int launch_stage_cost(const RolloutArgs& a, const GpSet& gs, const QueryWs& ws, cudaStream_t st);
+enum SumOrder { kSumPairs = 0, kSumLanes = 1, kSumBlock = 2 };
+TriJob tri_forward(const GpSet::One& G, const float* z, int Q, float* V);
+int launch_tri_forward(const TriJob& j, bool dependent, cudaStream_t st);
+int launch_tri_backward(const TriJob& j, bool dependent, cudaStream_t st);
+int launch_rowsum(const float* V, int ld, int Q, int N, SumOrder order, float* out, cudaStream_t st);
+int build_back_pieces(GpDevice& g, cudaStream_t st);
+// the chain with compensated terms (chain_fp32.cu): its sums in lane order, or by
+// the shuffle tree with the GPs mixed by their weights (terrain ensembles; the
+// adjoint, whose differences z - x are one rounding)
+enum ChainSums { kChainOrdered, kChainTree, kChainTreeFused };
+int launch_chain_fp32(const RolloutArgs& a, const GpSet& gs, ChainSums sums, const QueryWs& ws, cudaStream_t st);
+int launch_nominal_mean(const RolloutArgs& a, const QueryWs& ws, cudaStream_t st);
+// the squared norms |L^-1 k*|^2 on the tensor cores, for the queries of a rollout
+struct VarTcJob {
+    const float4* z;            // Q queries
+    int Q;
+    float* q;                   // M x nsplit x Q
+    int nsplit;
+    unsigned int* err;
+};
+constexpr int kMaxVarSplits = 8;
+int set_cB(GpDevice& g);
+int build_tc_pieces(GpDevice& g, int fmt);
+int var_tc_splits(const GpSet& gs, int Q, int nsm);
+int launch_var_tc(const GpSet& gs, const VarTcJob& j, int fmt, int nsm, bool dependent, cudaStream_t st);
+int launch_stage_cost(const RolloutArgs& a, const GpSet& gs, const QueryWs& ws, bool ensemble, cudaStream_t st);
 GpSet single_gp_set(const GpDevice& g, int o);
-int launch_rollout_fp32(const RolloutArgs& a, const CUtensorMap* tmap_w, bool trace,
-                        cudaStream_t st);
-// TMA tensor map over W (Np x Np floats) with the box the FP32 rollout reads
-int make_w_tensor_map(CUtensorMap* out, const float* W, int Np);
-// pipeline depth that fits shared memory (0 if none fits)
-int rollout_fp32_stages(int Np, int smem_optin);
 // after_rollout: the previous operation on st is the rollout kernel, and the
 // update's launch may overlap its tail (programmatic dependent launch)
 int launch_update(const UpdateArgs& a, int n_cta, cudaStream_t st, bool after_rollout);
 int launch_update_batched(const UpdateArgs* args, const int2* items, const int* ncta,
                           unsigned long long* iters, int nitems, int maxT, cudaStream_t st);
-int rollout_mma_smem(const MmaArgs& mm, int S, int O);
-// Batched persistent rollout: `grid` CTAs (one per SM) take items (controller,
-// tile, kind: 0 FP32 / 1 FP16 split / 2 BF16 split, producer threads per
-// sample) from the queue, advancing *head (zero before the launch).
-int launch_rollout_persistent(const RolloutArgs* args, const MmaArgs* mms, const CUtensorMap* tmaps,
-                              const int4* items, int nitems, unsigned int* head, int grid, int smem,
-                              cudaStream_t st);
+// a GP handle on the device made (1) or gone (-1): gp_predict's scratch lasts as long as any
+void scratch_user(int device, int change);
 int launch_gp_predict(const GpDevice& g, const float* Z, int M, float* mean, float* var,
                       cudaStream_t st);
 int gp_fit_device(GpDevice& g, const double* X, const double* Y, int N, cudaStream_t st);
+// Batched persistent rollout: `grid` CTAs (one per SM) take items (controller,
+// tile, operand format, producer threads per sample) from the queue, advancing
+// *head (zero before the launch).
+int launch_rollout_persistent(const RolloutArgs* args, const MmaArgs* mms, const int4* items, int nitems,
+                              unsigned int* head, int grid, int smem, cudaStream_t st);
+int launch_rollout_mma(const RolloutArgs& a, const MmaArgs& mm, int fmt, cudaStream_t st);
+int rollout_mma_smem(const MmaArgs& mm, int S, int O);
+int rollout_mma_stages(int NpM, int S, int O, int smem_optin, int lo_set, int parts, int M);
+int build_mma_tiles(GpDevice& g, int fmt);
+// The M GPs of a terrain ensemble as one block-diagonal factor: fills tr (ranges,
+// scales, weights 1) and allocates the stacked tiles and training set (caller
+// frees them).
+int build_mma_ensemble(GpDevice* const* gs, int M, int fmt, MmaTerrains& tr, uint16_t** hi, uint16_t** lo,
+                       uint16_t** mid, float** xa);
 int launch_philox(uint64_t seed, const uint32_t* ctr, int M, uint32_t* out, cudaStream_t st);
 int launch_noise(uint64_t seed, int K, int T, uint64_t it, float sv, float sw, float* eps,
                  cudaStream_t st);
-int launch_nominal(const RolloutArgs& a, float* sxy_out, cudaStream_t st);
-int rollout_fp32_smem_bytes(int Np, int mtp, int stages);
-int launch_rollout_mma(const RolloutArgs& a, const MmaArgs& mm, int fmt, bool trace, cudaStream_t st);
-int rollout_mma_stages(int NpM, int S, int O, int smem_optin, int lo_set, int parts, int M);
-int build_mma_tiles(GpDevice& g, int fmt);
-int build_cl_tiles(GpDevice& g, int fmt);
-// The M GPs of a terrain ensemble as one block-diagonal factor for the
-// streaming tensor-core rollout: fills tr (ranges, scales, weights 1) and
-// allocates the stacked tiles and training set (caller frees them).
-int build_mma_ensemble(GpDevice* const* gs, int M, int fmt, MmaTerrains& tr, uint16_t** hi, uint16_t** lo,
-                       uint16_t** mid, float** xa);
-int cl_smem_bytes(const ClArgs& cl, int S, int O);
-bool cl_schedulable(const ClArgs& cl, int S, int O, int device);
-int launch_rollout_cl(const RolloutArgs& a, const ClArgs& cl, int fmt, bool trace, cudaStream_t st);
+int launch_nominal_cov(const RolloutArgs& a, const GpSet& gs, const QueryWs& ws, float* sxy_out, cudaStream_t st);
 int launch_mma_selftest(int fmt, int N, int K, int variant, const uint16_t* A, const uint16_t* B,
                         float* D, unsigned int* err, cudaStream_t st);
-int rollout_fp32_mtp(int Np);
-int grad_smem_bytes(int Np, int C);
-int grad_samples_per_cta();
-int launch_grad(const GradArgs& g, int ncta, cudaStream_t st);
 // tr(D_d G_o) from G = [G_v; G_w] (2 Np x Np, column-major): one block per 8
 // columns, 8 partial sums per block; returns the number of blocks
 // the lengthscale Gram traces on the tensor cores (gram_tc.cu): nparts x 8
@@ -450,11 +425,10 @@ int launch_grad(const GradArgs& g, int ncta, cudaStream_t st);
 int gram_tc_parts(int Q, int Np, int nsm);
 int launch_gram_tc(const float* Bq, const float4* qbar, int Q, int Np, int N, const float* Xs, float sf2,
                    float* part, int nparts, unsigned int* err, int nsm, cudaStream_t st);
+int launch_grad_forward(const GradArgs& g, cudaStream_t st);
+int launch_grad_reverse(const GradArgs& g, cudaStream_t st);
 int launch_dk_alpha(const float* Xs, const float* alpha, int N, int Np, float sf2, float* ubar,
                     cudaStream_t st);
-int launch_transpose(const float* W, int Np, float* Wt, cudaStream_t st);
 int launch_grad_reduce(const GradReduceArgs& r, cudaStream_t st);
-int ens_smem_bytes(int Npmax);
-int launch_rollout_ens(const EnsArgs& e, bool trace, cudaStream_t st);
 
 }  // namespace gpm

@@ -2,11 +2,15 @@
 //
 // Sec. III-A fits two GPs (delta_v, delta_omega) on 4-D inputs; the rollout
 // needs, per output, alpha = K^-1 y and L^-1 with L = chol(K_XX + sn2 I)
-// (Rasmussen & Williams, Alg. 2.1).  The factorisation runs once per fit in
-// FP64 as a right-looking blocked Cholesky (32 x 32 blocks: diagonal factor,
-// panel solve, trailing update), followed by a column-block triangular
-// inverse and two matrix-vector products for alpha.  Results are then
-// converted to the FP32 layouts the rollout reads.
+// (Rasmussen & Williams, Alg. 2.1), never L itself.  So one blocked elimination
+// turns K into L^-1 in place (32 x 32 blocks): after block step k the block
+// columns up to k hold rows of the inverse's right-hand side and those past k
+// the trailing matrix, and the same rank-32 update serves both,
+//     M_ij -= L_ik V_j,   V_j = L_jk^T (j > k)  or  (L^-1)_kj (j <= k).
+// What bounds it: the FP64 pipe, two FMAs per clock and SM (N^3 / 3 of them:
+// 1.9 ms at N = 1500), once a step has more blocks than SMs; the diagonal
+// block of the next step is factored by the first CTA of an update while the
+// others work on the rest.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -22,149 +26,208 @@ namespace {
 
 constexpr int NB = 32;
 
-__global__ void k_build_kxx(const double* __restrict__ X, int N, double il0, double il1,
-                            double il2, double il3, double sf2, double sn2, double* __restrict__ A) {
-    const int i = blockIdx.y * 16 + threadIdx.y;
-    const int j = blockIdx.x * 16 + threadIdx.x;
+// K_XX + sn2 I in the lower triangle, zero above it.
+__global__ void k_build_kxx(const double* __restrict__ X, int N, double il0, double il1, double il2, double il3,
+                            double sf2, double sn2, double* __restrict__ M) {
+    const int i = blockIdx.y * 8 + threadIdx.y, j = blockIdx.x * 32 + threadIdx.x;
     if (i >= N || j >= N) return;
-    const double d0 = (X[i * 4 + 0] - X[j * 4 + 0]) * il0;
-    const double d1 = (X[i * 4 + 1] - X[j * 4 + 1]) * il1;
-    const double d2 = (X[i * 4 + 2] - X[j * 4 + 2]) * il2;
-    const double d3 = (X[i * 4 + 3] - X[j * 4 + 3]) * il3;
-    double v = sf2 * exp(-0.5 * (d0 * d0 + d1 * d1 + d2 * d2 + d3 * d3));
-    if (i == j) v += sn2;
-    A[(size_t)i * N + j] = v;
+    double v = 0.0;
+    if (j <= i) {
+        const double d0 = (X[i * 4 + 0] - X[j * 4 + 0]) * il0;
+        const double d1 = (X[i * 4 + 1] - X[j * 4 + 1]) * il1;
+        const double d2 = (X[i * 4 + 2] - X[j * 4 + 2]) * il2;
+        const double d3 = (X[i * 4 + 3] - X[j * 4 + 3]) * il3;
+        v = sf2 * exp(-0.5 * (d0 * d0 + d1 * d1 + d2 * d2 + d3 * d3));
+        if (i == j) v += sn2;
+    }
+    M[(size_t)i * N + j] = v;
 }
 
-// Unblocked Cholesky of the diagonal block at (kb, kb), size n <= 32.
-__global__ void k_potrf_diag(double* __restrict__ A, int N, int kb, int n, int* __restrict__ flag) {
-    __shared__ double a[NB][NB + 1];
+// a / b from r = 1 / b, correctly rounded (Markstein 1990: a faithful quotient
+// corrected by its exact remainder)
+__device__ __forceinline__ double quotient(double a, double b, double r) {
+    double q = a * r;
+    q = fma(fma(-q, b, a), r, q);
+    return fma(fma(-q, b, a), r, q);
+}
+
+// Cholesky factor of one 32 x 32 block, element (ty, tx) in m (the full
+// symmetric block): row c past the pivot serves, by symmetry, as column c, so a
+// step is one multiply-add a thread and one barrier.  D: the factor, lower
+// triangle.
+__device__ __forceinline__ void factor_diag(double m, double (*v)[NB + 1], double* __restrict__ D, int* flag) {
     const int tx = threadIdx.x, ty = threadIdx.y;
-    if (ty < n && tx < n) a[ty][tx] = A[(size_t)(kb + ty) * N + kb + tx];
-    __syncthreads();
-    for (int c = 0; c < n; ++c) {
-        if (tx == 0 && ty == 0) {
-            const double d = a[c][c];
+    for (int c = 0; c < NB; ++c) {
+        if (ty == c) {
+            double d = __shfl_sync(0xffffffffu, m, c);
             if (!(d > 0.0)) {
-                atomicExch(flag, 1);
-                a[c][c] = 1.0;   // keep going with finite values; the host reports NOT_PD
-            } else {
-                a[c][c] = sqrt(d);
+                if (tx == 0) atomicExch(flag, 1);   // the host reports NOT_PD; go on with finite values
+                d = 1.0;
             }
+            const double p = sqrt(d);
+            m = tx == c ? p : quotient(m, p, 1.0 / p);
+            v[c & 1][tx] = m;
+            if (tx >= c) D[tx * NB + c] = m;
         }
         __syncthreads();
-        if (tx == 0 && ty > c && ty < n) a[ty][c] /= a[c][c];
-        __syncthreads();
-        if (ty > c && ty < n && tx > c && tx <= ty) a[ty][tx] -= a[ty][c] * a[tx][c];
-        __syncthreads();
+        if (ty > c) m -= v[c & 1][ty] * v[c & 1][tx];
     }
-    if (ty < n && tx <= ty) A[(size_t)(kb + ty) * N + kb + tx] = a[ty][tx];
 }
 
-// Panel solve: rows below the diagonal block, X L_kk^T = B.
-__global__ void k_trsm_panel(double* __restrict__ A, int N, int kb, int n) {
-    __shared__ double l[NB][NB + 1];
-    __shared__ double b[NB][NB + 1];
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const int r0 = kb + n + blockIdx.x * NB;
-    const int rows = min(NB, N - r0);
-    if (ty < n && tx < n) l[ty][tx] = A[(size_t)(kb + ty) * N + kb + tx];
-    if (ty < rows && tx < n) b[ty][tx] = A[(size_t)(r0 + ty) * N + kb + tx];
-    __syncthreads();
-    for (int c = 0; c < n; ++c) {
-        if (tx == c && ty < rows) {
-            double s = b[ty][c];
-            for (int q = 0; q < c; ++q) s -= b[ty][q] * l[c][q];
-            b[ty][c] = s / l[c][c];
-        }
-        __syncthreads();
-    }
-    if (ty < rows && tx < n) A[(size_t)(r0 + ty) * N + kb + tx] = b[ty][tx];
+// element of block (kb, kb) with an identity extension beyond N
+__device__ __forceinline__ double diag_value(const double* M, int N, int kb) {
+    const int r = kb + max(threadIdx.x, threadIdx.y), c = kb + min(threadIdx.x, threadIdx.y);
+    return r < N ? M[(size_t)r * N + c] : (r == c ? 1.0 : 0.0);
 }
 
-// Trailing update A[ib][jb] -= P[ib] P[jb]^T for trailing blocks jb <= ib.
-__global__ void k_syrk(double* __restrict__ A, int N, int kb, int n) {
-    const int ib = blockIdx.y, jb = blockIdx.x;
-    if (jb > ib) return;
-    __shared__ double pi[NB][NB + 1];
-    __shared__ double pj[NB][NB + 1];
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const int t0 = kb + n;
-    const int ri = t0 + ib * NB + ty, rj = t0 + jb * NB + ty;
-    pi[ty][tx] = (ri < N && tx < n) ? A[(size_t)ri * N + kb + tx] : 0.0;
-    pj[ty][tx] = (rj < N && tx < n) ? A[(size_t)rj * N + kb + tx] : 0.0;
-    __syncthreads();
-    const int row = t0 + ib * NB + ty, col = t0 + jb * NB + tx;
-    if (row >= N || col >= N || col > row) return;
-    double s = 0.0;
+__global__ void __launch_bounds__(NB * NB) k_first_diag(const double* __restrict__ M, int N, double* __restrict__ D,
+                                                         int* __restrict__ flag) {
+    __shared__ double v[2][NB + 1];
+    factor_diag(diag_value(M, N, 0), v, D, flag);
+}
+
+// Step k's panel, from the factor D of its diagonal block, by substitution, one
+// warp a block: L_bk D^T = A_bk for the blocks b > k (to P, N x 32; a lane has a
+// row), D (L^-1)_kb = R_kb for b < k and D (L^-1)_kk = I (a lane has a column).
+// A value's updates go out as soon as it is known, which leaves up to 31
+// independent multiply-adds.
+__global__ void __launch_bounds__(NB) k_panel(double* __restrict__ M, int N, int k, const double* __restrict__ D,
+                                              double* __restrict__ P) {
+    __shared__ double d[NB][NB + 1], t[NB][NB + 1], rcp[NB];
+    const int tx = threadIdx.x, b = blockIdx.x, kb = NB * k, bb = NB * b;
 #pragma unroll 8
-    for (int q = 0; q < NB; ++q) s += pi[ty][q] * pj[tx][q];
-    A[(size_t)row * N + col] -= s;
-}
-
-// L entry with an identity extension beyond N (used by the inverse).
-__device__ __forceinline__ double lval(const double* L, int N, int r, int c) {
-    if (r < N && c < N) return c <= r ? L[(size_t)r * N + c] : 0.0;
-    return r == c ? 1.0 : 0.0;
-}
-
-// X = L^-1, one CTA per 32-column block cb: blocked forward substitution
-// X[ib][cb] = L[ib][ib]^-1 (I[ib][cb] - sum_{cb<=jb<ib} L[ib][jb] X[jb][cb]).
-__global__ void k_trtri(const double* __restrict__ L, int N, double* __restrict__ Xo) {
-    __shared__ double lb[NB][NB + 1];
-    __shared__ double xb[NB][NB + 1];
-    __shared__ double r[NB][NB + 1];
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const int cb = blockIdx.x;
-    const int nblk = (N + NB - 1) / NB;
-    const int col = cb * NB + tx;
-    for (int ib = cb; ib < nblk; ++ib) {
-        double acc = (ib == cb && ty == tx) ? 1.0 : 0.0;
-        for (int jb = cb; jb < ib; ++jb) {
-            __syncthreads();
-            lb[ty][tx] = lval(L, N, ib * NB + ty, jb * NB + tx);
-            const int xr = jb * NB + ty;
-            xb[ty][tx] = (xr < N && col < N) ? Xo[(size_t)xr * N + col] : 0.0;
-            __syncthreads();
-#pragma unroll 8
-            for (int q = 0; q < NB; ++q) acc -= lb[ty][q] * xb[q][tx];
-        }
-        __syncthreads();
-        lb[ty][tx] = lval(L, N, ib * NB + ty, ib * NB + tx);
-        r[ty][tx] = acc;
-        __syncthreads();
-        // forward substitution down the rows, one thread per column
-        if (ty == 0) {
-            for (int rr = 0; rr < NB; ++rr) {
-                double s = r[rr][tx];
-                for (int q = 0; q < rr; ++q) s -= lb[rr][q] * r[q][tx];
-                r[rr][tx] = s / lb[rr][rr];
-            }
-        }
-        __syncthreads();
-        const int row = ib * NB + ty;
-        if (row < N && col < N) Xo[(size_t)row * N + col] = r[ty][tx];
+    for (int i = 0; i < NB; ++i) {
+        d[i][tx] = D[i * NB + tx];                   // (the upper triangle is not read)
+        if (b > k)
+            t[i][tx] = bb + i < N ? M[(size_t)(bb + i) * N + kb + tx] : 0.0;
+        else if (b < k)
+            t[tx][i] = kb + i < N ? M[(size_t)(kb + i) * N + bb + tx] : 0.0;
+        else
+            t[tx][i] = i == tx ? 1.0 : 0.0;
+    }
+    __syncwarp();
+    rcp[tx] = 1.0 / d[tx][tx];
+    __syncwarp();
+    double x[NB];
+#pragma unroll
+    for (int i = 0; i < NB; ++i) x[i] = t[tx][i];
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+        x[q] = quotient(x[q], d[q][q], rcp[q]);
+#pragma unroll
+        for (int c = q + 1; c < NB; ++c) x[c] -= d[c][q] * x[q];
+    }
+    if (b > k) {
+#pragma unroll
+        for (int i = 0; i < NB; ++i) t[tx][i] = x[i];
+        __syncwarp();
+        for (int i = 0; i < NB && bb + i < N; ++i) P[(size_t)(bb + i) * NB + tx] = t[i][tx];
+    } else {
+#pragma unroll
+        for (int i = 0; i < NB; ++i)
+            if (kb + i < N && bb + tx < N) M[(size_t)(kb + i) * N + bb + tx] = x[i];
     }
 }
 
-// t = X y   (one thread per row)
-__global__ void k_matvec(const double* __restrict__ Xm, const double* __restrict__ y, int N,
-                         int ystride, double* __restrict__ t) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+// Step k's update of the blocks (i, j), k < i, j <= i, one CTA each; the first
+// CTA takes block (k + 1, k + 1) and factors it for the next step.
+__global__ void __launch_bounds__(NB * NB, 2) k_update(double* __restrict__ M, int N, int k, const double* __restrict__ P,
+                                                       double* __restrict__ D, int* __restrict__ flag) {
+    __shared__ double l[NB][NB + 1], v[NB][NB + 1];
+    const int tx = threadIdx.x, ty = threadIdx.y, kb = NB * k;
+    // block number in the triangle's row order, the next diagonal block first
+    const int first = (k + 1) * (k + 2) / 2;
+    int b = blockIdx.x;
+    b = b == 0 ? k + 1 : (b <= k + 1 ? b - 1 : b);
+    const int t = first + b;
+    int i = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
+    while ((i + 1) * (i + 2) / 2 <= t) ++i;
+    while (i * (i + 1) / 2 > t) --i;
+    const int j = t - i * (i + 1) / 2;
+    const int row = NB * i + ty, col = NB * j + tx;
+    double m = (j != k && row < N && col < N) ? M[(size_t)row * N + col] : 0.0;
+    l[ty][tx] = row < N ? P[(size_t)row * NB + tx] : 0.0;
+    if (j > k) {
+        const int r = NB * j + ty;
+        v[tx][ty] = r < N ? P[(size_t)r * NB + tx] : 0.0;
+    } else {
+        v[ty][tx] = M[(size_t)(kb + ty) * N + col];          // block row k lies below N: i > k has rows
+    }
+    __syncthreads();
+    if (j > k) {
+        double s = 0.0;
+#pragma unroll 8
+        for (int q = 0; q < NB; ++q) s += l[ty][q] * v[q][tx];
+        m -= s;
+    } else {
+#pragma unroll 8
+        for (int q = 0; q < NB; ++q) m -= l[ty][q] * v[q][tx];
+    }
+    if (blockIdx.x == 0) {
+        // identity beyond N; the block's lower half mirrored
+        if (row >= N || col >= N) m = row == col ? 1.0 : 0.0;
+        __syncthreads();
+        l[ty][tx] = m;
+        __syncthreads();
+        if (tx > ty) m = l[tx][ty];
+        factor_diag(m, v, D, flag);
+    } else if (row < N && col <= row) {
+        M[(size_t)row * N + col] = m;
+    }
+}
+
+// t = L^-1 y for both outputs' columns of y, one warp per row
+__global__ void k_alpha_fwd(const double* __restrict__ Xm, const double* __restrict__ y, int N, double* __restrict__ t) {
+    const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (i >= N) return;
-    double s = 0.0;
-    for (int j = 0; j <= i; ++j) s += Xm[(size_t)i * N + j] * y[(size_t)j * ystride];
-    t[i] = s;
+    double s0 = 0.0, s1 = 0.0;
+    for (int j = lane; j <= i; j += 32) {
+        const double x = Xm[(size_t)i * N + j];
+        s0 += x * y[2 * j];
+        s1 += x * y[2 * j + 1];
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+        s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+    }
+    if (lane == 0) {
+        t[2 * i] = s0;
+        t[2 * i + 1] = s1;
+    }
 }
 
-// a = X^T t   (one thread per column)
-__global__ void k_matvec_t(const double* __restrict__ Xm, const double* __restrict__ t, int N,
-                           double* __restrict__ a) {
+// alpha = L^-T t in kAlphaParts parts of the rows, 32 columns a CTA
+constexpr int kAlphaParts = 8;
+__global__ void k_alpha_bwd(const double* __restrict__ Xm, const double* __restrict__ t, int N, double* __restrict__ part) {
+    __shared__ double r0[8][33], r1[8][33];
+    const int tx = threadIdx.x, ty = threadIdx.y, j = blockIdx.x * 32 + tx;
+    const int rows = (N + kAlphaParts - 1) / kAlphaParts;
+    const int i0 = max(blockIdx.y * rows, blockIdx.x * 32), i1 = min(N, (blockIdx.y + 1) * rows);
+    double s0 = 0.0, s1 = 0.0;
+    if (j < N)
+        for (int i = i0 + ty; i < i1; i += 8) {
+            const double x = Xm[(size_t)i * N + j];          // zero above the diagonal
+            s0 += x * t[2 * i];
+            s1 += x * t[2 * i + 1];
+        }
+    r0[ty][tx] = s0;
+    r1[ty][tx] = s1;
+    __syncthreads();
+    if (ty == 0 && j < N) {
+        for (int q = 1; q < 8; ++q) {
+            s0 += r0[q][tx];
+            s1 += r1[q][tx];
+        }
+        part[((size_t)blockIdx.y * N + j) * 2] = s0;
+        part[((size_t)blockIdx.y * N + j) * 2 + 1] = s1;
+    }
+}
+__global__ void k_alpha_sum(const double* __restrict__ part, int N, int o, double* __restrict__ alpha) {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= N) return;
     double s = 0.0;
-    for (int i = j; i < N; ++i) s += Xm[(size_t)i * N + j] * t[i];
-    a[j] = s;
+    for (int q = 0; q < kAlphaParts; ++q) s += part[((size_t)q * N + j) * 2 + o];
+    alpha[j] = s;
 }
 
 // FP32 layouts for the rollout.
@@ -203,80 +266,6 @@ __global__ void k_pack_alpha(const double* __restrict__ a0, const double* __rest
     if (j >= N) return;
     out[j * 2 + 0] = (float)a0[j];
     out[j * 2 + 1] = (float)a1[j];
-}
-
-// ---------------------------------------------------------------------------
-// GP posterior at M queries, one CTA per query (FP32).
-// ---------------------------------------------------------------------------
-constexpr int PRED_THREADS = 128;
-
-__device__ float block_sum(float v, float* red) {
-    // deterministic: fixed shuffle tree, then warp partials summed in order
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    __syncthreads();
-    if (l == 0) red[w] = v;
-    __syncthreads();
-    float s = 0.0f;
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) s += red[i];
-    return s;
-}
-
-struct PredArgs {
-    const float* Xs[2];
-    const float* W[2];
-    const float* alpha;
-    float sf2[2];
-    float zscale[2][4];
-    int N, Np;
-    bool shared;
-};
-
-__global__ void k_gp_predict(PredArgs p, const float* __restrict__ Z, int M, float* __restrict__ mean,
-                             float* __restrict__ var) {
-    extern __shared__ float ks[];   // N floats
-    __shared__ float red[PRED_THREADS / 32];
-    const int q = blockIdx.x;
-    if (q >= M) return;
-    const int N = p.N;
-    float zq[4];
-    for (int o = 0; o < 2; ++o) {
-        if (o == 1 && p.shared) {
-            // identical kernel row: only the mean weights differ
-            float m = 0.0f;
-            for (int j = threadIdx.x; j < N; j += blockDim.x) m += ks[j] * p.alpha[j * 2 + 1];
-            m = block_sum(m, red);
-            if (threadIdx.x == 0) {
-                mean[q * 2 + 1] = m;
-                var[q * 2 + 1] = var[q * 2 + 0];
-            }
-            break;
-        }
-        for (int d = 0; d < 4; ++d) zq[d] = Z[q * 4 + d] * p.zscale[o][d];
-        const float* Xs = p.Xs[o];
-        __syncthreads();
-        float m = 0.0f;
-        for (int j = threadIdx.x; j < N; j += blockDim.x) {
-            const float4 x = reinterpret_cast<const float4*>(Xs)[j];
-            const float e0 = zq[0] - x.x, e1 = zq[1] - x.y, e2 = zq[2] - x.z, e3 = zq[3] - x.w;
-            const float k = p.sf2[o] * exp2f(-(e0 * e0 + e1 * e1 + e2 * e2 + e3 * e3));
-            ks[j] = k;
-            m += k * p.alpha[j * 2 + o];
-        }
-        m = block_sum(m, red);   // contains the barrier that publishes ks
-        float qf = 0.0f;
-        const float* W = p.W[o];
-        for (int i = threadIdx.x; i < N; i += blockDim.x) {
-            float v = 0.0f;
-            for (int j = 0; j <= i; ++j) v += W[(size_t)j * p.Np + i] * ks[j];
-            qf += v * v;
-        }
-        qf = block_sum(qf, red);
-        if (threadIdx.x == 0) {
-            mean[q * 2 + o] = m;
-            var[q * 2 + o] = fmaxf(0.0f, p.sf2[o] - qf);
-        }
-    }
 }
 
 // max |L^-1| over the lower triangle (positive doubles order like their bits)
@@ -332,58 +321,8 @@ __global__ void k_pack_mma(const double* __restrict__ Xm, int N, int NpM, int fm
     }
 }
 
-// Resident tiles of the cluster rollout.  Cluster rank r owns the 64-column
-// slices r and NS - 1 - r of cB L^-1 (NS = NpC / 64); chunk c (training points
-// 16c .. 16c + 15) of rank r is one piece: 128 rows (slice r then slice
-// NS - 1 - r) while both slices need it (c < 4 (r + 1)), else 64 rows (slice
-// NS - 1 - r alone, needed while c < 4 (NS - r)).  A piece is its hi part then
-// its lo part, each slab-major: slab sl (points 8 sl .. 8 sl + 7), row rr at
-// element sl * rows * 8 + rr * 8.  Pieces follow each other in chunk order;
-// rank r's pieces start at element offset base[r].
-__global__ void k_pack_cl(const double* __restrict__ Xm, int N, int NS, int fmt, double cB,
-                          const int4* __restrict__ pieces, int npieces, uint16_t* __restrict__ out) {
-    const int p = blockIdx.y;
-    if (p >= npieces) return;
-    const int4 d = pieces[p];            // (element offset, chunk, rank, rows per part)
-    const int rows = d.w, R2 = 2 * rows; // the piece holds the hi and the lo rows
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= R2 * 16) return;
-    const int sl = idx / (R2 * 8), rr = (idx / 8) % R2, e = idx % 8;
-    const int c = d.y, r = d.z;
-    const int j = 16 * c + 8 * sl + e;
-    const int lo_row = 64 * r, up_row = 64 * (NS - 1 - r);
-    // row order: [hi lower | hi upper | lo upper | lo lower] while both slices
-    // need the chunk (rows = 128), [hi upper | lo upper] after (rows = 64)
-    int i;
-    bool lo;
-    if (rows == 128) {
-        const int q = rr >> 6, o = rr & 63;
-        i = (q == 0 || q == 3) ? lo_row + o : up_row + o;
-        lo = q >= 2;
-    } else {
-        i = up_row + (rr & 63);
-        lo = rr >= 64;
-    }
-    double v = 0.0;
-    if (i < N && j < N && j <= i) v = cB * Xm[(size_t)i * N + j];
-    uint16_t h;
-    if (fmt == 0) {
-        const __half hh = __double2half(v);
-        h = lo ? __half_as_ushort(__double2half(v - (double)__half2float(hh))) : __half_as_ushort(hh);
-    } else {
-        const __nv_bfloat16 hh = __double2bfloat16(v);
-        h = lo ? __bfloat16_as_ushort(__double2bfloat16(v - (double)__bfloat162float(hh)))
-               : __bfloat16_as_ushort(hh);
-    }
-    out[(size_t)d.x + idx] = h;
-}
-
 }  // namespace
 
-// training inputs and alpha of the cluster rollout in pair layout: for points
-// 2p and 2p + 1, x[2p] = (x0, x0', x1, x1'), x[2p + 1] = (x2, x2', x3, x3') and
-// a[p] = (a_v, a_v', a_w, a_w') (primes: point 2p + 1); rows j >= N get a far
-// point (exp2 underflows to exactly 0) and alpha 0
 // Training inputs and alpha of one GP in pair layout: point j (j < npc; far
 // away with alpha 0 past N) at position J0 + j of an array of NpT points (a
 // single GP: J0 = 0, NpT = npc; J0 even).
@@ -409,46 +348,24 @@ __global__ void k_pack_xa(const float* __restrict__ Xs, const float* __restrict_
     ap[2] = al.y;
 }
 
-int build_cl_tiles(GpDevice& g, int fmt) {
-    if (g.cl_tiles[fmt] || g.N == 0) return GPMPPI_OK;
-    int rc = build_mma_tiles(g, fmt);      // sets cB (and the streaming tiles)
-    if (rc) return rc;
-    const int NpC = g.N <= 128 ? 128 : (g.N <= 256 ? 256 : 512);
-    if (g.N > 512) return fail(GPMPPI_ERR_UNSUPPORTED, "cluster tiles: N > 512");
-    const int NS = NpC / 64, CS = NS / 2;
-    std::vector<int4> pieces;
-    size_t off = 0;
-    for (int r = 0; r < CS; ++r) {
-        g.cl_base[r] = (int)off;
-        for (int c = 0; c < 4 * (NS - r); ++c) {
-            const int rows = (c < 4 * (r + 1)) ? 128 : 64;
-            pieces.push_back(make_int4((int)off, c, r, rows));
-            off += (size_t)rows * 16 * 2;
-        }
-        g.cl_bytes[r] = (int)((off - (size_t)g.cl_base[r]) * sizeof(uint16_t));
-    }
-    g.cl_npc = NpC;
-    int4* dp = nullptr;
-    GPM_CUDA(cudaMalloc(&dp, pieces.size() * sizeof(int4)));
-    cudaError_t e = cudaMemcpy(dp, pieces.data(), pieces.size() * sizeof(int4), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMalloc(&g.cl_tiles[fmt], off * sizeof(uint16_t));
+// Scale of the tensor-core operand cB L^-1: the largest power of two with
+// cB max|L^-1| <= 2^14 (16-bit range, room for the sums).
+int set_cB(GpDevice& g) {
+    if (g.cB != 0.0f || g.N == 0) return GPMPPI_OK;
+    unsigned long long* d = nullptr;
+    GPM_CUDA(cudaMalloc(&d, sizeof(unsigned long long)));
+    cudaError_t e = cudaMemset(d, 0, sizeof(unsigned long long));
     if (e == cudaSuccess) {
-        k_pack_cl<<<dim3(16, (unsigned)pieces.size()), 256>>>(g.Linv64[0], g.N, NS, fmt, (double)g.mma_cB, dp,
-                                                           (int)pieces.size(), g.cl_tiles[fmt]);
+        k_absmax<<<256, 256>>>(g.Linv64[0], (size_t)g.N * g.N, d);
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess) e = cudaDeviceSynchronize();
-    cudaFree(dp);
-    if (e != cudaSuccess) return cuda_fail(e, "build_cl_tiles");
-    if (!g.cl_xa) {
-        e = cudaMalloc(&g.cl_xa, sizeof(float) * 6 * (size_t)NpC);
-        if (e == cudaSuccess) {
-            k_pack_xa<<<(NpC + 127) / 128, 128>>>(g.Xs[0], g.alpha, g.N, NpC, 0, NpC, g.cl_xa);
-            e = cudaGetLastError();
-        }
-        if (e == cudaSuccess) e = cudaDeviceSynchronize();
-        if (e != cudaSuccess) return cuda_fail(e, "build_cl_tiles: training-set layout");
-    }
+    unsigned long long bits = 0;
+    if (e == cudaSuccess) e = cudaMemcpy(&bits, d, sizeof(bits), cudaMemcpyDeviceToHost);
+    cudaFree(d);
+    if (e != cudaSuccess) return cuda_fail(e, "tensor-core factor: absmax");
+    double mx = 0.0;
+    std::memcpy(&mx, &bits, sizeof(mx));
+    g.cB = (float)std::ldexp(1.0, (int)std::floor(std::log2(16384.0 / (mx > 0 ? mx : 1.0))));
     return GPMPPI_OK;
 }
 
@@ -456,29 +373,14 @@ int build_mma_tiles(GpDevice& g, int fmt) {
     if (g.mma_hi[fmt] || g.N == 0) return GPMPPI_OK;
     const int N = g.N;
     g.NpM = ((N + 127) / 128) * 128;
-    if (g.mma_cB == 0.0f) {
-        unsigned long long* d = nullptr;
-        GPM_CUDA(cudaMalloc(&d, sizeof(unsigned long long)));
-        cudaError_t e = cudaMemset(d, 0, sizeof(unsigned long long));
-        if (e == cudaSuccess) {
-            k_absmax<<<256, 256>>>(g.Linv64[0], (size_t)N * N, d);
-            e = cudaGetLastError();
-        }
-        unsigned long long bits = 0;
-        if (e == cudaSuccess) e = cudaMemcpy(&bits, d, sizeof(bits), cudaMemcpyDeviceToHost);
-        cudaFree(d);
-        if (e != cudaSuccess) return cuda_fail(e, "build_mma_tiles: absmax");
-        double mx = 0.0;
-        std::memcpy(&mx, &bits, sizeof(mx));
-        // largest power of two with cB * max|L^-1| <= 2^14 (16-bit range, room for the sums)
-        g.mma_cB = (float)std::ldexp(1.0, (int)std::floor(std::log2(16384.0 / (mx > 0 ? mx : 1.0))));
-    }
+    const int rc = set_cB(g);
+    if (rc) return rc;
     // 32-point stages x pairs of 128-row blocks x 256 rows x 32 points
     const size_t n = (size_t)(g.NpM / 32) * (size_t)((g.NpM / 128 + 1) / 2) * 8192;
     GPM_CUDA(cudaMalloc(&g.mma_hi[fmt], n * sizeof(uint16_t)));
     GPM_CUDA(cudaMalloc(&g.mma_lo[fmt], n * sizeof(uint16_t)));
     if (fmt == 2) GPM_CUDA(cudaMalloc(&g.mma_mid, n * sizeof(uint16_t)));
-    k_pack_mma<<<(unsigned)((n + 255) / 256), 256>>>(g.Linv64[0], N, g.NpM, fmt, (double)g.mma_cB, 0, 0,
+    k_pack_mma<<<(unsigned)((n + 255) / 256), 256>>>(g.Linv64[0], N, g.NpM, fmt, (double)g.cB, 0, 0,
                                                       (g.NpM / 128 + 1) / 2, g.mma_hi[fmt], g.mma_lo[fmt],
                                                       g.mma_mid);
     GPM_CUDA(cudaGetLastError());
@@ -507,7 +409,7 @@ int build_mma_ensemble(GpDevice* const* gs, int M, int fmt, MmaTerrains& tr, uin
         const int nbt = g.N == 0 ? 0 : 2 * ((g.NpM / 128 + 1) / 2);
         tr.blk0[t] = nb;
         nb += nbt;
-        const double r = (double)g.sf2[0] / (g.mma_cB > 0.0f ? (double)g.mma_cB : 1.0);
+        const double r = (double)g.sf2[0] / (g.cB > 0.0f ? (double)g.cB : 1.0);
         tr.qscale[t] = (float)(r * r);
         tr.sf2[t] = g.sf2[0];
         tr.w[t] = 1.0f;
@@ -531,35 +433,13 @@ int build_mma_ensemble(GpDevice* const* gs, int M, int fmt, MmaTerrains& tr, uin
         const int nbt = tr.blk0[t + 1] - tr.blk0[t];
         if (nbt == 0) continue;
         const size_t nt = (size_t)(nbt * 4) * (nbt / 2) * 8192;
-        k_pack_mma<<<(unsigned)((nt + 255) / 256), 256>>>(g.Linv64[0], g.N, nbt * 128, fmt, (double)g.mma_cB,
+        k_pack_mma<<<(unsigned)((nt + 255) / 256), 256>>>(g.Linv64[0], g.N, nbt * 128, fmt, (double)g.cB,
                                                            4 * tr.blk0[t], tr.blk0[t] / 2, NP, *hi, *lo, *mid);
         GPM_CUDA(cudaGetLastError());
         k_pack_xa<<<(nbt * 128 + 127) / 128, 128>>>(g.Xs[0], g.alpha, g.N, nbt * 128, 128 * tr.blk0[t], NpT, *xa);
         GPM_CUDA(cudaGetLastError());
     }
     GPM_CUDA(cudaDeviceSynchronize());
-    return GPMPPI_OK;
-}
-
-int launch_gp_predict(const GpDevice& g, const float* Z, int M, float* mean, float* var,
-                      cudaStream_t st) {
-    if (M == 0) return GPMPPI_OK;
-    PredArgs p;
-    for (int o = 0; o < 2; ++o) {
-        p.Xs[o] = g.Xs[o];
-        p.W[o] = g.W[o];
-        p.sf2[o] = g.sf2[o];
-        for (int d = 0; d < 4; ++d) p.zscale[o][d] = g.zscale[o][d];
-    }
-    p.alpha = g.alpha;
-    p.N = g.N;
-    p.Np = g.Np;
-    p.shared = g.shared;
-    const size_t smem = (size_t)(g.N > 0 ? g.N : 1) * sizeof(float);
-    GPM_CUDA(cudaFuncSetAttribute(k_gp_predict, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)smem));
-    k_gp_predict<<<M, PRED_THREADS, smem, st>>>(p, Z, M, mean, var);
-    GPM_CUDA(cudaGetLastError());
     return GPMPPI_OK;
 }
 
@@ -580,35 +460,44 @@ int gp_fit_device(GpDevice& g, const double* X, const double* Y, int N, cudaStre
     }
     const int nout = g.shared ? 1 : 2;
     const size_t nn = (size_t)N * N;
-    // device allocations owned by g (freed by the caller on any failure)
-    GPM_CUDA(cudaMalloc(&g.alpha, sizeof(float) * 2 * (N > 0 ? N : 1)));
+    // one allocation owned by g (freed by the caller on any failure), pieces on
+    // 256-byte boundaries: an allocation of its own for each costs as much as
+    // the fit of a small training set
+    size_t off = 0;
+    auto take = [&](size_t bytes) {
+        const size_t at = off;
+        off += (bytes + 255) & ~(size_t)255;
+        return at;
+    };
+    const size_t n1 = N > 0 ? (size_t)N : 1;
+    const size_t o_alpha = take(sizeof(float) * 2 * n1);
+    const size_t o_a64[2] = {take(sizeof(double) * n1), take(sizeof(double) * n1)};
+    size_t o_xs[2], o_w[2], o_l[2], o_xq[2], o_wb[2];
     for (int o = 0; o < nout; ++o) {
-        GPM_CUDA(cudaMalloc(&g.Xs[o], sizeof(float) * 4 * (N > 0 ? N : 1)));
-        GPM_CUDA(cudaMalloc(&g.W[o], sizeof(float) * (g.Np > 0 ? (size_t)g.Np * g.Np : 1)));
-        GPM_CUDA(cudaMalloc(&g.Linv64[o], sizeof(double) * (nn > 0 ? nn : 1)));
-        GPM_CUDA(cudaMalloc(&g.alpha64[o], sizeof(double) * (N > 0 ? N : 1)));
-        GPM_CUDA(cudaMalloc(&g.xq[o], sizeof(float) * 6 * (g.npad > 0 ? g.npad : 1)));
-        GPM_CUDA(cudaMalloc(&g.Wb[o], sizeof(float) * (nb > 0 ? nb * (nb + 1) / 2 * (128 * 128) : 1)));
+        o_xs[o] = take(sizeof(float) * 4 * n1);
+        o_w[o] = take(sizeof(float) * (size_t)g.Np * g.Np);
+        o_l[o] = take(sizeof(double) * nn);
+        o_xq[o] = take(sizeof(float) * 6 * (size_t)g.npad);
+        o_wb[o] = take(sizeof(float) * nb * (nb + 1) / 2 * (128 * 128));
     }
-    if (g.shared) {
-        g.Xs[1] = g.Xs[0];
-        g.W[1] = g.W[0];
-        g.Linv64[1] = g.Linv64[0];
-        g.xq[1] = g.xq[0];
-        g.Wb[1] = g.Wb[0];
-        GPM_CUDA(cudaMalloc(&g.alpha64[1], sizeof(double) * (N > 0 ? N : 1)));
+    GPM_CUDA(cudaMalloc(&g.mem, off));
+    char* mem = static_cast<char*>(g.mem);
+    g.alpha = reinterpret_cast<float*>(mem + o_alpha);
+    for (int o = 0; o < 2; ++o) {
+        const int s = o < nout ? o : 0;              // shared hyper-parameters: one factor
+        g.alpha64[o] = reinterpret_cast<double*>(mem + o_a64[o]);
+        g.Xs[o] = reinterpret_cast<float*>(mem + o_xs[s]);
+        g.W[o] = reinterpret_cast<float*>(mem + o_w[s]);
+        g.Linv64[o] = reinterpret_cast<double*>(mem + o_l[s]);
+        g.xq[o] = reinterpret_cast<float*>(mem + o_xq[s]);
+        g.Wb[o] = reinterpret_cast<float*>(mem + o_wb[s]);
     }
     if (N == 0) return GPMPPI_OK;
 
-    double *dX = nullptr, *dY = nullptr, *dA = nullptr, *dt = nullptr;
-    int* dflag = nullptr;
-    auto cleanup = [&]() {
-        cudaFree(dX);
-        cudaFree(dY);
-        cudaFree(dA);
-        cudaFree(dt);
-        cudaFree(dflag);
-    };
+    // one scratch allocation: X, y, t, alpha's parts, the panel, a diagonal block, the flag
+    const size_t n_x = 4 * (size_t)N, n_y = 2 * (size_t)N, n_part = 2 * (size_t)kAlphaParts * N, n_p = (size_t)NB * N;
+    double* scratch = nullptr;
+    auto cleanup = [&]() { cudaFree(scratch); };
     auto check = [&](cudaError_t e, const char* what) -> int {
         if (e != cudaSuccess) {
             cleanup();
@@ -617,11 +506,10 @@ int gp_fit_device(GpDevice& g, const double* X, const double* Y, int N, cudaStre
         return GPMPPI_OK;
     };
     int rc;
-    if ((rc = check(cudaMalloc(&dX, sizeof(double) * 4 * N), "cudaMalloc X"))) return rc;
-    if ((rc = check(cudaMalloc(&dY, sizeof(double) * 2 * N), "cudaMalloc Y"))) return rc;
-    if ((rc = check(cudaMalloc(&dA, sizeof(double) * nn), "cudaMalloc K"))) return rc;
-    if ((rc = check(cudaMalloc(&dt, sizeof(double) * N), "cudaMalloc t"))) return rc;
-    if ((rc = check(cudaMalloc(&dflag, sizeof(int)), "cudaMalloc flag"))) return rc;
+    if ((rc = check(cudaMalloc(&scratch, sizeof(double) * (n_x + 2 * n_y + n_part + n_p + NB * NB + 1)), "cudaMalloc scratch")))
+        return rc;
+    double *dX = scratch, *dY = dX + n_x, *dt = dY + n_y, *dpart = dt + n_y, *dP = dpart + n_part, *dD = dP + n_p;
+    int* dflag = reinterpret_cast<int*>(dD + NB * NB);
     if ((rc = check(cudaMemcpyAsync(dX, X, sizeof(double) * 4 * N, cudaMemcpyHostToDevice, st),
                     "copy X")))
         return rc;
@@ -632,40 +520,31 @@ int gp_fit_device(GpDevice& g, const double* X, const double* Y, int N, cudaStre
     for (int o = 0; o < nout; ++o) {
         const gpmppi_hyper& h = g.hyper[o];
         if ((rc = check(cudaMemsetAsync(dflag, 0, sizeof(int), st), "memset flag"))) return rc;
-        dim3 b16(16, 16), gK((N + 15) / 16, (N + 15) / 16);
-        k_build_kxx<<<gK, b16, 0, st>>>(dX, N, 1.0 / h.lengthscale[0], 1.0 / h.lengthscale[1],
-                                        1.0 / h.lengthscale[2], 1.0 / h.lengthscale[3],
-                                        h.signal_var, h.noise_var, dA);
-        for (int kb = 0; kb < N; kb += NB) {
-            const int n = (N - kb < NB) ? (N - kb) : NB;
-            k_potrf_diag<<<1, dim3(NB, NB), 0, st>>>(dA, N, kb, n, dflag);
-            const int rest = N - kb - n;
-            if (rest > 0) {
-                const int nb_rest = (rest + NB - 1) / NB;
-                k_trsm_panel<<<nb_rest, dim3(NB, NB), 0, st>>>(dA, N, kb, n);
-                k_syrk<<<dim3(nb_rest, nb_rest), dim3(NB, NB), 0, st>>>(dA, N, kb, n);
-            }
+        double* M = g.Linv64[o];
+        k_build_kxx<<<dim3(nblk, (N + 7) / 8), dim3(32, 8), 0, st>>>(
+            dX, N, 1.0 / h.lengthscale[0], 1.0 / h.lengthscale[1], 1.0 / h.lengthscale[2], 1.0 / h.lengthscale[3],
+            h.signal_var, h.noise_var, M);
+        k_first_diag<<<1, dim3(NB, NB), 0, st>>>(M, N, dD, dflag);
+        for (int k = 0; k < nblk; ++k) {
+            k_panel<<<nblk, NB, 0, st>>>(M, N, k, dD, dP);
+            const int blocks = nblk * (nblk + 1) / 2 - (k + 1) * (k + 2) / 2;
+            if (blocks > 0) k_update<<<blocks, dim3(NB, NB), 0, st>>>(M, N, k, dP, dD, dflag);
         }
-        if ((rc = check(cudaGetLastError(), "cholesky kernels"))) return rc;
+        if ((rc = check(cudaGetLastError(), "factorisation kernels"))) return rc;
         int hflag = 0;
         if ((rc = check(cudaMemcpyAsync(&hflag, dflag, sizeof(int), cudaMemcpyDeviceToHost, st),
                         "copy flag")))
             return rc;
-        if ((rc = check(cudaStreamSynchronize(st), "cholesky sync"))) return rc;
+        if ((rc = check(cudaStreamSynchronize(st), "factorisation sync"))) return rc;
         if (hflag) {
             cleanup();
             return fail(GPMPPI_ERR_NOT_PD, "gp_fit: K_XX + noise_var I is not positive definite");
         }
-        if ((rc = check(cudaMemsetAsync(g.Linv64[o], 0, sizeof(double) * nn, st), "memset Linv")))
-            return rc;
-        k_trtri<<<nblk, dim3(NB, NB), 0, st>>>(dA, N, g.Linv64[o]);
         const int tb = 128, gb = (N + tb - 1) / tb;
-        const int outs[2] = {o, g.shared ? 1 : -1};
-        for (int oo : outs) {
-            if (oo < 0) continue;
-            k_matvec<<<gb, tb, 0, st>>>(g.Linv64[o], dY + oo, N, 2, dt);
-            k_matvec_t<<<gb, tb, 0, st>>>(g.Linv64[o], dt, N, g.alpha64[oo]);
-        }
+        k_alpha_fwd<<<(N + 7) / 8, 256, 0, st>>>(M, dY, N, dt);
+        k_alpha_bwd<<<dim3(nblk, kAlphaParts), dim3(32, 8), 0, st>>>(M, dt, N, dpart);
+        k_alpha_sum<<<gb, tb, 0, st>>>(dpart, N, o, g.alpha64[o]);
+        if (g.shared) k_alpha_sum<<<gb, tb, 0, st>>>(dpart, N, 1, g.alpha64[1]);
         const double s = std::sqrt(0.5 * log2e);
         k_pack_x<<<gb, tb, 0, st>>>(dX, N, s / h.lengthscale[0], s / h.lengthscale[1],
                                     s / h.lengthscale[2], s / h.lengthscale[3], g.Xs[o]);

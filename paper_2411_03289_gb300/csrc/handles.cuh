@@ -19,7 +19,7 @@ struct gpmppi_ctrl_s {
     gpmppi_gp gp = nullptr;
     int device = 0;
     int O = 0, P = 0, S = 0;
-    int mt = 1, n_upd = 1;
+    int n_upd = 1;
     uint64_t it = 0;
     uint64_t wait_ns = 2000000000ull;   // FP32 rollout: limit of each tile-copy wait
     int expire_first = 0;               // FP32 rollout: failure-detection hook
@@ -30,12 +30,6 @@ struct gpmppi_ctrl_s {
     float* costs = nullptr;       // K, used when the caller passes no costs array
     float* hs_U = nullptr;        // mppi_step_host staging: U_nom then U_new (2 x T x 2)
     float* hs_w = nullptr;        // mppi_step_host staging: weights (K)
-    // a terrain ensemble on the tensor cores: the stacked factor tiles and
-    // training set of its GPs (owned by the controller)
-    uint16_t* ens_hi = nullptr;
-    uint16_t* ens_lo = nullptr;
-    uint16_t* ens_mid = nullptr;
-    float* ens_xa = nullptr;
     float2* u_tilde = nullptr;    // T x K
     float* partial = nullptr;     // n_upd x T x 2 update partials, then n_upd x 2 block statistics
     unsigned int* counter = nullptr;
@@ -49,17 +43,26 @@ struct gpmppi_ctrl_s {
     gpm::GpSet gset{};
     void* ws_buf = nullptr;
     int ws_Ks = 0;
+    float* vbuf = nullptr;        // FP32 and nominal rollouts: rows of v = L^-1 k* of up to v_q queries
+    int v_q = 0;
+    int nsplit = 1;               // parts of a variance (tensor cores: var_tc_splits)
+    int nsm = 0;                  // SMs of the device
     unsigned int* err = nullptr;  // device status word written by the rollout
-    int stages = 2;               // per-warp TMA pipeline depth
-    CUtensorMap tmW;              // TMA map over the GP's W
-    gpm::MmaArgs mm{};              // tensor-core tiles (split precisions)
-    int fmt = -1;                 // 0 = FP16, 1 = BF16 split, -1 = FP32 path
-    bool cl = false;              // split precisions with N <= 512: the cluster rollout
-    gpm::ClArgs cla{};
-    // terrain ensemble (Eq. 3): M >= 2 GPs mixed with weights tw on the
-    // ensemble rollout; M = 1 is the single GP `gp`
+    int fmt = -1;                 // 0 = FP16, 1 = BF16, 2 = three-part BF16 split, -1 = FP32
+    // the batched rollout's tiles of this controller (made with its first batch)
+    gpm::MmaArgs mm{};
+    bool mm_made = false;
+    // a terrain ensemble's stacked factor tiles and training set (owned by the controller)
+    uint16_t* ens_hi = nullptr;
+    uint16_t* ens_lo = nullptr;
+    uint16_t* ens_mid = nullptr;
+    float* ens_xa = nullptr;
+    int kind = GPMPPI_KERNEL_FP32;   // reported by mppi_rollout_kind
+    int rps = 2;                  // reported by mppi_batch_layout
+    // terrain ensemble (Eq. 3): M >= 2 GPs mixed with weights tw ;
+    // M = 1 is the single GP `gp`
     int M = 1;
-    bool ens = false;             // runs the ensemble rollout
+    bool ens = false;
     gpmppi_gp tgp[gpm::kMaxTerrains] = {};
     float tw[gpm::kMaxTerrains] = {};
     // adjoint-rollout scratch (allocated by the first mppi_grad call)
@@ -77,4 +80,7 @@ namespace gpm {
 RolloutArgs make_rollout_args(gpmppi_ctrl c, const float* state, const float* U);
 // Records of the samples [s0, s0 + Ks) in the controller's workspace.
 QueryWs make_query_ws(gpmppi_ctrl c, int s0, int Ks);
+// Alg. 1 Step 1 of controller c: costs and perturbed controls of all samples.
+int make_mma_args(gpmppi_ctrl c);
+int launch_query_rollout(gpmppi_ctrl c, const RolloutArgs& a, const GpSet& gs, cudaStream_t st);
 }  // namespace gpm

@@ -213,95 +213,52 @@ __global__ void k_noise(uint32_t key0, uint32_t key1, uint32_t it0, uint32_t it1
 }
 
 // ---------------------------------------------------------------------------
-// Alg. 1 Step 2: mean and covariance along the updated controls (no noise),
-// one CTA; records Sigma_XY(k+1) for the next iteration's tightening.
+// Alg. 1 Step 2: the means along the updated controls (no noise), one CTA,
+// recorded for the variances and the covariance (tri.cu, stage_cost.cu).
 // ---------------------------------------------------------------------------
 constexpr int NOM_THREADS = 256;
 
-__device__ float nom_block_sum(float v, float* red) {
-    v = warp_sum(v);
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    __syncthreads();
-    if (l == 0) red[w] = v;
-    __syncthreads();
-    float s = 0.0f;
-    for (int i = 0; i < NOM_THREADS / 32; ++i) s += red[i];
-    return s;
-}
-
-__global__ void __launch_bounds__(NOM_THREADS) k_nominal(const RolloutArgs a, const float* __restrict__ Uc,
-                                                         float* __restrict__ sxy_out) {
-    extern __shared__ __align__(16) float ks[];   // N floats
-    __shared__ float red[NOM_THREADS / 32];
-    __shared__ float4 zsh;
+__global__ void __launch_bounds__(NOM_THREADS) k_nominal_mean(const RolloutArgs a, const float* __restrict__ Uc,
+                                                              const QueryWs ws) {
+    __shared__ float2 red[2][NOM_THREADS / 32];
     float mu[5] = {a.x0[0], a.x0[1], a.x0[2], a.x0[3], a.x0[4]};
-    float S[5][5] = {};
     const int tid = threadIdx.x;
     for (int k = 0; k < a.T; ++k) {
         const float ux = fminf(fmaxf(Uc[2 * k], a.umin0), a.umax0);
         const float uy = fminf(fmaxf(Uc[2 * k + 1], a.umin1), a.umax1);
-        if (tid == 0)
-            zsh = make_float4(mu[3] * a.zscale[0], mu[4] * a.zscale[1], ux * a.zscale[2],
-                              uy * a.zscale[3]);
-        __syncthreads();
-        const float4 z = zsh;
+        const float z0 = mu[3] * a.zscale[0], z1 = mu[4] * a.zscale[1], z2 = ux * a.zscale[2], z3 = uy * a.zscale[3];
         float mv = 0.0f, mw = 0.0f;
         for (int j = tid; j < a.N; j += NOM_THREADS) {
-            const float4 x = reinterpret_cast<const float4*>(a.Xs)[j];
-            const float e0 = z.x - x.x, e1 = z.y - x.y, e2 = z.z - x.z, e3 = z.w - x.w;
+            const float4 x = __ldg(reinterpret_cast<const float4*>(a.Xs) + j);
+            const float2 al = __ldg(reinterpret_cast<const float2*>(a.alpha) + j);
+            const float e0 = z0 - x.x, e1 = z1 - x.y, e2 = z2 - x.z, e3 = z3 - x.w;
             const float kv = a.sf2 * exp2f(-(e0 * e0 + e1 * e1 + e2 * e2 + e3 * e3));
-            ks[j] = kv;
-            mv = fmaf(kv, a.alpha[2 * j], mv);
-            mw = fmaf(kv, a.alpha[2 * j + 1], mw);
+            mv = fmaf(kv, al.x, mv);
+            mw = fmaf(kv, al.y, mw);
         }
-        mv = nom_block_sum(mv, red);
-        mw = nom_block_sum(mw, red);
-        float q = 0.0f;
-        for (int i = tid; i < a.N; i += NOM_THREADS) {
-            float v = 0.0f;
-            for (int j = 0; j <= i; ++j) v = fmaf(a.W[(size_t)j * a.Np + i], ks[j], v);
-            q = fmaf(v, v, q);
+        // (two buffers: one barrier a step)
+        mv = warp_sum(mv);
+        mw = warp_sum(mw);
+        if ((tid & 31) == 0) red[k & 1][tid >> 5] = make_float2(mv, mw);
+        __syncthreads();
+        mv = 0.0f;
+        mw = 0.0f;
+        for (int i = 0; i < NOM_THREADS / 32; ++i) {
+            mv += red[k & 1][i].x;
+            mw += red[k & 1][i].y;
         }
-        q = nom_block_sum(q, red);
-        const float s = fmaxf(0.0f, a.sf2 - q);
         // every thread carries the (identical) single-trajectory state
         float sn, cs;
         sincosf(mu[2], &sn, &cs);
-        float A[5][5] = {};
-        for (int i = 0; i < 5; ++i) A[i][i] = 1.0f;
-        A[0][2] = -a.dt * mu[3] * sn;
-        A[0][3] = a.dt * cs;
-        A[1][2] = a.dt * mu[3] * cs;
-        A[1][3] = a.dt * sn;
-        A[2][4] = a.dt;
-        A[3][3] = a.av;
-        A[4][4] = a.aw;
-        float B[5][5];
-        for (int i = 0; i < 5; ++i)
-            for (int j = 0; j < 5; ++j) {
-                float acc = 0.0f;
-                for (int l = 0; l < 5; ++l) acc = fmaf(A[i][l], S[l][j], acc);
-                B[i][j] = acc;
-            }
-        for (int i = 0; i < 5; ++i)
-            for (int j = 0; j < 5; ++j) {
-                float acc = 0.0f;
-                for (int l = 0; l < 5; ++l) acc = fmaf(B[i][l], A[j][l], acc);
-                S[i][j] = acc;
-            }
-        S[3][3] += s;
-        S[4][4] += s;
         const float nX = mu[0] + a.dt * mu[3] * cs, nY = mu[1] + a.dt * mu[3] * sn;
         const float nT = mu[2] + a.dt * mu[4];
         const float nV = mu[3] + a.kv * (ux - mu[3]) + mv;
         const float nW = mu[4] + a.kw * (uy - mu[4]) + mw;
-        mu[0] = nX; mu[1] = nY; mu[2] = nT; mu[3] = nV; mu[4] = nW;
         if (tid == 0) {
-            sxy_out[3 * k] = S[0][0];
-            sxy_out[3 * k + 1] = S[0][1];
-            sxy_out[3 * k + 2] = S[1][1];
+            ws.zq[k] = make_float4(mu[3], mu[4], ux, uy);
+            ws.st[k] = make_float4(nX, nY, nT, nV);
         }
-        __syncthreads();
+        mu[0] = nX; mu[1] = nY; mu[2] = nT; mu[3] = nV; mu[4] = nW;
     }
 }
 
@@ -358,11 +315,9 @@ int launch_noise(uint64_t seed, int K, int T, uint64_t it, float sv, float sw, f
     return GPMPPI_OK;
 }
 
-int launch_nominal(const RolloutArgs& a, float* sxy_out, cudaStream_t st) {
-    const int smem = (a.N > 0 ? a.N : 1) * (int)sizeof(float);
-    GPM_CUDA(cudaFuncSetAttribute(k_nominal, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+int launch_nominal_mean(const RolloutArgs& a, const QueryWs& ws, cudaStream_t st) {
     // a.U holds the updated controls for this launch
-    k_nominal<<<1, NOM_THREADS, smem, st>>>(a, a.U, sxy_out);
+    k_nominal_mean<<<1, NOM_THREADS, 0, st>>>(a, a.U, ws);
     GPM_CUDA(cudaGetLastError());
     return GPMPPI_OK;
 }

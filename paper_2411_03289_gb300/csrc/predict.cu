@@ -1,0 +1,146 @@
+// The GP posterior at M queries (gp_predict), FP32: the triangular product of
+// tri.cu, then one CTA a query sums the squares and the mean.
+// M = 20000, N = 1000: 0.50 ms (48 TFLOP/s) against 3.29 ms of a CTA per query that
+// read the whole factor.
+#include <mutex>
+
+#include "query.cuh"
+
+namespace gpm {
+namespace {
+
+struct PredArgs {
+    const float* Z;          // queries, M x 4
+    const float* Xs;         // GpDevice::Xs, alpha
+    const float* alpha;
+    const float* V;          // M x npad
+    float* mean;
+    float* var;
+    int M, N, npad;
+    float sf2;
+    float zscale[4];
+    int out;                 // the output, or -1 for both (shared hyper-parameters)
+};
+
+// Stream-ordered scratch of gp_predict: one memory pool per device, for every
+// stream and thread.  It keeps up to kPoolKeep bytes between calls (mapping the
+// 80 MB of 20000 queries at N = 1000 anew costs more than the call) while GP
+// handles exist, and is given back with the last of them.
+constexpr uint64_t kPoolKeep = 256ull << 20;
+constexpr int kMaxDevices = 64;
+std::mutex g_pool_mu;
+cudaMemPool_t g_pool[kMaxDevices] = {};
+int g_pool_users[kMaxDevices] = {};
+
+int scratch_pool(int device, cudaMemPool_t* out) {
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    if (!g_pool[device]) {
+        cudaMemPoolProps props = {};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = device;
+        GPM_CUDA(cudaMemPoolCreate(&g_pool[device], &props));
+        uint64_t keep = kPoolKeep;
+        GPM_CUDA(cudaMemPoolSetAttribute(g_pool[device], cudaMemPoolAttrReleaseThreshold, &keep));
+    }
+    *out = g_pool[device];
+    return GPMPPI_OK;
+}
+
+constexpr int ST = 128;
+
+__device__ float block_sum(float v, float* red) {
+    // deterministic: fixed shuffle tree, then warp partials summed in order
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+    __syncthreads();
+    if (l == 0) red[w] = v;
+    __syncthreads();
+    float s = 0.0f;
+    for (int i = 0; i < ST / 32; ++i) s += red[i];
+    return s;
+}
+
+__global__ void __launch_bounds__(ST) k_pred_sum(const PredArgs p) {
+    __shared__ float red[ST / 32];
+    const int q = blockIdx.x;
+    float zq[4];
+    for (int d = 0; d < 4; ++d) zq[d] = p.Z[q * (size_t)4 + d] * p.zscale[d];
+    const int o0 = p.out < 0 ? 0 : p.out, o1 = p.out < 0 ? 1 : p.out;
+    float m0 = 0.0f, m1 = 0.0f, qf = 0.0f;
+    for (int j = threadIdx.x; j < p.N; j += ST) {
+        const float4 x = reinterpret_cast<const float4*>(p.Xs)[j];
+        const float e0 = zq[0] - x.x, e1 = zq[1] - x.y, e2 = zq[2] - x.z, e3 = zq[3] - x.w;
+        const float k = p.sf2 * exp2f(-(e0 * e0 + e1 * e1 + e2 * e2 + e3 * e3));
+        m0 += k * p.alpha[2 * j + o0];
+        m1 += k * p.alpha[2 * j + o1];
+        const float v = p.V[(size_t)q * p.npad + j];
+        qf = fmaf(v, v, qf);
+    }
+    m0 = block_sum(m0, red);
+    m1 = block_sum(m1, red);
+    qf = block_sum(qf, red);
+    if (threadIdx.x == 0) {
+        const float v = fmaxf(0.0f, p.sf2 - qf);
+        p.mean[2 * (size_t)q + o0] = m0;
+        p.var[2 * (size_t)q + o0] = v;
+        p.mean[2 * (size_t)q + o1] = m1;
+        p.var[2 * (size_t)q + o1] = v;
+    }
+}
+
+}  // namespace
+
+void scratch_user(int device, int change) {
+    if (device < 0 || device >= kMaxDevices) return;
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    g_pool_users[device] += change;
+    if (g_pool_users[device] == 0 && g_pool[device]) cudaMemPoolTrimTo(g_pool[device], 0);
+}
+
+int launch_gp_predict(const GpDevice& g, const float* Z, int M, float* mean, float* var, cudaStream_t st) {
+    if (M == 0) return GPMPPI_OK;
+    // V in stream-ordered scratch (calls from several threads or streams share
+    // nothing), at most 1 GB: more queries go in pieces
+    size_t piece = g.npad ? ((size_t)1 << 28) / g.npad / 64 * 64 : (size_t)M;
+    if (piece > (size_t)M) piece = (size_t)M;
+    float* V = nullptr;
+    if (g.npad) {
+        cudaMemPool_t pool = nullptr;
+        if (g.device < 0 || g.device >= kMaxDevices) return fail(GPMPPI_ERR_UNSUPPORTED, "gp_predict: device number");
+        const int rc0 = scratch_pool(g.device, &pool);
+        if (rc0) return rc0;
+        GPM_CUDA(cudaMallocFromPoolAsync((void**)&V, sizeof(float) * piece * g.npad, pool, st));
+    }
+    int rc = GPMPPI_OK;
+    for (int o = 0; o < (g.shared ? 1 : 2) && rc == GPMPPI_OK; ++o)
+        for (size_t q0 = 0; q0 < (size_t)M && rc == GPMPPI_OK; q0 += piece) {
+            PredArgs p;
+            p.Z = Z + 4 * q0;
+            p.Xs = g.Xs[o];
+            p.alpha = g.alpha;
+            p.V = V;
+            p.mean = mean + 2 * q0;
+            p.var = var + 2 * q0;
+            p.M = (int)((size_t)M - q0 < piece ? (size_t)M - q0 : piece);
+            p.N = g.N;
+            p.npad = g.npad;
+            p.sf2 = g.sf2[o];
+            for (int d = 0; d < 4; ++d) p.zscale[d] = g.zscale[o][d];
+            p.out = g.shared ? -1 : o;
+            TriJob j = tri_forward(single_gp_set(g, o).gp[0], p.Z, p.M, V);
+            j.fusez = 1;
+            rc = launch_tri_forward(j, false, st);
+            if (rc) break;
+            k_pred_sum<<<p.M, ST, 0, st>>>(p);
+            const cudaError_t e = cudaGetLastError();
+            if (e != cudaSuccess) rc = cuda_fail(e, "gp_predict");
+        }
+    if (V) {
+        const cudaError_t e = cudaFreeAsync(V, st);
+        if (e != cudaSuccess && rc == GPMPPI_OK) rc = cuda_fail(e, "gp_predict: scratch");
+    }
+    return rc;
+}
+
+}  // namespace gpm

@@ -1,4 +1,5 @@
-// Fused MPPI rollout with the GP variance contraction on the tensor cores
+// Batched MPPI rollout: many controllers' sample tiles in one persistent launch,
+// the GP variance contraction on the tensor cores
 // (tcgen05, split 16-bit operands, FP32 accumulation in TMEM).
 //
 // Same method as the FP32 rollout (Alg. 1 Step 1: noise, clamp, GP mean and
@@ -42,7 +43,6 @@
 #include <cfloat>
 
 #include "common.cuh"
-#include "rollout_fp32_body.cuh"
 #include "tc05.cuh"
 
 namespace gpm {
@@ -181,7 +181,7 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
 // batched kernel allocates once per CTA).
 constexpr uint32_t kTmemAlloc = 0xFFFFFFFFu;
 
-template <int FMT, int R, bool TRACE>
+template <int FMT, int R>
 __device__ __forceinline__ void rollout_mma_body(const RolloutArgs& a, const MmaArgs& mm, int tile,
                                                  unsigned char* sm, uint32_t tmem_given) {
     constexpr int MTC = NPROD / R;
@@ -646,25 +646,6 @@ __device__ __forceinline__ void rollout_mma_body(const RolloutArgs& a, const Mma
         stage += goal_cost(a, k, mu0, mu1);                           // Eq. 12 goal terms
         cost += stage;
         disc *= 0.9f;
-        if (TRACE && active && u == 0) {
-            const size_t sk = (size_t)s_me * a.T + k;
-            if (a.tr_mu) {
-                float* o = a.tr_mu + sk * 5;
-                o[0] = mu0; o[1] = mu1; o[2] = mu2; o[3] = mu3; o[4] = mu4;
-            }
-            if (a.tr_sig) {
-                float* o = a.tr_sig + sk * 15;
-                o[0] = S00; o[1] = S01; o[2] = S02; o[3] = S03; o[4] = S04;
-                o[5] = S11; o[6] = S12; o[7] = S13; o[8] = S14;
-                o[9] = S22; o[10] = S23; o[11] = S24;
-                o[12] = S33; o[13] = S34; o[14] = S44;
-            }
-            if (a.tr_stage) a.tr_stage[sk] = stage;
-            if (a.tr_margin) {
-                a.tr_margin[sk * 2] = lmargin;
-                a.tr_margin[sk * 2 + 1] = (a.O > 0) ? omargin : __int_as_float(0x7f800000);
-            }
-        }
     }
     if (active && u == 0 && a.costs) a.costs[s_me] = cost;
     // after an abort, give copies and MMAs in flight a bounded time to land
@@ -681,18 +662,17 @@ __device__ __forceinline__ void rollout_mma_body(const RolloutArgs& a, const Mma
     if (tmem_given == kTmemAlloc && warp == 0 && NB > 0) tc::tmem_dealloc(taddr, 512);
 }
 
-template <int FMT, int R, bool TRACE>
+template <int FMT, int R>
 __global__ void __launch_bounds__(THREADS, 1) k_rollout_mma(const RolloutArgs a, const MmaArgs mm) {
     extern __shared__ __align__(1024) unsigned char sm[];
-    rollout_mma_body<FMT, R, TRACE>(a, mm, blockIdx.x, sm, kTmemAlloc);
+    rollout_mma_body<FMT, R>(a, mm, blockIdx.x, sm, kTmemAlloc);
 }
 
 // ---------------------------------------------------------------------------
 // Batched step of many controllers as ONE persistent launch: one CTA per SM
 // takes items from an atomic work queue until it is empty.  An item is
-// (controller, sample tile, kind, producer threads per sample); kind 0 runs the
-// FP32 CUDA-core rollout body on warps 0-7 (warps 8-9 wait), kinds 1 and 2 the
-// tensor-core body with FP16 or BF16 split operands.  The queue holds the
+// (controller, sample tile, operand format, producer threads per sample).  The
+// queue holds the
 // items in decreasing order of their estimated time (longest first).  The CTA
 // holds its 512 TMEM columns for the whole launch; between items every role of
 // the CTA meets at a barrier and the previous item's mbarriers are
@@ -702,18 +682,8 @@ __device__ __forceinline__ void mbar_inval(uint64_t* bar) {
     asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(tc::smem_addr(bar)) : "memory");
 }
 
-__device__ __forceinline__ int fp32_mtp(int Np) { return Np <= 1024 ? 32 : (Np <= 2048 ? 16 : 8); }
-
 // invalidate the mbarriers an item initialised (thread 0, after every role is done)
-__device__ void inval_item_barriers(const RolloutArgs& a, const MmaArgs& mm, int kind, unsigned char* sm) {
-    if (kind == 0) {
-        const int mtp = fp32_mtp(a.Np);
-        const int off = mtp == 32 ? f32r::Smem<32>::bars(a.Np, a.stages)
-                                  : (mtp == 16 ? f32r::Smem<16>::bars(a.Np, a.stages) : f32r::Smem<8>::bars(a.Np, a.stages));
-        uint64_t* bars = reinterpret_cast<uint64_t*>(sm + off);
-        for (int i = 0; i < f32r::WARPS * a.stages; ++i) mbar_inval(bars + i);
-        return;
-    }
+__device__ void inval_item_barriers(const RolloutArgs& a, const MmaArgs& mm, unsigned char* sm) {
     const MLayout L = mma_layout(mm.stages, mm.nblocks * BLK, mm.scene_smem ? a.S : 0, mm.scene_smem ? a.O : 0,
                                  pairs_per_pass(mm.lo_set), mm.parts, mm.tr.M);
     uint64_t* a_full = reinterpret_cast<uint64_t*>(sm + L.bars);
@@ -731,17 +701,11 @@ __device__ void inval_item_barriers(const RolloutArgs& a, const MmaArgs& mm, int
 template <int FMT, int R>
 __device__ __noinline__ void persistent_mma_item(const RolloutArgs& a, const MmaArgs& mm, int tile,
                                                  unsigned char* sm, uint32_t taddr) {
-    rollout_mma_body<FMT, R, false>(a, mm, tile, sm, taddr);
+    rollout_mma_body<FMT, R>(a, mm, tile, sm, taddr);
 }
-template <int MTP>
-__device__ __noinline__ void persistent_fp32_item(const RolloutArgs& a, const CUtensorMap* tm, int tile,
-                                                  unsigned char* sm) {
-    f32r::rollout_fp32_body<MTP, false>(a, tm, tile, sm);
-}
-
 __global__ void __launch_bounds__(THREADS, 1)
     k_rollout_persistent(const RolloutArgs* __restrict__ args, const MmaArgs* __restrict__ mms,
-                         const CUtensorMap* __restrict__ tmaps, const int4* __restrict__ items, int nitems,
+                         const int4* __restrict__ items, int nitems,
                          unsigned int* __restrict__ head, int ctl_off) {
     // no static shared memory (it would move the dynamic region off the
     // alignment the bulk and tensor copies need): the CTA's own words (TMEM
@@ -766,7 +730,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         if (tid == 0) {
             if (prev >= 0) {
                 const int4 pi = items[prev];
-                inval_item_barriers(args[pi.x], mms[pi.x], pi.z, sm);
+                inval_item_barriers(args[pi.x], mms[pi.x], sm);
             }
             cur = (int)atomicAdd(head, 1u);
         }
@@ -775,28 +739,19 @@ __global__ void __launch_bounds__(THREADS, 1)
         if (item >= nitems) break;
         const int4 it = items[item];
         const RolloutArgs& a = args[it.x];
+        const MmaArgs& mm = mms[it.x];
         if (it.z == 0) {
-            if (warp < f32r::WARPS) {
-                const int mtp = fp32_mtp(a.Np);
-                if (mtp == 32) persistent_fp32_item<32>(a, tmaps + it.x, it.y, sm);
-                else if (mtp == 16) persistent_fp32_item<16>(a, tmaps + it.x, it.y, sm);
-                else persistent_fp32_item<8>(a, tmaps + it.x, it.y, sm);
-            }
+            if (it.w == 2) persistent_mma_item<0, 2>(a, mm, it.y, sm, taddr);
+            else if (it.w == 4) persistent_mma_item<0, 4>(a, mm, it.y, sm, taddr);
+            else persistent_mma_item<0, 8>(a, mm, it.y, sm, taddr);
+        } else if (it.z == 1) {
+            if (it.w == 2) persistent_mma_item<1, 2>(a, mm, it.y, sm, taddr);
+            else if (it.w == 4) persistent_mma_item<1, 4>(a, mm, it.y, sm, taddr);
+            else persistent_mma_item<1, 8>(a, mm, it.y, sm, taddr);
         } else {
-            const MmaArgs& mm = mms[it.x];
-            if (it.z == 1) {
-                if (it.w == 2) persistent_mma_item<0, 2>(a, mm, it.y, sm, taddr);
-                else if (it.w == 4) persistent_mma_item<0, 4>(a, mm, it.y, sm, taddr);
-                else persistent_mma_item<0, 8>(a, mm, it.y, sm, taddr);
-            } else if (it.z == 2) {
-                if (it.w == 2) persistent_mma_item<1, 2>(a, mm, it.y, sm, taddr);
-                else if (it.w == 4) persistent_mma_item<1, 4>(a, mm, it.y, sm, taddr);
-                else persistent_mma_item<1, 8>(a, mm, it.y, sm, taddr);
-            } else {
-                if (it.w == 2) persistent_mma_item<2, 2>(a, mm, it.y, sm, taddr);
-                else if (it.w == 4) persistent_mma_item<2, 4>(a, mm, it.y, sm, taddr);
-                else persistent_mma_item<2, 8>(a, mm, it.y, sm, taddr);
-            }
+            if (it.w == 2) persistent_mma_item<2, 2>(a, mm, it.y, sm, taddr);
+            else if (it.w == 4) persistent_mma_item<2, 4>(a, mm, it.y, sm, taddr);
+            else persistent_mma_item<2, 8>(a, mm, it.y, sm, taddr);
         }
         // every role of this CTA is done with the item (TMEM reads included)
         tc::fence_before_sync();
@@ -810,14 +765,13 @@ __global__ void __launch_bounds__(THREADS, 1)
 
 }  // namespace
 
-int launch_rollout_persistent(const RolloutArgs* args, const MmaArgs* mms, const CUtensorMap* tmaps,
-                              const int4* items, int nitems, unsigned int* head, int grid, int smem,
+int launch_rollout_persistent(const RolloutArgs* args, const MmaArgs* mms, const int4* items, int nitems, unsigned int* head, int grid, int smem,
                               cudaStream_t st) {
     if (nitems == 0) return GPMPPI_OK;
     const int ctl_off = ((smem + 15) / 16) * 16;
     const int total = ctl_off + 16;
     GPM_CUDA(cudaFuncSetAttribute(k_rollout_persistent, cudaFuncAttributeMaxDynamicSharedMemorySize, total));
-    k_rollout_persistent<<<grid, THREADS, total, st>>>(args, mms, tmaps, items, nitems, head, ctl_off);
+    k_rollout_persistent<<<grid, THREADS, total, st>>>(args, mms, items, nitems, head, ctl_off);
     GPM_CUDA(cudaGetLastError());
     return GPMPPI_OK;
 }
@@ -826,7 +780,7 @@ int rollout_mma_stages(int NpM, int S, int O, int smem_optin, int lo_set, int pa
     return mma_stages(NpM, S, O, smem_optin, pairs_per_pass(lo_set), parts, M);
 }
 
-int launch_rollout_mma(const RolloutArgs& a, const MmaArgs& mm, int fmt, bool trace, cudaStream_t st) {
+int launch_rollout_mma(const RolloutArgs& a, const MmaArgs& mm, int fmt, cudaStream_t st) {
     const int nstage = mm.stages;
     if (nstage < 2 || nstage > NSTAGE) return fail(GPMPPI_ERR_INVALID_ARG, "rollout: bad MMA pipeline depth");
     if (mm.rps != 2 && mm.rps != 4 && mm.rps != 8) return fail(GPMPPI_ERR_INVALID_ARG, "rollout: bad threads per sample");
@@ -838,25 +792,21 @@ int launch_rollout_mma(const RolloutArgs& a, const MmaArgs& mm, int fmt, bool tr
                                 pairs_per_pass(mm.lo_set), mm.parts, mm.tr.M).total;
     const int mtc = NPROD / mm.rps;
     const int grid = (a.K + mtc - 1) / mtc;
-#define GPM_LAUNCH_MMA(F, RR, TR)                                                                 \
+#define GPM_LAUNCH_MMA(F, RR)                                                                     \
     do {                                                                                          \
-        auto kern = k_rollout_mma<F, RR, TR>;                                                     \
+        auto kern = k_rollout_mma<F, RR>;                                                         \
         GPM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));  \
         kern<<<grid, THREADS, smem, st>>>(a, mm);                                                 \
     } while (0)
-#define GPM_LAUNCH_MMA_R(F, TR)                          \
-    do {                                                 \
-        if (mm.rps == 2) GPM_LAUNCH_MMA(F, 2, TR);       \
-        else if (mm.rps == 4) GPM_LAUNCH_MMA(F, 4, TR);  \
-        else GPM_LAUNCH_MMA(F, 8, TR);                   \
+#define GPM_LAUNCH_MMA_R(F)                          \
+    do {                                             \
+        if (mm.rps == 2) GPM_LAUNCH_MMA(F, 2);       \
+        else if (mm.rps == 4) GPM_LAUNCH_MMA(F, 4);  \
+        else GPM_LAUNCH_MMA(F, 8);                   \
     } while (0)
-    if (fmt == 0) {
-        if (trace) GPM_LAUNCH_MMA_R(0, true); else GPM_LAUNCH_MMA_R(0, false);
-    } else if (fmt == 1) {
-        if (trace) GPM_LAUNCH_MMA_R(1, true); else GPM_LAUNCH_MMA_R(1, false);
-    } else {
-        if (trace) GPM_LAUNCH_MMA_R(2, true); else GPM_LAUNCH_MMA_R(2, false);
-    }
+    if (fmt == 0) GPM_LAUNCH_MMA_R(0);
+    else if (fmt == 1) GPM_LAUNCH_MMA_R(1);
+    else GPM_LAUNCH_MMA_R(2);
 #undef GPM_LAUNCH_MMA_R
 #undef GPM_LAUNCH_MMA
     GPM_CUDA(cudaGetLastError());

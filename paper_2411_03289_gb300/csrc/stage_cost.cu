@@ -25,7 +25,8 @@ constexpr int CK = 16;                   // steps per chunk
 constexpr int SU = 8;                    // lane segments per round
 
 struct ScoreScale {
-    int M;
+    int M, nsplit;
+    bool two;            // the variances are added in a rounding of their own (FP32 terrain ensembles)
     float w2[kMaxTerrains], sf2[kMaxTerrains], qscale[kMaxTerrains];
 };
 
@@ -38,6 +39,40 @@ struct SLayout {
     static constexpr int disc = stage + 2 * CK * 32 * 4;     // CK floats
     static constexpr int obst = disc + 2 * CK * 4;           // O x 3 floats
 };
+
+// Sigma' = A Sigma A^T + diag(0, 0, 0, s, s) (Eq. 10), A the Jacobian of the
+// unicycle step at heading (sn, cs) and speed v
+__device__ __forceinline__ void cov_step(const RolloutArgs& a, bool two, float sn, float cs, float v, float s, float& S00,
+                                         float& S01, float& S02, float& S03, float& S04, float& S11, float& S12,
+                                         float& S13, float& S14, float& S22, float& S23, float& S24, float& S33,
+                                         float& S34, float& S44) {
+    const float a02 = -a.dt * v * sn, a03 = a.dt * cs;
+    const float a12 = a.dt * v * cs, a13 = a.dt * sn;
+    // B = A Sigma (rows), then Sigma' = B A^T + diag(0,0,0,s,s)
+    const float B00 = S00 + a02 * S02 + a03 * S03, B01 = S01 + a02 * S12 + a03 * S13,
+                B02 = S02 + a02 * S22 + a03 * S23, B03 = S03 + a02 * S23 + a03 * S33,
+                B04 = S04 + a02 * S24 + a03 * S34;
+    const float B11 = S11 + a12 * S12 + a13 * S13, B12 = S12 + a12 * S22 + a13 * S23,
+                B13 = S13 + a12 * S23 + a13 * S33, B14 = S14 + a12 * S24 + a13 * S34;
+    const float B22 = S22 + a.dt * S24, B23 = S23 + a.dt * S34, B24 = S24 + a.dt * S44;
+    const float B33 = a.av * S33, B34 = a.av * S34;
+    const float B44 = a.aw * S44;
+    S00 = B00 + a02 * B02 + a03 * B03;
+    S01 = B01 + a12 * B02 + a13 * B03;
+    S02 = B02 + a.dt * B04;
+    S03 = a.av * B03;
+    S04 = a.aw * B04;
+    S11 = B11 + a12 * B12 + a13 * B13;
+    S12 = B12 + a.dt * B14;
+    S13 = a.av * B13;
+    S14 = a.aw * B14;
+    S22 = B22 + a.dt * B24;
+    S23 = a.av * B23;
+    S24 = a.aw * B24;
+    S33 = two ? __fadd_rn(__fmul_rn(a.av, B33), s) : a.av * B33 + s;
+    S34 = a.aw * B34;
+    S44 = two ? __fadd_rn(__fmul_rn(a.aw, B44), s) : a.aw * B44 + s;
+}
 
 template <bool TRACE>
 __global__ void __launch_bounds__(ST) k_stage_cost(const RolloutArgs a, const ScoreScale sc, const QueryWs ws) {
@@ -77,8 +112,13 @@ __global__ void __launch_bounds__(ST) k_stage_cost(const RolloutArgs a, const Sc
                 v = p.w;
             }
             float s = 0.0f;
-            for (int t = 0; t < sc.M; ++t)
-                s += sc.w2[t] * fmaxf(0.0f, sc.sf2[t] - sc.qscale[t] * ws.q[t * Q + (size_t)k * Ks + l]);
+            const float* qp = ws.q + (size_t)k * Ks + l;
+            for (int t = 0; t < sc.M; ++t) {
+                float q = *qp;
+                qp += Q;
+                for (int j = 1; j < sc.nsplit; ++j, qp += Q) q += *qp;
+                s += sc.w2[t] * fmaxf(0.0f, sc.sf2[t] - sc.qscale[t] * q);
+            }
             float sn, cs;
             sincosf(th, &sn, &cs);
             pre[((c & 1) * CK + i) * 32 + lane] = make_float4(sn, cs, v, s);
@@ -95,32 +135,7 @@ __global__ void __launch_bounds__(ST) k_stage_cost(const RolloutArgs a, const Sc
                 if (k >= T) break;
                 const float4 p = pre[((c & 1) * CK + i) * 32 + lane];
                 const float sn = p.x, cs = p.y, v = p.z, s = p.w;
-                const float a02 = -a.dt * v * sn, a03 = a.dt * cs;
-                const float a12 = a.dt * v * cs, a13 = a.dt * sn;
-                // B = A Sigma (rows), then Sigma' = B A^T + diag(0,0,0,s,s)
-                const float B00 = S00 + a02 * S02 + a03 * S03, B01 = S01 + a02 * S12 + a03 * S13,
-                            B02 = S02 + a02 * S22 + a03 * S23, B03 = S03 + a02 * S23 + a03 * S33,
-                            B04 = S04 + a02 * S24 + a03 * S34;
-                const float B11 = S11 + a12 * S12 + a13 * S13, B12 = S12 + a12 * S22 + a13 * S23,
-                            B13 = S13 + a12 * S23 + a13 * S33, B14 = S14 + a12 * S24 + a13 * S34;
-                const float B22 = S22 + a.dt * S24, B23 = S23 + a.dt * S34, B24 = S24 + a.dt * S44;
-                const float B33 = a.av * S33, B34 = a.av * S34;
-                const float B44 = a.aw * S44;
-                S00 = B00 + a02 * B02 + a03 * B03;
-                S01 = B01 + a12 * B02 + a13 * B03;
-                S02 = B02 + a.dt * B04;
-                S03 = a.av * B03;
-                S04 = a.aw * B04;
-                S11 = B11 + a12 * B12 + a13 * B13;
-                S12 = B12 + a.dt * B14;
-                S13 = a.av * B13;
-                S14 = a.aw * B14;
-                S22 = B22 + a.dt * B24;
-                S23 = a.av * B23;
-                S24 = a.aw * B24;
-                S33 = a.av * B33 + s;
-                S34 = a.aw * B34;
-                S44 = a.aw * B44 + s;
+                cov_step(a, sc.two, sn, cs, v, s, S00, S01, S02, S03, S04, S11, S12, S13, S14, S22, S23, S24, S33, S34, S44);
                 float xx = S00, xy = S01, yy = S11;
                 if (a.nom_sxy) {
                     xx = __ldg(a.nom_sxy + 3 * k);
@@ -229,11 +244,51 @@ __global__ void __launch_bounds__(ST) k_stage_cost(const RolloutArgs a, const Sc
     }
 }
 
+// Alg. 1 Step 2: the covariance along the nominal trajectory, one warp.  Lanes
+// load 32 steps' states and variances at a time; every lane carries the
+// recurrence, lane 0 records Sigma_XY after each step.
+__global__ void __launch_bounds__(32) k_nominal_cov(const RolloutArgs a, float sf2, float qscale, const QueryWs ws,
+                                                    float* __restrict__ sxy) {
+    const int lane = threadIdx.x;
+    grid_wait();
+    float S00 = 0, S01 = 0, S02 = 0, S03 = 0, S04 = 0, S11 = 0, S12 = 0, S13 = 0, S14 = 0, S22 = 0, S23 = 0, S24 = 0,
+          S33 = 0, S34 = 0, S44 = 0;
+    for (int k0 = 0; k0 < a.T; k0 += 32) {
+        const int kl = min(k0 + lane, a.T - 1);
+        float th = a.x0[2], vl = a.x0[3];
+        if (kl > 0) {
+            const float4 p = ws.st[kl - 1];
+            th = p.z;
+            vl = p.w;
+        }
+        const float sl = fmaxf(0.0f, sf2 - qscale * ws.q[kl]);
+        float snl, csl;
+        sincosf(th, &snl, &csl);
+        for (int i = 0; i < 32 && k0 + i < a.T; ++i) {
+            const float sn = __shfl_sync(0xffffffffu, snl, i), cs = __shfl_sync(0xffffffffu, csl, i);
+            const float v = __shfl_sync(0xffffffffu, vl, i), s = __shfl_sync(0xffffffffu, sl, i);
+            cov_step(a, false, sn, cs, v, s, S00, S01, S02, S03, S04, S11, S12, S13, S14, S22, S23, S24, S33, S34, S44);
+            if (lane == 0) {
+                sxy[3 * (k0 + i)] = S00;
+                sxy[3 * (k0 + i) + 1] = S01;
+                sxy[3 * (k0 + i) + 2] = S11;
+            }
+        }
+    }
+}
+
 }  // namespace
 
-int launch_stage_cost(const RolloutArgs& a, const GpSet& gs, const QueryWs& ws, cudaStream_t st) {
+int launch_nominal_cov(const RolloutArgs& a, const GpSet& gs, const QueryWs& ws, float* sxy_out, cudaStream_t st) {
+    GPM_CUDA(launch_ex(k_nominal_cov, dim3(1), 32, 0, st, true, 1u, a, gs.gp[0].sf2, gs.gp[0].qscale, ws, sxy_out));
+    return GPMPPI_OK;
+}
+
+int launch_stage_cost(const RolloutArgs& a, const GpSet& gs, const QueryWs& ws, bool ensemble, cudaStream_t st) {
     ScoreScale sc = {};
     sc.M = gs.M;
+    sc.nsplit = ws.nsplit;
+    sc.two = ensemble;
     for (int t = 0; t < gs.M; ++t) {
         sc.w2[t] = gs.gp[t].w * gs.gp[t].w;
         sc.sf2[t] = gs.gp[t].sf2;
