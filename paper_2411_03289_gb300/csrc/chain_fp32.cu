@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(CT) k_chain32(const RolloutArgs a, const GpSet
             const float z0 = mu3 * P.zscale[0], z1 = mu4 * P.zscale[1], z2 = ut.x * P.zscale[2], z3 = ut.y * P.zscale[3];
             const float2* al = reinterpret_cast<const float2*>(xs + P.N);
             float mv = 0.0f, mw = 0.0f, cv = 0.0f, cw = 0.0f;
-#pragma unroll 2
+#pragma unroll 4
             for (int j = g; j < P.N; j += G) {
                 const float4 x = SMEM ? xs[j] : __ldg(reinterpret_cast<const float4*>(P.Xs) + j);
                 const float2 b = SMEM ? al[j] : __ldg(reinterpret_cast<const float2*>(P.alpha) + j);

@@ -23,9 +23,8 @@
 //   warp 20      rank 0 issues the MMAs of both CTAs; rank 1 tells it when its
 //                factor piece of a stage is in place
 //   warp 21      factor pieces and training points by bulk copies
-//   warps 22-23  make a stage's rows visible to the tensor core, in turn: the
-//                proxy fence takes about 1300 clocks here, a stage's MMAs 768,
-//                so that fences in the warps that make the rows set the pace
+//   warps 22-23  make a stage's rows visible to the tensor core and tell rank 0,
+//                in turn (in the warps that make the rows it cost 6 %)
 // What bounds it: the tensor pipe (three or six split products of the
 // triangle).
 #include <cuda_bf16.h>
@@ -122,8 +121,11 @@ __device__ __forceinline__ uint32_t mapa(const void* p, uint32_t rank) {
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(tc::smem_addr(p)), "r"(rank));
     return r;
 }
+// Arrive on a barrier of either CTA.  What it announces is operands of the async
+// proxy (behind a proxy fence, or bulk copies that have landed) or reads that are
+// done, so the arrival needs no cluster-scope release: with one it took 900 clocks.
 __device__ __forceinline__ void arrive_cluster(uint32_t bar) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 __device__ __forceinline__ void arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_addr(bar)) : "memory");
@@ -499,23 +501,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT, 1) k_var_tc(cons
         // ---------------- factor pieces and training points -------------------------
         // The points of a stage are fetched up to XR stages ahead: their slot is
         // free once the MMAs XR stages earlier are done.
-        int xi = pair, xpi = 0, xc = 0;                     // next stage whose points are fetched
+        int xi = pair, xpi = 0;                             // item and number of its next pass
+        int xc = 0, xns = 0;                                // stage and stages of the pass being fetched
+        const float* xsrc = nullptr;
         uint32_t xn = 0;
-        auto fetch_x = [&]() {
-            while (xi < nitems) {
+        auto next_x_pass = [&]() {
+            xc = xns = 0;
+            while (xi < nitems && xns == 0) {
                 const int ts = xi / ntiles;
                 const GpSet::One& G = gs.gp[ts / job.nsplit];
                 const int p = split_pass(pass_count(G.N), job.nsplit, ts % job.nsplit, xpi);
-                if (p >= 0 && xc < pass_stages(G.N, p)) {
-                    uint64_t* bar = x_full + xn % XR;
-                    tc::mbar_expect_tx(bar, KC * 16);
-                    bulk_g2s(tsm + L::x + (xn % XR) * (KC * 16), G.xq + (size_t)xc * (KC * 4), KC * 16, bar);
-                    ++xc;
-                    ++xn;
-                    return;
-                }
-                xc = 0;
                 if (p >= 0) {
+                    xns = pass_stages(G.N, p);
+                    xsrc = G.xq;
                     ++xpi;
                 } else {
                     xpi = 0;
@@ -523,6 +521,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT, 1) k_var_tc(cons
                 }
             }
         };
+        auto fetch_x = [&]() {
+            if (xns == 0) return;
+            uint64_t* bar = x_full + xn % XR;
+            tc::mbar_expect_tx(bar, KC * 16);
+            bulk_g2s(tsm + L::x + (xn % XR) * (KC * 16), xsrc + (size_t)xc * (KC * 4), KC * 16, bar);
+            ++xn;
+            if (++xc == xns) next_x_pass();
+        };
+        next_x_pass();
         for (int i = 0; i < XR; ++i) fetch_x();
         for (int item = pair; item < nitems && ok; item += npairs) {
             const int ts = item / ntiles;
