@@ -10,21 +10,21 @@
 // A pair of CTAs (cluster of two, one pair per SM pair, persistent) takes 256
 // queries, 128 in each CTA, and the factor's columns in passes of 256.  The MMAs
 // are cta_group::2, M = 256 x N <= 256 x K = 16: each CTA stages its own 128
-// kernel rows (A) and half of the factor piece (B), so a 32-point stage moves
-// 16 KiB of factor into each SM instead of 32 and shared memory feeds A and B
-// at half its bandwidth.  Columns above the diagonal are cut off by 64s (MMAs
-// of N = 256, 192, 128, 64 in a pass's last eight stages).
+// kernel rows (A) and half of the factor piece (B), so each SM takes in half of
+// the factor's bytes and shared memory feeds A and B at half its bandwidth.
+// Columns above the diagonal are cut off by 64s (MMAs of N = 256, 192, 128, 64
+// over a pass's last 256 points).
 //   warps 0-15   kernel rows, eight warps a stage in turn: a thread makes 8 points
-//                for two queries, so that a training point read from shared
-//                memory serves 64 of them a warp
+//                for two or four queries, so that a training point read from
+//                shared memory serves 64 or 128 of them a warp
 //   warps 16-19  squares: 64 columns as soon as their last MMA is done (the
-//                diagonal ends 0-63 six stages before 192-255), so that only the
+//                diagonal ends 0-63 192 points before 192-255), so that only the
 //                last quarter of a pass is read with the tensor pipe idle
 //   warp 20      rank 0 issues the MMAs of both CTAs; rank 1 tells it when its
 //                factor piece of a stage is in place
 //   warp 21      factor pieces and training points by bulk copies
-//   warps 22-23  make a stage's rows visible to the tensor core and tell rank 0,
-//                in turn (in the warps that make the rows it cost 6 %)
+//   warp 22      makes a stage's rows visible to the tensor core and tells rank 0
+//                (in the warps that make the rows it cost 6 %)
 // What bounds it: the tensor pipe (three or six split products of the
 // triangle).
 #include <cuda_bf16.h>
@@ -40,22 +40,25 @@ using namespace qr;
 constexpr int QM = 128;              // queries per CTA
 constexpr int PASS = 256;            // factor columns per pass
 constexpr int QUART = 64;            // columns per step of the diagonal
-constexpr int KC = 32;               // training points per stage
 constexpr int EPI_WARP = 16, MMA_WARP = 20, LOAD_WARP = 21;
-constexpr int NT = 768;              // threads
-constexpr int XR = 16;               // ring of the stages' training points
+constexpr int NT = 736;              // threads
+constexpr int XR = 8;                // ring of the stages' training points
+// training points per stage: 64 where the rings then hold three stages, which
+// halves every role's hand-offs per point
+__host__ __device__ constexpr int stage_points(int parts) { return parts == 2 ? 64 : 32; }
 constexpr uint32_t LO_COL = 256;     // TMEM column of the small products' set
 constexpr uint64_t kWaitNs = 2000000000ull;
 
 template <int PARTS>
 struct TcLayout {
-    static constexpr int na = PARTS == 2 ? 6 : 4, nb = PARTS == 2 ? 6 : 4;
-    static constexpr int a_part = QM * KC * 2;                    // kernel rows, one part
-    static constexpr int b_part = (PASS / 2) * KC * 2;            // factor piece (this CTA's half), one part
+    static constexpr int kc = stage_points(PARTS);
+    static constexpr int na = PARTS == 2 ? 3 : 4, nb = PARTS == 2 ? 3 : 4;
+    static constexpr int a_part = QM * kc * 2;                    // kernel rows, one part
+    static constexpr int b_part = (PASS / 2) * kc * 2;            // factor piece (this CTA's half), one part
     static constexpr int a_stage = PARTS * a_part, b_stage = PARTS * b_part;
     static constexpr int b = na * a_stage;
     static constexpr int x = b + nb * b_stage;
-    static constexpr int bars = x + XR * KC * 16;
+    static constexpr int bars = x + XR * kc * 16;
     // a_raw, a_full [na], b_full, done [nb], x_full [XR], q_done [4], t_free
     static constexpr int tslot = bars + 8 * (2 * na + 2 * nb + XR + 5);
     static constexpr int abort_flag = tslot + 4;
@@ -66,18 +69,21 @@ struct TcLayout {
 // pass p: columns 256 p .. 256 p + hi - 1, stages 0 .. pass_stages - 1; stage c
 // multiplies columns lo(c) .. hi - 1 (those below hold no point of the stage)
 __host__ __device__ inline int pass_count(int N) { return (N + PASS - 1) / PASS; }
-__host__ __device__ inline int pass_stages(int N, int p) {
-    const int n = (N + KC - 1) / KC;
-    return 8 * (p + 1) < n ? 8 * (p + 1) : n;
+__host__ __device__ inline int pass_stages(int N, int p, int kc) {
+    const int n = (N + kc - 1) / kc, full = PASS / kc * (p + 1);
+    return full < n ? full : n;
 }
 __host__ __device__ inline int pass_hi(int N, int p) {
     const int n = (N - PASS * p + QUART - 1) / QUART * QUART;
     return n < PASS ? n : PASS;
 }
-__host__ __device__ inline int stage_lo(int p, int c) { return c > 8 * p ? QUART * ((c - 8 * p) >> 1) : 0; }
-// position of (pass p, stage 0) in the packed factor, in columns x stages (only
+__host__ __device__ inline int stage_lo(int p, int c, int kc) {
+    const int d = kc * c - PASS * p;
+    return d > 0 ? QUART * (d / QUART) : 0;
+}
+// position of (pass p, stage 0) in the packed factor, in columns x points (only
 // the last pass is narrower, and nothing follows it)
-__host__ __device__ inline size_t pass_base(int p) { return (size_t)1024 * p * (p - 1) + (size_t)1280 * p; }
+__host__ __device__ inline size_t pass_base(int p) { return (size_t)32768 * p * (p - 1) + (size_t)40960 * p; }
 
 // The passes a split of a GP takes: dealt back and forth, largest first.
 __host__ __device__ inline int split_pass(int np, int nsplit, int split, int i) {
@@ -178,7 +184,7 @@ __device__ __forceinline__ void commit2_elect(uint64_t* bar) {
         : "memory");
 }
 
-// One stage (two K-steps) of the two-part split: A_hi B_hi into d, A_hi B_lo and
+// Two K-steps of the two-part split: A_hi B_hi into d, A_hi B_lo and
 // A_lo B_hi into d + LO_COL; the second K-step's operands sa and sb further on.
 // The first product of each set accumulates only if acc != 0.
 __device__ __forceinline__ void stage_split2(uint32_t d, uint64_t ah, uint64_t al, uint64_t bh, uint64_t bl,
@@ -227,7 +233,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT, 1) k_var_tc(cons
     extern __shared__ __align__(1024) unsigned char tsm[];
     constexpr int PARTS = FMT == 2 ? 3 : 2;
     using L = TcLayout<PARTS>;
-    constexpr int NA = L::na, NBP = L::nb;
+    constexpr int NA = L::na, NBP = L::nb, KC = L::kc;
     uint64_t* a_raw = reinterpret_cast<uint64_t*>(tsm + L::bars);
     uint64_t* a_full = a_raw + NA;
     uint64_t* b_full = a_full + NA;
@@ -289,7 +295,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT, 1) k_var_tc(cons
 
     if (warp < EPI_WARP) {
         // ---------------- kernel rows --------------------------------------------
-        const int slab = warp & 3, m0 = 64 * ((warp >> 2) & 1) + lane;
+        constexpr int SLABS = KC / 8, NQ = SLABS / 2;       // slabs of 8 points; queries per thread
+        const int slab = warp % SLABS, m0 = 32 * NQ * ((warp & 7) / SLABS) + lane;
         const uint32_t turn = (uint32_t)(warp >> 3);        // the stages this warp takes: n = turn (mod 2)
         grid_wait();
         const float4* zp = reinterpret_cast<const float4*>(job.z);
@@ -297,31 +304,25 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT, 1) k_var_tc(cons
             const int q = (item % ntiles) * (2 * QM) + (int)rank * QM + m;
             return __ldcg(zp + min(q, job.Q - 1));          // spare rows repeat the last query
         };
-        float4 za = make_float4(0, 0, 0, 0), zb = za;
-        if (pair < nitems) {
-            za = query(pair, m0);
-            zb = query(pair, m0 + 32);
-        }
+        float4 zn[NQ];
+#pragma unroll
+        for (int r = 0; r < NQ; ++r) zn[r] = pair < nitems ? query(pair, m0 + 32 * r) : make_float4(0, 0, 0, 0);
         for (int item = pair; item < nitems && ok; item += npairs) {
             const int ts = item / ntiles;
             const GpSet::One& G = gs.gp[ts / job.nsplit];
             const int split = ts % job.nsplit, np = pass_count(G.N);
-            uint64_t z0[4], z1[4];
-            {
-                const float a[4] = {za.x, za.y, za.z, za.w}, b[4] = {zb.x, zb.y, zb.z, zb.w};
+            float z[NQ][4];
 #pragma unroll
-                for (int d = 0; d < 4; ++d) {
-                    const float x = a[d] * G.zscale[d], y = b[d] * G.zscale[d];
-                    z0[d] = tc::f2pack(x, x);
-                    z1[d] = tc::f2pack(y, y);
-                }
-            }
-            if (item + npairs < nitems) {                  // the next tile's queries, in flight meanwhile
-                za = query(item + npairs, m0);
-                zb = query(item + npairs, m0 + 32);
+            for (int r = 0; r < NQ; ++r) {
+                z[r][0] = zn[r].x * G.zscale[0];
+                z[r][1] = zn[r].y * G.zscale[1];
+                z[r][2] = zn[r].z * G.zscale[2];
+                z[r][3] = zn[r].w * G.zscale[3];
+                // the next tile's queries, in flight meanwhile
+                if (item + npairs < nitems) zn[r] = query(item + npairs, m0 + 32 * r);
             }
             for (int i = 0, p; ok && (p = split_pass(np, job.nsplit, split, i)) >= 0; ++i) {
-                const int ns = pass_stages(G.N, p);
+                const int ns = pass_stages(G.N, p, KC);
                 for (int c = 0; c < ns; ++c) {
                     if ((n & 1u) != turn) {
                         advance();
@@ -329,31 +330,43 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT, 1) k_var_tc(cons
                     }
                     const bool got = wait(x_full + n % XR, (n / XR) & 1u);
                     const ulonglong2* x = reinterpret_cast<const ulonglong2*>(tsm + L::x + (n % XR) * (KC * 16)) + 8 * slab;
-                    uint32_t ha[4], la[4], hb[4], lb[4], ma[PARTS == 3 ? 4 : 1], mb[PARTS == 3 ? 4 : 1];
+                    // two queries at a time share the points' registers; the first two are
+                    // made before the slot is free
+                    uint32_t hi_[2][4], lo_[2][4], mid_[2][PARTS == 3 ? 4 : 1];
+                    bool room = true;
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const ulonglong2 xa = x[2 * q], xb = x[2 * q + 1];
-                        float k0, k1;
-                        kernel_pair(z0, xa, xb, k0, k1);
-                        if constexpr (PARTS == 3) split3(k0, k1, ha[q], ma[q], la[q]);
-                        else split2<FMT>(k0, k1, ha[q], la[q]);
-                        kernel_pair(z1, xa, xb, k0, k1);
-                        if constexpr (PARTS == 3) split3(k0, k1, hb[q], mb[q], lb[q]);
-                        else split2<FMT>(k0, k1, hb[q], lb[q]);
+                    for (int r0 = 0; r0 < NQ; r0 += 2) {
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const ulonglong2 xa = x[2 * q], xb = x[2 * q + 1];
+#pragma unroll
+                            for (int r = 0; r < 2; ++r) {
+                                uint64_t zz[4];
+#pragma unroll
+                                for (int d = 0; d < 4; ++d) zz[d] = tc::f2pack(z[r0 + r][d], z[r0 + r][d]);
+                                float k0, k1;
+                                kernel_pair(zz, xa, xb, k0, k1);
+                                if constexpr (PARTS == 3) split3(k0, k1, hi_[r][q], mid_[r][q], lo_[r][q]);
+                                else split2<FMT>(k0, k1, hi_[r][q], lo_[r][q]);
+                            }
+                        }
+                        if (r0 == 0) {
+                            room = n < (uint32_t)NA || wait(done + (n - NA) % NBP, ((n - NA) / NBP) & 1u);
+                            ok = __all_sync(0xffffffffu, got && room);
+                            if (!ok) break;
+                        }
+#pragma unroll
+                        for (int r = 0; r < 2; ++r) {
+                            unsigned char* dst = tsm + sa * L::a_stage + slab * (QM * 16) + (m0 + 32 * (r0 + r)) * 16;
+                            *reinterpret_cast<uint4*>(dst) = make_uint4(hi_[r][0], hi_[r][1], hi_[r][2], hi_[r][3]);
+                            if constexpr (PARTS == 3)
+                                *reinterpret_cast<uint4*>(dst + L::a_part) =
+                                    make_uint4(mid_[r][0], mid_[r][1], mid_[r][2], mid_[r][3]);
+                            *reinterpret_cast<uint4*>(dst + (PARTS - 1) * L::a_part) =
+                                make_uint4(lo_[r][0], lo_[r][1], lo_[r][2], lo_[r][3]);
+                        }
                     }
-                    const bool room = n < (uint32_t)NA || wait(done + (n - NA) % NBP, ((n - NA) / NBP) & 1u);
-                    if (!(ok = __all_sync(0xffffffffu, got && room))) break;
-                    unsigned char* dst = tsm + sa * L::a_stage + slab * (QM * 16) + m0 * 16;
-                    *reinterpret_cast<uint4*>(dst) = make_uint4(ha[0], ha[1], ha[2], ha[3]);
-                    *reinterpret_cast<uint4*>(dst + 512) = make_uint4(hb[0], hb[1], hb[2], hb[3]);
-                    dst += L::a_part;
-                    if constexpr (PARTS == 3) {
-                        *reinterpret_cast<uint4*>(dst) = make_uint4(ma[0], ma[1], ma[2], ma[3]);
-                        *reinterpret_cast<uint4*>(dst + 512) = make_uint4(mb[0], mb[1], mb[2], mb[3]);
-                        dst += L::a_part;
-                    }
-                    *reinterpret_cast<uint4*>(dst) = make_uint4(la[0], la[1], la[2], la[3]);
-                    *reinterpret_cast<uint4*>(dst + 512) = make_uint4(lb[0], lb[1], lb[2], lb[3]);
+                    if (!ok) break;
                     __syncwarp();
                     if (lane == 0) arrive(a_raw + sa);
                     advance();
@@ -416,7 +429,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT, 1) k_var_tc(cons
             const int N = gs.gp[ts / job.nsplit].N;
             const int split = ts % job.nsplit, np = pass_count(N);
             for (int i = 0, p; ok && (p = split_pass(np, job.nsplit, split, i)) >= 0; ++i, ++passes) {
-                const int ns = pass_stages(N, p), hi = pass_hi(N, p);
+                const int ns = pass_stages(N, p, KC), hi = pass_hi(N, p);
                 if (passes > 0) {
                     // both CTAs have read the last pass
                     if (!(ok = __all_sync(0xffffffffu, wait(t_free, (passes - 1) & 1u)))) break;
@@ -427,26 +440,29 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT, 1) k_var_tc(cons
                     go = go && wait(a_full + sa, pa);
                     if (!(ok = __all_sync(0xffffffffu, go))) break;
                     tc::fence_after_sync();
-                    const int lo = stage_lo(p, c), cols = hi - lo, h = cols / 2;
+                    const int lo = stage_lo(p, c, KC), cols = hi - lo, h = cols / 2;
                     const uint64_t ah = dA0 + (uint64_t)((sa * L::a_stage) >> 4);
                     const uint64_t bh = tc::smem_desc(tc::smem_addr(tsm) + (uint32_t)(L::b + sb * L::b_stage), (uint32_t)h * 16u, 128);
-                    const uint64_t bstep = (uint64_t)(4 * h);            // one part of the piece: 64 h bytes
+                    const uint64_t bstep = (uint64_t)(KC * h * 2 / 16);  // one part of the piece
                     const uint32_t idesc = idesc0 | ((uint32_t)(cols >> 3) << 17);
                     const uint64_t a1 = (uint64_t)(L::a_part >> 4);
                     const uint64_t ka = (uint64_t)((2 * QM * 16) >> 4), kb = (uint64_t)(2 * h);
                     if constexpr (PARTS == 2) {
-                        stage_split2(taddr + (uint32_t)lo, ah, ah + a1, bh, bh + bstep, ka, kb, idesc, c > 0 ? 1u : 0u);
+#pragma unroll
+                        for (int j = 0; j < KC / 16; j += 2)
+                            stage_split2(taddr + (uint32_t)lo, ah + j * ka, ah + a1 + j * ka, bh + j * kb, bh + bstep + j * kb,
+                                         ka, kb, idesc, c + j > 0 ? 1u : 0u);
                     } else {
 #pragma unroll
-                        for (int j = 0; j < 2; ++j)
+                        for (int j = 0; j < KC / 16; ++j)
                             step_split3(taddr + (uint32_t)lo, ah + j * ka, ah + a1 + j * ka, ah + 2 * a1 + j * ka,
                                         bh + j * kb, bh + bstep + j * kb, bh + 2 * bstep + j * kb, idesc,
                                         c + j > 0 ? 1u : 0u);
                     }
                     commit2_elect(done + sb);
                     // columns 64 j .. 64 j + 63 are complete after their diagonal's last stage
-                    const int d = c - 8 * p;
-                    if (d >= 0 && ((d & 1) || c == ns - 1)) commit2_elect(q_done + (d >> 1));
+                    const int d = KC * c - PASS * p;
+                    if (d >= 0 && ((d + KC) % QUART == 0 || c == ns - 1)) commit2_elect(q_done + d / QUART);
                     advance();
                 }
             }
@@ -467,7 +483,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT, 1) k_var_tc(cons
                 const int N = gs.gp[ts / job.nsplit].N;
                 const int split = ts % job.nsplit, np = pass_count(N);
                 for (int i = 0, p; ok && (p = split_pass(np, job.nsplit, split, i)) >= 0; ++i) {
-                    const int ns = pass_stages(N, p);
+                    const int ns = pass_stages(N, p, KC);
                     for (int c = 0; c < ns; ++c) {
                         if (!(ok = wait(b_full + sb, pb))) break;
                         arrive_cluster(peer0 + 8u * (uint32_t)sb);
@@ -479,19 +495,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT, 1) k_var_tc(cons
     } else if (warp > LOAD_WARP) {
         // ---------------- rows to the tensor core ------------------------------------
         if (lane == 0) {
-            const uint32_t a_full0 = mapa(a_full, 0u), turn = (uint32_t)(warp & 1);
+            const uint32_t a_full0 = mapa(a_full, 0u);
             for (int item = pair; item < nitems && ok; item += npairs) {
                 const int ts = item / ntiles;
                 const int N = gs.gp[ts / job.nsplit].N;
                 const int split = ts % job.nsplit, np = pass_count(N);
                 for (int i = 0, p; ok && (p = split_pass(np, job.nsplit, split, i)) >= 0; ++i) {
-                    const int ns = pass_stages(N, p);
+                    const int ns = pass_stages(N, p, KC);
                     for (int c = 0; c < ns; ++c) {
-                        if ((n & 1u) == turn) {
-                            if (!(ok = wait(a_raw + sa, pa))) break;
-                            tc::fence_proxy_async();
-                            arrive_cluster(a_full0 + 8u * (uint32_t)sa);
-                        }
+                        if (!(ok = wait(a_raw + sa, pa))) break;
+                        tc::fence_proxy_async();
+                        arrive_cluster(a_full0 + 8u * (uint32_t)sa);
                         advance();
                     }
                 }
@@ -512,7 +526,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT, 1) k_var_tc(cons
                 const GpSet::One& G = gs.gp[ts / job.nsplit];
                 const int p = split_pass(pass_count(G.N), job.nsplit, ts % job.nsplit, xpi);
                 if (p >= 0) {
-                    xns = pass_stages(G.N, p);
+                    xns = pass_stages(G.N, p, KC);
                     xsrc = G.xq;
                     ++xpi;
                 } else {
@@ -536,15 +550,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT, 1) k_var_tc(cons
             const GpSet::One& G = gs.gp[ts / job.nsplit];
             const int split = ts % job.nsplit, np = pass_count(G.N);
             for (int i = 0, p; ok && (p = split_pass(np, job.nsplit, split, i)) >= 0; ++i) {
-                const int ns = pass_stages(G.N, p), hi = pass_hi(G.N, p);
-                const unsigned char* src = reinterpret_cast<const unsigned char*>(G.Bt) + pass_base(p) * (64 * PARTS);
+                const int ns = pass_stages(G.N, p, KC), hi = pass_hi(G.N, p);
+                const unsigned char* src = reinterpret_cast<const unsigned char*>(G.Bt) + pass_base(p) * (2 * PARTS);
                 for (int c = 0; c < ns; ++c) {
                     if (n >= (uint32_t)NBP) {
                         if (!(ok = wait(done + sb, pb ^ 1u))) break;
                         fetch_x();
                     }
-                    const int cols = hi - stage_lo(p, c);
-                    const uint32_t bytes = (uint32_t)(32 * PARTS * cols);      // this CTA's half of the columns
+                    const int cols = hi - stage_lo(p, c, KC);
+                    const uint32_t bytes = (uint32_t)(KC * PARTS * cols);      // this CTA's half of the columns
                     tc::mbar_expect_tx(b_full + sb, bytes);
                     bulk_g2s(tsm + L::b + sb * L::b_stage, src + rank * bytes, bytes, b_full + sb);
                     src += 2 * bytes;
@@ -573,29 +587,29 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT, 1) k_var_tc(cons
 
 // cB L^-1 in the pieces of the passes: (pass, stage) holds, for each CTA of the
 // pair, its half of the stage's columns: the parts (hi, lo or hi, mid, lo) one
-// after the other, each as four slabs of 8 points x (columns / 2) rows.
+// after the other, each as slabs of 8 points x (columns / 2) rows.
 __global__ void k_pack_tc(const double* __restrict__ Xm, int N, int fmt, double cB, uint16_t* __restrict__ out) {
+    const int parts = fmt == 2 ? 3 : 2, kc = stage_points(parts);
     const int p = blockIdx.y, c = blockIdx.x;
-    if (c >= pass_stages(N, p)) return;
-    const int hi = pass_hi(N, p), lo = stage_lo(p, c), cols = hi - lo, h = cols / 2;
+    if (c >= pass_stages(N, p, kc)) return;
+    const int hi = pass_hi(N, p), lo = stage_lo(p, c, kc), cols = hi - lo, h = cols / 2;
     size_t off = pass_base(p);
-    for (int i = 0; i < c; ++i) off += (size_t)(hi - stage_lo(p, i));
-    const int parts = fmt == 2 ? 3 : 2;
-    uint16_t* dst = out + off * (32 * parts);
-    for (int idx = threadIdx.x; idx < cols * KC; idx += blockDim.x) {
-        const int e = idx % 8, row = (idx / 8) % h, sl = (idx / (8 * h)) % 4, r = idx / (32 * h);
-        const int i = PASS * p + lo + r * h + row, j = KC * c + 8 * sl + e;
+    for (int i = 0; i < c; ++i) off += (size_t)(hi - stage_lo(p, i, kc)) * kc;
+    uint16_t* dst = out + off * parts;
+    for (int idx = threadIdx.x; idx < cols * kc; idx += blockDim.x) {
+        const int e = idx % 8, row = (idx / 8) % h, sl = (idx / (8 * h)) % (kc / 8), r = idx / (kc * h);
+        const int i = PASS * p + lo + r * h + row, j = kc * c + 8 * sl + e;
         const double v = (i < N && j <= i) ? cB * Xm[(size_t)i * N + j] : 0.0;
-        uint16_t* o = dst + r * (parts * h * 32) + sl * (h * 8) + row * 8 + e;
+        uint16_t* o = dst + r * (parts * h * kc) + sl * (h * 8) + row * 8 + e;
         if (fmt == 0) {
             const __half a = __double2half(v);
             o[0] = __half_as_ushort(a);
-            o[h * 32] = __half_as_ushort(__double2half(v - (double)__half2float(a)));
+            o[h * kc] = __half_as_ushort(__double2half(v - (double)__half2float(a)));
         } else {
             double rest = v;
             for (int q = 0; q < parts; ++q) {              // each residual exact in double
                 const __nv_bfloat16 a = __double2bfloat16(rest);
-                o[q * h * 32] = __bfloat16_as_ushort(a);
+                o[q * h * kc] = __bfloat16_as_ushort(a);
                 rest -= (double)__bfloat162float(a);
             }
         }
@@ -609,10 +623,11 @@ int build_tc_pieces(GpDevice& g, int fmt) {
     const int rc = set_cB(g);
     if (rc) return rc;
     const int N = g.N, np = pass_count(N), p = np - 1;
-    size_t cols = pass_base(p);
-    for (int c = 0; c < pass_stages(N, p); ++c) cols += (size_t)(pass_hi(N, p) - stage_lo(p, c));
-    GPM_CUDA(cudaMalloc(&g.Bt[fmt], cols * (size_t)(64 * (fmt == 2 ? 3 : 2))));
-    k_pack_tc<<<dim3((unsigned)(8 * np), (unsigned)np), 256>>>(g.Linv64[0], N, fmt, (double)g.cB, g.Bt[fmt]);
+    const int parts = fmt == 2 ? 3 : 2, kc = stage_points(parts);
+    size_t n = pass_base(p);                     // columns x points
+    for (int c = 0; c < pass_stages(N, p, kc); ++c) n += (size_t)(pass_hi(N, p) - stage_lo(p, c, kc)) * kc;
+    GPM_CUDA(cudaMalloc(&g.Bt[fmt], n * (size_t)(2 * parts)));
+    k_pack_tc<<<dim3((unsigned)(PASS / kc * np), (unsigned)np), 256>>>(g.Linv64[0], N, fmt, (double)g.cB, g.Bt[fmt]);
     GPM_CUDA(cudaGetLastError());
     GPM_CUDA(cudaDeviceSynchronize());
     return GPMPPI_OK;
