@@ -323,11 +323,11 @@ int alloc_query_ws(gpmppi_ctrl c) {
     size_t npad = 0, rows = 0;
     for (size_t t = 0; t < M; ++t) npad = npad < (size_t)c->gset.gp[t].npad ? (size_t)c->gset.gp[t].npad : npad;
     if (c->fmt < 0) {
-        rows = npad ? ((size_t)1 << 27) / npad : n * T;
-        if (rows > n * T) rows = n * T;
+        rows = npad ? ((size_t)1 << 27) / npad / kTriTile * kTriTile : n * T;
+        if (rows > n * T) rows = (n * T + kTriTile - 1) / kTriTile * kTriTile;
         c->v_q = (int)rows;
     }
-    if (c->p.variance_mode == GPMPPI_VAR_NOMINAL && rows < T) rows = T;
+    if (c->p.variance_mode == GPMPPI_VAR_NOMINAL && rows < 4 * T) rows = 4 * T;     // 2 T N doubles
     cudaFree(c->vbuf);
     c->vbuf = nullptr;
     if (rows * npad > 0) {
@@ -376,10 +376,9 @@ int make_query_gp(GpDevice& g, int fmt, GpSet::One* out) {
     return GPMPPI_OK;
 }
 
-// Alg. 1 Step 2 as a query rollout of one trajectory without noise, in FP32
-// (args: the updated controls in U): its covariance tightens the next call.
+// Alg. 1 Step 2 as a query rollout of one trajectory without noise (args: the
+// updated controls in U): its covariance tightens the next call.
 int launch_nominal(gpmppi_ctrl c, const RolloutArgs& a, cudaStream_t st) {
-    const GpSet gs = single_gp_set(c->gp->g, 0);
     QueryWs ws;
     ws.zq = static_cast<float4*>(c->ws_buf);
     ws.st = ws.zq + (a.T + 1);
@@ -389,11 +388,8 @@ int launch_nominal(gpmppi_ctrl c, const RolloutArgs& a, cudaStream_t st) {
     ws.nsplit = 1;
     int rc;
     if ((rc = launch_nominal_mean(a, ws, st))) return rc;
-    TriJob j = tri_forward(gs.gp[0], reinterpret_cast<const float*>(ws.zq), a.T, c->vbuf);
-    j.err = a.err;
-    if ((rc = launch_tri_forward(j, true, st))) return rc;
-    if ((rc = launch_rowsum(c->vbuf, gs.gp[0].npad, a.T, a.N, kSumBlock, ws.q, st))) return rc;
-    return launch_nominal_cov(a, gs, ws, c->nom_sxy, st);
+    if ((rc = launch_nominal_var(c->gp->g, a.T, ws, reinterpret_cast<double*>(c->vbuf), st))) return rc;
+    return launch_nominal_cov(a, ws, c->nom_sxy, st);
 }
 
 }  // namespace
@@ -940,7 +936,7 @@ int mppi_grad(gpmppi_ctrl c, const float state[5], const float* U_nom, const flo
     const size_t o_st = take(sizeof(float4) * Q);
     const size_t o_qq = take(sizeof(float) * Q);
     const size_t o_rec = take(sizeof(float) * 16 * Q);
-    const size_t o_v = take(sizeof(float) * Q * g.npad);
+    const size_t o_v = take(sizeof(float) * ((Q + kTriTile - 1) / kTriTile * kTriTile) * g.npad);
     const size_t o_S = take(sizeof(float) * (size_t)K);
     const size_t o_dU = take(sizeof(float) * (size_t)2 * T * K);
     const size_t o_dl = take(sizeof(float) * (size_t)8 * K);

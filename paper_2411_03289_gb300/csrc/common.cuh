@@ -118,6 +118,7 @@ struct GpDevice {
     // FP64 factors kept for export: Linv64[o] N x N, alpha64[o] N
     double* Linv64[2] = {nullptr, nullptr};
     double* alpha64[2] = {nullptr, nullptr};
+    double* X64 = nullptr;       // N x 4 training inputs
     // tensor-core tiles of L^-T per operand format for the batched rollout (0 =
     // FP16 hi/lo, 1 = BF16 hi/lo, 2 = BF16 hi/mid/lo), built with a batch; NpM = N
     // rounded up to 128
@@ -345,15 +346,16 @@ struct GradArgs {
 // launchers (defined in the .cu files)
 int launch_chain(const RolloutArgs& a, const GpSet& gs, const QueryWs& ws, cudaStream_t st);
 // Triangular products and their row sums in FP32 (tri.cu)
+constexpr int kTriTile = 128;   // queries per tile of v
 struct TriJob {
-    const float* z;             // forward: Q x 4 queries (any 4-byte alignment); backward: Q x ldz rows of v
-    int ldz;
+    const float* z;             // forward: Q x 4 queries (any 4-byte alignment); backward: v
+    int ldz;                    // backward: columns of v
     const float* fac;           // GpDevice::Wb (forward), GpDevice::Lb (backward)
     const float* xq;
-    float* out;                 // Q x ldo
+    float* out;                 // forward: v, tiles of kTriTile queries, each ldo columns x kTriTile; backward: rows of ldo floats
     int ldo;
     int Q, N;
-    int rk, rkpad;              // rk != 0: row q goes to (q / rk) rkpad + q % rk
+    int rk, rkpad;              // backward: row q goes to (q / rk) rkpad + q % rk
     float sf2;
     float zscale[4];
     int fusez;                  // differences z - x with one rounding (gp_predict, the adjoint)
@@ -361,7 +363,7 @@ struct TriJob {
     unsigned long long wait_ns;
     int expire_first;
 };
-enum SumOrder { kSumPairs = 0, kSumLanes = 1, kSumBlock = 2 };
+enum SumOrder { kSumPairs = 0, kSumLanes = 1 };
 TriJob tri_forward(const GpSet::One& G, const float* z, int Q, float* V);
 int launch_tri_forward(const TriJob& j, bool dependent, cudaStream_t st);
 int launch_tri_backward(const TriJob& j, bool dependent, cudaStream_t st);
@@ -415,7 +417,9 @@ int build_mma_ensemble(GpDevice* const* gs, int M, int fmt, MmaTerrains& tr, uin
 int launch_philox(uint64_t seed, const uint32_t* ctr, int M, uint32_t* out, cudaStream_t st);
 int launch_noise(uint64_t seed, int K, int T, uint64_t it, float sv, float sw, float* eps,
                  cudaStream_t st);
-int launch_nominal_cov(const RolloutArgs& a, const GpSet& gs, const QueryWs& ws, float* sxy_out, cudaStream_t st);
+// variances of the T queries ws.zq in FP64 into ws.q; scratch: 2 T N doubles
+int launch_nominal_var(const GpDevice& g, int T, const QueryWs& ws, double* scratch, cudaStream_t st);
+int launch_nominal_cov(const RolloutArgs& a, const QueryWs& ws, float* sxy_out, cudaStream_t st);
 int launch_mma_selftest(int fmt, int N, int K, int variant, const uint16_t* A, const uint16_t* B,
                         float* D, unsigned int* err, cudaStream_t st);
 // tr(D_d G_o) from G = [G_v; G_w] (2 Np x Np, column-major): one block per 8

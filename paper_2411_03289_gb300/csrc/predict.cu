@@ -1,7 +1,5 @@
 // The GP posterior at M queries (gp_predict), FP32: the triangular product of
-// tri.cu, then one CTA a query sums the squares and the mean.
-// M = 20000, N = 1000: 0.50 ms (48 TFLOP/s) against 3.29 ms of a CTA per query that
-// read the whole factor.
+// tri.cu and its row sums, and the means with one CTA a query.
 #include <mutex>
 
 #include "query.cuh"
@@ -13,7 +11,7 @@ struct PredArgs {
     const float* Z;          // queries, M x 4
     const float* Xs;         // GpDevice::Xs, alpha
     const float* alpha;
-    const float* V;          // M x npad
+    const float* V;          // tiles of kTriTile queries, npad columns each
     float* mean;
     float* var;
     int M, N, npad;
@@ -61,32 +59,41 @@ __device__ float block_sum(float v, float* red) {
     return s;
 }
 
-__global__ void __launch_bounds__(ST) k_pred_sum(const PredArgs p) {
+// the means, one CTA a query
+__global__ void __launch_bounds__(ST) k_pred_mean(const PredArgs p) {
     __shared__ float red[ST / 32];
     const int q = blockIdx.x;
     float zq[4];
     for (int d = 0; d < 4; ++d) zq[d] = p.Z[q * (size_t)4 + d] * p.zscale[d];
     const int o0 = p.out < 0 ? 0 : p.out, o1 = p.out < 0 ? 1 : p.out;
-    float m0 = 0.0f, m1 = 0.0f, qf = 0.0f;
+    float m0 = 0.0f, m1 = 0.0f;
     for (int j = threadIdx.x; j < p.N; j += ST) {
         const float4 x = reinterpret_cast<const float4*>(p.Xs)[j];
         const float e0 = zq[0] - x.x, e1 = zq[1] - x.y, e2 = zq[2] - x.z, e3 = zq[3] - x.w;
         const float k = p.sf2 * exp2f(-(e0 * e0 + e1 * e1 + e2 * e2 + e3 * e3));
         m0 += k * p.alpha[2 * j + o0];
         m1 += k * p.alpha[2 * j + o1];
-        const float v = p.V[(size_t)q * p.npad + j];
-        qf = fmaf(v, v, qf);
     }
     m0 = block_sum(m0, red);
     m1 = block_sum(m1, red);
-    qf = block_sum(qf, red);
     if (threadIdx.x == 0) {
-        const float v = fmaxf(0.0f, p.sf2 - qf);
         p.mean[2 * (size_t)q + o0] = m0;
-        p.var[2 * (size_t)q + o0] = v;
         p.mean[2 * (size_t)q + o1] = m1;
-        p.var[2 * (size_t)q + o1] = v;
     }
+}
+
+// the variances from the rows of v, one thread a query: the squares as 128 threads
+// of a CTA would sum them, four warps' trees in order
+__global__ void __launch_bounds__(kTriTile) k_pred_var(const PredArgs p) {
+    qr::grid_wait();
+    const float* v = p.V + (size_t)blockIdx.x * p.npad * kTriTile + threadIdx.x;
+    float qf = 0.0f;
+    for (int w = 0; w < 4; ++w) qf += qr::lane_squares<128>(v, kTriTile, 32 * w, p.N);
+    const int q = blockIdx.x * kTriTile + threadIdx.x;
+    if (q >= p.M) return;
+    const float s = fmaxf(0.0f, p.sf2 - qf);
+    if (p.out != 1) p.var[2 * (size_t)q] = s;
+    if (p.out != 0) p.var[2 * (size_t)q + 1] = s;
 }
 
 }  // namespace
@@ -102,7 +109,7 @@ int launch_gp_predict(const GpDevice& g, const float* Z, int M, float* mean, flo
     if (M == 0) return GPMPPI_OK;
     // V in stream-ordered scratch (calls from several threads or streams share
     // nothing), at most 1 GB: more queries go in pieces
-    size_t piece = g.npad ? ((size_t)1 << 28) / g.npad / 64 * 64 : (size_t)M;
+    size_t piece = g.npad ? ((size_t)1 << 28) / g.npad / kTriTile * kTriTile : (size_t)M;
     if (piece > (size_t)M) piece = (size_t)M;
     float* V = nullptr;
     if (g.npad) {
@@ -110,7 +117,7 @@ int launch_gp_predict(const GpDevice& g, const float* Z, int M, float* mean, flo
         if (g.device < 0 || g.device >= kMaxDevices) return fail(GPMPPI_ERR_UNSUPPORTED, "gp_predict: device number");
         const int rc0 = scratch_pool(g.device, &pool);
         if (rc0) return rc0;
-        GPM_CUDA(cudaMallocFromPoolAsync((void**)&V, sizeof(float) * piece * g.npad, pool, st));
+        GPM_CUDA(cudaMallocFromPoolAsync((void**)&V, sizeof(float) * ((piece + kTriTile - 1) / kTriTile * kTriTile) * g.npad, pool, st));
     }
     int rc = GPMPPI_OK;
     for (int o = 0; o < (g.shared ? 1 : 2) && rc == GPMPPI_OK; ++o)
@@ -132,8 +139,11 @@ int launch_gp_predict(const GpDevice& g, const float* Z, int M, float* mean, flo
             j.fusez = 1;
             rc = launch_tri_forward(j, false, st);
             if (rc) break;
-            k_pred_sum<<<p.M, ST, 0, st>>>(p);
-            const cudaError_t e = cudaGetLastError();
+            cudaError_t e = launch_ex(k_pred_var, dim3((unsigned)((p.M + kTriTile - 1) / kTriTile)), kTriTile, 0, st, true, 1u, p);
+            if (e == cudaSuccess) {
+                k_pred_mean<<<p.M, ST, 0, st>>>(p);
+                e = cudaGetLastError();
+            }
             if (e != cudaSuccess) rc = cuda_fail(e, "gp_predict");
         }
     if (V) {

@@ -43,6 +43,27 @@ __device__ __forceinline__ void kernel_pair(const uint64_t (&zz)[4], const ulong
     k1 = ex2(-t1);
 }
 
+// Squares of a row of v (column i at v[i ld]) as a warp would sum them: 32 chains
+// over the columns i0 + l, i0 + l + STEP, ..., then the shuffle tree.
+template <int STEP>
+__device__ __forceinline__ float lane_squares(const float* v, int ld, int i0, int n) {
+    float s[32];
+#pragma unroll
+    for (int l = 0; l < 32; ++l) s[l] = 0.0f;
+    for (int i = i0; i < n; i += STEP) {
+#pragma unroll
+        for (int l = 0; l < 32; ++l) {
+            const float x = i + l < n ? __ldcg(v + (size_t)(i + l) * ld) : 0.0f;
+            s[l] = fmaf(x, x, s[l]);
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int l = 0; l < o; ++l) s[l] += s[l + o];
+    return s[0];
+}
+
 // wait for the kernel before this one in the stream (launched with programmatic
 // serialisation); a no-op after an ordinary launch
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

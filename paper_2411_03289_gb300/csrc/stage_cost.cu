@@ -245,9 +245,9 @@ __global__ void __launch_bounds__(ST) k_stage_cost(const RolloutArgs a, const Sc
 }
 
 // Alg. 1 Step 2: the covariance along the nominal trajectory, one warp.  Lanes
-// load 32 steps' states and variances at a time; every lane carries the
+// load 32 steps' states and variances (ws.q) at a time; every lane carries the
 // recurrence, lane 0 records Sigma_XY after each step.
-__global__ void __launch_bounds__(32) k_nominal_cov(const RolloutArgs a, float sf2, float qscale, const QueryWs ws,
+__global__ void __launch_bounds__(32) k_nominal_cov(const RolloutArgs a, const QueryWs ws,
                                                     float* __restrict__ sxy) {
     const int lane = threadIdx.x;
     grid_wait();
@@ -261,7 +261,7 @@ __global__ void __launch_bounds__(32) k_nominal_cov(const RolloutArgs a, float s
             th = p.z;
             vl = p.w;
         }
-        const float sl = fmaxf(0.0f, sf2 - qscale * ws.q[kl]);
+        const float sl = ws.q[kl];
         float snl, csl;
         sincosf(th, &snl, &csl);
         for (int i = 0; i < 32 && k0 + i < a.T; ++i) {
@@ -279,8 +279,8 @@ __global__ void __launch_bounds__(32) k_nominal_cov(const RolloutArgs a, float s
 
 }  // namespace
 
-int launch_nominal_cov(const RolloutArgs& a, const GpSet& gs, const QueryWs& ws, float* sxy_out, cudaStream_t st) {
-    GPM_CUDA(launch_ex(k_nominal_cov, dim3(1), 32, 0, st, true, 1u, a, gs.gp[0].sf2, gs.gp[0].qscale, ws, sxy_out));
+int launch_nominal_cov(const RolloutArgs& a, const QueryWs& ws, float* sxy_out, cudaStream_t st) {
+    GPM_CUDA(launch_ex(k_nominal_cov, dim3(1), 32, 0, st, true, 1u, a, ws, sxy_out));
     return GPMPPI_OK;
 }
 

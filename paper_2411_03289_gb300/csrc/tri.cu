@@ -2,13 +2,17 @@
 // of squares over their rows.
 //   forward   v_q = L^-1 k*_q   (query rollout, gp_predict, adjoint)
 //   backward  b_q = L^-T v_q = K^-1 k*_q   (adjoint)
-// An item is 64 queries x one 128-column block, reduced over the training points
+// An item is 128 queries x one 128-column block, reduced over the training points
 // of its triangle in chunks of 32: the factor piece (32 x 128 floats, contiguous)
-// and the chunk's points arrive by bulk copies in a ring, the CTA makes the
-// kernel values (forward) or transposes the rows of v (backward).  A thread
-// holds two columns x 16 queries, so that a step is 16 packed FMAs on four
-// broadcast reads; column sets past the diagonal are left out.  Items are very
-// uneven (one to N / 32 chunks) and go longest first, three CTAs an SM.
+// and the chunk's points (forward) or its rows of v (backward) arrive by bulk
+// copies in a ring.  A thread multiplies an 8-query x 8-column tile in registers
+// with packed FMAs (query pairs): 4 shared-memory reads for 32 of them, where 2
+// columns x 16 queries needed 12 and the reads, not the FMAs, bounded it.  Warp w
+// owns columns 16 w .. 16 w + 15 and leaves out the diagonal's rows that hold none
+// of them.  Items are very uneven (one to N / 32 chunks) and go longest first, two
+// CTAs an SM.  v is kept by tiles of 128 queries, query the fastest index, so that
+// it leaves in whole lines, comes back as operands by bulk copies and is summed
+// with a thread per query.
 // Every result is one FMA chain over the points in their order, so that it does
 // not depend on the split.  The GP variance is what remains of sf2 after nearly
 // all of it cancels: its last digits are the rounding of these chains and of the
@@ -23,61 +27,43 @@ namespace {
 using namespace qr;
 
 constexpr int PT = 256;              // threads
-constexpr int PQ = 64;               // queries per item
+constexpr int PQ = 128;              // queries per item (kTriTile)
 constexpr int CH = 32;               // training points per chunk
 constexpr int CB = 128;              // columns per block
 constexpr int NST = 3;               // ring stages
 constexpr int PIECE = CH * CB * 4;
-constexpr int XB = CH * 16;
-constexpr int STG = PIECE + XB;
-constexpr int OFF_A = NST * STG;                     // 2 x CH x PQ floats: kernel values (rows of v)
-constexpr int OFF_BAR = OFF_A + 2 * CH * PQ * 4;
-constexpr int SMEM = OFF_BAR + 8 * (NST + 1) + 16;
+constexpr int AB = CH * PQ * 4;      // a chunk's operand: kernel values or rows of v
+static_assert(PQ == kTriTile, "tile of v");
 
-// acc += a column's factor entries times the 16 queries' values, one chunk
-template <bool LO, bool HI>
-__device__ __forceinline__ void rows_fma(const float* A, const float* B, uint64_t (&lo)[8], uint64_t (&hi)[8]) {
-#pragma unroll 4
-    for (int k = 0; k < CH; ++k) {
-        uint64_t av[8];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(A + k * PQ + 4 * i);
-            av[2 * i] = a.x;
-            av[2 * i + 1] = a.y;
-        }
-        if (HI) {
-            const float b = B[k * CB + 64];
-            const uint64_t bb = tc::f2pack(b, b);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) hi[i] = tc::f2fma(av[i], bb, hi[i]);
-        }
-        if (LO) {
-            const float b = B[k * CB];
-            const uint64_t bb = tc::f2pack(b, b);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) lo[i] = tc::f2fma(av[i], bb, lo[i]);
-        }
-    }
-}
+// shared memory: ring (piece, then points or rows of v), kernel values, barriers
+template <bool BACK>
+struct TriLayout {
+    static constexpr int stage = PIECE + (BACK ? AB : CH * 16);
+    static constexpr int a = NST * stage;
+    static constexpr int bar = a + (BACK ? 0 : 2 * AB);
+    static constexpr int total = bar + 8 * (NST + 1) + 16;
+};
 
 // FUSEZ: a difference z - x is one rounding, fma(z, scale, -x), instead of two
 template <bool BACK, bool FUSEZ>
-__global__ void __launch_bounds__(PT, 3) k_tri(const TriJob p) {
+__global__ void __launch_bounds__(PT, 2) k_tri(const TriJob p) {
     extern __shared__ __align__(128) unsigned char psm[];
-    float* As = reinterpret_cast<float*>(psm + OFF_A);
-    uint64_t* full = reinterpret_cast<uint64_t*>(psm + OFF_BAR);
+    using L = TriLayout<BACK>;
+    float* As = reinterpret_cast<float*>(psm + L::a);
+    uint64_t* full = reinterpret_cast<uint64_t*>(psm + L::bar);
     uint64_t* never = full + NST;
     int* copies_on = reinterpret_cast<int*>(never + 1);
-    const int tid = threadIdx.x, warp = tid >> 5;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int nb = (int)gridDim.y, nrow = (p.N + CH - 1) / CH;
     const int cb = BACK ? (int)blockIdx.y : nb - 1 - (int)blockIdx.y;          // longest first
-    const int q0 = blockIdx.x * PQ;
+    const int tile = blockIdx.x, q0 = tile * PQ;
     // chunks r0 .. r1 - 1 of the points, and the block's first piece
     const int r0 = BACK ? (CB / CH) * cb : 0;
     const int r1 = BACK ? nrow : min((CB / CH) * (cb + 1), nrow);
     const int nr = r1 - r0;
     const float* fac = p.fac + (BACK ? (size_t)cb * nb - (size_t)cb * (cb - 1) / 2 : (size_t)cb * (cb + 1) / 2) * (CB * CB);
+    // rows of v of this tile (backward): npad x 128 floats
+    const float* vt = p.z + ((size_t)tile * p.ldz + CH * r0) * PQ;
 
     if (tid == 0) {
         for (int i = 0; i < NST; ++i) tc::mbar_init(full + i, 1);
@@ -92,29 +78,24 @@ __global__ void __launch_bounds__(PT, 3) k_tri(const TriJob p) {
     bool on = *copies_on != 0;
     int fetched = 0;
     auto fetch = [&](int r) {
-        unsigned char* dst = psm + (r % NST) * STG;
+        unsigned char* dst = psm + (r % NST) * L::stage;
         uint64_t* bar = full + r % NST;
         ++fetched;
-        tc::mbar_expect_tx(bar, BACK ? PIECE : STG);
+        tc::mbar_expect_tx(bar, L::stage);
         bulk_g2s(dst, fac + (size_t)r * (CH * CB), PIECE, bar);
-        if (!BACK) bulk_g2s(dst + PIECE, p.xq + (size_t)r * (CH * 4), XB, bar);
+        if (BACK) bulk_g2s(dst + PIECE, vt + (size_t)r * (CH * PQ), AB, bar);
+        else bulk_g2s(dst + PIECE, p.xq + (size_t)r * (CH * 4), CH * 16, bar);
     };
-    // the factor does not depend on the previous kernel: fetch before it ends
+    // the factor and the points do not depend on the previous kernel (v does)
+    if (BACK) grid_wait();
     if (tid == 0 && on)
         for (int r = 0; r < NST && r < nr; ++r) fetch(r);
-    grid_wait();
+    if (!BACK) grid_wait();
 
-    const int m = tid % PQ, h = tid / PQ;            // query m, points 8 h .. 8 h + 7 of a chunk
-    const int qm = min(q0 + m, p.Q - 1);
+    const int m = tid % PQ, h = tid / PQ;            // kernel values: query m, points 16 h .. 16 h + 15 of a chunk
     uint64_t zz[4], zs[4];
-    float4 va, vb;                                   // (backward) the next chunk's 8 values
-    const float* vrow = nullptr;
-    if (BACK) {
-        vrow = p.z + (size_t)qm * p.ldz + CH * r0 + 8 * h;
-        va = __ldcg(reinterpret_cast<const float4*>(vrow));
-        vb = __ldcg(reinterpret_cast<const float4*>(vrow) + 1);
-    } else {
-        const float* z = p.z + 4 * (size_t)qm;
+    if (!BACK) {
+        const float* z = p.z + 4 * (size_t)min(q0 + m, p.Q - 1);
 #pragma unroll
         for (int d = 0; d < 4; ++d) {
             const float v = FUSEZ ? __ldcg(z + d) : __ldcg(z + d) * p.zscale[d];
@@ -122,22 +103,15 @@ __global__ void __launch_bounds__(PT, 3) k_tri(const TriJob p) {
             zs[d] = tc::f2pack(p.zscale[d], p.zscale[d]);
         }
     }
-    auto make = [&](int r) {
+    auto arrived = [&](int r) {
         if (on) on = tc::mbar_wait(full + r % NST, (uint32_t)(r / NST) & 1u, p.wait_ns, p.err);
-        float* dst = As + (r & 1) * (CH * PQ) + h * 8 * PQ + m;
-        if (BACK) {
-            const float v[8] = {va.x, va.y, va.z, va.w, vb.x, vb.y, vb.z, vb.w};
+    };
+    auto make = [&](int r) {
+        arrived(r);
+        const ulonglong2* x = reinterpret_cast<const ulonglong2*>(psm + (r % NST) * L::stage + PIECE) + h * 16;
+        float* dst = As + (r & 1) * (CH * PQ) + h * 16 * PQ + m;
 #pragma unroll
-            for (int i = 0; i < 8; ++i) dst[i * PQ] = v[i];
-            if (r + 1 < nr) {
-                va = __ldcg(reinterpret_cast<const float4*>(vrow + CH * (r + 1)));
-                vb = __ldcg(reinterpret_cast<const float4*>(vrow + CH * (r + 1)) + 1);
-            }
-            return;
-        }
-        const ulonglong2* x = reinterpret_cast<const ulonglong2*>(psm + (r % NST) * STG + PIECE) + h * 8;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
+        for (int i = 0; i < 8; ++i) {
             // k = sf2 2^-(e0 e0 + e1 e1 + e2 e2 + e3 e3), the sum as one chain
             // that starts with the product of e1
             const ulonglong2 a = x[2 * i], b = x[2 * i + 1];
@@ -156,26 +130,43 @@ __global__ void __launch_bounds__(PT, 3) k_tri(const TriJob p) {
         }
     };
 
-    const int g = tid >> 6, c = tid & 63, wc = warp & 1;     // queries 16 g .., columns c and c + 64
-    uint64_t lo[8], hi[8];
+    const int lq = lane & 15, c0 = 16 * warp + 8 * (lane >> 4);
+    uint64_t acc[4][8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        lo[i] = 0ull;
-        hi[i] = 0ull;
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int c = 0; c < 8; ++c) acc[i][c] = 0ull;
+    if (!BACK) {
+        make(0);
+        __syncthreads();
     }
-    make(0);
-    __syncthreads();
     for (int r = 0; r < nr; ++r) {
-        if (r + 1 < nr) make(r + 1);
-        const float* A = As + (r & 1) * (CH * PQ) + 16 * g;
-        const float* B = reinterpret_cast<const float*>(psm + (r % NST) * STG) + c;
-        // chunk d of the diagonal block (points 32 d ..): forward, columns below
-        // 32 d are zero; backward, columns past 32 d + 31
-        const int d = BACK ? r : r - (CB / CH) * cb;
-        const bool dolo = BACK ? d >= wc : d <= wc, dohi = BACK ? d >= wc + 2 : d <= wc + 2;
-        if (dolo && dohi) rows_fma<true, true>(A, B, lo, hi);
-        else if (dolo) rows_fma<true, false>(A, B, lo, hi);
-        else if (dohi) rows_fma<false, true>(A, B, lo, hi);
+        if (BACK) arrived(r);
+        else if (r + 1 < nr) make(r + 1);
+        const unsigned char* stage = psm + (r % NST) * L::stage;
+        const float* A = BACK ? reinterpret_cast<const float*>(stage + PIECE) : As + (r & 1) * (CH * PQ);
+        const float* B = reinterpret_cast<const float*>(stage) + c0;
+        // rows of the diagonal block that hold none of this warp's columns: forward
+        // those past its last column, backward those before its first
+        const int d = BACK ? CH * r : CH * (r - (CB / CH) * cb);
+        const int k0 = BACK ? min(CH, max(0, 16 * warp - d)) : 0;
+        const int k1 = BACK ? CH : min(CH, 16 * warp + 16 - d);
+#pragma unroll 4
+        for (int k = k0; k < k1; ++k) {
+            uint64_t av[4];
+            const ulonglong2 a0 = *reinterpret_cast<const ulonglong2*>(A + k * PQ + 4 * lq);
+            const ulonglong2 a1 = *reinterpret_cast<const ulonglong2*>(A + k * PQ + 64 + 4 * lq);
+            av[0] = a0.x; av[1] = a0.y; av[2] = a1.x; av[3] = a1.y;
+            const float4 b0 = *reinterpret_cast<const float4*>(B + k * CB);
+            const float4 b1 = *reinterpret_cast<const float4*>(B + k * CB + 4);
+            const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                const uint64_t bb = tc::f2pack(b[c], b[c]);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) acc[i][c] = tc::f2fma(av[i], bb, acc[i][c]);
+            }
+        }
         __syncthreads();
         if (tid == 0 && on && r + NST < nr) {
             tc::fence_proxy_async();                 // the CTA's reads of this stage precede the refill
@@ -188,91 +179,62 @@ __global__ void __launch_bounds__(PT, 3) k_tri(const TriJob p) {
             while (!tc::mbar_try_wait(full + r % NST, (uint32_t)(r / NST) & 1u) && tc::global_ns() - t0 < 200000000ull) {
             }
     }
-    const int col = CB * cb + c;
+    float o[8][8];                                   // query, column
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        float l[2], u[2];
-        tc::f2unpack(lo[i], l[0], l[1]);
-        tc::f2unpack(hi[i], u[0], u[1]);
+    for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            const int q = q0 + 16 * g + 2 * i + e;
-            if (q >= p.Q) continue;
-            // row q, or its place among rows padded from rk to rkpad
-            const size_t row = p.rk ? (size_t)(q / p.rk) * p.rkpad + q % p.rk : (size_t)q;
-            float* o = p.out + row * p.ldo + col;
-            if (col < p.ldo) o[0] = l[e];
-            if (col + 64 < p.ldo) o[64] = u[e];
-        }
-    }
-}
-
-__device__ __forceinline__ float warp_sum(float v) {
+        for (int c = 0; c < 8; ++c) tc::f2unpack(acc[i][c], o[2 * i][c], o[2 * i + 1][c]);
+    if (!BACK) {
+        float* v = p.out + ((size_t)tile * p.ldo + CB * cb + c0) * PQ + 4 * lq;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
-// |v_q|^2 of the rows of V, one warp a query
-//   kSumPairs  pairs of 8-column groups from both ends of the Np columns (equal
-//              triangular work), each pair one chain, the pairs in order
-//   kSumLanes  lane l the columns l mod 32, then the shuffle tree
-template <int ORDER>
-__global__ void __launch_bounds__(256) k_rowsum(const float* __restrict__ V, int ld, int Q, int Np, float* __restrict__ out) {
-    const int q = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    grid_wait();
-    if (q >= Q) return;
-    const float* v = V + (size_t)q * ld;
-    float s = 0.0f;
-    if (ORDER == kSumPairs) {
-        const int np = Np / 16;
-        for (int p0 = 0; p0 < np; p0 += 32) {
-            const int p = p0 + lane;
-            float t = 0.0f;
-            if (p < np) {
-                float a[8], b[8];
-                *reinterpret_cast<float4*>(a) = __ldcg(reinterpret_cast<const float4*>(v + 8 * p));
-                *reinterpret_cast<float4*>(a + 4) = __ldcg(reinterpret_cast<const float4*>(v + 8 * p + 4));
-                *reinterpret_cast<float4*>(b) = __ldcg(reinterpret_cast<const float4*>(v + Np - 8 * (p + 1)));
-                *reinterpret_cast<float4*>(b + 4) = __ldcg(reinterpret_cast<const float4*>(v + Np - 8 * (p + 1) + 4));
-#pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    t = fmaf(a[c], a[c], t);
-                    t = fmaf(b[c], b[c], t);
-                }
-            }
-            const int n = min(32, np - p0);
-            for (int i = 0; i < n; ++i) s += __shfl_sync(0xffffffffu, t, i);
+        for (int c = 0; c < 8; ++c) {
+            *reinterpret_cast<float4*>(v + c * PQ) = make_float4(o[0][c], o[1][c], o[2][c], o[3][c]);
+            *reinterpret_cast<float4*>(v + c * PQ + 64) = make_float4(o[4][c], o[5][c], o[6][c], o[7][c]);
         }
     } else {
-        for (int i = lane; i < Np; i += 32) {
-            const float x = __ldcg(v + i);
-            s = fmaf(x, x, s);
+        // row q, at its place among rows padded from rk to rkpad; 8 columns at a
+        // time (ldo is a multiple of 16)
+        const int col = CB * cb + c0;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int q = q0 + (i >> 2) * 64 + 4 * lq + (i & 3);
+            if (q >= p.Q || col >= p.ldo) continue;
+            float* b = p.out + ((size_t)(q / p.rk) * p.rkpad + q % p.rk) * p.ldo + col;
+            *reinterpret_cast<float4*>(b) = make_float4(o[i][0], o[i][1], o[i][2], o[i][3]);
+            *reinterpret_cast<float4*>(b + 4) = make_float4(o[i][4], o[i][5], o[i][6], o[i][7]);
         }
-        s = warp_sum(s);
     }
-    if (lane == 0) out[q] = s;
 }
 
-// the same, thread i mod 256 of a CTA per query, warps in order
-__global__ void __launch_bounds__(256) k_rowsum_block(const float* __restrict__ V, int ld, int N, float* __restrict__ out) {
-    __shared__ float red[8];
-    const int tid = threadIdx.x;
+// |v_q|^2, one thread a query
+//   kSumPairs  pairs of 8-column groups from both ends of the Np columns (equal
+//              triangular work), each pair one chain, the pairs in order
+//   kSumLanes  32 chains over the columns l mod 32, added as a tree
+template <int ORDER>
+__global__ void __launch_bounds__(PQ) k_rowsum(const float* __restrict__ V, int ld, int Q, int Np, float* __restrict__ out) {
     grid_wait();
-    const float* v = V + (size_t)blockIdx.x * ld;
+    const float* v = V + (size_t)blockIdx.x * ld * PQ + threadIdx.x;
     float s = 0.0f;
-    for (int i = tid; i < N; i += 256) {
-        const float x = __ldcg(v + i);
-        s = fmaf(x, x, s);
+    if (ORDER == kSumPairs) {
+        for (int p = 0; p < Np / 16; ++p) {
+            float a[8], b[8], t = 0.0f;
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                a[c] = __ldcg(v + (size_t)(8 * p + c) * PQ);
+                b[c] = __ldcg(v + (size_t)(Np - 8 * (p + 1) + c) * PQ);
+            }
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                t = fmaf(a[c], a[c], t);
+                t = fmaf(b[c], b[c], t);
+            }
+            s += t;
+        }
+    } else {
+        s = lane_squares<32>(v, PQ, 0, Np);
     }
-    s = warp_sum(s);
-    if ((tid & 31) == 0) red[tid >> 5] = s;
-    __syncthreads();
-    if (tid == 0) {
-        float t = 0.0f;
-        for (int i = 0; i < 8; ++i) t += red[i];
-        out[blockIdx.x] = t;
-    }
+    const int q = blockIdx.x * PQ + threadIdx.x;
+    if (q < Q) out[q] = s;
 }
 
 // L^-1 in the pieces of the backward product: block column cb holds rows
@@ -290,14 +252,15 @@ template <bool BACK>
 int launch_tri(const TriJob& j, bool dependent, cudaStream_t st) {
     const dim3 grid((unsigned)((j.Q + PQ - 1) / PQ), (unsigned)((j.N + CB - 1) / CB));
     auto kern = j.fusez ? k_tri<BACK, true> : k_tri<BACK, false>;
-    GPM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM));
-    GPM_CUDA(launch_ex(kern, grid, PT, SMEM, st, dependent, 1u, j));
+    const int smem = TriLayout<BACK>::total;
+    GPM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    GPM_CUDA(launch_ex(kern, grid, PT, smem, st, dependent, 1u, j));
     return GPMPPI_OK;
 }
 
 }  // namespace
 
-// the forward product of GP g's output o at Q queries (z: Q x 4) into V (Q x npad)
+// the forward product of a GP at Q queries (z: Q x 4) into V (tiles of 128 queries x npad)
 TriJob tri_forward(const GpSet::One& G, const float* z, int Q, float* V) {
     TriJob j = {};
     j.z = z;
@@ -324,13 +287,8 @@ int launch_rowsum(const float* V, int ld, int Q, int N, SumOrder order, float* o
     if (Q <= 0) return GPMPPI_OK;
     int Np = (N + 15) / 16 * 16;
     if (Np > 0 && Np < 64) Np = 64;
-    const dim3 grid((unsigned)((Q + 7) / 8));
-    if (order == kSumBlock)
-        GPM_CUDA(launch_ex(k_rowsum_block, dim3((unsigned)Q), 256, 0, st, true, 1u, V, ld, N, out));
-    else if (order == kSumPairs)
-        GPM_CUDA(launch_ex(k_rowsum<kSumPairs>, grid, 256, 0, st, true, 1u, V, ld, Q, Np, out));
-    else
-        GPM_CUDA(launch_ex(k_rowsum<kSumLanes>, grid, 256, 0, st, true, 1u, V, ld, Q, Np, out));
+    auto kern = order == kSumPairs ? k_rowsum<kSumPairs> : k_rowsum<kSumLanes>;
+    GPM_CUDA(launch_ex(kern, dim3((unsigned)((Q + PQ - 1) / PQ)), PQ, 0, st, true, 1u, V, ld, Q, Np, out));
     return GPMPPI_OK;
 }
 
