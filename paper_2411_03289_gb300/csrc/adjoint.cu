@@ -340,6 +340,7 @@ __global__ void __launch_bounds__(GT) k_grad_rev(const GradArgs g) {
                     z2 = zq.z * a.zscale[2], z3 = zq.w * a.zscale[3];
         float zb[4] = {0.f, 0.f, 0.f, 0.f};
         float lb[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
         for (int j = lane; j < a.N; j += 32) {
             const float4 x = ldg4(a.Xs + 4 * j);
             const float d[4] = {z0 - x.x, z1 - x.y, z2 - x.z, z3 - x.w};

@@ -64,8 +64,12 @@ __device__ __forceinline__ void factor_diag(double m, double (*v)[NB + 1], doubl
                 if (tx == 0) atomicExch(flag, 1);   // the host reports NOT_PD; go on with finite values
                 d = 1.0;
             }
-            const double p = sqrt(d);
-            m = tx == c ? p : quotient(m, p, 1.0 / p);
+            // square root by its remainder (Markstein) from the reciprocal root, which
+            // then also serves the quotients: a third of the chain of sqrt and 1 / p
+            const double y = rsqrt(d);
+            double p = d * y;
+            p = fma(fma(-p, p, d), 0.5 * y, p);
+            m = tx == c ? p : quotient(m, p, y);
             v[c & 1][tx] = m;
             if (tx >= c) D[tx * NB + c] = m;
         }
@@ -86,46 +90,54 @@ __global__ void __launch_bounds__(NB * NB) k_first_diag(const double* __restrict
     factor_diag(diag_value(M, N, 0), v, D, flag);
 }
 
-// Step k's panel, from the factor D of its diagonal block, by substitution, one
-// warp a block: L_bk D^T = A_bk for the blocks b > k (to P, N x 32; a lane has a
-// row), D (L^-1)_kb = R_kb for b < k and D (L^-1)_kk = I (a lane has a column).
-// A value's updates go out as soon as it is known, which leaves up to 31
-// independent multiply-adds.
-__global__ void __launch_bounds__(NB) k_panel(double* __restrict__ M, int N, int k, const double* __restrict__ D,
-                                              double* __restrict__ P) {
+// Step k's panel, from the factor D of its diagonal block, by substitution:
+// L_bk D^T = A_bk for the blocks b > k (to P, N x 32; a vector is a row), D
+// (L^-1)_kb = R_kb for b < k and D (L^-1)_kk = I (a vector is a column).  A warp
+// takes 8 of a block's 32 vectors, four lanes a vector, lane g its elements g,
+// g + 4, ...: a value's updates go out as soon as it is known.  What bounds it is
+// the FP64 pipe's rate for one warp, 64 clocks an instruction, on the critical
+// path of every step: about 300 instructions (10 us), where a lane per vector took
+// 700 (40 us).
+__global__ void __launch_bounds__(128) k_panel(double* __restrict__ M, int N, int k, const double* __restrict__ D,
+                                               double* __restrict__ P) {
     __shared__ double d[NB][NB + 1], t[NB][NB + 1], rcp[NB];
-    const int tx = threadIdx.x, b = blockIdx.x, kb = NB * k, bb = NB * b;
-#pragma unroll 8
-    for (int i = 0; i < NB; ++i) {
-        d[i][tx] = D[i * NB + tx];                   // (the upper triangle is not read)
-        if (b > k)
-            t[i][tx] = bb + i < N ? M[(size_t)(bb + i) * N + kb + tx] : 0.0;
-        else if (b < k)
-            t[tx][i] = kb + i < N ? M[(size_t)(kb + i) * N + bb + tx] : 0.0;
-        else
-            t[tx][i] = i == tx ? 1.0 : 0.0;
-    }
-    __syncwarp();
-    rcp[tx] = 1.0 / d[tx][tx];
-    __syncwarp();
-    double x[NB];
+    const int tid = threadIdx.x, lane = tid & 31, b = blockIdx.x, kb = NB * k, bb = NB * b;
 #pragma unroll
-    for (int i = 0; i < NB; ++i) x[i] = t[tx][i];
+    for (int i = tid >> 5; i < NB; i += 4) {
+        d[i][lane] = D[i * NB + lane];                   // (the upper triangle is not read)
+        if (b > k)
+            t[i][lane] = bb + i < N ? M[(size_t)(bb + i) * N + kb + lane] : 0.0;
+        else if (b < k)
+            t[lane][i] = kb + i < N ? M[(size_t)(kb + i) * N + bb + lane] : 0.0;
+        else
+            t[lane][i] = i == lane ? 1.0 : 0.0;
+    }
+    __syncthreads();
+    if (tid < NB) rcp[tid] = 1.0 / d[tid][tid];
+    __syncthreads();
+    const int vec = 8 * (tid >> 5) + (lane >> 2), g = lane & 3;
+    double x[NB / 4];
+#pragma unroll
+    for (int e = 0; e < NB / 4; ++e) x[e] = t[vec][4 * e + g];
 #pragma unroll
     for (int q = 0; q < NB; ++q) {
-        x[q] = quotient(x[q], d[q][q], rcp[q]);
+        const int e = q >> 2;
+        const double xq = __shfl_sync(0xffffffffu, quotient(x[e], d[q][q], rcp[q]), (lane & ~3) | (q & 3));
+        if (g == (q & 3)) x[e] = xq;
+        const double u = x[e] - d[4 * e + g][q] * xq;
+        if (g > (q & 3)) x[e] = u;
 #pragma unroll
-        for (int c = q + 1; c < NB; ++c) x[c] -= d[c][q] * x[q];
+        for (int f = e + 1; f < NB / 4; ++f) x[f] -= d[4 * f + g][q] * xq;
     }
-    if (b > k) {
 #pragma unroll
-        for (int i = 0; i < NB; ++i) t[tx][i] = x[i];
-        __syncwarp();
-        for (int i = 0; i < NB && bb + i < N; ++i) P[(size_t)(bb + i) * NB + tx] = t[i][tx];
-    } else {
-#pragma unroll
-        for (int i = 0; i < NB; ++i)
-            if (kb + i < N && bb + tx < N) M[(size_t)(kb + i) * N + bb + tx] = x[i];
+    for (int e = 0; e < NB / 4; ++e) t[vec][4 * e + g] = x[e];
+    __syncthreads();
+    for (int i = tid >> 5; i < NB; i += 4) {
+        if (b > k) {
+            if (bb + i < N) P[(size_t)(bb + i) * NB + lane] = t[i][lane];
+        } else if (kb + i < N && bb + lane < N) {
+            M[(size_t)(kb + i) * N + bb + lane] = t[lane][i];
+        }
     }
 }
 
@@ -528,7 +540,7 @@ int gp_fit_device(GpDevice& g, const double* X, const double* Y, int N, cudaStre
             h.signal_var, h.noise_var, M);
         k_first_diag<<<1, dim3(NB, NB), 0, st>>>(M, N, dD, dflag);
         for (int k = 0; k < nblk; ++k) {
-            k_panel<<<nblk, NB, 0, st>>>(M, N, k, dD, dP);
+            k_panel<<<nblk, 128, 0, st>>>(M, N, k, dD, dP);
             const int blocks = nblk * (nblk + 1) / 2 - (k + 1) * (k + 2) / 2;
             if (blocks > 0) k_update<<<blocks, dim3(NB, NB), 0, st>>>(M, N, k, dP, dD, dflag);
         }

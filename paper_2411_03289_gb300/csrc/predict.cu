@@ -82,15 +82,18 @@ __global__ void __launch_bounds__(ST) k_pred_mean(const PredArgs p) {
     }
 }
 
-// the variances from the rows of v, one thread a query: the squares as 128 threads
-// of a CTA would sum them, four warps' trees in order
-__global__ void __launch_bounds__(kTriTile) k_pred_var(const PredArgs p) {
+// the variances from the rows of v: the squares as 128 threads of a CTA would sum
+// them, four threads a query for the four warps' trees, added in order
+__global__ void __launch_bounds__(4 * kTriTile) k_pred_var(const PredArgs p) {
+    __shared__ float red[4][kTriTile];
+    const int w = threadIdx.x / kTriTile, l = threadIdx.x % kTriTile;
     qr::grid_wait();
-    const float* v = p.V + (size_t)blockIdx.x * p.npad * kTriTile + threadIdx.x;
+    red[w][l] = qr::lane_squares<128>(p.V + (size_t)blockIdx.x * p.npad * kTriTile + l, kTriTile, 32 * w, p.N);
+    __syncthreads();
+    const int q = blockIdx.x * kTriTile + l;
+    if (w > 0 || q >= p.M) return;
     float qf = 0.0f;
-    for (int w = 0; w < 4; ++w) qf += qr::lane_squares<128>(v, kTriTile, 32 * w, p.N);
-    const int q = blockIdx.x * kTriTile + threadIdx.x;
-    if (q >= p.M) return;
+    for (int i = 0; i < 4; ++i) qf += red[i][l];
     const float s = fmaxf(0.0f, p.sf2 - qf);
     if (p.out != 1) p.var[2 * (size_t)q] = s;
     if (p.out != 0) p.var[2 * (size_t)q + 1] = s;
@@ -139,7 +142,7 @@ int launch_gp_predict(const GpDevice& g, const float* Z, int M, float* mean, flo
             j.fusez = 1;
             rc = launch_tri_forward(j, false, st);
             if (rc) break;
-            cudaError_t e = launch_ex(k_pred_var, dim3((unsigned)((p.M + kTriTile - 1) / kTriTile)), kTriTile, 0, st, true, 1u, p);
+            cudaError_t e = launch_ex(k_pred_var, dim3((unsigned)((p.M + kTriTile - 1) / kTriTile)), 4 * kTriTile, 0, st, true, 1u, p);
             if (e == cudaSuccess) {
                 k_pred_mean<<<p.M, ST, 0, st>>>(p);
                 e = cudaGetLastError();
