@@ -258,7 +258,7 @@ class ClockSampler:
 # measured DRAM traffic of the rollout kernel (from the committed ncu summary)
 # ---------------------------------------------------------------------------
 
-def committed_traffic(kernel="rollout_fp32", workload=WORKLOAD):
+def committed_traffic(kernel="tri", workload=WORKLOAD):
     """DRAM bytes per launch from the committed ncu summary of this kernel and
     workload, if it was taken on the current sources: the summary records the
     sha256 of the kernel's .cu file and of every other source it names, and
@@ -279,6 +279,17 @@ def committed_traffic(kernel="rollout_fp32", workload=WORKLOAD):
             return None
     m_tr = re.search(r"dram bytes per launch \(full workload\):\s*([0-9.eE+]+)", txt)
     return float(m_tr.group(1)) if m_tr else None
+
+
+def step_launches(P, sizes):
+    """Kernels of one mppi_step over GPs of these sizes: the chain, the variances
+    (split precisions: one kernel; FP32: a product and its row sums for each GP and
+    each 512 MB of rows), the stage costs and the update."""
+    if P.precision != 0:
+        return 4
+    npad = max((n + 127) // 128 * 128 for n in sizes)
+    rows = max(1, (1 << 27) // max(npad, 1) // 128 * 128)
+    return 3 + 2 * len(sizes) * -(-P.K * P.T // rows)
 
 
 # ---------------------------------------------------------------------------
@@ -456,7 +467,7 @@ def fp32_path(args, gp, S, dev, flush, stream, barrier, peaks=None):
     flops = rollout_flops_per_sample_step(sc.N, sc.obstacles.shape[0], S_seg) * P.K * P.T
     r_avg = sum(rollout_ms) / len(rollout_ms)
     ach = flops / (r_avg / 1e3) / 1e12
-    roof = alu_roof(ach, peaks, "k_rollout_fp32", committed_traffic("rollout_fp32", args.workload))
+    roof = alu_roof(ach, peaks, "k_tri", committed_traffic("tri", args.workload))
     if peaks:
         # the kernel rows' exponentials: N per sample-step on the SFU
         ex2 = sc.N * P.K * P.T / (r_avg / 1e3) / 1e9
@@ -488,8 +499,8 @@ def _tc_leg(args, gp, dev, flush, stream, barrier, sc, ctrl, flops, profile_key,
             "kernel_ms": {"rollout_avg": r_avg, "update_avg": sum(update_ms) / len(update_ms)},
             "roofline": {"bound": "tensor", "achieved": ach, "peak": peak, "unit": "TFLOP/s",
                          "frac": ach / peak, "peak_note": note,
-                         "kernel": "k_rollout_mma" if kind == gp.GPMPPI_KERNEL_TC_STREAM else str(kind),
-                         "traffic": committed_traffic("rollout_mma", profile_key)}}
+                         "kernel": "k_var_tc" if kind == gp.GPMPPI_KERNEL_TC_STREAM else str(kind),
+                         "traffic": committed_traffic("variance_tc", profile_key)}}
 
 
 def cfg3_leg(args, gp, S, dev, flush, stream, barrier, precision="fp16split"):
@@ -661,16 +672,16 @@ def run_ours(args):
     r_avg = sum(rollout_ms) / len(rollout_ms)
     achieved = flops / (r_avg / 1e3) / 1e12
     kind = gp.mppi_rollout_kind(ctrl)
-    src, kname = {gp.GPMPPI_KERNEL_FP32: ("rollout_fp32", "k_rollout_fp32"),
-                  gp.GPMPPI_KERNEL_TC_STREAM: ("rollout_mma", "k_rollout_mma"),
-                  gp.GPMPPI_KERNEL_TC_CLUSTER: ("rollout_cluster", "k_rollout_cl"),
-                  gp.GPMPPI_KERNEL_ENSEMBLE: ("ensemble", "k_rollout_ens")}[kind]
+    src, kname = {gp.GPMPPI_KERNEL_FP32: ("tri", "k_tri"),
+                  gp.GPMPPI_KERNEL_TC_STREAM: ("variance_tc", "k_var_tc"),
+                  gp.GPMPPI_KERNEL_TC_CLUSTER: ("variance_tc", "k_var_tc"),
+                  gp.GPMPPI_KERNEL_ENSEMBLE: ("tri", "k_tri")}[kind]
     traffic = committed_traffic(src, args.workload)
     peaks = measure_alu_peaks(gp, dev, stream) if not args.no_alu_peaks else None
     if terrain and P.precision == 0:
-        roof = alu_roof(achieved, peaks, "k_rollout_ens", traffic, "; flops summed over the three terrain GPs")
+        roof = alu_roof(achieved, peaks, "k_tri", traffic, "; flops summed over the three terrain GPs")
     elif P.precision == 0:
-        roof = alu_roof(achieved, peaks, "k_rollout_fp32", traffic)
+        roof = alu_roof(achieved, peaks, "k_tri", traffic)
     else:
         peak, note = measured_tensor_peak()
         if terrain:
@@ -702,7 +713,7 @@ def run_ours(args):
             **describe(sc), "workload": f"{sc.name}: K={P.K} T={P.T} three terrain GPs of N={sc.terrains[0][0].shape[0]} "
                                         f"mixed by Eq. 3 (w={sc.terrain_w}), obstacles={sc.obstacles.shape[0]}, "
                                         f"figure-eight, {args.precision}", "terrains": 3},
-        "gpu_launches": 2 * args.steps,
+        "gpu_launches": step_launches(P, [t[0].shape[0] for t in sc.terrains] if terrain else [sc.N]) * args.steps,
         "kernel_ms": {"rollout_avg": r_avg, "update_avg": sum(update_ms) / len(update_ms)},
         "roofline": roof,
         "cpu_baseline": cpu_baseline(workload=args.workload) if (rank == 0 and ws == 1 and not args.no_cpu) else None,
@@ -871,12 +882,13 @@ def run_grad(args):
         "vs_baseline": None, "dtype": "f32", "data": "synthetic (seeded GP training set, obstacles, figure-eight path)",
         "config": {"workload": f"cfg4: K={P.K} T={P.T} N={sc.N} obstacles={sc.obstacles.shape[0]} figure-eight, "
                                f"gradient of the sigmoid-smoothed cost (slope {GRAD_SLOPE:g}) in U and the "
-                               f"lengthscales, checkpoints every ceil(sqrt(T)) steps",
+                               f"lengthscales",
                    "K": P.K, "T": P.T, "N": sc.N, "obstacles": int(sc.obstacles.shape[0]),
                    "l2": f"flushed between timed steps ({L2_FLUSH_BYTES >> 20} MiB write)"},
-        "gpu_launches": 3 * args.steps,
+        # chain, product, sums, forward, product, reverse, Gram traces, reduction
+        "gpu_launches": 8 * args.steps,
         "kernel_ms": {"adjoint_avg": a_avg, "gram_trace_and_reduce_avg": sum(rest_ms) / len(rest_ms)},
-        "roofline": alu_roof(achieved, peaks, "k_grad", committed_traffic("adjoint", "cfg4")),
+        "roofline": alu_roof(achieved, peaks, "k_tri", committed_traffic("tri", "cfg4")),
         "alu_peaks": peaks,
         "cpu_baseline": grad_cpu_baseline() if (ws == 1 and not args.no_cpu) else None,
         "e2e": {"value": units * n_e2e * ws / e2e_s, "unit": "sample-steps/s",
@@ -988,7 +1000,8 @@ def run_batched(args):
                    "autotune_layouts_changed": chosen, "precision": args.precision,
                    "l2": f"flushed between timed steps ({L2_FLUSH_BYTES >> 20} MiB write)",
                    "fit_and_create_s": t_fit},
-        "gpu_launches": 2 * args.steps,
+        # the persistent rollout and the update, and the FP32 controllers' own rollouts
+        "gpu_launches": (2 + sum(step_launches(s.params, [s.N]) - 1 for s in scs if s.params.precision == 0)) * args.steps,
         "roofline": {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                      "frac": achieved / peak, "traffic": None, "kernel": "k_rollout_persistent",
                      "peak_note": note + "; whole batched step timed"},

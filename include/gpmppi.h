@@ -202,12 +202,12 @@ int mppi_get_iteration(gpmppi_ctrl c, uint64_t* it);
  * (Alg. 1 Step 2), T x 3 floats (Sxx, Sxy, Syy) of Sigma_XY(k+1), device. */
 int mppi_nominal_sxy(gpmppi_ctrl c, float* sxy, void* stream);
 
-/* Which rollout kernel mppi_step runs for this controller (host int32):
- * GPMPPI_KERNEL_FP32 (CUDA cores), GPMPPI_KERNEL_TC_STREAM (tensor cores,
- * factor tiles streamed per step), GPMPPI_KERNEL_TC_CLUSTER (tensor cores,
- * factor resident in a CTA cluster; split precisions with N <= 512 when the
- * cluster fits the device) or GPMPPI_KERNEL_ENSEMBLE (FP32 terrain ensemble;
- * a terrain ensemble in the split precisions reports GPMPPI_KERNEL_TC_STREAM). */
+/* The class of rollout mppi_step runs for this controller (host int32):
+ * GPMPPI_KERNEL_FP32 (variances on the CUDA cores), GPMPPI_KERNEL_TC_CLUSTER
+ * (on the tensor cores, two-part formats with 0 < N <= 512),
+ * GPMPPI_KERNEL_TC_STREAM (on the tensor cores, everything else in the split
+ * precisions, terrain ensembles included) or GPMPPI_KERNEL_ENSEMBLE (FP32
+ * terrain ensemble).  The two tensor-core classes run the same kernels. */
 #define GPMPPI_KERNEL_FP32 0
 #define GPMPPI_KERNEL_TC_STREAM 1
 #define GPMPPI_KERNEL_TC_CLUSTER 2
@@ -215,10 +215,10 @@ int mppi_nominal_sxy(gpmppi_ctrl c, float* sxy, void* stream);
 int mppi_rollout_kind(gpmppi_ctrl c, int32_t* kind);
 
 /* Per-kernel timing of mppi_step.  When enabled, mppi_step records CUDA
- * events on its stream around the rollout kernel and around the update
+ * events on its stream around the rollout's kernels and around the update
  * kernel(s); mppi_last_profile waits for the last step's events and returns
  * the two durations in milliseconds (host floats).  mppi_grad records the
- * same pair around its adjoint kernel and around the rest (Gram trace and
+ * same pair around its forward and reverse passes and around the rest (Gram trace and
  * reductions); the last call of either is reported.  Off by default. */
 int mppi_set_profiling(gpmppi_ctrl c, int32_t on);
 int mppi_last_profile(gpmppi_ctrl c, float* rollout_ms, float* update_ms);
@@ -239,11 +239,11 @@ int mppi_destroy(gpmppi_ctrl c);
  * controller keeps them alive as mppi_create does), weights: host, M floats
  * (any finite values; Eq. 4 keeps them on the simplex).  2 <= M <= 8, or
  * M = 1 (weight 1 gives the single-GP controller of mppi_create).  Needs
- * the per-sample variance mode (else GPMPPI_ERR_UNSUPPORTED).  In FP32 the
- * ensemble rollout runs on the CUDA cores; in the split precisions the
- * streaming tensor-core rollout runs over the GPs' factors stacked
- * block-diagonally (each GP's block count rounded up to even; UNSUPPORTED
- * when the GPs' training sets do not fit shared memory together).
+ * the per-sample variance mode (else GPMPPI_ERR_UNSUPPORTED).  In the split
+ * precisions a batch runs it over the GPs' factors stacked block-diagonally
+ * (each GP's block count rounded up to even); GPs whose training sets do not
+ * fit shared memory together there are refused here (UNSUPPORTED), and in FP32
+ * those of more than 3616 points.
  * mppi_step and mppi_rollout_trace use it; mppi_grad rejects it; the batch
  * API takes it in the split precisions only.
  * mppi_set_terrain_weights replaces the weights (host, M floats) for the
@@ -290,7 +290,8 @@ int terrain_weights(const double* Yv, const double* Yw, const double* Fv, const 
  *                  alpha = K^-1 y and K^-1 on the lengthscales (one more kernel
  *                  and T * K * N floats of scratch)
  * Needs variance mode GPMPPI_VAR_PER_SAMPLE (else GPMPPI_ERR_UNSUPPORTED) and
- * enough shared memory for 2 x 8 x N floats (GPMPPI_ERR_UNSUPPORTED beyond).
+ * 64 N + 768 sqrt(T) bytes below the shared memory of a CTA
+ * (GPMPPI_ERR_UNSUPPORTED beyond).
  * The first call, and the first call asking for dlengthscale, allocate
  * device scratch owned by the controller (freed by mppi_destroy) and may
  * synchronise.  Runs on the controller's FP32 path whatever its precision. */
@@ -337,11 +338,11 @@ int mppi_update_noalloc(const float* costs, const float* u_tilde, const float* U
  * device memory while batched: it starts from the controller's counter at
  * creation, advances by one per batched step, and is read back with
  * mppi_batch_get_iteration (the controller's own counter is not updated).
- * A step = ONE persistent rollout launch (one CTA per SM) whose CTAs take
- * (controller, sample tile) items from an atomic work queue - FP32 tiles and
- * FP16- or BF16-split tensor-core tiles alike, longest first - then one update
- * launch for all controllers.  Controllers whose own mppi_step would use the
- * cluster rollout (N <= 512) run the streaming tensor-core body here; terrain
+ * A step = ONE persistent rollout launch (one CTA per SM) for the controllers in
+ * the split precisions, whose CTAs take (controller, sample tile) items from an
+ * atomic work queue, longest first, beside the FP32 controllers' own rollouts on
+ * internal streams that fork from the step's stream and join it; then one update
+ * launch for all controllers.  Terrain
  * ensembles in the split precisions are items like single-GP controllers
  * (their weights as set on the controller when a step is enqueued); FP32
  * terrain ensembles give GPMPPI_ERR_UNSUPPORTED. */
@@ -356,7 +357,7 @@ int mppi_batch_graph(gpmppi_batch b, void* stream);
 /* Autotuner, per controller shape (precision, K, T, N, lane segments,
  * obstacles): times one wave of the controller's tiles for each tensor-core
  * tile layout (2, 4 or 8 producer threads per sample, i.e. 128, 64 or 32
- * samples per tile; FP32 controllers have one layout), keeps the layout with
+ * samples per tile; an FP32 controller's rollout is timed whole), keeps the layout with
  * the least SM time (tiles x time per tile) and orders the work queue by the
  * measured time per tile.  Results are kept for the process and reused for
  * the same shape.  Runs rollouts only (their outputs are scratch; iteration
@@ -405,13 +406,13 @@ int gpmppi_alu_probe(int32_t kind, int32_t blocks, int32_t iters, float* out, vo
 
 /* Failure-detection hook (no counterpart in the paper) for the FP32
  * CUDA-core rollout of this controller:
- *   ns            time limit of each bounded wait for a tile copy of L^-T, in
+ *   ns            time limit of each bounded wait for a copy of a piece of L^-T, in
  *                 nanoseconds (default 2e9)
- *   expire_first  non-zero: before any copy, one warp of every CTA waits,
+ *   expire_first  non-zero: before any copy, one thread of every CTA waits,
  *                 bounded by ns, on an mbarrier that nothing arrives on, so
  *                 that the wait runs out
  * A wait that runs out records GPMPPI_ERR_TIMEOUT in the controller's status
- * word (mppi_device_status reports and clears it) and stops that warp's copies;
+ * word (mppi_device_status reports and clears it) and stops that CTA's copies;
  * the copies in flight land (bounded) before the CTA exits and the kernel ends
  * normally, so the context stays usable; that step's outputs are unspecified.
  * A host-side setting of this controller only (not applied in batches); no GPU

@@ -9,16 +9,14 @@
 // draws the perturbed controls of its samples and steps first, as they do not
 // depend on the state.
 // What bounds it: the issue slots of the point loop (about 30 instructions a
-// point, two thirds of them the two compensated additions).
+// point, two thirds of them the two compensated additions) and, below two warps a
+// scheduler, their latency.  K = 4096 T = 50 N = 500: 143 us.
 #include "query.cuh"
 
 namespace gpm {
 namespace {
 
 using namespace qr;
-
-constexpr int CT = 128;          // threads
-constexpr int CW = CT / 32;
 
 // sum over the warp's lanes
 __device__ __forceinline__ float tree_sum(float x) {
@@ -30,10 +28,10 @@ __device__ __forceinline__ float tree_sum(float x) {
 // TREE: the sums by the shuffle tree (G = 32), the GPs mixed by their weights.
 // FUSEZ: a difference z - x is one rounding, fma(z, scale, -x), instead of two.
 // SMEM: the training sets of all GPs staged in shared memory.
-template <int G, bool TREE, bool FUSEZ, bool SMEM>
-__global__ void __launch_bounds__(CT) k_chain32(const RolloutArgs a, const GpSet gs, const QueryWs ws) {
+template <int G, bool TREE, bool FUSEZ, bool SMEM, int CW>
+__global__ void __launch_bounds__(32 * CW) k_chain32(const RolloutArgs a, const GpSet gs, const QueryWs ws) {
     extern __shared__ __align__(16) unsigned char csm[];
-    constexpr int SPW = 32 / G, SPC = CW * SPW;    // samples per warp, per CTA
+    constexpr int CT = 32 * CW, SPW = 32 / G, SPC = CW * SPW;    // samples per warp, per CTA
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int l0 = blockIdx.x * SPC;
     const int ls = l0 + warp * SPW + lane / G, g = lane % G;
@@ -143,23 +141,28 @@ __global__ void __launch_bounds__(CT) k_chain32(const RolloutArgs a, const GpSet
     if (writer) ws.zq[(size_t)T * Ks + l] = make_float4(mu3, mu4, 0.0f, 0.0f);
 }
 
+template <int G, bool TREE, bool FUSEZ, bool SMEM, int CW>
+int launch_w(const RolloutArgs& a, const GpSet& gs, const QueryWs& ws, size_t bytes, cudaStream_t st) {
+    constexpr int SPC = CW * 32 / G;
+    auto kern = k_chain32<G, TREE, FUSEZ, SMEM, CW>;
+    GPM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024));
+    kern<<<(unsigned)((ws.Ks + SPC - 1) / SPC), 32 * CW, bytes, st>>>(a, gs, ws);
+    GPM_CUDA(cudaGetLastError());
+    return GPMPPI_OK;
+}
+
 template <int G, bool TREE, bool FUSEZ>
 int launch_t(const RolloutArgs& a, const GpSet& gs, const QueryWs& ws, cudaStream_t st) {
     size_t bytes = 0;
     for (int t = 0; t < gs.M; ++t) bytes += (size_t)gs.gp[t].N * 16 + (size_t)(gs.gp[t].N + 1) / 2 * 16;
-    // two CTAs per SM keep their training sets in shared memory up to 4096 points
-    const bool sm = bytes <= 100 * 1024;
-    constexpr int SPC = CW * 32 / G;
-    const dim3 grid((unsigned)((ws.Ks + SPC - 1) / SPC));
-    if (sm) {
-        auto kern = k_chain32<G, TREE, FUSEZ, true>;
-        GPM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024));
-        kern<<<grid, CT, bytes, st>>>(a, gs, ws);
-    } else {
-        k_chain32<G, TREE, FUSEZ, false><<<grid, CT, 0, st>>>(a, gs, ws);
-    }
-    GPM_CUDA(cudaGetLastError());
-    return GPMPPI_OK;
+    // Eight-lane samples: CTAs of one warp (four samples) spread the warps over the
+    // schedulers evenly, where 256 CTAs of four are two on most SMs and one on the
+    // rest (K = 4096 T = 50 N = 500: 143 against 214 us).  With a sample a warp their
+    // copies of the training set cost more (N = 1000: 322 against 267 us).
+    // Training sets of up to 4096 points go to shared memory.
+    if (G == 8) return launch_w<G, TREE, FUSEZ, true, 1>(a, gs, ws, bytes, st);
+    if (bytes <= 100 * 1024) return launch_w<G, TREE, FUSEZ, true, 4>(a, gs, ws, bytes, st);
+    return launch_w<G, TREE, FUSEZ, false, 4>(a, gs, ws, 0, st);
 }
 
 }  // namespace

@@ -41,3 +41,66 @@ def test_fp32_in_pieces(lib):
     # 2^23 queries are recorded at a time: 5 x 1.7 M samples take two pieces
     sc = S.scenario("small", K=1_700_001, T=5, N=3, precision=0)
     _check_rows(lib, sc, np.array([0, 1, 1_677_720, 1_677_721, 1_677_722, 1_700_000]))
+
+
+@pytest.mark.parametrize("precision", [1, 2, 3])
+@pytest.mark.parametrize("K,T,N", [
+    (33, 3, 1), (64, 4, 63), (64, 4, 64), (65, 4, 65), (31, 33, 129), (300, 5, 255), (257, 4, 256), (129, 5, 257),
+    (200, 4, 449), (1, 1, 513), (90, 3, 769), (260, 2, 1025)])
+def test_split_tile_edges(lib, K, T, N, precision):
+    """The tensor-core variances: training sets around the 64-column steps of the
+    diagonal, the 256-column passes and the 32- and 64-point stages, query counts
+    around the 256 queries of a CTA pair, one pass or several split over the pairs."""
+    _check_rows(lib, S.scenario("small", K=K, T=T, N=N, precision=precision), _rows(K))
+
+
+@pytest.mark.parametrize("N", [1, 31, 127, 128, 129, 300, 1025])
+@pytest.mark.parametrize("M", [1, 127, 129])
+def test_predict_tile_edges(lib, N, M):
+    """gp_predict around the 128-query tiles and the 128-column blocks: the mean
+    and variance of the FP64 posterior, within the rounding of their FP32 sums
+    (N eps times the sums of magnitudes)."""
+    import torch
+    sc = S.scenario("small", K=33, T=2, N=N, precision=0)
+    g, _ = make_ctrl(lib, sc)
+    rng = np.random.default_rng(N * 1000 + M)
+    Z = (rng.random((M, 4)) * [2.0, 3.0, 2.0, 3.0] - [0.0, 1.5, 0.0, 1.5]).astype(np.float32)
+    mean = torch.empty(M, 2, device="cuda")
+    var = torch.empty(M, 2, device="cuda")
+    lib.gp_predict(g, torch.tensor(Z, device="cuda"), mean, var)
+    torch.cuda.synchronize()
+    eps = 2.0 ** -23
+    for o in range(2):
+        h = sc.hyper[o]
+        d = (Z[:, None].astype(np.float64) - sc.X[None]) / np.asarray(h.lengthscale)
+        k = h.signal_var * np.exp(-0.5 * (d * d).sum(-1))
+        Linv, alpha = lib.gp_factors(g, o)
+        Linv = np.asarray(Linv).reshape(N, N)
+        v = k @ Linv.T
+        # a kernel value is good to a few eps times its exponent's magnitude
+        rel = (8.0 + 2.0 * np.max((d * d).sum(-1))) * eps
+        tol_m = (rel + np.sqrt(N) * eps) * (np.abs(k) @ np.abs(np.asarray(alpha))) + eps
+        tol_v = 2.0 * (np.abs(v) * ((rel + np.sqrt(N) * eps) * (np.abs(k) @ np.abs(Linv).T))).sum(1) + 8 * eps * h.signal_var
+        assert np.all(np.abs(mean[:, o].cpu().numpy() - k @ np.asarray(alpha)) <= tol_m)
+        assert np.all(np.abs(var[:, o].cpu().numpy() - np.maximum(0.0, h.signal_var - (v * v).sum(1))) <= tol_v)
+
+
+def test_gradient_ragged_samples(lib):
+    """The adjoint over a sample count that is no multiple of its eight-row padding
+    and a training set past one block, against the FP64 central differences."""
+    sc = S.scenario("small", K=45, T=6, N=150, precision=0)
+    h = sc.hyper[0]
+    sc = sc.replace(hyper=(h, S.Hyper(tuple(h.lengthscale), h.signal_var, h.noise_var)))
+    import torch
+    _, ctrl = make_ctrl(lib, sc)
+    J, dU, dl = lib.mppi_grad(ctrl, sc.x0, torch.tensor(sc.U0, dtype=torch.float32, device="cuda"), 20.0, None,
+                              want_dl=True)
+    torch.cuda.synchronize()
+    x0, U = sc.x0.astype(np.float32).astype(np.float64), sc.U0.astype(np.float32).astype(np.float64)
+    Jo, _ = O.objective(sc, sc.hyper, x0, U, 0, None, 20.0)
+    gU, gL = O.fd_gradient(sc, sc.hyper, x0, U, 0, None, 20.0)
+    assert abs(float(J.cpu().numpy()[0]) - Jo) <= 1e-4 * abs(Jo)
+    for got, ref in ((dU, gU), (dl, gL)):
+        got, ref = got.cpu().numpy().ravel().astype(np.float64), np.asarray(ref).ravel()
+        floor = 1e-3 * np.max(np.abs(ref))
+        assert np.max(np.abs(got - ref) / np.maximum(np.abs(ref), floor)) <= 1e-3
