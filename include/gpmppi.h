@@ -56,7 +56,7 @@ extern "C" {
 #define GPMPPI_BF16_SPLIT 1   /* tensor cores: BF16 hi/lo operands, 3 products, FP32 sums */
 #define GPMPPI_FP16_SPLIT 2   /* tensor cores: FP16 hi/lo operands, 3 products, FP32 sums */
 #define GPMPPI_BF16_SPLIT3 3  /* tensor cores: BF16 hi/mid/lo operands, 6 products, FP32 sums
-                                 (the streaming rollout at every N; 24 operand bits)     */
+                                 (24 operand bits)                                         */
 
 /* limits of this library */
 #define GPMPPI_MAX_N 4096         /* GP training points      */

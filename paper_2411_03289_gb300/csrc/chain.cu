@@ -108,30 +108,22 @@ __global__ void __launch_bounds__(CT) k_chain(const RolloutArgs a, const GpSet g
         }
     }
     // clamped perturbed controls (Eq. 8) of this CTA's samples, every step
-    if (a.u_tilde) {
-        const int n = min(SPC, Ks - l0);
-        for (int i = tid; i < SPC * T; i += CT) {
-            const int k = i / SPC, q = i % SPC;
-            if (q >= n) continue;
-            const float2 e = control_eps((uint32_t)k, (uint32_t)(ws.s0 + l0 + q), it0, it1, a.key0, a.key1, a.sig_v,
-                                         a.sig_w);
-            float2 u;
-            u.x = fminf(fmaxf(__ldg(a.U + 2 * k) + e.x, a.umin0), a.umax0);
-            u.y = fminf(fmaxf(__ldg(a.U + 2 * k + 1) + e.y, a.umin1), a.umax1);
-            a.u_tilde[(size_t)k * K + ws.s0 + l0 + q] = u;
-        }
+    const int n = min(SPC, Ks - l0);
+    for (int i = tid; i < SPC * T; i += CT) {
+        const int k = i / SPC, q = i % SPC;
+        if (q >= n) continue;
+        const float2 e = control_eps((uint32_t)k, (uint32_t)(ws.s0 + l0 + q), it0, it1, a.key0, a.key1, a.sig_v,
+                                     a.sig_w);
+        float2 u;
+        u.x = fminf(fmaxf(__ldg(a.U + 2 * k) + e.x, a.umin0), a.umax0);
+        u.y = fminf(fmaxf(__ldg(a.U + 2 * k + 1) + e.y, a.umin1), a.umax1);
+        a.u_tilde[(size_t)k * K + ws.s0 + l0 + q] = u;
     }
     __syncthreads();
-    // the control of step k (no sampled controls: the nominal trajectory)
-    auto control = [&](int k) {
-        if (a.u_tilde) return a.u_tilde[(size_t)k * K + s];
-        return make_float2(fminf(fmaxf(__ldg(a.U + 2 * k), a.umin0), a.umax0),
-                           fminf(fmaxf(__ldg(a.U + 2 * k + 1), a.umin1), a.umax1));
-    };
-    float2 un = control(0);
+    float2 un = a.u_tilde[s];
     for (int k = 0; k < T; ++k) {
         const float2 ut = un;
-        if (k + 1 < T) un = control(k + 1);
+        if (k + 1 < T) un = a.u_tilde[(size_t)(k + 1) * K + s];
         if (lane < SG) zs[lane] = make_float4(mu3, mu4, ut.x, ut.y);
         __syncwarp();
         float mean_v = 0.0f, mean_w = 0.0f;

@@ -138,92 +138,12 @@ __device__ __forceinline__ void mma_commit_elect(uint64_t* bar) {
         : "memory");
 }
 
-// The same commit arriving on the mbarrier at bar's offset in every CTA of
-// the cluster whose bit is set in cta_mask (not in this CTA unless its bit is
-// set): a peer learns that this CTA's earlier MMAs have completed.
-__device__ __forceinline__ void mma_commit_mc_elect(uint64_t* bar, uint16_t cta_mask) {
-    asm volatile(
-        "{\n\t.reg .pred e;\n\t"
-        "elect.sync _|e, 0xffffffff;\n\t"
-        "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n\t}" ::"r"(
-            smem_addr(bar)),
-        "h"(cta_mask)
-        : "memory");
-}
-
-// One ring stage of four 16-point chunks, A from tensor memory: for chunk
-// j = 0 .. 3 the products A_hi,j x B_j (instruction descriptor i_hi) and
-// A_lo,j x B_j (i_lo), all into d_tmem, then the commit that arrives on bar
-// once they completed.  A_hi,j and A_lo,j start at TMEM columns a + 16 j and
-// a + 16 j + 8; B_j's descriptor is b0 + j * bstep.  The first product
-// accumulates only if acc0 != 0.  Warp-collective: one elect.sync picks the
-// lane that issues all nine instructions, which keeps the issue cost per MMA
-// below the tensor pipe's time for these small shapes.
-__device__ __forceinline__ void mma_stage4_elect(uint32_t d_tmem, uint32_t a, uint64_t b0, uint64_t bstep,
-                                                 uint64_t* bar, uint32_t acc0, uint32_t i_hi, uint32_t i_lo) {
-    asm volatile(
-        "{\n\t.reg .pred e, p0, p1;\n\t"
-        ".reg .b32 a1, a2, a3, a4, a5, a6, a7;\n\t"
-        ".reg .b64 b1, b2, b3;\n\t"
-        "add.u32 a1, %1, 8;\n\tadd.u32 a2, %1, 16;\n\tadd.u32 a3, %1, 24;\n\t"
-        "add.u32 a4, %1, 32;\n\tadd.u32 a5, %1, 40;\n\tadd.u32 a6, %1, 48;\n\t"
-        "add.u32 a7, %1, 56;\n\t"
-        "add.u64 b1, %2, %3;\n\tadd.u64 b2, b1, %3;\n\tadd.u64 b3, b2, %3;\n\t"
-        "elect.sync _|e, 0xffffffff;\n\t"
-        "setp.ne.b32 p0, %5, 0;\n\t"
-        "setp.ne.b32 p1, 1, 0;\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %6, p0;\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [a1], %2, %7, p1;\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [a2], b1, %6, p1;\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [a3], b1, %7, p1;\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [a4], b2, %6, p1;\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [a5], b2, %7, p1;\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [a6], b3, %6, p1;\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [a7], b3, %7, p1;\n\t"
-        "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%4];\n\t}" ::"r"(d_tmem),
-        "r"(a), "l"(b0), "l"(bstep), "r"(smem_addr(bar)), "r"(acc0), "r"(i_hi), "r"(i_lo)
-        : "memory");
-}
-
-// The same four chunks with A in shared memory: A_hi,j at descriptor a_j,
-// A_lo,j at a_j + lo_off; every product accumulates; no commit.
-__device__ __forceinline__ void mma_stage4_sa_elect(uint32_t d_tmem, uint64_t a0, uint64_t a1, uint64_t a2,
-                                                    uint64_t a3, uint64_t lo_off, uint64_t b0, uint64_t bstep,
-                                                    uint32_t i_hi, uint32_t i_lo) {
-    asm volatile(
-        "{\n\t.reg .pred e, p1;\n\t"
-        ".reg .b64 l0, l1, l2, l3, b1, b2, b3;\n\t"
-        "add.u64 l0, %1, %5;\n\tadd.u64 l1, %2, %5;\n\tadd.u64 l2, %3, %5;\n\tadd.u64 l3, %4, %5;\n\t"
-        "add.u64 b1, %6, %7;\n\tadd.u64 b2, b1, %7;\n\tadd.u64 b3, b2, %7;\n\t"
-        "elect.sync _|e, 0xffffffff;\n\t"
-        "setp.ne.b32 p1, 1, 0;\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %6, %8, p1;\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], l0, %6, %9, p1;\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %2, b1, %8, p1;\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], l1, b1, %9, p1;\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %3, b2, %8, p1;\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], l2, b2, %9, p1;\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %4, b3, %8, p1;\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], l3, b3, %9, p1;\n\t}" ::"r"(d_tmem),
-        "l"(a0), "l"(a1), "l"(a2), "l"(a3), "l"(lo_off), "l"(b0), "l"(bstep), "r"(i_hi), "r"(i_lo)
-        : "memory");
-}
-
 // Four consecutive 32-bit columns of this thread's TMEM lane (warp-collective;
 // warp w writes lanes 32 (w % 4) .. 32 (w % 4) + 31, encoded in taddr).
 __device__ __forceinline__ void tmem_st4(uint32_t taddr, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3) {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(taddr), "r"(r0), "r"(r1),
                  "r"(r2), "r"(r3)
                  : "memory");
-}
-// Sixteen consecutive 32-bit columns of this thread's TMEM lane (warp-collective).
-__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
-        "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};" ::"r"(taddr),
-        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
-        "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
-        : "memory");
 }
 // Wait until this thread's tcgen05.st writes are complete.
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
@@ -386,14 +306,6 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint64
 __device__ __forceinline__ void fence_proxy_async() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
-__device__ __forceinline__ void tma_load_2d(void* dst, const void* tmap, int x, int y, uint64_t* bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%2, %3}], [%4];" ::"r"(smem_addr(dst)),
-        "l"(reinterpret_cast<uint64_t>(tmap)), "r"(x), "r"(y), "r"(smem_addr(bar))
-        : "memory");
-}
-
 // Packed FP32 pairs (f32x2: two lanes per 64-bit register, element 0 in the
 // low half).  The kernel rows are computed two training points at a time, so
 // one packed instruction does the work of two scalar ones.
