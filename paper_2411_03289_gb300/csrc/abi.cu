@@ -313,27 +313,38 @@ int alloc_query_ws(gpmppi_ctrl c) {
     const size_t T = (size_t)c->p.T, M = (size_t)c->gset.M;
     size_t n = ((size_t)1 << 23) / T;
     if (n > (size_t)c->p.K) n = (size_t)c->p.K;
-    c->ws_Ks = (int)n;
     c->nsplit = c->fmt < 0 ? 1 : var_tc_splits(c->gset, (int)(n * T), c->nsm);
     cudaFree(c->ws_buf);
     c->ws_buf = nullptr;
-    cudaError_t e = cudaMalloc(&c->ws_buf, n * (16 * (2 * T + 1) + 4 * M * c->nsplit * T));
+    cudaError_t e;
+    // on a full device smaller pieces of the samples (the results are the same)
+    while ((e = cudaMalloc(&c->ws_buf, n * (16 * (2 * T + 1) + 4 * M * c->nsplit * T))) == cudaErrorMemoryAllocation &&
+           n > 64) {
+        cudaGetLastError();
+        n = (n / 2 + 31) / 32 * 32;
+    }
     if (e != cudaSuccess) return cuda_fail(e, "mppi_create: rollout workspace");
+    c->ws_Ks = (int)n;
     // rows of v: up to 512 MB at a time
     size_t npad = 0, rows = 0;
     for (size_t t = 0; t < M; ++t) npad = npad < (size_t)c->gset.gp[t].npad ? (size_t)c->gset.gp[t].npad : npad;
     if (c->fmt < 0) {
         rows = npad ? ((size_t)1 << 27) / npad / kTriTile * kTriTile : n * T;
         if (rows > n * T) rows = (n * T + kTriTile - 1) / kTriTile * kTriTile;
-        c->v_q = (int)rows;
     }
-    if (c->p.variance_mode == GPMPPI_VAR_NOMINAL && rows < 4 * T) rows = 4 * T;     // 2 T N doubles
+    const size_t least = c->p.variance_mode == GPMPPI_VAR_NOMINAL ? 4 * T : 0;      // 2 T N doubles
     cudaFree(c->vbuf);
     c->vbuf = nullptr;
-    if (rows * npad > 0) {
-        e = cudaMalloc(&c->vbuf, sizeof(float) * rows * npad);
+    if ((rows > least ? rows : least) * npad > 0) {
+        while ((e = cudaMalloc(&c->vbuf, sizeof(float) * (rows > least ? rows : least) * npad)) ==
+                   cudaErrorMemoryAllocation &&
+               rows > kTriTile) {
+            cudaGetLastError();
+            rows = (rows / 2 + kTriTile - 1) / kTriTile * kTriTile;
+        }
         if (e != cudaSuccess) return cuda_fail(e, "mppi_create: rollout workspace");
     }
+    if (c->fmt < 0) c->v_q = (int)rows;
     return GPMPPI_OK;
 }
 

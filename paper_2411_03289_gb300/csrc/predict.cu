@@ -101,8 +101,12 @@ __global__ void __launch_bounds__(4 * kTriTile) k_pred_var(const PredArgs p) {
 
 }  // namespace
 
+// A GP handle more or less on the device.  The first makes the pool, which a call
+// under stream capture may not.
 void scratch_user(int device, int change) {
     if (device < 0 || device >= kMaxDevices) return;
+    cudaMemPool_t pool = nullptr;
+    if (change > 0) scratch_pool(device, &pool);     // a failure is reported by the call that needs it
     std::lock_guard<std::mutex> lock(g_pool_mu);
     g_pool_users[device] += change;
     if (g_pool_users[device] == 0 && g_pool[device]) cudaMemPoolTrimTo(g_pool[device], 0);
@@ -111,7 +115,7 @@ void scratch_user(int device, int change) {
 int launch_gp_predict(const GpDevice& g, const float* Z, int M, float* mean, float* var, cudaStream_t st) {
     if (M == 0) return GPMPPI_OK;
     // V in stream-ordered scratch (calls from several threads or streams share
-    // nothing), at most 1 GB: more queries go in pieces
+    // nothing), at most 1 GB: more queries go in pieces, smaller ones on a full device
     size_t piece = g.npad ? ((size_t)1 << 28) / g.npad / kTriTile * kTriTile : (size_t)M;
     if (piece > (size_t)M) piece = (size_t)M;
     float* V = nullptr;
@@ -120,7 +124,15 @@ int launch_gp_predict(const GpDevice& g, const float* Z, int M, float* mean, flo
         if (g.device < 0 || g.device >= kMaxDevices) return fail(GPMPPI_ERR_UNSUPPORTED, "gp_predict: device number");
         const int rc0 = scratch_pool(g.device, &pool);
         if (rc0) return rc0;
-        GPM_CUDA(cudaMallocFromPoolAsync((void**)&V, sizeof(float) * ((piece + kTriTile - 1) / kTriTile * kTriTile) * g.npad, pool, st));
+        cudaError_t e;
+        while ((e = cudaMallocFromPoolAsync(
+                    (void**)&V, sizeof(float) * ((piece + kTriTile - 1) / kTriTile * kTriTile) * g.npad, pool, st)) ==
+                   cudaErrorMemoryAllocation &&
+               piece > kTriTile) {
+            cudaGetLastError();
+            piece = (piece / 2 + kTriTile - 1) / kTriTile * kTriTile;
+        }
+        if (e != cudaSuccess) return cuda_fail(e, "gp_predict: scratch");
     }
     int rc = GPMPPI_OK;
     for (int o = 0; o < (g.shared ? 1 : 2) && rc == GPMPPI_OK; ++o)

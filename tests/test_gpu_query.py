@@ -104,3 +104,38 @@ def test_gradient_ragged_samples(lib):
         got, ref = got.cpu().numpy().ravel().astype(np.float64), np.asarray(ref).ravel()
         floor = 1e-3 * np.max(np.abs(ref))
         assert np.max(np.abs(got - ref) / np.maximum(np.abs(ref), floor)) <= 1e-3
+
+
+@pytest.mark.parametrize("precision", [0, 2])
+def test_prediction_and_step_under_capture(lib, precision):
+    """gp_predict, as the first call on a fitted GP, and mppi_step may be captured
+    into a CUDA graph: the replay gives what the direct calls give, bit for bit."""
+    import torch
+    sc = S.scenario("small", K=70, T=5, N=130, precision=precision)
+    g, ctrl = make_ctrl(lib, sc)
+    x0 = sc.x0.astype(np.float32)
+    Z = torch.rand(150, 4, device="cuda")
+    U = torch.tensor(sc.U0.astype(np.float32), device="cuda")
+    bufs = [torch.zeros(n, device="cuda") for n in (300, 300, U.numel(), 70, 70)]
+    mean, var, Un, w, costs = (b.view(-1, 2) if i < 3 else b for i, b in enumerate(bufs))
+
+    def calls(stream):
+        lib.gp_predict(g, Z, mean, var, stream=stream)
+        lib.mppi_set_iteration(ctrl, 4)
+        lib.mppi_step(ctrl, x0, U, Un, w, costs, stream=stream)
+
+    s = torch.cuda.Stream()
+    graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=s):
+        calls(s)
+    for _ in range(2):
+        graph.replay()
+    torch.cuda.synchronize()
+    replayed = [b.cpu().numpy().copy() for b in bufs]
+    for b in bufs:
+        b.zero_()
+    calls(None)
+    torch.cuda.synchronize()
+    for a, b in zip(replayed, bufs):
+        assert a.any() and np.array_equal(a, b.cpu().numpy())
