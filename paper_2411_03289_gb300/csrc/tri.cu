@@ -7,9 +7,9 @@
 // and the chunk's points (forward) or its rows of v (backward) arrive by bulk
 // copies in a ring.  A thread multiplies an 8-query x 8-column tile in registers
 // with packed FMAs (query pairs): 4 shared-memory reads for 32 of them, where 2
-// columns x 16 queries needed 12 and the reads, not the FMAs, bounded it.  Warp w
-// owns columns 16 w .. 16 w + 15 and leaves out the diagonal's rows that hold none
-// of them.  Items are very uneven (one to N / 32 chunks) and go longest first, two
+// columns x 16 queries needed 12 and the reads, not the FMAs, bounded it.  A warp
+// owns 16 columns, leaves out the diagonal's rows that hold none of them, and does
+// nothing past N.  Items are very uneven (one to N / 32 chunks) and go longest first, two
 // CTAs an SM.  v is kept by tiles of 128 queries, query the fastest index, so that
 // it leaves in whole lines, comes back as operands by bulk copies and is summed
 // with a thread per query.
@@ -17,8 +17,13 @@
 // not depend on the split.  The GP variance is what remains of sf2 after nearly
 // all of it cancels: its last digits are the rounding of these chains and of the
 // sums of squares, whose orders (SumOrder) are part of the results.
-// Bound: the FP32 FMA pipe (N (N + 1) / 2 FMAs a query); v is written once
-// (4 N bytes a query) and read back once by the sums.
+// Bound: the FP32 FMA pipe (N (N + 1) / 2 FMAs a query; three quarters active), the rest
+// the barriers around a chunk; v is written once (4 N bytes a query) and read back once
+// by the sums.  204,800 queries, forward: N = 500 0.98 ms (52 TFLOP/s; 1.32 with 2
+// columns x 16 queries; 2.5 inside the rollout that carried a sample tile through the
+// horizon), N = 1000 3.74 ms; backward, N = 1000: 3.57 ms (57 TFLOP/s).  81,920 queries
+// of N = 400: 0.29 ms (0.41 with the columns past N multiplied).  Barriers in shared
+// memory that let warps drift a chunk apart: 8 % slower.
 #include "query.cuh"
 
 namespace gpm {
@@ -130,7 +135,12 @@ __global__ void __launch_bounds__(PT, 2) k_tri(const TriJob p) {
         }
     };
 
-    const int lq = lane & 15, c0 = 16 * warp + 8 * (lane >> 4);
+    // The warp's columns: 16 w for warps 0-3 and from the other end for 4-7, so that
+    // the two warps of every scheduler share the diagonal's work evenly; none past N.
+    const int w0 = 16 * (warp < 4 ? warp : 11 - warp);
+    // first row (backward) or last row (forward) of the block's first 128 that it needs
+    const int edge = CB * cb + w0 >= (BACK ? p.ldo : p.N) ? (BACK ? 1 << 20 : -(1 << 20)) : BACK ? w0 : w0 + 16;
+    const int lq = lane & 15, c0 = w0 + 8 * (lane >> 4);
     uint64_t acc[4][8];
 #pragma unroll
     for (int i = 0; i < 4; ++i)
@@ -141,17 +151,20 @@ __global__ void __launch_bounds__(PT, 2) k_tri(const TriJob p) {
         __syncthreads();
     }
     for (int r = 0; r < nr; ++r) {
+        // kernel values of the next chunk: one of a scheduler's two warps before its
+        // products, the other after, so that they overlap
         if (BACK) arrived(r);
-        else if (r + 1 < nr) make(r + 1);
+        else if (warp < 4 && r + 1 < nr) make(r + 1);
         const unsigned char* stage = psm + (r % NST) * L::stage;
         const float* A = BACK ? reinterpret_cast<const float*>(stage + PIECE) : As + (r & 1) * (CH * PQ);
         const float* B = reinterpret_cast<const float*>(stage) + c0;
         // rows of the diagonal block that hold none of this warp's columns: forward
         // those past its last column, backward those before its first
         const int d = BACK ? CH * r : CH * (r - (CB / CH) * cb);
-        const int k0 = BACK ? min(CH, max(0, 16 * warp - d)) : 0;
-        const int k1 = BACK ? CH : min(CH, 16 * warp + 16 - d);
-#pragma unroll 4
+        const int k0 = BACK ? min(CH, max(0, edge - d)) : 0;
+        const int k1 = BACK ? CH : min(CH, edge - d);
+        // 16 points of loads and FMAs in flight (4 points: 1.05 against 0.98 ms at N = 500)
+#pragma unroll 16
         for (int k = k0; k < k1; ++k) {
             uint64_t av[4];
             const ulonglong2 a0 = *reinterpret_cast<const ulonglong2*>(A + k * PQ + 4 * lq);
@@ -167,6 +180,7 @@ __global__ void __launch_bounds__(PT, 2) k_tri(const TriJob p) {
                 for (int i = 0; i < 4; ++i) acc[i][c] = tc::f2fma(av[i], bb, acc[i][c]);
             }
         }
+        if (!BACK && warp >= 4 && r + 1 < nr) make(r + 1);
         __syncthreads();
         if (tid == 0 && on && r + NST < nr) {
             tc::fence_proxy_async();                 // the CTA's reads of this stage precede the refill
