@@ -284,7 +284,7 @@ int gpm::launch_query_rollout(gpmppi_ctrl c, const RolloutArgs& a, const GpSet& 
                 }
         } else {
             if ((rc = launch_chain(a, gs, ws, st))) return rc;
-            const VarTcJob j = {ws.zq, Q, ws.q, ws.nsplit, a.err};
+            const VarTcJob j = {ws.zq, Q, ws.q, ws.nsplit, ws.nparts, ws.rps, ws.even, a.err};
             if ((rc = launch_var_tc(gs, j, c->fmt, c->nsm, true, st))) return rc;
         }
         if ((rc = launch_stage_cost(a, gs, ws, c->ens && c->fmt < 0, st))) return rc;
@@ -301,6 +301,11 @@ QueryWs gpm::make_query_ws(gpmppi_ctrl c, int s0, int Ks) {
     ws.s0 = s0;
     ws.Ks = Ks;
     ws.nsplit = c->nsplit;
+    ws.nparts = c->nparts;
+    // The sums of the batched rollout wherever both kernels give the small products
+    // their own column set, so that their products agree to the bit.
+    ws.rps = c->fmt >= 0 && c->mm.lo_set ? c->rps : 0;
+    ws.even = c->ens ? 1 : 0;
     return ws;
 }
 
@@ -313,12 +318,22 @@ int alloc_query_ws(gpmppi_ctrl c) {
     const size_t T = (size_t)c->p.T, M = (size_t)c->gset.M;
     size_t n = ((size_t)1 << 23) / T;
     if (n > (size_t)c->p.K) n = (size_t)c->p.K;
-    c->nsplit = c->fmt < 0 ? 1 : var_tc_splits(c->gset, (int)(n * T), c->nsm);
+    if (n < (size_t)c->p.K && n > 32) n = n / 32 * 32;     // (every piece starts a warp of the chain)
+    c->nsplit = c->nparts = c->fmt < 0 ? 1 : var_tc_splits(c->gset, (int)(n * T), c->nsm);
+    if (c->fmt >= 0 && c->mm.lo_set && c->nsplit > 1) {
+        // a split's sums are put in the batched rollout's order afterwards, from a part
+        // for every 32 columns; not worth the room beyond 64 MB, where splits gain
+        // little (they fill the last wave)
+        int N = 0;
+        for (size_t t = 0; t < M; ++t) N = N < c->gset.gp[t].N ? c->gset.gp[t].N : N;
+        c->nparts = 8 * ((N + 255) / 256);
+        if ((size_t)c->nparts * M * n * T > ((size_t)1 << 24)) c->nsplit = c->nparts = 1;
+    }
     cudaFree(c->ws_buf);
     c->ws_buf = nullptr;
     cudaError_t e;
     // on a full device smaller pieces of the samples (the results are the same)
-    while ((e = cudaMalloc(&c->ws_buf, n * (16 * (2 * T + 1) + 4 * M * c->nsplit * T))) == cudaErrorMemoryAllocation &&
+    while ((e = cudaMalloc(&c->ws_buf, n * (16 * (2 * T + 1) + 4 * M * c->nparts * T))) == cudaErrorMemoryAllocation &&
            n > 64) {
         cudaGetLastError();
         n = (n / 2 + 31) / 32 * 32;
@@ -396,7 +411,8 @@ int launch_nominal(gpmppi_ctrl c, const RolloutArgs& a, cudaStream_t st) {
     ws.q = reinterpret_cast<float*>(ws.st + a.T);
     ws.s0 = 0;
     ws.Ks = 1;
-    ws.nsplit = 1;
+    ws.nsplit = ws.nparts = 1;
+    ws.rps = ws.even = 0;
     int rc;
     if ((rc = launch_nominal_mean(a, ws, st))) return rc;
     if ((rc = launch_nominal_var(c->gp->g, a.T, ws, reinterpret_cast<double*>(c->vbuf), st))) return rc;
@@ -847,10 +863,6 @@ int mppi_create_ensemble(const gpmppi_params* p, const float* obstacles, int32_t
         c->gset.gp[i].w = weights[i];
     }
     c->gset.M = M;
-    if (M > 1 && (rc = alloc_query_ws(c))) {   // room for every terrain's variance
-        mppi_destroy(c);
-        return rc;
-    }
     if (ens) {
         c->kind = c->fmt < 0 ? GPMPPI_KERNEL_ENSEMBLE : GPMPPI_KERNEL_TC_STREAM;
         if (c->fmt >= 0) {
@@ -861,12 +873,18 @@ int mppi_create_ensemble(const gpmppi_params* p, const float* obstacles, int32_t
                 lo = lo || gps[i]->g.N > kLoSetMinN;
             }
             c->mm.lo_set = lo ? 1 : 0;
-            GPM_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device));
-            if (!mma_layout_of(points, M, c->S, O, optin, &c->mm)) {
+            const cudaError_t e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device);
+            if (e != cudaSuccess || !mma_layout_of(points, M, c->S, O, optin, &c->mm)) {
                 mppi_destroy(c);
+                if (e != cudaSuccess) return cuda_fail(e, "mppi_create_ensemble");
                 return fail(GPMPPI_ERR_UNSUPPORTED, "mppi_create_ensemble: the GPs' training sets do not fit shared memory");
             }
         }
+    }
+    // room for every terrain's variance, in the parts of the ensemble's sums
+    if (ens && (rc = alloc_query_ws(c))) {
+        mppi_destroy(c);
+        return rc;
     }
     *out = c;
     return GPMPPI_OK;
@@ -977,7 +995,7 @@ int mppi_grad(gpmppi_ctrl c, const float state[5], const float* U_nom, const flo
     ga.ws.zq = reinterpret_cast<float4*>(base + o_zq);
     ga.ws.st = reinterpret_cast<float4*>(base + o_st);
     ga.ws.q = reinterpret_cast<float*>(base + o_qq);
-    ga.ws.nsplit = 1;
+    ga.ws.nsplit = ga.ws.nparts = 1;
     ga.rec = reinterpret_cast<float*>(base + o_rec);
     ga.S_out = reinterpret_cast<float*>(base + o_S);
     ga.dU_out = reinterpret_cast<float*>(base + o_dU);

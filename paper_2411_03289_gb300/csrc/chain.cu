@@ -67,16 +67,37 @@ __device__ __forceinline__ int sum_lane(int i) {
     return lane;
 }
 
+// A warp's partial sums (R > 0): 2 SG R chains, 16 or 32 stages at a time (a batch's
+// hand-over costs as much as the sums of some 20 stages), a word of padding between
+// chains; 1 to 4 KB.
+__host__ __device__ constexpr int batch_parts(int SG, int R) { return SG == 1 ? R : R / 2; }    // parts a lane
+__host__ __device__ constexpr int batch_stages(int SG, int R) { return R ? batch_parts(SG, R) * 32 / R : 0; }
+__host__ __device__ constexpr int part_bytes(int SG, int R) { return R ? (2 * SG * R * (batch_stages(SG, R) + 1) * 4 + 15) / 16 * 16 : 0; }
+
 // SMEM: the training sets of all GPs staged in shared memory (x in two arrays
 // of 16-byte halves, so that neighbouring lanes read neighbouring lines).
-template <int SG, bool SMEM>
+// R = 0: every lane sums its own pairs, the lanes' sums are added as a tree.
+// R > 0: the sums of the batched rollout's R threads a sample (rollout_mma.cu),
+// so that a controller's costs are the same bits there and here: R parts of 32 / R
+// points of every 32-point stage, each one chain of products, added with
+// compensation in the order of the stages; the R sums plainly.  A lane forms the
+// parts of its stages, and a lane a chain then adds them: a serial sum of N / 32
+// terms a step that the tree does not have.  K = 16384 T = 100 N = 2048 (R = 2):
+// 1.64 ms (1.64 as R = 0); K = 5000 T = 60 N = 1500 (R = 8): 397 us (313); K = 1500
+// T = 37 N = 777 (R = 8): 77 us (55).
+template <int SG, int R, bool SMEM>
 __global__ void __launch_bounds__(CT) k_chain(const RolloutArgs a, const GpSet gs, const QueryWs ws) {
     extern __shared__ __align__(16) unsigned char csm[];
     constexpr int SPC = CW * SG;               // samples per CTA
     constexpr int NV = 2 * SG;
+    constexpr int RR = R ? R : 1;
+    constexpr int PU = 16 / RR;                // pairs of a part
+    constexpr int SPB = batch_stages(SG, R);   // stages of a batch
+    constexpr int LD = SPB + 1, NCH = NV * RR; // chains and their spacing
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     float4* zs = reinterpret_cast<float4*>(csm) + warp * SG;            // the warp's queries
-    ulonglong2* xs = reinterpret_cast<ulonglong2*>(csm + CW * SG * 16);
+    float* ps = reinterpret_cast<float*>(csm + CW * SG * 16 + warp * part_bytes(SG, R));
+    ulonglong2* xs = reinterpret_cast<ulonglong2*>(csm + CW * (SG * 16 + part_bytes(SG, R)));
     const int l0 = blockIdx.x * SPC;
     const int j = lane % SG;                                            // the sample whose state this lane carries
     const int l = min(l0 + warp * SG + j, ws.Ks - 1);                   // spare ones repeat the last sample
@@ -100,9 +121,11 @@ __global__ void __launch_bounds__(CT) k_chain(const RolloutArgs a, const GpSet g
             const int np = gs.gp[t].npad / 2;           // pairs
             const ulonglong2* src = reinterpret_cast<const ulonglong2*>(gs.gp[t].xq);
             for (int i = tid; i < np; i += CT) {
-                dst[i] = __ldg(src + 2 * i);
-                dst[np + i] = __ldg(src + 2 * i + 1);
-                dst[2 * np + i] = __ldg(src + 2 * np + i);
+                // R > 0: the pairs of the lanes' parts next to each other
+                const int to = R ? (i % PU) * (np / PU) + i / PU : i;
+                dst[to] = __ldg(src + 2 * i);
+                dst[np + to] = __ldg(src + 2 * i + 1);
+                dst[2 * np + to] = __ldg(src + 2 * np + i);
             }
             dst += 3 * np;
         }
@@ -143,6 +166,89 @@ __global__ void __launch_bounds__(CT) k_chain(const RolloutArgs a, const GpSet g
                 zz[q][2] = tc::f2pack(z2, z2);
                 zz[q][3] = tc::f2pack(z3, z3);
             }
+            const float wsf = G.w * G.sf2;
+            if constexpr (R > 0) {
+                const int C = (G.N + 31) / 32, U = C * R;       // stages and parts
+                float cs_[(NCH + 31) / 32], cc_[(NCH + 31) / 32];
+#pragma unroll
+                for (int h = 0; h < (NCH + 31) / 32; ++h) {
+                    cs_[h] = 0.0f;
+                    cc_[h] = 0.0f;
+                }
+                for (int c0 = 0; c0 < C; c0 += SPB) {
+                    // IU parts of a lane interleaved; past the last one that part again
+                    constexpr int IU = SG < 4 && batch_parts(SG, R) > 1 ? 2 : 1;
+                    for (int b0 = 0; b0 < batch_parts(SG, R) && c0 * R + 32 * b0 < U; b0 += IU) {
+                        uint64_t pv[IU][SG], pw[IU][SG];
+                        int at[IU];
+#pragma unroll
+                        for (int b = 0; b < IU; ++b) {
+                            const int unit = min(c0 * R + 32 * (b0 + b) + lane, U - 1);
+                            at[b] = SMEM ? unit : unit * PU;
+#pragma unroll
+                            for (int q = 0; q < SG; ++q) {
+                                pv[b][q] = 0ull;
+                                pw[b][q] = 0ull;
+                            }
+                        }
+#pragma unroll
+                        for (int i = 0; i < PU; ++i) {
+#pragma unroll
+                            for (int b = 0; b < IU; ++b) {
+                                const int p = SMEM ? i * (np / PU) + at[b] : at[b] + i;
+                                const ulonglong2 xa = SMEM ? base[p] : __ldg(xg + 2 * p);
+                                const ulonglong2 xb = SMEM ? base[np + p] : __ldg(xg + 2 * p + 1);
+                                const ulonglong2 al = SMEM ? base[2 * np + p] : __ldg(xg + 2 * np + p);
+#pragma unroll
+                                for (int q = 0; q < SG; ++q) {
+                                    float k0, k1;
+                                    kernel_pair(zz[q], xa, xb, k0, k1);
+                                    const uint64_t kk = tc::f2pack(k0, k1);
+                                    pv[b][q] = tc::f2fma(kk, al.x, pv[b][q]);
+                                    pw[b][q] = tc::f2fma(kk, al.y, pw[b][q]);
+                                }
+                            }
+                        }
+#pragma unroll
+                        for (int b = 0; b < IU; ++b) {
+                            float* o = ps + (lane % R) * LD + (32 / RR) * (b0 + b) + lane / R;
+#pragma unroll
+                            for (int q = 0; q < SG; ++q) {
+                                float x, y;
+                                tc::f2unpack(pv[b][q], x, y);
+                                o[2 * q * R * LD] = x + y;
+                                tc::f2unpack(pw[b][q], x, y);
+                                o[(2 * q + 1) * R * LD] = x + y;
+                            }
+                        }
+                    }
+                    __syncwarp();
+                    const int nc = min(SPB, C - c0);
+#pragma unroll
+                    for (int h = 0; h < (NCH + 31) / 32; ++h)
+                        if (lane + 32 * h < NCH) {
+                            const float* o = ps + (lane + 32 * h) * LD;
+#pragma unroll 8
+                            for (int c = 0; c < nc; ++c) kahan_add(cs_[h], cc_[h], o[c]);
+                        }
+                    __syncwarp();
+                }
+#pragma unroll
+                for (int h = 0; h < (NCH + 31) / 32; ++h)
+                    if (lane + 32 * h < NCH) ps[lane + 32 * h] = cs_[h] + cc_[h];
+                __syncwarp();
+                float mv = ps[2 * j * R], mw = ps[(2 * j + 1) * R];
+#pragma unroll
+                for (int u = 1; u < R; ++u) {
+                    mv += ps[2 * j * R + u];
+                    mw += ps[(2 * j + 1) * R + u];
+                }
+                mean_v += wsf * mv;
+                mean_w += wsf * mw;
+                __syncwarp();                      // read before the next GP's parts
+                base += 3 * np;
+                continue;
+            }
             float v[NV], c[NV];
 #pragma unroll
             for (int i = 0; i < NV; ++i) {
@@ -181,14 +287,14 @@ __global__ void __launch_bounds__(CT) k_chain(const RolloutArgs a, const GpSet g
                 }
             }
             scatter_sum<NV>(v, c);
-            const float wsf = G.w * G.sf2;
             mean_v += wsf * __shfl_sync(0xffffffffu, v[0], sum_lane<NV>(2 * j));
             mean_w += wsf * __shfl_sync(0xffffffffu, v[0], sum_lane<NV>(2 * j + 1));
             base += 3 * np;
         }
         float sn, cs;
         sincosf(mu2, &sn, &cs);
-        const float nX = mu0 + a.dt * mu3 * cs;
+        // R > 0: the two roundings of the batched rollout
+        const float nX = R ? __fadd_rn(mu0, __fmul_rn(__fmul_rn(a.dt, mu3), cs)) : mu0 + a.dt * mu3 * cs;
         const float nY = mu1 + a.dt * mu3 * sn;
         const float nT = mu2 + a.dt * mu4;
         const float nV = mu3 + a.kv * (ut.x - mu3) + mean_v;
@@ -215,22 +321,30 @@ int launch_chain(const RolloutArgs& a, const GpSet& gs, const QueryWs& ws, cudaS
     // 20; K = 1000 T = 40 N = 300: 34 / 36 / 40 / 54; K = 4096 T = 50 N = 500:
     // 114 / 98 / 87 / 87; K = 16384 T = 100 N = 2048: 2379 / 1683 / 1414 / 1509.
     int sg = 1;
-    while (sg < 4 && ws.Ks / (2 * sg) >= 900) sg *= 2;
-#define GPM_CHAIN(L)                                                                                            \
+    while (sg < 4 && a.K / (2 * sg) >= 900) sg *= 2;     // (a.K: the same in every piece of the samples)
+#define GPM_CHAIN(L, R)                                                                                         \
     do {                                                                                                        \
         const dim3 grid((unsigned)((ws.Ks + CW * L - 1) / (CW * L)));                                           \
-        const size_t smem = CW * L * 16 + (sm ? points * 24 : 0);                                               \
+        const size_t smem = CW * (L * 16 + part_bytes(L, R)) + (sm ? points * 24 : 0);                          \
         if (sm) {                                                                                               \
-            GPM_CUDA(cudaFuncSetAttribute(k_chain<L, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,        \
-                                          101 * 1024));                                                         \
-            k_chain<L, true><<<grid, CT, smem, st>>>(a, gs, ws);                                                \
+            GPM_CUDA(cudaFuncSetAttribute(k_chain<L, R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,     \
+                                          120 * 1024));                                                         \
+            k_chain<L, R, true><<<grid, CT, smem, st>>>(a, gs, ws);                                             \
         } else {                                                                                                \
-            k_chain<L, false><<<grid, CT, smem, st>>>(a, gs, ws);                                               \
+            k_chain<L, R, false><<<grid, CT, smem, st>>>(a, gs, ws);                                            \
         }                                                                                                       \
     } while (0)
-    if (sg == 1) GPM_CHAIN(1);
-    else if (sg == 2) GPM_CHAIN(2);
-    else GPM_CHAIN(4);
+#define GPM_CHAIN_R(R)                     \
+    do {                                   \
+        if (sg == 1) GPM_CHAIN(1, R);      \
+        else if (sg == 2) GPM_CHAIN(2, R); \
+        else GPM_CHAIN(4, R);              \
+    } while (0)
+    if (ws.rps == 0) GPM_CHAIN_R(0);
+    else if (ws.rps == 2) GPM_CHAIN_R(2);
+    else if (ws.rps == 4) GPM_CHAIN_R(4);
+    else GPM_CHAIN_R(8);
+#undef GPM_CHAIN_R
 #undef GPM_CHAIN
     GPM_CUDA(cudaGetLastError());
     return GPMPPI_OK;

@@ -321,9 +321,12 @@ struct GpSet {
 struct QueryWs {
     float4* zq;                 // (T + 1) x Ks: (v, omega, u~_v, u~_omega) before step k
     float4* st;                 // T x Ks: (X, Y, theta, v) after step k
-    float* q;                   // M x nsplit x T x Ks: parts of |L_t^-1 k*|^2 over the variance kernel's scale
+    float* q;                   // M x nparts x T x Ks: parts of |L_t^-1 k*|^2 over the variance kernel's scale
     int s0, Ks;
-    int nsplit;                 // parts a variance comes in (their sum in this order)
+    int nsplit;                 // CTA pairs that share a query's passes (variance_tc.cu)
+    int nparts;                 // parts a variance comes in: nsplit, or (rps > 0) 1 or a part for every 32 columns
+    int rps;                    // > 0: the sums of the batched rollout with rps threads a sample
+    int even;                   // with rps: the batched rollout pads every GP to pairs of 128-column blocks
 };
 
 // Adjoint (gradient of the smoothed cost) of the samples [s0, s0 + Ks); see adjoint.cu.
@@ -379,8 +382,9 @@ int launch_nominal_mean(const RolloutArgs& a, const QueryWs& ws, cudaStream_t st
 struct VarTcJob {
     const float4* z;            // Q queries
     int Q;
-    float* q;                   // M x nsplit x Q
+    float* q;                   // M x nparts x Q
     int nsplit;
+    int nparts, rps, even;      // as in QueryWs
     unsigned int* err;
 };
 constexpr int kMaxVarSplits = 8;

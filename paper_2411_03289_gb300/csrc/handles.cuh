@@ -45,7 +45,8 @@ struct gpmppi_ctrl_s {
     int ws_Ks = 0;
     float* vbuf = nullptr;        // FP32 and nominal rollouts: rows of v = L^-1 k* of up to v_q queries
     int v_q = 0;
-    int nsplit = 1;               // parts of a variance (tensor cores: var_tc_splits)
+    int nsplit = 1;               // pairs of CTAs a query's variance is split over (var_tc_splits)
+    int nparts = 1;               // parts a variance comes in (QueryWs)
     int nsm = 0;                  // SMs of the device
     unsigned int* err = nullptr;  // device status word written by the rollout
     int fmt = -1;                 // 0 = FP16, 1 = BF16, 2 = three-part BF16 split, -1 = FP32

@@ -89,8 +89,11 @@ __host__ __device__ inline int stage_lo(int p, int c, int kc) {
 // the last pass is narrower, and nothing follows it)
 __host__ __device__ inline size_t pass_base(int p) { return (size_t)32768 * p * (p - 1) + (size_t)40960 * p; }
 
-// The passes a split of a GP takes: dealt back and forth, largest first.
+// The passes a split of a GP takes: dealt back and forth, largest first; without a
+// split and with the batched rollout's sums (BSUM) in their order.
+template <bool BSUM>
 __host__ __device__ inline int split_pass(int np, int nsplit, int split, int i) {
+    if (BSUM && nsplit == 1) return i < np ? i : -1;
     return np - 1 - (i * nsplit + ((i & 1) ? nsplit - 1 - split : split));
 }
 
@@ -231,8 +234,15 @@ __device__ __forceinline__ void step_split3(uint32_t d, uint64_t ah, uint64_t am
         : "memory");
 }
 
-// FMT: 0 = FP16 hi/lo, 1 = BF16 hi/lo, 2 = BF16 hi/mid/lo
-template <int FMT>
+// FMT: 0 = FP16 hi/lo, 1 = BF16 hi/lo, 2 = BF16 hi/mid/lo.  BSUM: the squares in the
+// order of the batched rollout (rollout_mma.cu), where the two halves of a pass's
+// columns are summed apart, 32 columns at a time in four chains, pass after pass.
+// The MMAs of a column are the same products in the same order there and here, so
+// that q is the same bits (what is cut off here are products with zero).  With a
+// split the 32-column sums go out, and the stage costs add them.  11.3 ms at
+// K = 16384, T = 100, N = 2048, FP16, as in the other order (4 % more with chains
+// packed across registers that are not loaded as pairs).
+template <int FMT, bool BSUM>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT, 1) k_var_tc(const GpSet gs, const VarTcJob job) {
     extern __shared__ __align__(1024) unsigned char tsm[];
     constexpr int PARTS = FMT == 2 ? 3 : 2;
@@ -325,7 +335,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT, 1) k_var_tc(cons
                 // the next tile's queries, in flight meanwhile
                 if (item + npairs < nitems) zn[r] = query(item + npairs, m0 + 32 * r);
             }
-            for (int i = 0, p; ok && (p = split_pass(np, job.nsplit, split, i)) >= 0; ++i) {
+            for (int i = 0, p; ok && (p = split_pass<BSUM>(np, job.nsplit, split, i)) >= 0; ++i) {
                 const int ns = pass_stages(G.N, p, KC);
                 for (int c = 0; c < ns; ++c) {
                     if ((n & 1u) != turn) {
@@ -387,14 +397,51 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT, 1) k_var_tc(cons
             const int ts = item / ntiles, tile = item % ntiles;
             const GpSet::One& G = gs.gp[ts / job.nsplit];
             const int split = ts % job.nsplit, np = pass_count(G.N);
-            float sum = 0.0f;
-            for (int i = 0, p; ok && (p = split_pass(np, job.nsplit, split, i)) >= 0; ++i) {
+            const int q = tile * (2 * QM) + (int)rank * QM + 32 * e + lane;
+            float sum = 0.0f, half2 = 0.0f;
+            for (int i = 0, p; ok && (p = split_pass<BSUM>(np, job.nsplit, split, i)) >= 0; ++i) {
                 const int nq = pass_hi(G.N, p) / QUART;
                 for (int j = 0; j < nq; ++j) {
                     ok = __all_sync(0xffffffffu, wait(q_done + j, (qph >> j) & 1u));
                     if (!ok) break;
                     qph ^= 1u << j;
                     tc::fence_after_sync();
+                    if constexpr (BSUM) {
+                        const bool second = j >= (job.even ? 2 : (nq + 1) / 2);
+#pragma unroll
+                        for (int cc = 0; cc < QUART; cc += 32) {
+                            float g[4];
+#pragma unroll
+                            for (int h = 0; h < 2; ++h) {
+                                float v[16], w[16];
+                                const uint32_t col = row + (uint32_t)(QUART * j + cc + 16 * h);
+                                tc::tmem_ld16x2(col, col + LO_COL, v, w);
+                                // pairs of neighbouring columns (a register pair as loaded)
+                                // are added, each chain's squares one by one
+                                float x[16], s0 = 0.0f, s1 = 0.0f;
+#pragma unroll
+                                for (int k = 0; k < 16; k += 2)
+                                    tc::f2unpack(tc::f2add(tc::f2pack(v[k], v[k + 1]), tc::f2pack(w[k], w[k + 1])), x[k], x[k + 1]);
+#pragma unroll
+                                for (int k = 0; k < 8; ++k) {
+                                    s0 = fmaf(x[k], x[k], s0);
+                                    s1 = fmaf(x[8 + k], x[8 + k], s1);
+                                }
+                                g[2 * h] = s0;
+                                g[2 * h + 1] = s1;
+                            }
+                            const float s32 = (g[0] + g[1]) + (g[2] + g[3]);
+                            if (job.nparts > 1) {
+                                if (q < job.Q)
+                                    job.q[((size_t)(ts / job.nsplit) * job.nparts + 8 * p + 2 * j + cc / 32) * job.Q + q] = s32;
+                            } else if (second) {
+                                half2 += s32;
+                            } else {
+                                sum += s32;
+                            }
+                        }
+                        continue;
+                    }
 #pragma unroll
                     for (int cc = 0; cc < QUART; cc += 16) {
                         float v[16], w[16];
@@ -419,8 +466,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT, 1) k_var_tc(cons
                 __syncwarp();
                 if (lane == 0) arrive_cluster(t_free0);
             }
-            const int q = tile * (2 * QM) + (int)rank * QM + 32 * e + lane;
-            if (ok && q < job.Q) job.q[(size_t)ts * job.Q + q] = sum;
+            if (BSUM && job.nparts > 1) continue;
+            if (ok && q < job.Q) job.q[(size_t)ts * job.Q + q] = BSUM ? sum + half2 : sum;
         }
     } else if (warp == MMA_WARP && rank == 0) {
         // ---------------- MMA issuer -----------------------------------------------
@@ -432,7 +479,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT, 1) k_var_tc(cons
             const int ts = item / ntiles;
             const int N = gs.gp[ts / job.nsplit].N;
             const int split = ts % job.nsplit, np = pass_count(N);
-            for (int i = 0, p; ok && (p = split_pass(np, job.nsplit, split, i)) >= 0; ++i, ++passes) {
+            for (int i = 0, p; ok && (p = split_pass<BSUM>(np, job.nsplit, split, i)) >= 0; ++i, ++passes) {
                 const int ns = pass_stages(N, p, KC), hi = pass_hi(N, p);
                 if (passes > 0) {
                     // both CTAs have read the last pass
@@ -486,7 +533,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT, 1) k_var_tc(cons
                 const int ts = item / ntiles;
                 const int N = gs.gp[ts / job.nsplit].N;
                 const int split = ts % job.nsplit, np = pass_count(N);
-                for (int i = 0, p; ok && (p = split_pass(np, job.nsplit, split, i)) >= 0; ++i) {
+                for (int i = 0, p; ok && (p = split_pass<BSUM>(np, job.nsplit, split, i)) >= 0; ++i) {
                     const int ns = pass_stages(N, p, KC);
                     for (int c = 0; c < ns; ++c) {
                         if (!(ok = wait(b_full + sb, pb))) break;
@@ -504,7 +551,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT, 1) k_var_tc(cons
                 const int ts = item / ntiles;
                 const int N = gs.gp[ts / job.nsplit].N;
                 const int split = ts % job.nsplit, np = pass_count(N);
-                for (int i = 0, p; ok && (p = split_pass(np, job.nsplit, split, i)) >= 0; ++i) {
+                for (int i = 0, p; ok && (p = split_pass<BSUM>(np, job.nsplit, split, i)) >= 0; ++i) {
                     const int ns = pass_stages(N, p, KC);
                     for (int c = 0; c < ns; ++c) {
                         if (!(ok = wait(a_raw + sa, pa))) break;
@@ -528,7 +575,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT, 1) k_var_tc(cons
             while (xi < nitems && xns == 0) {
                 const int ts = xi / ntiles;
                 const GpSet::One& G = gs.gp[ts / job.nsplit];
-                const int p = split_pass(pass_count(G.N), job.nsplit, ts % job.nsplit, xpi);
+                const int p = split_pass<BSUM>(pass_count(G.N), job.nsplit, ts % job.nsplit, xpi);
                 if (p >= 0) {
                     xns = pass_stages(G.N, p, KC);
                     xsrc = G.xq;
@@ -553,7 +600,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT, 1) k_var_tc(cons
             const int ts = item / ntiles;
             const GpSet::One& G = gs.gp[ts / job.nsplit];
             const int split = ts % job.nsplit, np = pass_count(G.N);
-            for (int i = 0, p; ok && (p = split_pass(np, job.nsplit, split, i)) >= 0; ++i) {
+            for (int i = 0, p; ok && (p = split_pass<BSUM>(np, job.nsplit, split, i)) >= 0; ++i) {
                 const int ns = pass_stages(G.N, p, KC), hi = pass_hi(G.N, p);
                 const unsigned char* src = reinterpret_cast<const unsigned char*>(G.Bt) + pass_base(p) * (2 * PARTS);
                 for (int c = 0; c < ns; ++c) {
@@ -651,7 +698,7 @@ int var_tc_splits(const GpSet& gs, int Q, int nsm) {
             const int np = pass_count(gs.gp[t].N);
             for (int j = 0; j < s; ++j) {
                 int w = 0;
-                for (int i = 0, p; (p = split_pass(np, s, j, i)) >= 0; ++i) w += 8 * p + 6;
+                for (int i = 0, p; (p = split_pass<false>(np, s, j, i)) >= 0; ++i) w += 8 * p + 6;
                 longest = w > longest ? w : longest;
             }
         }
@@ -668,7 +715,9 @@ int launch_var_tc(const GpSet& gs, const VarTcJob& j, int fmt, int nsm, bool dep
     if (j.Q <= 0) return GPMPPI_OK;
     const long long items = (long long)((j.Q + 2 * QM - 1) / (2 * QM)) * gs.M * j.nsplit;
     const int pairs = (int)(items < nsm / 2 ? items : nsm / 2);
-    auto kern = fmt == 0 ? k_var_tc<0> : (fmt == 1 ? k_var_tc<1> : k_var_tc<2>);
+    auto kern = fmt == 2   ? k_var_tc<2, true>
+                : j.rps > 0 ? (fmt == 0 ? k_var_tc<0, true> : k_var_tc<1, true>)
+                            : (fmt == 0 ? k_var_tc<0, false> : k_var_tc<1, false>);
     const int smem = fmt == 2 ? TcLayout<3>::total : TcLayout<2>::total;
     GPM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     GPM_CUDA(launch_ex(kern, dim3((unsigned)(2 * pairs)), NT, smem, st, dependent, 1u, gs, j));
