@@ -274,11 +274,11 @@ int terrain_weights(const double* Yv, const double* Yw, const double* Fv, const 
  * logistic sigmoids of slope * (e - r_bar) and -slope * min_j d_bar_j, and the
  * control noise fixed at the draws of the controller's current iteration
  * (the counter is not advanced).  The gradient is exact for that smoothed
- * cost up to FP32 rounding, taken by a reverse pass over the horizon that
- * stores the state every ceil(sqrt(T)) steps and recomputes each segment;
- * derivatives of sqrt(lambda_max) and sqrt(n^T Sigma n) are taken as zero
- * where their argument is zero (Sigma_XY(1) = 0), and those of the clamps
- * (Eq. 8, the variance at zero) as zero outside the box.
+ * cost up to FP32 rounding, taken by a reverse pass over the horizon from the
+ * recorded states, v = L^-1 k* and K^-1 k* of every step; derivatives of
+ * sqrt(lambda_max) and sqrt(n^T Sigma n) are taken as zero where their argument
+ * is zero (Sigma_XY(1) = 0), and those of the clamps (Eq. 8, the variance at
+ * zero) as zero outside the box.
  *   state          host, 5 floats (x0)
  *   U_nom          device, T x 2 floats
  *   sample_weights device, K floats w_s, or NULL for w_s = 1/K
@@ -287,14 +287,16 @@ int terrain_weights(const double* Yv, const double* Yw, const double* Fv, const 
  *   dU             device, T x 2 floats dJ/dU (output), or NULL to evaluate J only
  *   dlengthscale   device, 2 x 4 floats dJ/dl_{o,d} for output o (v, omega) and
  *                  GP input d (output), or NULL.  It includes the dependence of
- *                  alpha = K^-1 y and K^-1 on the lengthscales (one more kernel
- *                  and T * K * N floats of scratch)
+ *                  alpha = K^-1 y and K^-1 on the lengthscales (one more kernel)
  * Needs variance mode GPMPPI_VAR_PER_SAMPLE (else GPMPPI_ERR_UNSUPPORTED) and
  * 64 N + 768 sqrt(T) bytes below the shared memory of a CTA
  * (GPMPPI_ERR_UNSUPPORTED beyond).
  * The first call, and the first call asking for dlengthscale, allocate
  * device scratch owned by the controller (freed by mppi_destroy) and may
- * synchronise.  Runs on the controller's FP32 path whatever its precision. */
+ * synchronise: 2 T K N floats for as many samples at a time as fit 2 GB, fewer
+ * on a full device (J and dU are the same bits, dlengthscale up to the order of
+ * its sums).  Runs on the
+ * controller's FP32 path whatever its precision. */
 int mppi_grad(gpmppi_ctrl c, const float state[5], const float* U_nom, const float* sample_weights,
               float slope, float* J, float* dU, float* dlengthscale, void* stream);
 

@@ -940,47 +940,62 @@ int mppi_grad(gpmppi_ctrl c, const float state[5], const float* U_nom, const flo
         if (N > 0 && (rc = launch_dk_alpha(g.Xs[0], g.alpha, N, Np, g.sf2[0], g.ubar, st))) return rc;
         GPM_CUDA(cudaStreamSynchronize(st));
     }
-    // samples at a time: rows of v and b of up to 8 GB
-    size_t piece = ((size_t)1 << 31) / ((size_t)T * (g.npad + Np + 64));
-    piece = piece < 8 ? 8 : piece / 8 * 8;
-    const int Ks = piece < (size_t)K ? (int)piece : K;
-    const int Kpad = (Ks + 7) / 8 * 8;
     const GpSet gs = single_gp_set(g, 0);
-    // scratch layout (bytes, each piece 256-aligned)
     int nsm = 0;
     GPM_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device));
-    size_t off = 0;
-    auto take = [&](size_t bytes) {
-        const size_t o = off;
-        off += (bytes + 255) & ~(size_t)255;
-        return o;
-    };
+    // Samples at a time: rows of v and b of up to 2 GB, fewer on a full device.  The
+    // count is kept with the scratch: every later call takes the same pieces.
+    size_t piece = ((size_t)1 << 29) / ((size_t)T * (g.npad + Np + 64));
+    piece = piece < 8 ? 8 : piece / 8 * 8;
+    int Ks = c->grad_Ks > 0 ? c->grad_Ks : (piece < (size_t)K ? (int)piece : K);
     auto kpad_of = [&](int s0) { return ((K - s0 < Ks ? K - s0 : Ks) + 7) / 8 * 8; };
+    // scratch layout (bytes, each piece 256-aligned)
+    size_t off = 0, o_ut = 0, o_zq = 0, o_st = 0, o_qq = 0, o_rec = 0, o_v = 0, o_S = 0, o_dU = 0, o_dl = 0, o_B = 0,
+           o_q = 0, o_p = 0;
     int nparts = 0;
-    if (want_l)
-        for (int s0 = 0; s0 < K; s0 += Ks) nparts += gram_tc_parts(T * kpad_of(s0), Np, nsm);
-    const size_t Q = (size_t)T * Ks;
-    const size_t o_ut = take(sizeof(float2) * (size_t)T * K);
-    const size_t o_zq = take(sizeof(float4) * (Q + Ks));
-    const size_t o_st = take(sizeof(float4) * Q);
-    const size_t o_qq = take(sizeof(float) * Q);
-    const size_t o_rec = take(sizeof(float) * 16 * Q);
-    const size_t o_v = take(sizeof(float) * ((Q + kTriTile - 1) / kTriTile * kTriTile) * g.npad);
-    const size_t o_S = take(sizeof(float) * (size_t)K);
-    const size_t o_dU = take(sizeof(float) * (size_t)2 * T * K);
-    const size_t o_dl = take(sizeof(float) * (size_t)8 * K);
-    size_t o_B = 0, o_q = 0, o_p = 0;
-    if (dU) o_B = take(sizeof(float) * (size_t)T * Kpad * Np);
-    if (want_l) {
-        o_q = take(sizeof(float4) * (size_t)T * Kpad);
-        o_p = take(sizeof(float) * 8 * (size_t)nparts);
-    }
+    auto layout = [&]() {
+        off = 0;
+        auto take = [&](size_t bytes) {
+            const size_t o = off;
+            off += (bytes + 255) & ~(size_t)255;
+            return o;
+        };
+        const size_t Q = (size_t)T * Ks, Qpad = (size_t)T * kpad_of(0);
+        o_ut = take(sizeof(float2) * (size_t)T * K);
+        o_zq = take(sizeof(float4) * (Q + Ks));
+        o_st = take(sizeof(float4) * Q);
+        o_qq = take(sizeof(float) * Q);
+        o_rec = take(sizeof(float) * 16 * Q);
+        o_v = take(sizeof(float) * ((Q + kTriTile - 1) / kTriTile * kTriTile) * g.npad);
+        o_S = take(sizeof(float) * (size_t)K);
+        o_dU = take(sizeof(float) * (size_t)2 * T * K);
+        o_dl = take(sizeof(float) * (size_t)8 * K);
+        if (dU) o_B = take(sizeof(float) * Qpad * Np);
+        nparts = 0;
+        if (want_l) {
+            for (int s0 = 0; s0 < K; s0 += Ks) nparts += gram_tc_parts(T * kpad_of(s0), Np, nsm);
+            o_q = take(sizeof(float4) * Qpad);
+            o_p = take(sizeof(float) * 8 * (size_t)nparts);
+        }
+    };
+    layout();
     if (off > c->grad_bytes) {
         cudaFree(c->grad_scr);
         c->grad_scr = nullptr;
         c->grad_bytes = 0;
-        GPM_CUDA(cudaMalloc(&c->grad_scr, off));
+        c->grad_Ks = 0;
+        cudaError_t e;
+        while ((e = cudaMalloc(&c->grad_scr, off)) == cudaErrorMemoryAllocation && Ks > 8) {
+            cudaGetLastError();
+            Ks = (Ks / 2 + 7) / 8 * 8;
+            layout();
+        }
+        if (e != cudaSuccess) {
+            c->grad_scr = nullptr;
+            return cuda_fail(e, "mppi_grad: scratch");
+        }
         c->grad_bytes = off;
+        c->grad_Ks = Ks;
     }
     char* base = static_cast<char*>(c->grad_scr);
     GradArgs ga;

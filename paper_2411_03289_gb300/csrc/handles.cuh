@@ -69,6 +69,7 @@ struct gpmppi_ctrl_s {
     // adjoint-rollout scratch (allocated by the first mppi_grad call)
     void* grad_scr = nullptr;
     size_t grad_bytes = 0;
+    int grad_Ks = 0;              // samples at a time that it was made for
     bool profiling = false;
     bool profiled = false;
     cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};

@@ -1,0 +1,56 @@
+"""Scratch that is made by a first call or shrinks on a full device: the results do
+not depend on it."""
+import numpy as np
+import pytest
+
+import scenarios as S
+from parity import make_ctrl
+
+pytestmark = pytest.mark.gpu
+
+
+class _Full:
+    """All but `left` bytes of the device held by one allocation."""
+
+    def __init__(self, left):
+        import torch
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        free, _ = torch.cuda.mem_get_info()
+        self.hold = torch.empty(max(0, free - left), dtype=torch.uint8, device="cuda")
+
+    def __enter__(self):
+        return self
+
+    def __exit__(self, *exc):
+        import torch
+        del self.hold
+        torch.cuda.empty_cache()
+
+
+def _grad(lib, ctrl, sc, want_dl=True):
+    import torch
+    U = torch.tensor(sc.U0, dtype=torch.float32, device="cuda")
+    out = lib.mppi_grad(ctrl, sc.x0, U, 20.0, None, want_dl=want_dl)
+    return [x.cpu().numpy() for x in out if x is not None]
+
+
+@pytest.mark.parametrize("K,T,N,left", [
+    (4001, 40, 500, 300 << 20),       # 0.7 GB of rows: one piece, and a few with a ragged last one
+    (6001, 60, 1000, 500 << 20)])     # 3 GB: two pieces, and more
+def test_gradient_on_a_full_device(lib, K, T, N, left):
+    """Fewer samples at a time: J and dU are per-sample terms added in the samples'
+    order, the same bits; the lengthscales' Gram sums are FP32 sums of thousands of
+    products in another grouping (1e-4 of the largest)."""
+    sc = S.scenario("small", K=K, T=T, N=N, precision=0)
+    _, ctrl = make_ctrl(lib, sc)
+    free = _grad(lib, ctrl, sc)
+    _, ctrl = make_ctrl(lib, sc)
+    with _Full(left):
+        full = _grad(lib, ctrl, sc)
+        again = _grad(lib, ctrl, sc)
+    assert all(np.all(np.isfinite(x)) for x in free)
+    assert np.array_equal(free[0], full[0]) and np.array_equal(free[1], full[1])
+    assert np.max(np.abs(free[2] - full[2])) <= 1e-4 * np.max(np.abs(free[2]))
+    assert all(np.array_equal(a, b) for a, b in zip(full, again))
+
