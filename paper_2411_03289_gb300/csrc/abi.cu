@@ -933,8 +933,9 @@ int mppi_grad(gpmppi_ctrl c, const float state[5], const float* U_nom, const flo
         return fail(GPMPPI_ERR_UNSUPPORTED, "mppi_grad: GP too large for the adjoint kernel's shared memory");
     cudaStream_t st = (cudaStream_t)stream;
     const bool want_l = dlengthscale != nullptr;
-    // per-GP factors of the adjoint, built once
-    if (dU && (rc = build_back_pieces(g, st))) return rc;
+    // per-GP factors of the adjoint, built once (with the first call of any kind, so
+    // that a later one may be captured)
+    if ((rc = build_back_pieces(g, st))) return rc;
     if (want_l && !g.ubar) {
         GPM_CUDA(cudaMalloc(&g.ubar, sizeof(float) * 8 * (size_t)(Np > 0 ? Np : 1)));
         if (N > 0 && (rc = launch_dk_alpha(g.Xs[0], g.alpha, N, Np, g.sf2[0], g.ubar, st))) return rc;
@@ -970,7 +971,7 @@ int mppi_grad(gpmppi_ctrl c, const float state[5], const float* U_nom, const flo
         o_S = take(sizeof(float) * (size_t)K);
         o_dU = take(sizeof(float) * (size_t)2 * T * K);
         o_dl = take(sizeof(float) * (size_t)8 * K);
-        if (dU) o_B = take(sizeof(float) * Qpad * Np);
+        o_B = take(sizeof(float) * Qpad * Np);
         nparts = 0;
         if (want_l) {
             for (int s0 = 0; s0 < K; s0 += Ks) nparts += gram_tc_parts(T * kpad_of(s0), Np, nsm);

@@ -1,5 +1,5 @@
 """Scratch that is made by a first call or shrinks on a full device: the results do
-not depend on it."""
+not depend on it, and what a first call prepared lets later ones be captured."""
 import numpy as np
 import pytest
 
@@ -54,3 +54,22 @@ def test_gradient_on_a_full_device(lib, K, T, N, left):
     assert np.max(np.abs(free[2] - full[2])) <= 1e-4 * np.max(np.abs(free[2]))
     assert all(np.array_equal(a, b) for a, b in zip(full, again))
 
+
+def test_gradient_after_a_cost_may_be_captured(lib):
+    """A first call for J alone makes what a call for dU needs."""
+    import torch
+    sc = S.scenario("small", K=70, T=5, N=130, precision=0)
+    _, ctrl = make_ctrl(lib, sc)
+    U = torch.tensor(sc.U0, dtype=torch.float32, device="cuda")
+    J, dU = torch.zeros(1, device="cuda"), torch.zeros(5, 2, device="cuda")
+    lib.mppi_grad(ctrl, sc.x0, U, 20.0, None, J, want_dU=False)
+    s = torch.cuda.Stream()
+    graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=s):
+        lib.mppi_grad(ctrl, sc.x0, U, 20.0, None, J, dU, want_dl=False, stream=s)
+    J.zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    ref = _grad(lib, ctrl, sc, want_dl=False)
+    assert np.array_equal(J.cpu().numpy(), ref[0]) and np.array_equal(dU.cpu().numpy(), ref[1]) and ref[1].any()
