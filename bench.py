@@ -284,11 +284,11 @@ def committed_traffic(kernel="tri", workload=WORKLOAD):
 def step_launches(P, sizes):
     """Kernels of one mppi_step over GPs of these sizes: the chain, the variances
     (split precisions: one kernel; FP32: a product and its row sums for each GP and
-    each 512 MB of rows), the stage costs and the update."""
+    each 256 MB of rows), the stage costs and the update."""
     if P.precision != 0:
         return 4
     npad = max((n + 127) // 128 * 128 for n in sizes)
-    rows = max(1, (1 << 27) // max(npad, 1) // 128 * 128)
+    rows = max(1, (1 << 26) // max(npad, 1) // 128 * 128)
     return 3 + 2 * len(sizes) * -(-P.K * P.T // rows)
 
 

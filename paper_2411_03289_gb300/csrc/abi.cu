@@ -311,6 +311,12 @@ QueryWs gpm::make_query_ws(gpmppi_ctrl c, int s0, int Ks) {
 
 namespace {
 
+// Bytes of rows of v that an FP32 controller holds at most.  Every controller of a
+// fleet holds its own, so it is kept to what costs little: steps of K = 4096 T = 50
+// N = 500 / K = 8000 T = 50 N = 1500 take 1237 / 16510 us with 512 MB, 1239 / 16850
+// with 256, 1287 / 17500 with 128 (the tails of the pieces' triangular products).
+constexpr size_t kVRows = (size_t)256 << 20;
+
 // The workspace of the query rollout: the records of ws_Ks samples, all of
 // them up to 2^23 queries (36 bytes each for a single GP), beyond which a
 // rollout goes through its samples in pieces.
@@ -340,12 +346,13 @@ int alloc_query_ws(gpmppi_ctrl c) {
     }
     if (e != cudaSuccess) return cuda_fail(e, "mppi_create: rollout workspace");
     c->ws_Ks = (int)n;
-    // rows of v: up to 512 MB at a time
+    // rows of v: up to kVRows bytes at a time, in pieces of one size
     size_t npad = 0, rows = 0;
     for (size_t t = 0; t < M; ++t) npad = npad < (size_t)c->gset.gp[t].npad ? (size_t)c->gset.gp[t].npad : npad;
     if (c->fmt < 0) {
-        rows = npad ? ((size_t)1 << 27) / npad / kTriTile * kTriTile : n * T;
-        if (rows > n * T) rows = (n * T + kTriTile - 1) / kTriTile * kTriTile;
+        const size_t most = npad ? kVRows / 4 / npad / kTriTile * kTriTile : n * T;
+        const size_t pieces = (n * T + most - 1) / most;
+        rows = ((n * T + pieces - 1) / pieces + kTriTile - 1) / kTriTile * kTriTile;
     }
     const size_t least = c->p.variance_mode == GPMPPI_VAR_NOMINAL ? 4 * T : 0;      // 2 T N doubles
     cudaFree(c->vbuf);

@@ -115,8 +115,9 @@ void scratch_user(int device, int change) {
 int launch_gp_predict(const GpDevice& g, const float* Z, int M, float* mean, float* var, cudaStream_t st) {
     if (M == 0) return GPMPPI_OK;
     // V in stream-ordered scratch (calls from several threads or streams share
-    // nothing), at most 1 GB: more queries go in pieces, smaller ones on a full device
-    size_t piece = g.npad ? ((size_t)1 << 28) / g.npad / kTriTile * kTriTile : (size_t)M;
+    // nothing), at most what the pool keeps: more queries go in pieces, smaller ones on
+    // a full device
+    size_t piece = g.npad ? kPoolKeep / 4 / g.npad / kTriTile * kTriTile : (size_t)M;
     if (piece > (size_t)M) piece = (size_t)M;
     float* V = nullptr;
     if (g.npad) {

@@ -73,3 +73,16 @@ def test_gradient_after_a_cost_may_be_captured(lib):
     torch.cuda.synchronize()
     ref = _grad(lib, ctrl, sc, want_dl=False)
     assert np.array_equal(J.cpu().numpy(), ref[0]) and np.array_equal(dU.cpu().numpy(), ref[1]) and ref[1].any()
+
+
+@pytest.mark.parametrize("K,T,N", [(4096, 50, 500), (16384, 100, 300)])
+def test_memory_of_an_fp32_controller(lib, K, T, N):
+    """256 MB of rows of v at most, whatever K and T, beside 36 bytes of records and
+    the 8 of the perturbed control for every query (and 2 MB granules)."""
+    import torch
+    sc = S.scenario("small", K=K, T=T, N=N, precision=0)
+    g, _ = make_ctrl(lib, S.scenario("small", K=33, T=2, N=N, precision=0))
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    _, ctrl = make_ctrl(lib, sc, g)
+    assert before - torch.cuda.mem_get_info()[0] <= (256 << 20) + 44 * K * T + (32 << 20)
