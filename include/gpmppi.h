@@ -133,7 +133,9 @@ int gp_factors(gpmppi_gp gp, int32_t j, double* Linv, double* alpha);
  *   Z     device, M x 4 floats
  *   mean  device, M x 2 floats (output)
  *   var   device, M x 2 floats (output)
- * FP32 arithmetic on the FP32 factors. */
+ * FP32 arithmetic on the FP32 factors.  Scratch of up to 256 MB in the stream's
+ * order, from a pool kept while a GP exists; none under stream capture, nor where
+ * the device has no room (slower, the same results). */
 int gp_predict(gpmppi_gp gp, const float* Z, int32_t M, float* mean, float* var, void* stream);
 
 /* Create a controller for one robot.  The radius tightening factors of the

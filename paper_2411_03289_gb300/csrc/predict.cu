@@ -1,5 +1,6 @@
 // The GP posterior at M queries (gp_predict), FP32: the triangular product of
-// tri.cu and its row sums, and the means with one CTA a query.
+// tri.cu and its row sums (or, without scratch, one CTA a query), and the means
+// with one CTA a query.
 #include <mutex>
 
 #include "query.cuh"
@@ -11,6 +12,7 @@ struct PredArgs {
     const float* Z;          // queries, M x 4
     const float* Xs;         // GpDevice::Xs, alpha
     const float* alpha;
+    const float* Wb;         // GpDevice::Wb
     const float* V;          // tiles of kTriTile queries, npad columns each
     float* mean;
     float* var;
@@ -99,14 +101,42 @@ __global__ void __launch_bounds__(4 * kTriTile) k_pred_var(const PredArgs p) {
     if (p.out != 0) p.var[2 * (size_t)q + 1] = s;
 }
 
+// The variances without scratch, one CTA a query: the same sums in the same order (v
+// one chain over the points, the squares as above), every query reading the whole
+// factor: 20000 queries at N = 1000 in 3.3 ms, 0.4 by way of V.  For calls under
+// stream capture, where scratch would be an allocation node, with which a graph may
+// neither be instantiated twice at a time nor be a child of another, and for a
+// device without room for 128 rows.
+__global__ void __launch_bounds__(ST) k_pred_direct(const PredArgs p) {
+    extern __shared__ float ks[];                    // N floats
+    __shared__ float red[ST / 32];
+    const float* z = p.Z + 4 * (size_t)blockIdx.x;
+    for (int j = threadIdx.x; j < p.N; j += ST) {
+        const float4 x = reinterpret_cast<const float4*>(p.Xs)[j];
+        const float e0 = fmaf(z[0], p.zscale[0], -x.x), e1 = fmaf(z[1], p.zscale[1], -x.y);
+        const float e2 = fmaf(z[2], p.zscale[2], -x.z), e3 = fmaf(z[3], p.zscale[3], -x.w);
+        ks[j] = p.sf2 * qr::ex2(-fmaf(e3, e3, fmaf(e2, e2, fmaf(e0, e0, e1 * e1))));
+    }
+    __syncthreads();
+    float qf = 0.0f;
+    for (int i = threadIdx.x; i < p.N; i += ST) {
+        const int cb = i / 128;
+        const float* w = p.Wb + (size_t)cb * (cb + 1) / 2 * (128 * 128) + i % 128;
+        float v = 0.0f;
+        for (int j = 0; j <= i; ++j) v = fmaf(ks[j], w[j * 128], v);
+        qf = fmaf(v, v, qf);
+    }
+    qf = block_sum(qf, red);
+    const float s = fmaxf(0.0f, p.sf2 - qf);
+    if (threadIdx.x == 0 && p.out != 1) p.var[2 * (size_t)blockIdx.x] = s;
+    if (threadIdx.x == 0 && p.out != 0) p.var[2 * (size_t)blockIdx.x + 1] = s;
+}
+
 }  // namespace
 
-// A GP handle more or less on the device.  The first makes the pool, which a call
-// under stream capture may not.
+// a GP handle more or less on the device
 void scratch_user(int device, int change) {
     if (device < 0 || device >= kMaxDevices) return;
-    cudaMemPool_t pool = nullptr;
-    if (change > 0) scratch_pool(device, &pool);     // a failure is reported by the call that needs it
     std::lock_guard<std::mutex> lock(g_pool_mu);
     g_pool_users[device] += change;
     if (g_pool_users[device] == 0 && g_pool[device]) cudaMemPoolTrimTo(g_pool[device], 0);
@@ -120,7 +150,9 @@ int launch_gp_predict(const GpDevice& g, const float* Z, int M, float* mean, flo
     size_t piece = g.npad ? kPoolKeep / 4 / g.npad / kTriTile * kTriTile : (size_t)M;
     if (piece > (size_t)M) piece = (size_t)M;
     float* V = nullptr;
-    if (g.npad) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    GPM_CUDA(cudaStreamIsCapturing(st, &cap));
+    if (g.npad && cap == cudaStreamCaptureStatusNone) {
         cudaMemPool_t pool = nullptr;
         if (g.device < 0 || g.device >= kMaxDevices) return fail(GPMPPI_ERR_UNSUPPORTED, "gp_predict: device number");
         const int rc0 = scratch_pool(g.device, &pool);
@@ -133,8 +165,13 @@ int launch_gp_predict(const GpDevice& g, const float* Z, int M, float* mean, flo
             cudaGetLastError();
             piece = (piece / 2 + kTriTile - 1) / kTriTile * kTriTile;
         }
-        if (e != cudaSuccess) return cuda_fail(e, "gp_predict: scratch");
+        if (e != cudaSuccess && e != cudaErrorMemoryAllocation) return cuda_fail(e, "gp_predict: scratch");
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            V = nullptr;
+        }
     }
+    if (!V) piece = (size_t)M;
     int rc = GPMPPI_OK;
     for (int o = 0; o < (g.shared ? 1 : 2) && rc == GPMPPI_OK; ++o)
         for (size_t q0 = 0; q0 < (size_t)M && rc == GPMPPI_OK; q0 += piece) {
@@ -142,6 +179,7 @@ int launch_gp_predict(const GpDevice& g, const float* Z, int M, float* mean, flo
             p.Z = Z + 4 * q0;
             p.Xs = g.Xs[o];
             p.alpha = g.alpha;
+            p.Wb = g.Wb[o];
             p.V = V;
             p.mean = mean + 2 * q0;
             p.var = var + 2 * q0;
@@ -151,11 +189,17 @@ int launch_gp_predict(const GpDevice& g, const float* Z, int M, float* mean, flo
             p.sf2 = g.sf2[o];
             for (int d = 0; d < 4; ++d) p.zscale[d] = g.zscale[o][d];
             p.out = g.shared ? -1 : o;
-            TriJob j = tri_forward(single_gp_set(g, o).gp[0], p.Z, p.M, V);
-            j.fusez = 1;
-            rc = launch_tri_forward(j, false, st);
-            if (rc) break;
-            cudaError_t e = launch_ex(k_pred_var, dim3((unsigned)((p.M + kTriTile - 1) / kTriTile)), 4 * kTriTile, 0, st, true, 1u, p);
+            cudaError_t e;
+            if (V) {
+                TriJob j = tri_forward(single_gp_set(g, o).gp[0], p.Z, p.M, V);
+                j.fusez = 1;
+                rc = launch_tri_forward(j, false, st);
+                if (rc) break;
+                e = launch_ex(k_pred_var, dim3((unsigned)((p.M + kTriTile - 1) / kTriTile)), 4 * kTriTile, 0, st, true, 1u, p);
+            } else {
+                k_pred_direct<<<p.M, ST, sizeof(float) * (g.N > 0 ? g.N : 1), st>>>(p);
+                e = cudaGetLastError();
+            }
             if (e == cudaSuccess) {
                 k_pred_mean<<<p.M, ST, 0, st>>>(p);
                 e = cudaGetLastError();

@@ -1,5 +1,7 @@
 """Scratch that is made by a first call or shrinks on a full device: the results do
 not depend on it, and what a first call prepared lets later ones be captured."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -17,7 +19,12 @@ class _Full:
         torch.cuda.synchronize()
         torch.cuda.empty_cache()
         free, _ = torch.cuda.mem_get_info()
-        self.hold = torch.empty(max(0, free - left), dtype=torch.uint8, device="cuda")
+        for more in range(0, 256 << 20, 2 << 20):
+            try:
+                self.hold = torch.empty(max(0, free - left - more), dtype=torch.uint8, device="cuda")
+                return
+            except torch.cuda.OutOfMemoryError:
+                pass
 
     def __enter__(self):
         return self
@@ -86,3 +93,66 @@ def test_memory_of_an_fp32_controller(lib, K, T, N):
     before = torch.cuda.mem_get_info()[0]
     _, ctrl = make_ctrl(lib, sc, g)
     assert before - torch.cuda.mem_get_info()[0] <= (256 << 20) + 44 * K * T + (32 << 20)
+
+
+@pytest.mark.parametrize("shared", [True, False])
+@pytest.mark.parametrize("N", [0, 1, 127, 130, 1025])
+def test_prediction_in_a_graph_instantiated_twice(lib, N, shared):
+    """A captured gp_predict is kernels alone, so that its graph may be instantiated
+    as often as one likes: both replays give the direct call's bits."""
+    import torch
+    cu = ctypes.CDLL("libcuda.so.1")
+    sc = S.scenario("small", K=33, T=2, N=N, precision=0)
+    h = sc.hyper[0]
+    other = h if shared else S.Hyper(tuple(1.3 * x for x in h.lengthscale), 0.7 * h.signal_var, h.noise_var)
+    g = lib.gp_fit(sc.X, sc.Y, (h, S.Hyper(tuple(other.lengthscale), other.signal_var, other.noise_var)))
+    Z = torch.rand(300, 4, device="cuda") * 2.0
+    mean, var = torch.zeros(300, 2, device="cuda"), torch.zeros(300, 2, device="cuda")
+    st = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    s = ctypes.c_void_p(st.cuda_stream)
+    graph, execs = ctypes.c_void_p(), [ctypes.c_void_p(), ctypes.c_void_p()]
+    assert cu.cuStreamBeginCapture_v2(s, 0) == 0
+    lib.gp_predict(g, Z, mean, var, stream=st)
+    assert cu.cuStreamEndCapture(s, ctypes.byref(graph)) == 0
+    for e in execs:
+        assert cu.cuGraphInstantiateWithFlags(ctypes.byref(e), graph, ctypes.c_ulonglong(0)) == 0
+    got = []
+    for e in execs:
+        mean.zero_()
+        var.zero_()
+        torch.cuda.synchronize()
+        assert cu.cuGraphLaunch(e, s) == 0
+        st.synchronize()
+        got.append((mean.cpu().numpy(), var.cpu().numpy()))
+    for e in execs:
+        cu.cuGraphExecDestroy(e)
+    cu.cuGraphDestroy(graph)
+    lib.gp_predict(g, Z, mean, var)
+    torch.cuda.synchronize()
+    for m, v in got:
+        assert np.array_equal(m, mean.cpu().numpy()) and np.array_equal(v, var.cpu().numpy()) and v.any()
+
+
+def test_prediction_on_a_full_device(lib):
+    """Smaller pieces, down to no scratch at all: the same bits."""
+    import torch
+    sc = S.scenario("small", K=33, T=2, N=1025, precision=0)
+    g = lib.gp_fit(sc.X, sc.Y, sc.hyper)
+    Z = torch.rand(60000, 4, device="cuda") * 2.0
+    mean, var = torch.zeros(60000, 2, device="cuda"), torch.zeros(60000, 2, device="cuda")
+    small = [torch.zeros(200, 2, device="cuda") for _ in range(2)]
+    lib.gp_predict(g, Z, mean, var)
+    torch.cuda.synchronize()
+    want = mean.cpu().numpy(), var.cpu().numpy()
+    del g                                 # (what its predictions left in the pool goes with it)
+    g2 = lib.gp_fit(sc.X, sc.Y, sc.hyper)
+    for left in (100 << 20, 2 << 20):
+        mean.zero_()
+        var.zero_()
+        with _Full(left):
+            lib.gp_predict(g2, Z, mean, var)
+            lib.gp_predict(g2, Z[:200], *small)
+            torch.cuda.synchronize()
+        assert np.array_equal(mean.cpu().numpy(), want[0]) and np.array_equal(var.cpu().numpy(), want[1])
+        assert np.array_equal(small[1].cpu().numpy(), want[1][:200])
