@@ -414,7 +414,8 @@ int gpmppi_alu_probe(int32_t kind, int32_t blocks, int32_t iters, float* out, vo
  *                 nanoseconds (default 2e9)
  *   expire_first  non-zero: before any copy, one thread of every CTA waits,
  *                 bounded by ns, on an mbarrier that nothing arrives on, so
- *                 that the wait runs out
+ *                 that the wait runs out (CTAs that start after the timeout is
+ *                 recorded do not wait: a step takes about ns longer)
  * A wait that runs out records GPMPPI_ERR_TIMEOUT in the controller's status
  * word (mppi_device_status reports and clears it) and stops that CTA's copies;
  * the copies in flight land (bounded) before the CTA exits and the kernel ends
