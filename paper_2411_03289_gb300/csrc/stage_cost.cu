@@ -321,7 +321,9 @@ int launch_stage_cost(const RolloutArgs& a, const GpSet& gs, const QueryWs& ws, 
     const int smem = SLayout::obst + 12 * a.O;
     const bool trace = a.tr_mu || a.tr_sig || a.tr_stage || a.tr_margin;
     auto kern = trace ? k_stage_cost<true> : k_stage_cost<false>;
-    if (smem > 48 * 1024) GPM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    // the same limit whatever O is: it belongs to the function, which other threads launch too
+    GPM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  SLayout::obst + 12 * GPMPPI_MAX_OBSTACLES));
     GPM_CUDA(launch_ex(kern, dim3((unsigned)((ws.Ks + 31) / 32)), ST, smem, st, true, 1u, a, sc, ws));
     return GPMPPI_OK;
 }
