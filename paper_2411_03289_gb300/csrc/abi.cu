@@ -26,6 +26,7 @@ int fail(int code, const std::string& msg) {
 }
 
 int cuda_fail(cudaError_t e, const char* what) {
+    cudaGetLastError();      // reported here: the next call's check of its launches must not find it again
     g_err = std::string(what) + ": " + cudaGetErrorString(e);
     return e == cudaErrorMemoryAllocation ? GPMPPI_ERR_OOM : GPMPPI_ERR_CUDA;
 }

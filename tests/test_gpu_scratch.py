@@ -156,3 +156,22 @@ def test_prediction_on_a_full_device(lib):
             torch.cuda.synchronize()
         assert np.array_equal(mean.cpu().numpy(), want[0]) and np.array_equal(var.cpu().numpy(), want[1])
         assert np.array_equal(small[1].cpu().numpy(), want[1][:200])
+
+
+def test_a_failed_allocation_ends_with_its_call(lib):
+    """A controller that does not fit is OOM; the calls after it are not."""
+    import torch
+    sc = S.scenario("small", K=60, T=4, N=70, precision=0)
+    big = S.scenario("small", K=1 << 20, T=64, N=70, precision=0)
+    g, ctrl = make_ctrl(lib, sc)
+    U = torch.tensor(sc.U0, dtype=torch.float32, device="cuda")
+    want, got = torch.empty_like(U), torch.empty_like(U)
+    lib.mppi_step(ctrl, sc.x0, U, want)
+    with _Full(64 << 20):
+        with pytest.raises(lib.GpmppiError) as ei:
+            make_ctrl(lib, big, g)
+        assert ei.value.code == lib.GPMPPI_ERR_OOM
+        g2, ctrl = make_ctrl(lib, sc)
+        lib.mppi_step(ctrl, sc.x0, U, got)
+        torch.cuda.synchronize()
+    assert torch.equal(got, want)
