@@ -336,37 +336,37 @@ int alloc_query_ws(gpmppi_ctrl c) {
         c->nparts = 8 * ((N + 255) / 256);
         if ((size_t)c->nparts * M * n * T > ((size_t)1 << 24)) c->nsplit = c->nparts = 1;
     }
-    cudaFree(c->ws_buf);
-    c->ws_buf = nullptr;
-    cudaError_t e;
-    // on a full device smaller pieces of the samples (the results are the same)
-    while ((e = cudaMalloc(&c->ws_buf, n * (16 * (2 * T + 1) + 4 * M * c->nparts * T))) == cudaErrorMemoryAllocation &&
-           n > 64) {
-        cudaGetLastError();
-        n = (n / 2 + 31) / 32 * 32;
-    }
-    if (e != cudaSuccess) return cuda_fail(e, "mppi_create: rollout workspace");
-    c->ws_Ks = (int)n;
-    // rows of v: up to kVRows bytes at a time, in pieces of one size
+    // On a full device smaller pieces: the rows of v down to a tile, then the samples
+    // of the records and the rows anew (the results are the same).
     size_t npad = 0, rows = 0;
     for (size_t t = 0; t < M; ++t) npad = npad < (size_t)c->gset.gp[t].npad ? (size_t)c->gset.gp[t].npad : npad;
-    if (c->fmt < 0) {
-        const size_t most = npad ? kVRows / 4 / npad / kTriTile * kTriTile : n * T;
-        const size_t pieces = (n * T + most - 1) / most;
-        rows = ((n * T + pieces - 1) / pieces + kTriTile - 1) / kTriTile * kTriTile;
-    }
     const size_t least = c->p.variance_mode == GPMPPI_VAR_NOMINAL ? 4 * T : 0;      // 2 T N doubles
-    cudaFree(c->vbuf);
-    c->vbuf = nullptr;
-    if ((rows > least ? rows : least) * npad > 0) {
-        while ((e = cudaMalloc(&c->vbuf, sizeof(float) * (rows > least ? rows : least) * npad)) ==
-                   cudaErrorMemoryAllocation &&
-               rows > kTriTile) {
-            cudaGetLastError();
-            rows = (rows / 2 + kTriTile - 1) / kTriTile * kTriTile;
+    for (;; n = (n / 2 + 31) / 32 * 32) {
+        cudaFree(c->ws_buf);
+        cudaFree(c->vbuf);
+        c->ws_buf = nullptr;
+        c->vbuf = nullptr;
+        cudaError_t e = cudaMalloc(&c->ws_buf, n * (16 * (2 * T + 1) + 4 * M * c->nparts * T));
+        if (e == cudaSuccess) {
+            if (c->fmt < 0) {
+                // up to kVRows bytes of rows at a time, in pieces of one size
+                const size_t most = npad ? kVRows / 4 / npad / kTriTile * kTriTile : n * T;
+                const size_t pieces = (n * T + most - 1) / most;
+                rows = ((n * T + pieces - 1) / pieces + kTriTile - 1) / kTriTile * kTriTile;
+            }
+            if ((rows > least ? rows : least) * npad > 0)
+                while ((e = cudaMalloc(&c->vbuf, sizeof(float) * (rows > least ? rows : least) * npad)) ==
+                           cudaErrorMemoryAllocation &&
+                       rows > kTriTile) {
+                    cudaGetLastError();
+                    rows = (rows / 2 + kTriTile - 1) / kTriTile * kTriTile;
+                }
         }
-        if (e != cudaSuccess) return cuda_fail(e, "mppi_create: rollout workspace");
+        if (e == cudaSuccess) break;
+        if (e != cudaErrorMemoryAllocation || n <= 64) return cuda_fail(e, "mppi_create: rollout workspace");
+        cudaGetLastError();
     }
+    c->ws_Ks = (int)n;
     if (c->fmt < 0) c->v_q = (int)rows;
     return GPMPPI_OK;
 }
