@@ -45,8 +45,9 @@ __global__ void k_build_kxx(const double* __restrict__ X, int N, double il0, dou
     M[(size_t)i * N + j] = v;
 }
 
-// a / b from r = 1 / b, correctly rounded (Markstein 1990: a faithful quotient
-// corrected by its exact remainder)
+// a / b from r near 1 / b: two corrections by the exact remainder (Markstein 1990).
+// Correctly rounded where r is the rounded reciprocal (the panels); within a unit in
+// the last place with r a few of them off (the pivot's reciprocal root)
 __device__ __forceinline__ double quotient(double a, double b, double r) {
     double q = a * r;
     q = fma(fma(-q, b, a), r, q);
