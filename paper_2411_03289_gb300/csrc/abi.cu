@@ -203,7 +203,6 @@ RolloutArgs gpm::make_rollout_args(gpmppi_ctrl c, const float* state, const floa
     std::memset(&a, 0, sizeof(a));
     a.Xs = g.Xs[0];
     a.alpha = g.alpha;
-    a.W = g.W[0];
     a.obst = c->obst;
     a.seg = c->seg;
     a.seg_il2 = c->seg_il2;

@@ -390,11 +390,6 @@ __global__ void __launch_bounds__(GT) k_grad_rev(const GradArgs g) {
     }
 }
 
-// ---- Gram trace: sum_ij dK/dl_d[i][j] G_o[i][j], G_o = sum_q sbar_o,q b_q b_q^T ----
-// tr(D_d G_o) for d = 0..3, o = v, w, with D_d[i][j] = sf2 2^-|xs_i - xs_j|^2
-// (xs_id - xs_jd)^2 (dK/dl_d up to the factor 2 ln2 / l_d) and G = [G_v; G_w]
-// (2 Np x Np, column-major, symmetric blocks): warp w of block b takes column
-// j = 8 b + w, lanes the rows i (coalesced); 8 partial sums per block.
 // ubar[(o*4+d)][i] = sum_j Kf_ij (xs_id - xs_jd)^2 alpha_o[j]: (dK/dl_d) alpha_o
 // up to the factor 2 ln2 / l_d; one warp per row i.
 __global__ void k_dk_alpha(const float* __restrict__ Xs, const float* __restrict__ alpha, int N, int Np,

@@ -103,16 +103,14 @@ int check_dev_ptr(const void* p, const char* name, bool nullable);
 // ---------------------------------------------------------------------------
 struct GpDevice {
     int N = 0;        // training points
-    int Np = 0;       // N rounded up to a multiple of 16, at least 64 (W is Np x Np)
+    int Np = 0;       // N rounded up to a multiple of 16, at least 64
     int device = 0;
     bool shared = true;          // both outputs share their hyper-parameters
     float sf2[2] = {0, 0};       // signal variances
     void* mem = nullptr;         // the allocation of the fit's arrays below
     // per output o: Xs[o] = N x 4 floats, X scaled by sqrt(log2(e)/2)/l_d so
-    // that k = sf2 * exp2(-|xs - zs|^2); W[o] = Np x Np floats, W[j][i] =
-    // (L^-1)[i][j] for i >= j, zero elsewhere (row j of L^-T).
+    // that k = sf2 * exp2(-|xs - zs|^2)
     float* Xs[2] = {nullptr, nullptr};
-    float* W[2] = {nullptr, nullptr};
     float* alpha = nullptr;      // N x 2 floats (alpha_v, alpha_w) per point
     float zscale[2][4] = {};     // the per-input scale applied to queries
     // FP64 factors kept for export: Linv64[o] N x N, alpha64[o] N
@@ -132,8 +130,8 @@ struct GpDevice {
     // Layouts of the query rollout (query.cuh), built by the fit, per distinct
     // output: npad = N rounded up to 128 points; xq[o] = the scaled inputs in
     // pair layout (npad x 4 floats: two points per 32 bytes, far points past
-    // N) then alpha (npad x 2 floats, both outputs, 0 past N); Wb[o] = L^-T in
-    // 16 x 128 pieces, block column cb holding rows 0 .. 128 (cb + 1) - 1.
+    // N) then alpha (npad x 2 floats, both outputs, 0 past N); Wb[o] = L^-T by
+    // block columns of 128, cb holding rows 0 .. 128 (cb + 1) - 1.
     int npad = 0;
     float* xq[2] = {nullptr, nullptr};
     float* Wb[2] = {nullptr, nullptr};
@@ -153,7 +151,6 @@ struct GpDevice {
 struct RolloutArgs {
     const float* Xs;        // N x 4 scaled GP inputs
     const float* alpha;     // N x 2
-    const float* W;         // Np x Np
     const float* obst;      // O x 3 (cx, cy, r)
     const float4* seg;      // S segments: (ax, ay, bx - ax, by - ay)
     const float* seg_il2;   // S: 1 / |b - a|^2, or 0 for a degenerate segment
@@ -426,8 +423,6 @@ int launch_nominal_var(const GpDevice& g, int T, const QueryWs& ws, double* scra
 int launch_nominal_cov(const RolloutArgs& a, const QueryWs& ws, float* sxy_out, cudaStream_t st);
 int launch_mma_selftest(int fmt, int N, int K, int variant, const uint16_t* A, const uint16_t* B,
                         float* D, unsigned int* err, cudaStream_t st);
-// tr(D_d G_o) from G = [G_v; G_w] (2 Np x Np, column-major): one block per 8
-// columns, 8 partial sums per block; returns the number of blocks
 // the lengthscale Gram traces on the tensor cores (gram_tc.cu): nparts x 8
 // partial traces, nparts = gram_tc_parts(Q, Np, nsm)
 int gram_tc_parts(int Q, int Np, int nsm);

@@ -245,24 +245,20 @@ __global__ void k_alpha_sum(const double* __restrict__ part, int N, int o, doubl
     alpha[j] = s;
 }
 
-// FP32 layouts for the rollout.
-__global__ void k_pack_w(const double* __restrict__ Xm, int N, int Np, float* __restrict__ W) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;   // column of W (row of L^-1)
-    const int j = blockIdx.y;                              // row of W
-    if (i >= Np) return;
-    float v = 0.0f;
-    if (i < N && j < N && i >= j) v = (float)Xm[(size_t)i * N + j];
-    W[(size_t)j * Np + i] = v;
-}
-
-// L^-T in the pieces of the query rollout's variance (GpDevice::Wb): block
-// column cb = blockIdx.y holds rows 0 .. 128 (cb + 1) - 1, 128 columns each.
-__global__ void k_pack_wb(const float* __restrict__ W, int Np, float* __restrict__ Wb) {
-    const int cb = blockIdx.y;
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (cb + 1) * 128 * 128) return;
-    const int j = idx / 128, i = 128 * cb + idx % 128;
-    Wb[(size_t)cb * (cb + 1) / 2 * (128 * 128) + idx] = (j < Np && i < Np) ? W[(size_t)j * Np + i] : 0.0f;
+// L^-T in the pieces of the query rollout's variance (GpDevice::Wb): block column
+// cb holds rows 0 .. 128 (cb + 1) - 1, 128 columns each.  32 x 32 tiles turned in
+// shared memory; blockIdx: tile of the points j, of the columns i.
+__global__ void __launch_bounds__(256) k_pack_wb(const double* __restrict__ Xm, int N, float* __restrict__ Wb) {
+    __shared__ float t[32][33];
+    const int tx = threadIdx.x, ty = threadIdx.y, j0 = 32 * blockIdx.x, i0 = 32 * blockIdx.y, cb = i0 / 128;
+    if (j0 / 128 > cb) return;
+    for (int r = ty; r < 32; r += 8) {
+        const int i = i0 + r, j = j0 + tx;
+        t[r][tx] = (i < N && j <= i) ? (float)Xm[(size_t)i * N + j] : 0.0f;
+    }
+    __syncthreads();
+    float* out = Wb + (size_t)cb * (cb + 1) / 2 * (128 * 128) + i0 % 128 + tx;
+    for (int r = ty; r < 32; r += 8) out[(size_t)(j0 + r) * 128] = t[tx][r];
 }
 
 __global__ void k_pack_x(const double* __restrict__ X, int N, double s0, double s1, double s2,
@@ -461,8 +457,8 @@ int build_mma_ensemble(GpDevice* const* gs, int M, int fmt, MmaTerrains& tr, uin
 // Fit both outputs.  X (N x 4) and Y (N x 2) are host arrays; g.hyper is set.
 int gp_fit_device(GpDevice& g, const double* X, const double* Y, int N, cudaStream_t st) {
     g.N = N;
-    // rows of W padded to a multiple of 16, at least 64 so that every TMA box
-    // of the rollout fits inside the tensor; N = 0 has no W at all
+    // columns of the sums of squares and of the adjoint's b: a multiple of 16, at least
+    // 64 (the orders of both are part of the results); none at N = 0
     g.Np = (N > 0) ? ((N + 15) / 16) * 16 : 0;
     if (g.Np > 0 && g.Np < 64) g.Np = 64;
     g.npad = ((N + 127) / 128) * 128;
@@ -488,10 +484,9 @@ int gp_fit_device(GpDevice& g, const double* X, const double* Y, int N, cudaStre
     const size_t o_alpha = take(sizeof(float) * 2 * n1);
     const size_t o_a64[2] = {take(sizeof(double) * n1), take(sizeof(double) * n1)};
     const size_t o_x64 = take(sizeof(double) * 4 * n1);
-    size_t o_xs[2], o_w[2], o_l[2], o_xq[2], o_wb[2];
+    size_t o_xs[2], o_l[2], o_xq[2], o_wb[2];
     for (int o = 0; o < nout; ++o) {
         o_xs[o] = take(sizeof(float) * 4 * n1);
-        o_w[o] = take(sizeof(float) * (size_t)g.Np * g.Np);
         o_l[o] = take(sizeof(double) * nn);
         o_xq[o] = take(sizeof(float) * 6 * (size_t)g.npad);
         o_wb[o] = take(sizeof(float) * nb * (nb + 1) / 2 * (128 * 128));
@@ -504,7 +499,6 @@ int gp_fit_device(GpDevice& g, const double* X, const double* Y, int N, cudaStre
         const int s = o < nout ? o : 0;              // shared hyper-parameters: one factor
         g.alpha64[o] = reinterpret_cast<double*>(mem + o_a64[o]);
         g.Xs[o] = reinterpret_cast<float*>(mem + o_xs[s]);
-        g.W[o] = reinterpret_cast<float*>(mem + o_w[s]);
         g.Linv64[o] = reinterpret_cast<double*>(mem + o_l[s]);
         g.xq[o] = reinterpret_cast<float*>(mem + o_xq[s]);
         g.Wb[o] = reinterpret_cast<float*>(mem + o_wb[s]);
@@ -565,13 +559,12 @@ int gp_fit_device(GpDevice& g, const double* X, const double* Y, int N, cudaStre
         const double s = std::sqrt(0.5 * log2e);
         k_pack_x<<<gb, tb, 0, st>>>(dX, N, s / h.lengthscale[0], s / h.lengthscale[1],
                                     s / h.lengthscale[2], s / h.lengthscale[3], g.Xs[o]);
-        k_pack_w<<<dim3((g.Np + 127) / 128, g.Np), 128, 0, st>>>(g.Linv64[o], N, g.Np, g.W[o]);
         if ((rc = check(cudaGetLastError(), "inverse kernels"))) return rc;
     }
     k_pack_alpha<<<(N + 127) / 128, 128, 0, st>>>(g.alpha64[0], g.alpha64[1], N, g.alpha);
     for (int o = 0; o < nout; ++o) {
         k_pack_xa<<<(g.npad + 127) / 128, 128, 0, st>>>(g.Xs[o], g.alpha, N, g.npad, 0, g.npad, g.xq[o]);
-        k_pack_wb<<<dim3((unsigned)(nb * 64), (unsigned)nb), 256, 0, st>>>(g.W[o], g.Np, g.Wb[o]);
+        k_pack_wb<<<dim3((unsigned)(4 * nb), (unsigned)(4 * nb)), dim3(32, 8), 0, st>>>(g.Linv64[o], N, g.Wb[o]);
     }
     if ((rc = check(cudaGetLastError(), "pack alpha"))) return rc;
     if ((rc = check(cudaStreamSynchronize(st), "gp_fit sync"))) return rc;

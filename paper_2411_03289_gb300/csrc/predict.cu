@@ -195,7 +195,7 @@ int launch_gp_predict(const GpDevice& g, const float* Z, int M, float* mean, flo
                 j.fusez = 1;
                 rc = launch_tri_forward(j, false, st);
                 if (rc) break;
-                e = launch_ex(k_pred_var, dim3((unsigned)((p.M + kTriTile - 1) / kTriTile)), 4 * kTriTile, 0, st, true, 1u, p);
+                e = launch_ex(k_pred_var, dim3((unsigned)((p.M + kTriTile - 1) / kTriTile)), 4 * kTriTile, 0, st, true, p);
             } else {
                 k_pred_direct<<<p.M, ST, sizeof(float) * (g.N > 0 ? g.N : 1), st>>>(p);
                 e = cudaGetLastError();

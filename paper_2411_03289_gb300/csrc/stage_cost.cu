@@ -301,7 +301,7 @@ __global__ void __launch_bounds__(32) k_nominal_cov(const RolloutArgs a, const Q
 }  // namespace
 
 int launch_nominal_cov(const RolloutArgs& a, const QueryWs& ws, float* sxy_out, cudaStream_t st) {
-    GPM_CUDA(launch_ex(k_nominal_cov, dim3(1), 32, 0, st, true, 1u, a, ws, sxy_out));
+    GPM_CUDA(launch_ex(k_nominal_cov, dim3(1), 32, 0, st, true, a, ws, sxy_out));
     return GPMPPI_OK;
 }
 
@@ -324,7 +324,7 @@ int launch_stage_cost(const RolloutArgs& a, const GpSet& gs, const QueryWs& ws, 
     // the same limit whatever O is: it belongs to the function, which other threads launch too
     GPM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   SLayout::obst + 12 * GPMPPI_MAX_OBSTACLES));
-    GPM_CUDA(launch_ex(kern, dim3((unsigned)((ws.Ks + 31) / 32)), ST, smem, st, true, 1u, a, sc, ws));
+    GPM_CUDA(launch_ex(kern, dim3((unsigned)((ws.Ks + 31) / 32)), ST, smem, st, true, a, sc, ws));
     return GPMPPI_OK;
 }
 

@@ -270,7 +270,7 @@ int launch_tri(const TriJob& j, bool dependent, cudaStream_t st) {
     auto kern = j.fusez ? k_tri<BACK, true> : k_tri<BACK, false>;
     const int smem = TriLayout<BACK>::total;
     GPM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    GPM_CUDA(launch_ex(kern, grid, PT, smem, st, dependent, 1u, j));
+    GPM_CUDA(launch_ex(kern, grid, PT, smem, st, dependent, j));
     return GPMPPI_OK;
 }
 
@@ -304,7 +304,7 @@ int launch_rowsum(const float* V, int ld, int Q, int N, SumOrder order, float* o
     int Np = (N + 15) / 16 * 16;
     if (Np > 0 && Np < 64) Np = 64;
     auto kern = order == kSumPairs ? k_rowsum<kSumPairs> : k_rowsum<kSumLanes>;
-    GPM_CUDA(launch_ex(kern, dim3((unsigned)((Q + PQ - 1) / PQ)), PQ, 0, st, true, 1u, V, ld, Q, Np, out));
+    GPM_CUDA(launch_ex(kern, dim3((unsigned)((Q + PQ - 1) / PQ)), PQ, 0, st, true, V, ld, Q, Np, out));
     return GPMPPI_OK;
 }
 

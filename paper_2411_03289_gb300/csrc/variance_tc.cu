@@ -365,6 +365,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT, 1) k_var_tc(cons
                             }
                         }
                         if (r0 == 0) {
+                            // A warp takes every second stage, so that with a ring of three its
+                            // waits on a slot all have one parity.  The phase before is over all
+                            // the same: two stages ago it saw the commit of stage n - NA - 2, and
+                            // the slot's last use, stage n - NA - NBP, was committed before that.
+                            static_assert(NBP >= 2, "the slot's last use is older than the last commit seen");
                             room = n < (uint32_t)NA || wait(done + (n - NA) % NBP, ((n - NA) / NBP) & 1u);
                             ok = __all_sync(0xffffffffu, got && room);
                             if (!ok) break;
@@ -720,7 +725,7 @@ int launch_var_tc(const GpSet& gs, const VarTcJob& j, int fmt, int nsm, bool dep
                             : (fmt == 0 ? k_var_tc<0, false> : k_var_tc<1, false>);
     const int smem = fmt == 2 ? TcLayout<3>::total : TcLayout<2>::total;
     GPM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    GPM_CUDA(launch_ex(kern, dim3((unsigned)(2 * pairs)), NT, smem, st, dependent, 1u, gs, j));
+    GPM_CUDA(launch_ex(kern, dim3((unsigned)(2 * pairs)), NT, smem, st, dependent, gs, j));
     return GPMPPI_OK;
 }
 
