@@ -944,9 +944,16 @@ int mppi_grad(gpmppi_ctrl c, const float state[5], const float* U_nom, const flo
     // that a later one may be captured)
     if ((rc = build_back_pieces(g, st))) return rc;
     if (want_l && !g.ubar) {
-        GPM_CUDA(cudaMalloc(&g.ubar, sizeof(float) * 8 * (size_t)(Np > 0 ? Np : 1)));
-        if (N > 0 && (rc = launch_dk_alpha(g.Xs[0], g.alpha, N, Np, g.sf2[0], g.ubar, st))) return rc;
-        GPM_CUDA(cudaStreamSynchronize(st));
+        float* ubar = nullptr;
+        GPM_CUDA(cudaMalloc(&ubar, sizeof(float) * 8 * (size_t)(Np > 0 ? Np : 1)));
+        rc = N > 0 ? launch_dk_alpha(g.Xs[0], g.alpha, N, Np, g.sf2[0], ubar, st) : GPMPPI_OK;
+        const cudaError_t e = rc ? cudaSuccess : cudaStreamSynchronize(st);
+        if (e != cudaSuccess) rc = cuda_fail(e, "mppi_grad: (dK/dl) alpha");
+        if (rc) {
+            cudaFree(ubar);
+            return rc;
+        }
+        g.ubar = ubar;
     }
     const GpSet gs = single_gp_set(g, 0);
     int nsm = 0;

@@ -380,28 +380,41 @@ int set_cB(GpDevice& g) {
     return GPMPPI_OK;
 }
 
+// The tiles belong to the GP once all of them are there: after a failure the next call
+// starts anew.
 int build_mma_tiles(GpDevice& g, int fmt) {
     if (g.mma_hi[fmt] || g.N == 0) return GPMPPI_OK;
-    const int N = g.N;
-    g.NpM = ((N + 127) / 128) * 128;
+    const int N = g.N, NpM = ((N + 127) / 128) * 128;
     const int rc = set_cB(g);
     if (rc) return rc;
     // 32-point stages x pairs of 128-row blocks x 256 rows x 32 points
-    const size_t n = (size_t)(g.NpM / 32) * (size_t)((g.NpM / 128 + 1) / 2) * 8192;
-    GPM_CUDA(cudaMalloc(&g.mma_hi[fmt], n * sizeof(uint16_t)));
-    GPM_CUDA(cudaMalloc(&g.mma_lo[fmt], n * sizeof(uint16_t)));
-    if (fmt == 2) GPM_CUDA(cudaMalloc(&g.mma_mid, n * sizeof(uint16_t)));
-    k_pack_mma<<<(unsigned)((n + 255) / 256), 256>>>(g.Linv64[0], N, g.NpM, fmt, (double)g.cB, 0, 0,
-                                                      (g.NpM / 128 + 1) / 2, g.mma_hi[fmt], g.mma_lo[fmt],
-                                                      g.mma_mid);
-    GPM_CUDA(cudaGetLastError());
-    if (!g.mma_xa) {
-        // the streaming rollout's training inputs and alpha in pair layout
-        GPM_CUDA(cudaMalloc(&g.mma_xa, sizeof(float) * 6 * (size_t)g.NpM));
-        k_pack_xa<<<(g.NpM + 127) / 128, 128>>>(g.Xs[0], g.alpha, g.N, g.NpM, 0, g.NpM, g.mma_xa);
-        GPM_CUDA(cudaGetLastError());
+    const size_t n = (size_t)(NpM / 32) * (size_t)((NpM / 128 + 1) / 2) * 8192;
+    uint16_t *hi = nullptr, *lo = nullptr, *mid = nullptr;
+    float* xa = g.mma_xa;
+    cudaError_t e = cudaMalloc(&hi, n * sizeof(uint16_t));
+    if (e == cudaSuccess) e = cudaMalloc(&lo, n * sizeof(uint16_t));
+    if (e == cudaSuccess && fmt == 2) e = cudaMalloc(&mid, n * sizeof(uint16_t));
+    if (e == cudaSuccess && !xa) e = cudaMalloc(&xa, sizeof(float) * 6 * (size_t)NpM);
+    if (e == cudaSuccess) {
+        k_pack_mma<<<(unsigned)((n + 255) / 256), 256>>>(g.Linv64[0], N, NpM, fmt, (double)g.cB, 0, 0,
+                                                          (NpM / 128 + 1) / 2, hi, lo, mid);
+        // the batched rollout's training inputs and alpha in pair layout
+        if (!g.mma_xa) k_pack_xa<<<(NpM + 127) / 128, 128>>>(g.Xs[0], g.alpha, N, NpM, 0, NpM, xa);
+        e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaDeviceSynchronize();
     }
-    GPM_CUDA(cudaDeviceSynchronize());
+    if (e != cudaSuccess) {
+        cudaFree(hi);
+        cudaFree(lo);
+        cudaFree(mid);
+        if (!g.mma_xa) cudaFree(xa);
+        return cuda_fail(e, "batched rollout: factor tiles");
+    }
+    g.NpM = NpM;
+    g.mma_hi[fmt] = hi;
+    g.mma_lo[fmt] = lo;
+    if (fmt == 2) g.mma_mid = mid;
+    g.mma_xa = xa;
     return GPMPPI_OK;
 }
 
@@ -430,27 +443,33 @@ int build_mma_ensemble(GpDevice* const* gs, int M, int fmt, MmaTerrains& tr, uin
     if (nb == 0) return GPMPPI_OK;
     const int NpT = nb * 128, NP = nb / 2;
     const size_t n = (size_t)(NpT / 32) * NP * 8192;
-    GPM_CUDA(cudaMalloc(hi, n * sizeof(uint16_t)));
-    GPM_CUDA(cudaMalloc(lo, n * sizeof(uint16_t)));
-    GPM_CUDA(cudaMemset(*hi, 0, n * sizeof(uint16_t)));
-    GPM_CUDA(cudaMemset(*lo, 0, n * sizeof(uint16_t)));
-    if (fmt == 2) {
-        GPM_CUDA(cudaMalloc(mid, n * sizeof(uint16_t)));
-        GPM_CUDA(cudaMemset(*mid, 0, n * sizeof(uint16_t)));
-    }
-    GPM_CUDA(cudaMalloc(xa, sizeof(float) * 6 * (size_t)NpT));
-    for (int t = 0; t < M; ++t) {
+    cudaError_t e = cudaMalloc(hi, n * sizeof(uint16_t));
+    if (e == cudaSuccess) e = cudaMalloc(lo, n * sizeof(uint16_t));
+    if (e == cudaSuccess && fmt == 2) e = cudaMalloc(mid, n * sizeof(uint16_t));
+    if (e == cudaSuccess) e = cudaMalloc(xa, sizeof(float) * 6 * (size_t)NpT);
+    if (e == cudaSuccess) e = cudaMemset(*hi, 0, n * sizeof(uint16_t));
+    if (e == cudaSuccess) e = cudaMemset(*lo, 0, n * sizeof(uint16_t));
+    if (e == cudaSuccess && fmt == 2) e = cudaMemset(*mid, 0, n * sizeof(uint16_t));
+    for (int t = 0; t < M && e == cudaSuccess; ++t) {
         const GpDevice& g = *gs[t];
         const int nbt = tr.blk0[t + 1] - tr.blk0[t];
         if (nbt == 0) continue;
         const size_t nt = (size_t)(nbt * 4) * (nbt / 2) * 8192;
         k_pack_mma<<<(unsigned)((nt + 255) / 256), 256>>>(g.Linv64[0], g.N, nbt * 128, fmt, (double)g.cB,
                                                            4 * tr.blk0[t], tr.blk0[t] / 2, NP, *hi, *lo, *mid);
-        GPM_CUDA(cudaGetLastError());
         k_pack_xa<<<(nbt * 128 + 127) / 128, 128>>>(g.Xs[0], g.alpha, g.N, nbt * 128, 128 * tr.blk0[t], NpT, *xa);
-        GPM_CUDA(cudaGetLastError());
+        e = cudaGetLastError();
     }
-    GPM_CUDA(cudaDeviceSynchronize());
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    if (e != cudaSuccess) {
+        cudaFree(*hi);
+        cudaFree(*lo);
+        cudaFree(*mid);
+        cudaFree(*xa);
+        *hi = *lo = *mid = nullptr;
+        *xa = nullptr;
+        return cuda_fail(e, "batched rollout: stacked factor tiles");
+    }
     return GPMPPI_OK;
 }
 

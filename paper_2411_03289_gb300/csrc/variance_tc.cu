@@ -682,10 +682,16 @@ int build_tc_pieces(GpDevice& g, int fmt) {
     const int parts = fmt == 2 ? 3 : 2, kc = stage_points(parts);
     size_t n = pass_base(p);                     // columns x points
     for (int c = 0; c < pass_stages(N, p, kc); ++c) n += (size_t)(pass_hi(N, p) - stage_lo(p, c, kc)) * kc;
-    GPM_CUDA(cudaMalloc(&g.Bt[fmt], n * (size_t)(2 * parts)));
-    k_pack_tc<<<dim3((unsigned)(PASS / kc * np), (unsigned)np), 256>>>(g.Linv64[0], N, fmt, (double)g.cB, g.Bt[fmt]);
-    GPM_CUDA(cudaGetLastError());
-    GPM_CUDA(cudaDeviceSynchronize());
+    uint16_t* Bt = nullptr;
+    GPM_CUDA(cudaMalloc(&Bt, n * (size_t)(2 * parts)));
+    k_pack_tc<<<dim3((unsigned)(PASS / kc * np), (unsigned)np), 256>>>(g.Linv64[0], N, fmt, (double)g.cB, Bt);
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    if (e != cudaSuccess) {
+        cudaFree(Bt);
+        return cuda_fail(e, "tensor-core factor pieces");
+    }
+    g.Bt[fmt] = Bt;
     return GPMPPI_OK;
 }
 

@@ -175,3 +175,36 @@ def test_a_failed_allocation_ends_with_its_call(lib):
         lib.mppi_step(ctrl, sc.x0, U, got)
         torch.cuda.synchronize()
     assert torch.equal(got, want)
+
+
+@pytest.mark.parametrize("precision,terrains", [(2, 1), (3, 1), (3, 2)])
+def test_batch_after_a_failed_one(lib, precision, terrains):
+    """A batch whose factor tiles do not fit is OOM, whichever of them fails; made again
+    with room it steps as the controller does on its own."""
+    import torch
+    N = 1500
+    if terrains == 1:
+        sc = S.scenario("small", K=70, T=3, N=N, precision=precision)
+    else:
+        sc = S.terrain_scenario("small", M=terrains, N=N, K=70, T=3, precision=precision)
+    _, ctrl = make_ctrl(lib, sc)
+    U = torch.tensor(sc.U0, dtype=torch.float32, device="cuda")
+    want, w, c = torch.empty_like(U), torch.empty(70, device="cuda"), torch.empty(70, device="cuda")
+    failed = 0
+    for left in (2, 6, 10, 14, 18, 24):           # a part is 5 MB, of the stacked factor 18
+        with _Full(left << 20):
+            try:
+                b = lib.mppi_batch_create([ctrl])
+                del b
+            except lib.GpmppiError as e:
+                assert e.code == lib.GPMPPI_ERR_OOM
+                failed += 1
+    assert failed >= 2
+    lib.mppi_set_iteration(ctrl, 4)
+    b = lib.mppi_batch_create([ctrl])
+    b.state[0].copy_(torch.tensor(sc.x0, dtype=torch.float32))
+    b.U_nom[0].copy_(U)
+    lib.mppi_step(ctrl, sc.x0.astype(np.float32), U, want, w, c)
+    lib.mppi_batch_step(b)
+    torch.cuda.synchronize()
+    assert torch.equal(b.U_new[0], want) and torch.equal(b.weights[0], w) and want.any()
