@@ -103,10 +103,11 @@ __global__ void __launch_bounds__(4 * kTriTile) k_pred_var(const PredArgs p) {
 
 // The variances without scratch, one CTA a query: the same sums in the same order (v
 // one chain over the points, the squares as above), every query reading the whole
-// factor: 20000 queries at N = 1000 in 3.3 ms, 0.4 by way of V.  For calls under
-// stream capture, where scratch would be an allocation node, with which a graph may
-// neither be instantiated twice at a time nor be a child of another, and for a
-// device without room for 128 rows.
+// factor.  In all, 20000 queries at N = 1000: 1.83 ms, 0.44 by way of V; 200: 152
+// against 111 us; 200 at N = 300: 25 against 36.  For calls under stream capture,
+// where scratch would be an allocation node, with which a graph may neither be
+// instantiated twice at a time nor be a child of another, and for a device without
+// room for 128 rows.
 __global__ void __launch_bounds__(ST) k_pred_direct(const PredArgs p) {
     extern __shared__ float ks[];                    // N floats
     __shared__ float red[ST / 32];
