@@ -106,6 +106,7 @@ void free_gp(gpmppi_gp h) {
     if (!h) return;
     GpDevice& g = h->g;
     cudaFree(g.mem);
+    for (int f = 0; f < 2; ++f) cudaFree(g.Bs[f]);
     for (int f = 0; f < 3; ++f) {
         cudaFree(g.Bt[f]);
         cudaFree(g.mma_hi[f]);
@@ -284,12 +285,16 @@ int gpm::launch_query_rollout(gpmppi_ctrl c, const RolloutArgs& a, const GpSet& 
                 }
         } else {
             if ((rc = launch_chain(a, gs, ws, st))) return rc;
-            const VarTcJob j = {ws.zq, Q, ws.q, ws.nsplit, ws.nparts, ws.rps, ws.even, a.err};
+            const VarTcJob j = {ws.zq, Q, ws.q, ws.nsplit, ws.nparts, ws.sums, ws.even, a.err};
             if ((rc = launch_var_tc(gs, j, c->fmt, c->nsm, true, st))) return rc;
         }
         if ((rc = launch_stage_cost(a, gs, ws, c->ens && c->fmt < 0, st))) return rc;
     }
     return GPMPPI_OK;
+}
+
+static VarSums sums_of(gpmppi_ctrl c) {
+    return c->kind == GPMPPI_KERNEL_TC_CLUSTER ? kSumsShares : c->mm.lo_set ? kSumsTwo : kSumsOne;
 }
 
 QueryWs gpm::make_query_ws(gpmppi_ctrl c, int s0, int Ks) {
@@ -302,9 +307,8 @@ QueryWs gpm::make_query_ws(gpmppi_ctrl c, int s0, int Ks) {
     ws.Ks = Ks;
     ws.nsplit = c->nsplit;
     ws.nparts = c->nparts;
-    // The sums of the batched rollout wherever both kernels give the small products
-    // their own column set, so that their products agree to the bit.
-    ws.rps = c->fmt >= 0 && c->mm.lo_set ? c->rps : 0;
+    ws.sums = sums_of(c);
+    ws.rps = c->rps;
     ws.even = c->ens ? 1 : 0;
     return ws;
 }
@@ -326,13 +330,13 @@ int alloc_query_ws(gpmppi_ctrl c) {
     if (n > (size_t)c->p.K) n = (size_t)c->p.K;
     if (n < (size_t)c->p.K && n > 32) n = n / 32 * 32;     // (every piece starts a warp of the chain)
     c->nsplit = c->nparts = c->fmt < 0 ? 1 : var_tc_splits(c->gset, (int)(n * T), c->nsm);
-    if (c->fmt >= 0 && c->mm.lo_set && c->nsplit > 1) {
-        // a split's sums are put in the batched rollout's order afterwards, from a part
-        // for every 32 columns; not worth the room beyond 64 MB, where splits gain
-        // little (they fill the last wave)
+    if (c->nsplit > 1) {
+        // a split's sums are put in their order afterwards, from a part for every 32 or
+        // 64 columns; not worth the room beyond 64 MB, where splits gain little (they
+        // fill the last wave)
         int N = 0;
         for (size_t t = 0; t < M; ++t) N = N < c->gset.gp[t].N ? c->gset.gp[t].N : N;
-        c->nparts = 8 * ((N + 255) / 256);
+        c->nparts = (sums_of(c) == kSumsTwo ? 8 : 4) * ((N + 255) / 256);
         if ((size_t)c->nparts * M * n * T > ((size_t)1 << 24)) c->nsplit = c->nparts = 1;
     }
     // On a full device smaller pieces: the rows of v down to a tile, then the samples
@@ -398,13 +402,13 @@ constexpr int kMaxFp32EnsembleN = 3616;
 
 // GP g as the query rollout reads it, in format fmt (-1: FP32); builds the
 // format's tensor-core pieces on first use.
-int make_query_gp(GpDevice& g, int fmt, GpSet::One* out) {
+int make_query_gp(GpDevice& g, int fmt, bool shares, GpSet::One* out) {
     *out = single_gp_set(g, 0).gp[0];
     if (fmt < 0) return GPMPPI_OK;
     int rc;
-    if ((rc = build_tc_pieces(g, fmt))) return rc;
+    if ((rc = build_tc_pieces(g, fmt, shares))) return rc;
     const double r = (double)g.sf2[0] / (g.cB > 0.0f ? (double)g.cB : 1.0);
-    out->Bt = g.Bt[fmt];
+    out->Bt = shares ? g.Bs[fmt] : g.Bt[fmt];
     out->qscale = (float)(r * r);
     return GPMPPI_OK;
 }
@@ -419,7 +423,7 @@ int launch_nominal(gpmppi_ctrl c, const RolloutArgs& a, cudaStream_t st) {
     ws.s0 = 0;
     ws.Ks = 1;
     ws.nsplit = ws.nparts = 1;
-    ws.rps = ws.even = 0;
+    ws.sums = ws.rps = ws.even = 0;
     int rc;
     if ((rc = launch_nominal_mean(a, ws, st))) return rc;
     if ((rc = launch_nominal_var(c->gp->g, a.T, ws, reinterpret_cast<double*>(c->vbuf), st))) return rc;
@@ -707,9 +711,10 @@ int mppi_create(const gpmppi_params* p, const float* obstacles, int32_t O, const
             }
         }
         if (fmt >= 0) {
-            // what mppi_rollout_kind and mppi_batch_layout report: the class of the
-            // workload (training sets of up to 512 points in two parts apart) and
-            // the layout's threads per sample, fewest that give every SM a tile
+            // the class of the workload (training sets of up to 512 points in two parts
+            // apart), which sets the order of its sums (VarSums) and is what
+            // mppi_rollout_kind reports, and the batched layout's threads per sample,
+            // fewest that give every SM a tile
             const char* no_cl = std::getenv("GPMPPI_NO_CLUSTER");
             const bool small = fmt < 2 && gp->g.N > 0 && gp->g.N <= 512 && !(no_cl && no_cl[0] == '1');
             c->kind = small ? GPMPPI_KERNEL_TC_CLUSTER : GPMPPI_KERNEL_TC_STREAM;
@@ -723,7 +728,7 @@ int mppi_create(const gpmppi_params* p, const float* obstacles, int32_t O, const
             }
         }
         c->gset.M = 1;
-        if ((rc = make_query_gp(gp->g, c->fmt, &c->gset.gp[0])) || (rc = alloc_query_ws(c))) {
+        if ((rc = make_query_gp(gp->g, c->fmt, c->kind == GPMPPI_KERNEL_TC_CLUSTER, &c->gset.gp[0])) || (rc = alloc_query_ws(c))) {
             free_ctrl(c);
             return rc;
         }
@@ -862,8 +867,9 @@ int mppi_create_ensemble(const gpmppi_params* p, const float* obstacles, int32_t
         c->tw[i] = weights[i];
         if (i > 0) gps[i]->g.n_controllers++;
     }
+    if (ens) c->kind = c->fmt < 0 ? GPMPPI_KERNEL_ENSEMBLE : GPMPPI_KERNEL_TC_STREAM;
     for (int i = 0; i < M; ++i) {
-        if ((rc = make_query_gp(gps[i]->g, c->fmt, &c->gset.gp[i]))) {
+        if ((rc = make_query_gp(gps[i]->g, c->fmt, c->kind == GPMPPI_KERNEL_TC_CLUSTER, &c->gset.gp[i]))) {
             mppi_destroy(c);
             return rc;
         }
@@ -871,7 +877,6 @@ int mppi_create_ensemble(const gpmppi_params* p, const float* obstacles, int32_t
     }
     c->gset.M = M;
     if (ens) {
-        c->kind = c->fmt < 0 ? GPMPPI_KERNEL_ENSEMBLE : GPMPPI_KERNEL_TC_STREAM;
         if (c->fmt >= 0) {
             int points = 0, optin = 0;
             bool lo = c->fmt == 2;

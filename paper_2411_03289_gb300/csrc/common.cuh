@@ -138,6 +138,7 @@ struct GpDevice {
     // tensor-core pieces of cB L^-1 per operand format (variance_tc.cu), built
     // on first use by a controller
     uint16_t* Bt[3] = {nullptr, nullptr, nullptr};
+    uint16_t* Bs[2] = {nullptr, nullptr};      // the same in the stage order of kSumsShares
     float cB = 0.0f;
     // adjoint, built on first use: L^-1 in the pieces of the backward product and the
     // vectors (dK/dl_d) alpha_o (8 x Np)
@@ -305,7 +306,7 @@ struct GpSet {
         const float* Wb;        // GpDevice::Wb
         const float* Xs;        // GpDevice::Xs, alpha
         const float* alpha;
-        const uint16_t* Bt;     // GpDevice::Bt of the controller's format
+        const uint16_t* Bt;     // GpDevice::Bt or Bs of the controller's format
         int N, npad;
         float sf2, w;
         float qscale;           // variance = sf2 - qscale * (what the variance kernel stored)
@@ -320,11 +321,24 @@ struct QueryWs {
     float4* st;                 // T x Ks: (X, Y, theta, v) after step k
     float* q;                   // M x nparts x T x Ks: parts of |L_t^-1 k*|^2 over the variance kernel's scale
     int s0, Ks;
+    // split precisions
     int nsplit;                 // CTA pairs that share a query's passes (variance_tc.cu)
-    int nparts;                 // parts a variance comes in: nsplit, or (rps > 0) 1 or a part for every 32 columns
-    int rps;                    // > 0: the sums of the batched rollout with rps threads a sample
-    int even;                   // with rps: the batched rollout pads every GP to pairs of 128-column blocks
+    int nparts;                 // parts a variance comes in: 1, or one for every 32 or 64 columns
+    int sums;                   // VarSums
+    int rps;                    // threads a sample whose sums of the mean the chain forms (chain.cu)
+    int even;                   // terrain ensembles: every GP padded to pairs of 128-column blocks
 };
+// The orders of the sums of a split-precision rollout, which are part of its results
+// (a mean or a margin in the last bit decides an indicator now and then):
+//   kSumsTwo     hi.hi and the small products in column sets of their own, as in the
+//                batched rollout: more than 768 points, the three-part format
+//   kSumsOne     all three products in one set, as in the batched rollout: other
+//                training sets of more than 512 points, terrain ensembles
+//   kSumsShares  training sets of up to 512 points in two parts: 64-column slices in
+//                pairs (s, last - s), each pair with its own order of the stages and its
+//                own share of the mean's 16-point chunks (the batched rollout runs
+//                these as kSumsOne)
+enum VarSums { kSumsTwo = 0, kSumsOne = 1, kSumsShares = 2 };
 
 // Adjoint (gradient of the smoothed cost) of the samples [s0, s0 + Ks); see adjoint.cu.
 struct GradArgs {
@@ -381,12 +395,12 @@ struct VarTcJob {
     int Q;
     float* q;                   // M x nparts x Q
     int nsplit;
-    int nparts, rps, even;      // as in QueryWs
+    int nparts, sums, even;     // as in QueryWs
     unsigned int* err;
 };
 constexpr int kMaxVarSplits = 8;
 int set_cB(GpDevice& g);
-int build_tc_pieces(GpDevice& g, int fmt);
+int build_tc_pieces(GpDevice& g, int fmt, bool shares);
 int var_tc_splits(const GpSet& gs, int Q, int nsm);
 int launch_var_tc(const GpSet& gs, const VarTcJob& j, int fmt, int nsm, bool dependent, cudaStream_t st);
 int launch_stage_cost(const RolloutArgs& a, const GpSet& gs, const QueryWs& ws, bool ensemble, cudaStream_t st);

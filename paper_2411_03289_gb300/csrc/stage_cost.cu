@@ -27,8 +27,6 @@ constexpr int SU = 8;                    // lane segments per round
 struct ScoreScale {
     int M, nparts;
     bool two;            // the variances are added in a rounding of their own (FP32 terrain ensembles)
-    bool half;           // the parts are 32 columns each, the halves of every pass summed apart (QueryWs::rps)
-    int even, N[kMaxTerrains];
     float w2[kMaxTerrains], sf2[kMaxTerrains], qscale[kMaxTerrains];
 };
 
@@ -116,28 +114,8 @@ __global__ void __launch_bounds__(ST) k_stage_cost(const RolloutArgs a, const Sc
             float s = 0.0f;
             const float* qp = ws.q + (size_t)k * Ks + l;
             for (int t = 0; t < sc.M; ++t) {
-                float q;
-                if (sc.half) {
-                    float h0 = 0.0f, h1 = 0.0f;
-                    const float* gp = qp;
-                    for (int n = (sc.N[t] + 63) / 64 * 2; n > 0; n -= 8) {      // a pass: 8 parts, or what is left
-                        const int h = sc.even || n >= 8 ? 4 : (n + 2) / 4 * 2;
-                        float g[8];
-#pragma unroll
-                        for (int j = 0; j < 8; ++j, gp += Q) g[j] = j < n ? *gp : 0.0f;
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) {
-                            if (j < n && j < h) h0 += g[j];
-                            if (j < n && j >= h) h1 += g[j];
-                        }
-                    }
-                    q = h0 + h1;
-                    qp += (size_t)sc.nparts * Q;
-                } else {
-                    q = *qp;
-                    qp += Q;
-                    for (int j = 1; j < sc.nparts; ++j, qp += Q) q += *qp;
-                }
+                const float q = *qp;
+                qp += (size_t)sc.nparts * Q;
                 s += sc.w2[t] * fmaxf(0.0f, sc.sf2[t] - sc.qscale[t] * q);
             }
             float sn, cs;
@@ -309,14 +287,11 @@ int launch_stage_cost(const RolloutArgs& a, const GpSet& gs, const QueryWs& ws, 
     ScoreScale sc = {};
     sc.M = gs.M;
     sc.nparts = ws.nparts;
-    sc.half = ws.rps > 0 && ws.nparts > 1;
-    sc.even = ws.even;
     sc.two = ensemble;
     for (int t = 0; t < gs.M; ++t) {
         sc.w2[t] = gs.gp[t].w * gs.gp[t].w;
         sc.sf2[t] = gs.gp[t].sf2;
         sc.qscale[t] = gs.gp[t].qscale;
-        sc.N[t] = gs.gp[t].N;
     }
     const int smem = SLayout::obst + 12 * a.O;
     const bool trace = a.tr_mu || a.tr_sig || a.tr_stage || a.tr_margin;

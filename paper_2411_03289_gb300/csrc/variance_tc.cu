@@ -70,13 +70,16 @@ struct TcLayout {
 };
 
 // ---- the passes of one GP of N points ---------------------------------------
-// pass p: columns 256 p .. 256 p + hi - 1, stages 0 .. pass_stages - 1; stage c
-// multiplies columns lo(c) .. hi - 1 (those below hold no point of the stage)
+// pass p: columns 256 p .. 256 p + hi - 1, in 64-column quarters; entry c of a pass
+// multiplies one stage of points with some of them (those that hold none of its points
+// are left out).  In the order of the points (kSumsTwo, kSumsOne) entry c is stage c
+// and the quarters lo(c) / 64 on.  kSumsShares gives every quarter the order that it
+// had when a cluster of CTAs held the factor and each CTA took its stages as its share
+// of the mean came first: of 257 to 512 points quarter 5 in the order 0 3 4 5 1 2, 6 in
+// 0 6 1 .. 5, 7 in 0 7 1 .. 6, of 129 to 256 points quarter 3 in 0 3 1 2, the others
+// ascending.  A pass is a common sequence of its quarters' orders, in which some stages
+// come twice (11 entries instead of 8 for the last pass of 512 points).
 __host__ __device__ inline int pass_count(int N) { return (N + PASS - 1) / PASS; }
-__host__ __device__ inline int pass_stages(int N, int p, int kc) {
-    const int n = (N + kc - 1) / kc, full = PASS / kc * (p + 1);
-    return full < n ? full : n;
-}
 __host__ __device__ inline int pass_hi(int N, int p) {
     const int n = (N - PASS * p + QUART - 1) / QUART * QUART;
     return n < PASS ? n : PASS;
@@ -85,15 +88,58 @@ __host__ __device__ inline int stage_lo(int p, int c, int kc) {
     const int d = kc * c - PASS * p;
     return d > 0 ? QUART * (d / QUART) : 0;
 }
+
+// kSumsShares: entry c of a pass in hexadecimal digit c (of two words of eight)
+struct Digits {
+    unsigned int lo, hi;
+    __host__ __device__ int operator[](int c) const { return (int)((c < 8 ? lo >> 4 * c : hi >> 4 * (c - 8)) & 15u); }
+};
+struct Shares {
+    int n;
+    Digits stage;           // its stage
+    Digits quarters;        // the quarters it multiplies
+    Digits done;            // those that are complete after it
+    unsigned int order;     // the quarters as they become complete
+};
+__host__ __device__ inline Shares shares_of(int N, int p) {
+    const int h = pass_hi(N, p) / QUART;
+    if (p == 1) {
+        if (h == 1) return {5, {0x43210u, 0u}, {0x11111u, 0u}, {0x10000u, 0u}, 0x0u};
+        if (h == 2) return {8, {0x21543210u, 0u}, {0x22233113u, 0u}, {0x20010000u, 0u}, 0x10u};
+        if (h == 3) return {9, {0x15432160u, 0x2u}, {0x26775547u, 0x2u}, {0x04100000u, 0x2u}, 0x120u};
+        return {11, {0x54321670u, 0x216u}, {0xEFFDD48Fu, 0x228u}, {0x41000000u, 0x208u}, 0x1320u};
+    }
+    if (h == 4 && N <= PASS) return {4, {0x2130u, 0u}, {0xCE8Fu, 0u}, {0xC201u, 0u}, 0x3210u};
+    const unsigned int all = (1u << h) - 1u;
+    return {h, {0x3210u, 0u}, {0x8CEFu & all * 0x1111u, 0u}, {0x8421u, 0u}, 0x3210u};
+}
+// the bits set in a digit
+__host__ __device__ inline int quarter_count(int q) { return (q & 1) + (q >> 1 & 1) + (q >> 2 & 1) + (q >> 3); }
+
+template <int SUMS>
+__host__ __device__ inline int pass_stages(int N, int p, int kc) {
+    if (SUMS == kSumsShares) return shares_of(N, p).n;
+    const int n = (N + kc - 1) / kc, full = PASS / kc * (p + 1);
+    return full < n ? full : n;
+}
+// columns of entry c
+template <int SUMS>
+__host__ __device__ inline int stage_cols(int N, int p, int c, int kc) {
+    if (SUMS == kSumsShares) return QUART * quarter_count(shares_of(N, p).quarters[c]);
+    return pass_hi(N, p) - stage_lo(p, c, kc);
+}
+template <int SUMS>
+__host__ __device__ inline int stage_id(int N, int p, int c) {
+    return SUMS == kSumsShares ? shares_of(N, p).stage[c] : c;
+}
 // position of (pass p, stage 0) in the packed factor, in columns x points (only
 // the last pass is narrower, and nothing follows it)
 __host__ __device__ inline size_t pass_base(int p) { return (size_t)32768 * p * (p - 1) + (size_t)40960 * p; }
 
 // The passes a split of a GP takes: dealt back and forth, largest first; without a
-// split and with the batched rollout's sums (BSUM) in their order.
-template <bool BSUM>
+// split in their order.
 __host__ __device__ inline int split_pass(int np, int nsplit, int split, int i) {
-    if (BSUM && nsplit == 1) return i < np ? i : -1;
+    if (nsplit == 1) return i < np ? i : -1;
     return np - 1 - (i * nsplit + ((i & 1) ? nsplit - 1 - split : split));
 }
 
@@ -191,26 +237,28 @@ __device__ __forceinline__ void commit2_elect(uint64_t* bar) {
         : "memory");
 }
 
-// Two K-steps of the two-part split: A_hi B_hi into d, A_hi B_lo and
-// A_lo B_hi into d + LO_COL; the second K-step's operands sa and sb further on.
-// The first product of each set accumulates only if acc != 0.
-__device__ __forceinline__ void stage_split2(uint32_t d, uint64_t ah, uint64_t al, uint64_t bh, uint64_t bl,
-                                             uint64_t sa, uint64_t sb, uint32_t idesc, uint32_t acc) {
+// Two K-steps of the two-part split: A_hi B_hi into d, A_hi B_lo into d + hl and
+// A_lo B_hi into d + lh; the second K-step's operands sa and sb further on.  The first
+// product accumulates only if acc != 0, the second only if acc_hl != 0.
+__device__ __forceinline__ void stage_split2(uint32_t d, uint32_t hl, uint32_t lh, uint64_t ah, uint64_t al, uint64_t bh,
+                                             uint64_t bl, uint64_t sa, uint64_t sb, uint32_t idesc, uint32_t acc,
+                                             uint32_t acc_hl) {
     asm volatile(
-        "{\n\t.reg .pred e, p0, p1;\n\t"
-        ".reg .b32 dl;\n\t.reg .b64 ah1, al1, bh1, bl1;\n\t"
-        "add.u32 dl, %0, 256;\n\t"
+        "{\n\t.reg .pred e, p0, p1, p2;\n\t"
+        ".reg .b32 d2, d3;\n\t.reg .b64 ah1, al1, bh1, bl1;\n\t"
+        "add.u32 d2, %0, %9;\n\tadd.u32 d3, %0, %10;\n\t"
         "add.u64 ah1, %1, %5;\n\tadd.u64 al1, %2, %5;\n\tadd.u64 bh1, %3, %6;\n\tadd.u64 bl1, %4, %6;\n\t"
         "elect.sync _|e, 0xffffffff;\n\t"
         "setp.ne.b32 p0, %8, 0;\n\t"
+        "setp.ne.b32 p2, %11, 0;\n\t"
         "setp.ne.b32 p1, 1, 0;\n\t"
         "@e tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %3, %7, p0;\n\t"
-        "@e tcgen05.mma.cta_group::2.kind::f16 [dl], %1, %4, %7, p0;\n\t"
-        "@e tcgen05.mma.cta_group::2.kind::f16 [dl], %2, %3, %7, p1;\n\t"
+        "@e tcgen05.mma.cta_group::2.kind::f16 [d2], %1, %4, %7, p2;\n\t"
+        "@e tcgen05.mma.cta_group::2.kind::f16 [d3], %2, %3, %7, p1;\n\t"
         "@e tcgen05.mma.cta_group::2.kind::f16 [%0], ah1, bh1, %7, p1;\n\t"
-        "@e tcgen05.mma.cta_group::2.kind::f16 [dl], ah1, bl1, %7, p1;\n\t"
-        "@e tcgen05.mma.cta_group::2.kind::f16 [dl], al1, bh1, %7, p1;\n\t}" ::"r"(d),
-        "l"(ah), "l"(al), "l"(bh), "l"(bl), "l"(sa), "l"(sb), "r"(idesc), "r"(acc)
+        "@e tcgen05.mma.cta_group::2.kind::f16 [d2], ah1, bl1, %7, p1;\n\t"
+        "@e tcgen05.mma.cta_group::2.kind::f16 [d3], al1, bh1, %7, p1;\n\t}" ::"r"(d),
+        "l"(ah), "l"(al), "l"(bh), "l"(bl), "l"(sa), "l"(sb), "r"(idesc), "r"(acc), "r"(hl), "r"(lh), "r"(acc_hl)
         : "memory");
 }
 
@@ -234,15 +282,20 @@ __device__ __forceinline__ void step_split3(uint32_t d, uint64_t ah, uint64_t am
         : "memory");
 }
 
-// FMT: 0 = FP16 hi/lo, 1 = BF16 hi/lo, 2 = BF16 hi/mid/lo.  BSUM: the squares in the
-// order of the batched rollout (rollout_mma.cu), where the two halves of a pass's
-// columns are summed apart, 32 columns at a time in four chains, pass after pass.
-// The MMAs of a column are the same products in the same order there and here, so
-// that q is the same bits (what is cut off here are products with zero).  With a
-// split the 32-column sums go out, and the stage costs add them.  11.3 ms at
-// K = 16384, T = 100, N = 2048, FP16, as in the other order (4 % more with chains
-// packed across registers that are not loaded as pairs).
-template <int FMT, bool BSUM>
+// FMT: 0 = FP16 hi/lo, 1 = BF16 hi/lo, 2 = BF16 hi/mid/lo.  SUMS: which products share
+// a column set, the order of a column's MMAs and of the squares.
+//   kSumsTwo     hi.hi apart; the two halves of a pass's columns summed apart, 32
+//                columns at a time in four chains, pass after pass
+//   kSumsOne     all in one set; the halves of 512 columns, 64 at a time in four chains
+//   kSumsShares  hi.lo apart; 64 columns at a time in eight chains, the outermost of
+//                the slices first
+// The products of a column are the same in the same order as in the batched rollout
+// (kSumsShares: as in the cluster of CTAs that had the rollout), so that q is the same
+// bits; what is cut off here are products with zero.  With a split the sums of 32 or 64
+// columns go out, and k_var_parts adds them.  11.3 ms at K = 16384, T = 100, N =
+// 2048, FP16, as with the squares in any order (4 % more with chains packed across
+// registers that are not loaded as pairs).
+template <int FMT, int SUMS>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT, 1) k_var_tc(const GpSet gs, const VarTcJob job) {
     extern __shared__ __align__(1024) unsigned char tsm[];
     constexpr int PARTS = FMT == 2 ? 3 : 2;
@@ -335,8 +388,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT, 1) k_var_tc(cons
                 // the next tile's queries, in flight meanwhile
                 if (item + npairs < nitems) zn[r] = query(item + npairs, m0 + 32 * r);
             }
-            for (int i = 0, p; ok && (p = split_pass<BSUM>(np, job.nsplit, split, i)) >= 0; ++i) {
-                const int ns = pass_stages(G.N, p, KC);
+            for (int i = 0, p; ok && (p = split_pass(np, job.nsplit, split, i)) >= 0; ++i) {
+                const int ns = pass_stages<SUMS>(G.N, p, KC);
                 for (int c = 0; c < ns; ++c) {
                     if ((n & 1u) != turn) {
                         advance();
@@ -403,24 +456,44 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT, 1) k_var_tc(cons
             const GpSet::One& G = gs.gp[ts / job.nsplit];
             const int split = ts % job.nsplit, np = pass_count(G.N);
             const int q = tile * (2 * QM) + (int)rank * QM + 32 * e + lane;
-            float sum = 0.0f, half2 = 0.0f;
-            for (int i = 0, p; ok && (p = split_pass<BSUM>(np, job.nsplit, split, i)) >= 0; ++i) {
+            float sum = 0.0f, half2 = 0.0f, slice[SUMS == kSumsShares ? 8 : 1] = {};
+            for (int i = 0, p; ok && (p = split_pass(np, job.nsplit, split, i)) >= 0; ++i) {
                 const int nq = pass_hi(G.N, p) / QUART;
-                for (int j = 0; j < nq; ++j) {
+                // of the 128-column blocks of a pass of 256 (kSumsOne: 512) columns, those
+                // whose halves are summed apart: the first half ends after so many quarters
+                int edge = job.even ? 2 : (nq + 1) / 2;
+                if (SUMS == kSumsOne) {
+                    const int left = (G.N - 2 * PASS * (p / 2) + QUART - 1) / QUART;      // quarters of the 512
+                    edge = left >= 8 ? 4 : job.even ? 2 * ((left + 3) / 4) : (left + 1) / 2;
+                    edge -= 4 * (p & 1);
+                }
+                unsigned int order = 0x3210u;
+                if constexpr (SUMS == kSumsShares) order = shares_of(G.N, p).order;
+                for (int jj = 0; jj < nq; ++jj) {
+                    const int j = (int)(order >> 4 * jj & 15u);
                     ok = __all_sync(0xffffffffu, wait(q_done + j, (qph >> j) & 1u));
                     if (!ok) break;
                     qph ^= 1u << j;
                     tc::fence_after_sync();
-                    if constexpr (BSUM) {
-                        const bool second = j >= (job.even ? 2 : (nq + 1) / 2);
+                    const uint32_t col0 = row + (uint32_t)(QUART * j);
+                    float* part = job.q + ((size_t)(ts / job.nsplit) * job.nparts) * job.Q + q;    // with a split
+                    auto add = [&](float g, int at) {
+                        if (job.nparts > 1) {
+                            if (q < job.Q) part[(size_t)at * job.Q] = g;
+                        } else if (j >= edge) {
+                            half2 += g;
+                        } else {
+                            sum += g;
+                        }
+                    };
+                    if constexpr (SUMS == kSumsTwo) {
 #pragma unroll
                         for (int cc = 0; cc < QUART; cc += 32) {
                             float g[4];
 #pragma unroll
                             for (int h = 0; h < 2; ++h) {
                                 float v[16], w[16];
-                                const uint32_t col = row + (uint32_t)(QUART * j + cc + 16 * h);
-                                tc::tmem_ld16x2(col, col + LO_COL, v, w);
+                                tc::tmem_ld16x2(col0 + cc + 16 * h, col0 + cc + 16 * h + LO_COL, v, w);
                                 // pairs of neighbouring columns (a register pair as loaded)
                                 // are added, each chain's squares one by one
                                 float x[16], s0 = 0.0f, s1 = 0.0f;
@@ -435,35 +508,45 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT, 1) k_var_tc(cons
                                 g[2 * h] = s0;
                                 g[2 * h + 1] = s1;
                             }
-                            const float s32 = (g[0] + g[1]) + (g[2] + g[3]);
-                            if (job.nparts > 1) {
-                                if (q < job.Q)
-                                    job.q[((size_t)(ts / job.nsplit) * job.nparts + 8 * p + 2 * j + cc / 32) * job.Q + q] = s32;
-                            } else if (second) {
-                                half2 += s32;
-                            } else {
-                                sum += s32;
+                            add((g[0] + g[1]) + (g[2] + g[3]), 8 * p + 2 * j + cc / 32);
+                        }
+                    } else if constexpr (SUMS == kSumsOne) {
+                        float g[4];
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            float v[16], w[16], s0 = 0.0f, s1 = 0.0f;
+                            tc::tmem_ld16x2(col0 + 32 * h, col0 + 32 * h + 16, v, w);
+#pragma unroll
+                            for (int k = 0; k < 16; ++k) {
+                                s0 = fmaf(v[k], v[k], s0);
+                                s1 = fmaf(w[k], w[k], s1);
+                            }
+                            g[2 * h] = s0;
+                            g[2 * h + 1] = s1;
+                        }
+                        add((g[0] + g[1]) + (g[2] + g[3]), 4 * p + j);
+                    } else {
+                        uint64_t s[4] = {0ull, 0ull, 0ull, 0ull};
+#pragma unroll
+                        for (int cc = 0; cc < QUART; cc += 16) {
+                            float v[16], w[16];
+                            tc::tmem_ld16x2(col0 + cc, col0 + cc + LO_COL, v, w);
+#pragma unroll
+                            for (int k = 0; k < 16; k += 2) {
+                                const uint64_t x = tc::f2add(tc::f2pack(v[k], v[k + 1]), tc::f2pack(w[k], w[k + 1]));
+                                s[k / 2 % 4] = tc::f2fma(x, x, s[k / 2 % 4]);
                             }
                         }
-                        continue;
-                    }
+                        float g[8];
 #pragma unroll
-                    for (int cc = 0; cc < QUART; cc += 16) {
-                        float v[16], w[16];
-                        const uint32_t col = row + (uint32_t)(QUART * j + cc);
-                        tc::tmem_ld16x2(col, col + LO_COL, v, w);
-                        uint64_t s0 = 0ull, s1 = 0ull;
+                        for (int k = 0; k < 4; ++k) tc::f2unpack(s[k], g[2 * k], g[2 * k + 1]);
+                        const float g64 = ((g[0] + g[1]) + (g[2] + g[3])) + ((g[4] + g[5]) + (g[6] + g[7]));
+                        if (job.nparts > 1) {
+                            add(g64, 4 * p + j);
+                        } else {
 #pragma unroll
-                        for (int k = 0; k < 16; k += 4) {
-                            const uint64_t x0 = tc::f2add(tc::f2pack(v[k], v[k + 1]), tc::f2pack(w[k], w[k + 1]));
-                            const uint64_t x1 = tc::f2add(tc::f2pack(v[k + 2], v[k + 3]), tc::f2pack(w[k + 2], w[k + 3]));
-                            s0 = tc::f2fma(x0, x0, s0);
-                            s1 = tc::f2fma(x1, x1, s1);
+                            for (int k = 0; k < 8; ++k) slice[k] = k == 4 * p + j ? g64 : slice[k];
                         }
-                        float a0, a1, b0, b1;
-                        tc::f2unpack(s0, a0, a1);
-                        tc::f2unpack(s1, b0, b1);
-                        sum += (a0 + a1) + (b0 + b1);
                     }
                 }
                 if (!ok) break;
@@ -471,8 +554,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT, 1) k_var_tc(cons
                 __syncwarp();
                 if (lane == 0) arrive_cluster(t_free0);
             }
-            if (BSUM && job.nparts > 1) continue;
-            if (ok && q < job.Q) job.q[(size_t)ts * job.Q + q] = BSUM ? sum + half2 : sum;
+            if (!ok || job.nparts > 1 || q >= job.Q) continue;
+            if constexpr (SUMS == kSumsShares) {
+                const int last = G.N <= 128 ? 1 : G.N <= 256 ? 3 : 7;
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    if (2 * r >= last) break;
+                    sum += slice[r];
+                    sum += last == 1 ? slice[1 - r] : last == 3 ? slice[3 - r > 0 ? 3 - r : 0] : slice[7 - r];
+                }
+            }
+            job.q[(size_t)ts * job.Q + q] = sum + half2;
         }
     } else if (warp == MMA_WARP && rank == 0) {
         // ---------------- MMA issuer -----------------------------------------------
@@ -484,8 +576,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT, 1) k_var_tc(cons
             const int ts = item / ntiles;
             const int N = gs.gp[ts / job.nsplit].N;
             const int split = ts % job.nsplit, np = pass_count(N);
-            for (int i = 0, p; ok && (p = split_pass<BSUM>(np, job.nsplit, split, i)) >= 0; ++i, ++passes) {
-                const int ns = pass_stages(N, p, KC), hi = pass_hi(N, p);
+            for (int i = 0, p; ok && (p = split_pass(np, job.nsplit, split, i)) >= 0; ++i, ++passes) {
+                const int ns = pass_stages<SUMS>(N, p, KC), hi = pass_hi(N, p);
+                Shares sh = {};
+                if constexpr (SUMS == kSumsShares) sh = shares_of(N, p);
                 if (passes > 0) {
                     // both CTAs have read the last pass
                     if (!(ok = __all_sync(0xffffffffu, wait(t_free, (passes - 1) & 1u)))) break;
@@ -496,29 +590,53 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT, 1) k_var_tc(cons
                     go = go && wait(a_full + sa, pa);
                     if (!(ok = __all_sync(0xffffffffu, go))) break;
                     tc::fence_after_sync();
-                    const int lo = stage_lo(p, c, KC), cols = hi - lo, h = cols / 2;
                     const uint64_t ah = dA0 + (uint64_t)((sa * L::a_stage) >> 4);
-                    const uint64_t bh = tc::smem_desc(tc::smem_addr(tsm) + (uint32_t)(L::b + sb * L::b_stage), (uint32_t)h * 16u, 128);
-                    const uint64_t bstep = (uint64_t)(KC * h * 2 / 16);  // one part of the piece
-                    const uint32_t idesc = idesc0 | ((uint32_t)(cols >> 3) << 17);
-                    const uint64_t a1 = (uint64_t)(L::a_part >> 4);
-                    const uint64_t ka = (uint64_t)((2 * QM * 16) >> 4), kb = (uint64_t)(2 * h);
-                    if constexpr (PARTS == 2) {
+                    const uint64_t a1 = (uint64_t)(L::a_part >> 4), ka = (uint64_t)((2 * QM * 16) >> 4);
+                    // the entry's columns, in one run of quarters or (kSumsShares) two
+                    int lo = stage_lo(p, c, KC), cols = hi - lo, left = 0;
+                    if constexpr (SUMS == kSumsShares) {
+                        left = sh.quarters[c];
+                        lo = QUART * (__ffs(left) - 1);
+                        cols = QUART * (__ffs(~(left >> lo / QUART)) - 1);
+                        left &= -1 << (lo + cols) / QUART;
+                    }
+                    uint32_t bs = (uint32_t)(L::b + sb * L::b_stage);
+                    while (true) {
+                        const int h = cols / 2;
+                        const uint64_t bh = tc::smem_desc(tc::smem_addr(tsm) + bs, (uint32_t)h * 16u, 128);
+                        const uint64_t bstep = (uint64_t)(KC * h * 2 / 16);  // one part of the piece
+                        const uint64_t kb = (uint64_t)(2 * h);
+                        const uint32_t idesc = idesc0 | ((uint32_t)(cols >> 3) << 17);
+                        if constexpr (PARTS == 2) {
+                            constexpr uint32_t HL = SUMS == kSumsOne ? 0u : LO_COL, LH = SUMS == kSumsTwo ? LO_COL : 0u;
 #pragma unroll
-                        for (int j = 0; j < KC / 16; j += 2)
-                            stage_split2(taddr + (uint32_t)lo, ah + j * ka, ah + a1 + j * ka, bh + j * kb, bh + bstep + j * kb,
-                                         ka, kb, idesc, c + j > 0 ? 1u : 0u);
-                    } else {
+                            for (int j = 0; j < KC / 16; j += 2)
+                                stage_split2(taddr + (uint32_t)lo, HL, LH, ah + j * ka, ah + a1 + j * ka, bh + j * kb,
+                                             bh + bstep + j * kb, ka, kb, idesc, c + j > 0 ? 1u : 0u,
+                                             SUMS == kSumsOne || c + j > 0 ? 1u : 0u);
+                        } else {
 #pragma unroll
-                        for (int j = 0; j < KC / 16; ++j)
-                            step_split3(taddr + (uint32_t)lo, ah + j * ka, ah + a1 + j * ka, ah + 2 * a1 + j * ka,
-                                        bh + j * kb, bh + bstep + j * kb, bh + 2 * bstep + j * kb, idesc,
-                                        c + j > 0 ? 1u : 0u);
+                            for (int j = 0; j < KC / 16; ++j)
+                                step_split3(taddr + (uint32_t)lo, ah + j * ka, ah + a1 + j * ka, ah + 2 * a1 + j * ka,
+                                            bh + j * kb, bh + bstep + j * kb, bh + 2 * bstep + j * kb, idesc,
+                                            c + j > 0 ? 1u : 0u);
+                        }
+                        if (SUMS != kSumsShares || left == 0) break;
+                        bs += (uint32_t)(KC * PARTS * cols);      // this CTA's half of the first run
+                        lo = QUART * (__ffs(left) - 1);
+                        cols = QUART * (__ffs(~(left >> lo / QUART)) - 1);
+                        left = 0;
                     }
                     commit2_elect(done + sb);
-                    // columns 64 j .. 64 j + 63 are complete after their diagonal's last stage
-                    const int d = KC * c - PASS * p;
-                    if (d >= 0 && ((d + KC) % QUART == 0 || c == ns - 1)) commit2_elect(q_done + d / QUART);
+                    // quarters are complete after their last entry
+                    if constexpr (SUMS == kSumsShares) {
+                        const int over = sh.done[c];
+                        for (int j = 0; j < 4; ++j)
+                            if (over >> j & 1) commit2_elect(q_done + j);
+                    } else {
+                        const int d = KC * c - PASS * p;
+                        if (d >= 0 && ((d + KC) % QUART == 0 || c == ns - 1)) commit2_elect(q_done + d / QUART);
+                    }
                     advance();
                 }
             }
@@ -538,8 +656,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT, 1) k_var_tc(cons
                 const int ts = item / ntiles;
                 const int N = gs.gp[ts / job.nsplit].N;
                 const int split = ts % job.nsplit, np = pass_count(N);
-                for (int i = 0, p; ok && (p = split_pass<BSUM>(np, job.nsplit, split, i)) >= 0; ++i) {
-                    const int ns = pass_stages(N, p, KC);
+                for (int i = 0, p; ok && (p = split_pass(np, job.nsplit, split, i)) >= 0; ++i) {
+                    const int ns = pass_stages<SUMS>(N, p, KC);
                     for (int c = 0; c < ns; ++c) {
                         if (!(ok = wait(b_full + sb, pb))) break;
                         arrive_cluster(peer0 + 8u * (uint32_t)sb);
@@ -556,8 +674,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT, 1) k_var_tc(cons
                 const int ts = item / ntiles;
                 const int N = gs.gp[ts / job.nsplit].N;
                 const int split = ts % job.nsplit, np = pass_count(N);
-                for (int i = 0, p; ok && (p = split_pass<BSUM>(np, job.nsplit, split, i)) >= 0; ++i) {
-                    const int ns = pass_stages(N, p, KC);
+                for (int i = 0, p; ok && (p = split_pass(np, job.nsplit, split, i)) >= 0; ++i) {
+                    const int ns = pass_stages<SUMS>(N, p, KC);
                     for (int c = 0; c < ns; ++c) {
                         if (!(ok = wait(a_raw + sa, pa))) break;
                         tc::fence_proxy_async();
@@ -572,7 +690,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT, 1) k_var_tc(cons
         // The points of a stage are fetched up to XR stages ahead: their slot is
         // free once the MMAs XR stages earlier are done.
         int xi = pair, xpi = 0;                             // item and number of its next pass
-        int xc = 0, xns = 0;                                // stage and stages of the pass being fetched
+        int xc = 0, xns = 0, xp = 0, xN = 0;                // entry and entries of the pass being fetched, its pass and GP
         const float* xsrc = nullptr;
         uint32_t xn = 0;
         auto next_x_pass = [&]() {
@@ -580,10 +698,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT, 1) k_var_tc(cons
             while (xi < nitems && xns == 0) {
                 const int ts = xi / ntiles;
                 const GpSet::One& G = gs.gp[ts / job.nsplit];
-                const int p = split_pass<BSUM>(pass_count(G.N), job.nsplit, ts % job.nsplit, xpi);
+                const int p = split_pass(pass_count(G.N), job.nsplit, ts % job.nsplit, xpi);
                 if (p >= 0) {
-                    xns = pass_stages(G.N, p, KC);
+                    xns = pass_stages<SUMS>(G.N, p, KC);
                     xsrc = G.xq;
+                    xp = p;
+                    xN = G.N;
                     ++xpi;
                 } else {
                     xpi = 0;
@@ -595,7 +715,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT, 1) k_var_tc(cons
             if (xns == 0) return;
             uint64_t* bar = x_full + xn % XR;
             tc::mbar_expect_tx(bar, KC * 16);
-            bulk_g2s(tsm + L::x + (xn % XR) * (KC * 16), xsrc + (size_t)xc * (KC * 4), KC * 16, bar);
+            bulk_g2s(tsm + L::x + (xn % XR) * (KC * 16), xsrc + (size_t)stage_id<SUMS>(xN, xp, xc) * (KC * 4), KC * 16, bar);
             ++xn;
             if (++xc == xns) next_x_pass();
         };
@@ -605,16 +725,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT, 1) k_var_tc(cons
             const int ts = item / ntiles;
             const GpSet::One& G = gs.gp[ts / job.nsplit];
             const int split = ts % job.nsplit, np = pass_count(G.N);
-            for (int i = 0, p; ok && (p = split_pass<BSUM>(np, job.nsplit, split, i)) >= 0; ++i) {
-                const int ns = pass_stages(G.N, p, KC), hi = pass_hi(G.N, p);
+            for (int i = 0, p; ok && (p = split_pass(np, job.nsplit, split, i)) >= 0; ++i) {
+                const int ns = pass_stages<SUMS>(G.N, p, KC);
                 const unsigned char* src = reinterpret_cast<const unsigned char*>(G.Bt) + pass_base(p) * (2 * PARTS);
                 for (int c = 0; c < ns; ++c) {
                     if (n >= (uint32_t)NBP) {
                         if (!(ok = wait(done + sb, pb ^ 1u))) break;
                         fetch_x();
                     }
-                    const int cols = hi - stage_lo(p, c, KC);
-                    const uint32_t bytes = (uint32_t)(KC * PARTS * cols);      // this CTA's half of the columns
+                    // this CTA's half of the columns
+                    const uint32_t bytes = (uint32_t)(KC * PARTS * stage_cols<SUMS>(G.N, p, c, KC));
                     tc::mbar_expect_tx(b_full + sb, bytes);
                     bulk_g2s(tsm + L::b + sb * L::b_stage, src + rank * bytes, bytes, b_full + sb);
                     src += 2 * bytes;
@@ -641,22 +761,82 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NT, 1) k_var_tc(cons
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;" ::"r"(taddr) : "memory");
 }
 
-// cB L^-1 in the pieces of the passes: (pass, stage) holds, for each CTA of the
-// pair, its half of the stage's columns: the parts (hi, lo or hi, mid, lo) one
-// after the other, each as slabs of 8 points x (columns / 2) rows.
+// |V_m|^2 of a query from its parts (stride Q): a part for every 32 columns (kSumsTwo)
+// or 64, added in the order of one CTA pair.
+__device__ float parts_sum(int sums, int even, const float* qp, size_t Q, int N) {
+    float h0 = 0.0f, h1 = 0.0f;
+    const int ns = (N + 63) / 64;
+    if (sums == kSumsShares) {
+        const int last = N <= 128 ? 1 : N <= 256 ? 3 : 7;
+        for (int r = 0; 2 * r < last; ++r) {
+            if (r < ns) h0 += qp[(size_t)r * Q];
+            if (last - r < ns) h0 += qp[(size_t)(last - r) * Q];
+        }
+        return h0;
+    }
+    // eight parts at a time: a pass of 256 columns in 32s or of 512 in 64s, its halves
+    // (of the 128-column blocks that it has) apart
+    const bool two = sums == kSumsTwo;
+    for (int n = two ? 2 * ns : ns; n > 0; n -= 8, qp += 8 * Q) {
+        int h = 4;
+        if (two) h = even || n >= 8 ? 4 : (n + 2) / 4 * 2;
+        else if (n < 8) h = even ? 2 * ((n + 3) / 4) : (n + 1) / 2;
+        float g[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) g[j] = j < n ? qp[j * Q] : 0.0f;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            if (j < n && j < h) h0 += g[j];
+            if (j < n && j >= h) h1 += g[j];
+        }
+    }
+    return h0 + h1;
+}
+
+// after a split: the first part of every query and GP becomes its sum.  A launch of its
+// own: in the stage costs' loads the parts' loop cost 15 to 70 us.
+__global__ void __launch_bounds__(256) k_var_parts(const GpSet gs, const VarTcJob job) {
+    grid_wait();
+    const int q = blockIdx.x * 256 + threadIdx.x;
+    if (q >= job.Q) return;
+    float* p = job.q + (size_t)blockIdx.y * job.nparts * job.Q + q;
+    *p = parts_sum(job.sums, job.even, p, (size_t)job.Q, gs.gp[blockIdx.y].N);
+}
+
+// cB L^-1 in the pieces of the passes: (pass, entry) holds, for each CTA of the
+// pair, its half of every run of the entry's columns, a run's parts (hi, lo or hi, mid,
+// lo) one after the other, each as slabs of 8 points x (columns / 2) rows.
+template <int SUMS>
 __global__ void k_pack_tc(const double* __restrict__ Xm, int N, int fmt, double cB, uint16_t* __restrict__ out) {
     const int parts = fmt == 2 ? 3 : 2, kc = stage_points(parts);
     const int p = blockIdx.y, c = blockIdx.x;
-    if (c >= pass_stages(N, p, kc)) return;
-    const int hi = pass_hi(N, p), lo = stage_lo(p, c, kc), cols = hi - lo, h = cols / 2;
+    if (c >= pass_stages<SUMS>(N, p, kc)) return;
+    const int cols = stage_cols<SUMS>(N, p, c, kc), st = stage_id<SUMS>(N, p, c);
+    // the runs of quarters: start and columns of the first, start of the second
+    int lo = stage_lo(p, c, kc), n0 = cols, lo1 = 0;
+    if (SUMS == kSumsShares) {
+        const int q = shares_of(N, p).quarters[c];
+        lo = QUART * (__ffs(q) - 1);
+        n0 = QUART * (__ffs(~(q >> lo / QUART)) - 1);
+        const int rest = q & (-1 << (lo + n0) / QUART);
+        lo1 = rest ? QUART * (__ffs(rest) - 1) : 0;
+    }
     size_t off = pass_base(p);
-    for (int i = 0; i < c; ++i) off += (size_t)(hi - stage_lo(p, i, kc)) * kc;
-    uint16_t* dst = out + off * parts;
+    for (int i = 0; i < c; ++i) off += (size_t)stage_cols<SUMS>(N, p, i, kc) * kc;
     for (int idx = threadIdx.x; idx < cols * kc; idx += blockDim.x) {
-        const int e = idx % 8, row = (idx / 8) % h, sl = (idx / (8 * h)) % (kc / 8), r = idx / (kc * h);
-        const int i = PASS * p + lo + r * h + row, j = kc * c + 8 * sl + e;
+        const int r = idx / (kc * cols / 2);
+        int in = idx % (kc * cols / 2);
+        uint16_t* dst = out + off * parts + (size_t)r * (parts * kc * cols / 2);
+        const bool second = in >= kc * n0 / 2;
+        if (second) {
+            in -= kc * n0 / 2;
+            dst += parts * kc * n0 / 2;
+        }
+        const int h = (second ? cols - n0 : n0) / 2;
+        const int e = in % 8, row = (in / 8) % h, sl = in / (8 * h);
+        const int i = PASS * p + (second ? lo1 : lo) + r * h + row, j = kc * st + 8 * sl + e;
         const double v = (i < N && j <= i) ? cB * Xm[(size_t)i * N + j] : 0.0;
-        uint16_t* o = dst + r * (parts * h * kc) + sl * (h * 8) + row * 8 + e;
+        uint16_t* o = dst + sl * (h * 8) + row * 8 + e;
         if (fmt == 0) {
             const __half a = __double2half(v);
             o[0] = __half_as_ushort(a);
@@ -674,24 +854,28 @@ __global__ void k_pack_tc(const double* __restrict__ Xm, int N, int fmt, double 
 
 }  // namespace
 
-int build_tc_pieces(GpDevice& g, int fmt) {
-    if (g.Bt[fmt] || g.N == 0) return GPMPPI_OK;
+int build_tc_pieces(GpDevice& g, int fmt, bool shares) {
+    uint16_t*& made = shares ? g.Bs[fmt] : g.Bt[fmt];
+    if (made || g.N == 0) return GPMPPI_OK;
     const int rc = set_cB(g);
     if (rc) return rc;
     const int N = g.N, np = pass_count(N), p = np - 1;
     const int parts = fmt == 2 ? 3 : 2, kc = stage_points(parts);
-    size_t n = pass_base(p);                     // columns x points
-    for (int c = 0; c < pass_stages(N, p, kc); ++c) n += (size_t)(pass_hi(N, p) - stage_lo(p, c, kc)) * kc;
+    // columns x points: the same for either order
+    size_t n = pass_base(p);
+    for (int c = 0; c < pass_stages<kSumsTwo>(N, p, kc); ++c) n += (size_t)stage_cols<kSumsTwo>(N, p, c, kc) * kc;
     uint16_t* Bt = nullptr;
     GPM_CUDA(cudaMalloc(&Bt, n * (size_t)(2 * parts)));
-    k_pack_tc<<<dim3((unsigned)(PASS / kc * np), (unsigned)np), 256>>>(g.Linv64[0], N, fmt, (double)g.cB, Bt);
+    const dim3 grid((unsigned)(shares ? 11 : PASS / kc * np), (unsigned)np);
+    auto kern = shares ? k_pack_tc<kSumsShares> : k_pack_tc<kSumsTwo>;
+    kern<<<grid, 256>>>(g.Linv64[0], N, fmt, (double)g.cB, Bt);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
         cudaFree(Bt);
         return cuda_fail(e, "tensor-core factor pieces");
     }
-    g.Bt[fmt] = Bt;
+    made = Bt;
     return GPMPPI_OK;
 }
 
@@ -709,7 +893,7 @@ int var_tc_splits(const GpSet& gs, int Q, int nsm) {
             const int np = pass_count(gs.gp[t].N);
             for (int j = 0; j < s; ++j) {
                 int w = 0;
-                for (int i = 0, p; (p = split_pass<false>(np, s, j, i)) >= 0; ++i) w += 8 * p + 6;
+                for (int i = 0, p; (p = split_pass(np, s, j, i)) >= 0; ++i) w += 8 * p + 6;
                 longest = w > longest ? w : longest;
             }
         }
@@ -726,12 +910,15 @@ int launch_var_tc(const GpSet& gs, const VarTcJob& j, int fmt, int nsm, bool dep
     if (j.Q <= 0) return GPMPPI_OK;
     const long long items = (long long)((j.Q + 2 * QM - 1) / (2 * QM)) * gs.M * j.nsplit;
     const int pairs = (int)(items < nsm / 2 ? items : nsm / 2);
-    auto kern = fmt == 2   ? k_var_tc<2, true>
-                : j.rps > 0 ? (fmt == 0 ? k_var_tc<0, true> : k_var_tc<1, true>)
-                            : (fmt == 0 ? k_var_tc<0, false> : k_var_tc<1, false>);
+    auto kern = fmt == 2               ? k_var_tc<2, kSumsTwo>
+                : j.sums == kSumsTwo ? (fmt == 0 ? k_var_tc<0, kSumsTwo> : k_var_tc<1, kSumsTwo>)
+                : j.sums == kSumsOne ? (fmt == 0 ? k_var_tc<0, kSumsOne> : k_var_tc<1, kSumsOne>)
+                                     : (fmt == 0 ? k_var_tc<0, kSumsShares> : k_var_tc<1, kSumsShares>);
     const int smem = fmt == 2 ? TcLayout<3>::total : TcLayout<2>::total;
     GPM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     GPM_CUDA(launch_ex(kern, dim3((unsigned)(2 * pairs)), NT, smem, st, dependent, gs, j));
+    if (j.nparts > 1)
+        GPM_CUDA(launch_ex(k_var_parts, dim3((unsigned)((j.Q + 255) / 256), (unsigned)gs.M), 256, 0, st, true, gs, j));
     return GPMPPI_OK;
 }
 
