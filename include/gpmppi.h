@@ -209,7 +209,8 @@ int mppi_nominal_sxy(gpmppi_ctrl c, float* sxy, void* stream);
  * (on the tensor cores, two-part formats with 0 < N <= 512),
  * GPMPPI_KERNEL_TC_STREAM (on the tensor cores, everything else in the split
  * precisions, terrain ensembles included) or GPMPPI_KERNEL_ENSEMBLE (FP32
- * terrain ensemble).  The two tensor-core classes run the same kernels. */
+ * terrain ensemble).  The two tensor-core classes run the same kernels with the
+ * sums in another order. */
 #define GPMPPI_KERNEL_FP32 0
 #define GPMPPI_KERNEL_TC_STREAM 1
 #define GPMPPI_KERNEL_TC_CLUSTER 2

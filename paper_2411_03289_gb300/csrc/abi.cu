@@ -343,7 +343,7 @@ int alloc_query_ws(gpmppi_ctrl c) {
     // of the records and the rows anew (the results are the same).
     size_t npad = 0, rows = 0;
     for (size_t t = 0; t < M; ++t) npad = npad < (size_t)c->gset.gp[t].npad ? (size_t)c->gset.gp[t].npad : npad;
-    const size_t least = c->p.variance_mode == GPMPPI_VAR_NOMINAL ? 4 * T : 0;      // 2 T N doubles
+    const size_t least = c->p.variance_mode == GPMPPI_VAR_NOMINAL ? (T + kTriTile - 1) / kTriTile * kTriTile : 0;
     for (;; n = (n / 2 + 31) / 32 * 32) {
         cudaFree(c->ws_buf);
         cudaFree(c->vbuf);
@@ -426,7 +426,11 @@ int launch_nominal(gpmppi_ctrl c, const RolloutArgs& a, cudaStream_t st) {
     ws.sums = ws.rps = ws.even = 0;
     int rc;
     if ((rc = launch_nominal_mean(a, ws, st))) return rc;
-    if ((rc = launch_nominal_var(c->gp->g, a.T, ws, reinterpret_cast<double*>(c->vbuf), st))) return rc;
+    const GpSet::One& G = c->gset.gp[0];
+    TriJob j = tri_forward(G, reinterpret_cast<const float*>(ws.zq), a.T, c->vbuf);
+    j.err = a.err;
+    if ((rc = launch_tri_forward(j, false, st))) return rc;
+    if ((rc = launch_block_variance(c->vbuf, G.npad, a.T, G.N, G.sf2, ws.q, st))) return rc;
     return launch_nominal_cov(a, ws, c->nom_sxy, st);
 }
 

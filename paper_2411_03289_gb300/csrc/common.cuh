@@ -116,7 +116,6 @@ struct GpDevice {
     // FP64 factors kept for export: Linv64[o] N x N, alpha64[o] N
     double* Linv64[2] = {nullptr, nullptr};
     double* alpha64[2] = {nullptr, nullptr};
-    double* X64 = nullptr;       // N x 4 training inputs
     // tensor-core tiles of L^-T per operand format for the batched rollout (0 =
     // FP16 hi/lo, 1 = BF16 hi/lo, 2 = BF16 hi/mid/lo), built with a batch; NpM = N
     // rounded up to 128
@@ -382,6 +381,8 @@ TriJob tri_forward(const GpSet::One& G, const float* z, int Q, float* V);
 int launch_tri_forward(const TriJob& j, bool dependent, cudaStream_t st);
 int launch_tri_backward(const TriJob& j, bool dependent, cudaStream_t st);
 int launch_rowsum(const float* V, int ld, int Q, int N, SumOrder order, float* out, cudaStream_t st);
+// max(0, sf2 - |v_q|^2), the squares as 256 threads of a CTA would sum them
+int launch_block_variance(const float* V, int ld, int Q, int N, float sf2, float* out, cudaStream_t st);
 int build_back_pieces(GpDevice& g, cudaStream_t st);
 // the chain with compensated terms (chain_fp32.cu): its sums in lane order, or by
 // the shuffle tree with the GPs mixed by their weights (terrain ensembles; the
@@ -432,8 +433,6 @@ int build_mma_ensemble(GpDevice* const* gs, int M, int fmt, MmaTerrains& tr, uin
 int launch_philox(uint64_t seed, const uint32_t* ctr, int M, uint32_t* out, cudaStream_t st);
 int launch_noise(uint64_t seed, int K, int T, uint64_t it, float sv, float sw, float* eps,
                  cudaStream_t st);
-// variances of the T queries ws.zq in FP64 into ws.q; scratch: 2 T N doubles
-int launch_nominal_var(const GpDevice& g, int T, const QueryWs& ws, double* scratch, cudaStream_t st);
 int launch_nominal_cov(const RolloutArgs& a, const QueryWs& ws, float* sxy_out, cudaStream_t st);
 int launch_mma_selftest(int fmt, int N, int K, int variant, const uint16_t* A, const uint16_t* B,
                         float* D, unsigned int* err, cudaStream_t st);

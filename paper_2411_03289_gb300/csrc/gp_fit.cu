@@ -502,7 +502,6 @@ int gp_fit_device(GpDevice& g, const double* X, const double* Y, int N, cudaStre
     const size_t n1 = N > 0 ? (size_t)N : 1;
     const size_t o_alpha = take(sizeof(float) * 2 * n1);
     const size_t o_a64[2] = {take(sizeof(double) * n1), take(sizeof(double) * n1)};
-    const size_t o_x64 = take(sizeof(double) * 4 * n1);
     size_t o_xs[2], o_l[2], o_xq[2], o_wb[2];
     for (int o = 0; o < nout; ++o) {
         o_xs[o] = take(sizeof(float) * 4 * n1);
@@ -513,7 +512,6 @@ int gp_fit_device(GpDevice& g, const double* X, const double* Y, int N, cudaStre
     GPM_CUDA(cudaMalloc(&g.mem, off));
     char* mem = static_cast<char*>(g.mem);
     g.alpha = reinterpret_cast<float*>(mem + o_alpha);
-    g.X64 = reinterpret_cast<double*>(mem + o_x64);
     for (int o = 0; o < 2; ++o) {
         const int s = o < nout ? o : 0;              // shared hyper-parameters: one factor
         g.alpha64[o] = reinterpret_cast<double*>(mem + o_a64[o]);
@@ -524,7 +522,7 @@ int gp_fit_device(GpDevice& g, const double* X, const double* Y, int N, cudaStre
     }
     if (N == 0) return GPMPPI_OK;
 
-    // one scratch allocation: y, t, alpha's parts, the panel, a diagonal block, the flag
+    // one scratch allocation: x, y, t, alpha's parts, the panel, a diagonal block, the flag
     const size_t n_y = 2 * (size_t)N, n_part = 2 * (size_t)kAlphaParts * N, n_p = (size_t)NB * N;
     double* scratch = nullptr;
     auto cleanup = [&]() { cudaFree(scratch); };
@@ -536,9 +534,9 @@ int gp_fit_device(GpDevice& g, const double* X, const double* Y, int N, cudaStre
         return GPMPPI_OK;
     };
     int rc;
-    if ((rc = check(cudaMalloc(&scratch, sizeof(double) * (2 * n_y + n_part + n_p + NB * NB + 1)), "cudaMalloc scratch")))
+    if ((rc = check(cudaMalloc(&scratch, sizeof(double) * (4 * n_y + n_part + n_p + NB * NB + 1)), "cudaMalloc scratch")))
         return rc;
-    double *dX = g.X64, *dY = scratch, *dt = dY + n_y, *dpart = dt + n_y, *dP = dpart + n_part, *dD = dP + n_p;
+    double *dX = scratch, *dY = dX + 2 * n_y, *dt = dY + n_y, *dpart = dt + n_y, *dP = dpart + n_part, *dD = dP + n_p;
     int* dflag = reinterpret_cast<int*>(dD + NB * NB);
     if ((rc = check(cudaMemcpyAsync(dX, X, sizeof(double) * 4 * N, cudaMemcpyHostToDevice, st),
                     "copy X")))

@@ -226,7 +226,9 @@ __global__ void __launch_bounds__(NOM_THREADS) k_nominal_mean(const RolloutArgs 
     for (int k = 0; k < a.T; ++k) {
         const float ux = fminf(fmaxf(Uc[2 * k], a.umin0), a.umax0);
         const float uy = fminf(fmaxf(Uc[2 * k + 1], a.umin1), a.umax1);
-        const float z0 = mu[3] * a.zscale[0], z1 = mu[4] * a.zscale[1], z2 = ux * a.zscale[2], z3 = uy * a.zscale[3];
+        // (rounded before the difference, as in the products for the variances)
+        const float z0 = __fmul_rn(mu[3], a.zscale[0]), z1 = __fmul_rn(mu[4], a.zscale[1]);
+        const float z2 = __fmul_rn(ux, a.zscale[2]), z3 = __fmul_rn(uy, a.zscale[3]);
         float mv = 0.0f, mw = 0.0f;
         for (int j = tid; j < a.N; j += NOM_THREADS) {
             const float4 x = __ldg(reinterpret_cast<const float4*>(a.Xs) + j);
@@ -260,57 +262,6 @@ __global__ void __launch_bounds__(NOM_THREADS) k_nominal_mean(const RolloutArgs 
         }
         mu[0] = nX; mu[1] = nY; mu[2] = nT; mu[3] = nV; mu[4] = nW;
     }
-}
-
-// The variances along that trajectory in FP64: T queries of N (N + 1) / 2
-// multiply-adds (5 us of the FP64 pipe at T = 45, N = 350).  The FP32 products of
-// a rollout would do for its samples; here one trajectory's covariance goes to
-// the caller, and what is left of the signal variance is its rounding.
-__global__ void k_nominal_k64(const double* __restrict__ X, int N, int T, const float4* __restrict__ zq, double il0,
-                              double il1, double il2, double il3, double sf2, double* __restrict__ K) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x, t = blockIdx.y;
-    if (j >= N) return;
-    const float4 z = zq[t];
-    const double d0 = (z.x - X[4 * j]) * il0, d1 = (z.y - X[4 * j + 1]) * il1;
-    const double d2 = (z.z - X[4 * j + 2]) * il2, d3 = (z.w - X[4 * j + 3]) * il3;
-    K[(size_t)t * N + j] = sf2 * exp(-0.5 * (d0 * d0 + d1 * d1 + d2 * d2 + d3 * d3));
-}
-
-constexpr int NQ64 = 8;              // queries per warp: a factor entry read serves all of them
-
-// V[t][i] = (L^-1 k_t)_i squared, one warp per row i and NQ64 queries
-__global__ void __launch_bounds__(256) k_nominal_v64(const double* __restrict__ L, int N, int T, const double* __restrict__ K,
-                                                     double* __restrict__ V) {
-    const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31, t0 = blockIdx.y * NQ64;
-    if (i >= N) return;
-    const int n = min(NQ64, T - t0);
-    double v[NQ64];
-#pragma unroll
-    for (int q = 0; q < NQ64; ++q) v[q] = 0.0;
-    for (int j = lane; j <= i; j += 32) {
-        const double l = L[(size_t)i * N + j];
-#pragma unroll
-        for (int q = 0; q < NQ64; ++q) v[q] += l * K[(size_t)(t0 + min(q, n - 1)) * N + j];
-    }
-#pragma unroll
-    for (int q = 0; q < NQ64; ++q) {
-        for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
-        if (lane == 0 && q < n) V[(size_t)(t0 + q) * N + i] = v[q] * v[q];
-    }
-}
-
-// variance of query t: max(0, sf2 - sum_i V[t][i])
-__global__ void __launch_bounds__(256) k_nominal_s64(const double* __restrict__ V, int N, double sf2, float* __restrict__ out) {
-    __shared__ double red[256];
-    double s = 0.0;
-    for (int i = threadIdx.x; i < N; i += 256) s += V[(size_t)blockIdx.x * N + i];
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) out[blockIdx.x] = (float)fmax(0.0, sf2 - red[0]);
 }
 
 }  // namespace
@@ -369,21 +320,6 @@ int launch_noise(uint64_t seed, int K, int T, uint64_t it, float sv, float sw, f
 int launch_nominal_mean(const RolloutArgs& a, const QueryWs& ws, cudaStream_t st) {
     // a.U holds the updated controls for this launch
     k_nominal_mean<<<1, NOM_THREADS, 0, st>>>(a, a.U, ws);
-    GPM_CUDA(cudaGetLastError());
-    return GPMPPI_OK;
-}
-
-int launch_nominal_var(const GpDevice& g, int T, const QueryWs& ws, double* scratch, cudaStream_t st) {
-    const gpmppi_hyper& h = g.hyper[0];
-    double *K = scratch, *V = scratch + (size_t)T * g.N;
-    if (g.N > 0) {
-        k_nominal_k64<<<dim3((unsigned)((g.N + 127) / 128), (unsigned)T), 128, 0, st>>>(
-            g.X64, g.N, T, ws.zq, 1.0 / h.lengthscale[0], 1.0 / h.lengthscale[1], 1.0 / h.lengthscale[2],
-            1.0 / h.lengthscale[3], h.signal_var, K);
-        k_nominal_v64<<<dim3((unsigned)((g.N + 7) / 8), (unsigned)((T + NQ64 - 1) / NQ64)), 256, 0, st>>>(
-            g.Linv64[0], g.N, T, K, V);
-    }
-    k_nominal_s64<<<T, 256, 0, st>>>(V, g.N, h.signal_var, ws.q);
     GPM_CUDA(cudaGetLastError());
     return GPMPPI_OK;
 }

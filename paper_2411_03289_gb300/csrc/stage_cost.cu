@@ -245,13 +245,13 @@ __global__ void __launch_bounds__(ST) k_stage_cost(const RolloutArgs a, const Sc
 
 // Alg. 1 Step 2: the covariance along the nominal trajectory, one warp.  Lanes
 // load 32 steps' states and variances (ws.q) at a time; every lane carries the
-// recurrence, lane 0 records Sigma_XY after each step.
+// recurrence, lane 0 records Sigma_XY after each step.  Sigma in full, its two
+// triangles by themselves: their roundings differ, and both go into the next step.
 __global__ void __launch_bounds__(32) k_nominal_cov(const RolloutArgs a, const QueryWs ws,
                                                     float* __restrict__ sxy) {
     const int lane = threadIdx.x;
     grid_wait();
-    float S00 = 0, S01 = 0, S02 = 0, S03 = 0, S04 = 0, S11 = 0, S12 = 0, S13 = 0, S14 = 0, S22 = 0, S23 = 0, S24 = 0,
-          S33 = 0, S34 = 0, S44 = 0;
+    float S[5][5] = {};
     for (int k0 = 0; k0 < a.T; k0 += 32) {
         const int kl = min(k0 + lane, a.T - 1);
         float th = a.x0[2], vl = a.x0[3];
@@ -266,11 +266,30 @@ __global__ void __launch_bounds__(32) k_nominal_cov(const RolloutArgs a, const Q
         for (int i = 0; i < 32 && k0 + i < a.T; ++i) {
             const float sn = __shfl_sync(0xffffffffu, snl, i), cs = __shfl_sync(0xffffffffu, csl, i);
             const float v = __shfl_sync(0xffffffffu, vl, i), s = __shfl_sync(0xffffffffu, sl, i);
-            cov_step(a, false, sn, cs, v, s, S00, S01, S02, S03, S04, S11, S12, S13, S14, S22, S23, S24, S33, S34, S44);
+            const float a02 = -a.dt * v * sn, a03 = a.dt * cs, a12 = a.dt * v * cs, a13 = a.dt * sn;
+            float B[5][5];                     // A Sigma
+#pragma unroll
+            for (int j = 0; j < 5; ++j) {
+                B[0][j] = fmaf(a03, S[3][j], fmaf(a02, S[2][j], S[0][j]));
+                B[1][j] = fmaf(a13, S[3][j], fmaf(a12, S[2][j], S[1][j]));
+                B[2][j] = fmaf(a.dt, S[4][j], S[2][j]);
+                B[3][j] = a.av * S[3][j];
+                B[4][j] = a.aw * S[4][j];
+            }
+#pragma unroll
+            for (int r = 0; r < 5; ++r) {      // times A^T
+                S[r][0] = fmaf(B[r][3], a03, fmaf(B[r][2], a02, B[r][0]));
+                S[r][1] = fmaf(B[r][3], a13, fmaf(B[r][2], a12, B[r][1]));
+                S[r][2] = fmaf(B[r][4], a.dt, B[r][2]);
+                S[r][3] = __fmul_rn(B[r][3], a.av);
+                S[r][4] = __fmul_rn(B[r][4], a.aw);
+            }
+            S[3][3] = __fadd_rn(S[3][3], s);
+            S[4][4] = __fadd_rn(S[4][4], s);
             if (lane == 0) {
-                sxy[3 * (k0 + i)] = S00;
-                sxy[3 * (k0 + i) + 1] = S01;
-                sxy[3 * (k0 + i) + 2] = S11;
+                sxy[3 * (k0 + i)] = S[0][0];
+                sxy[3 * (k0 + i) + 1] = S[0][1];
+                sxy[3 * (k0 + i) + 2] = S[1][1];
             }
         }
     }

@@ -253,6 +253,22 @@ __global__ void __launch_bounds__(PQ) k_rowsum(const float* __restrict__ V, int 
     if (q < Q) out[q] = s;
 }
 
+// max(0, sf2 - |v_q|^2): 256 chains over the columns mod 256, eight threads a query for
+// the trees of their warps, which are added in order
+__global__ void __launch_bounds__(8 * PQ) k_block_variance(const float* __restrict__ V, int ld, int Q, int N, float sf2,
+                                                           float* __restrict__ out) {
+    __shared__ float red[8][PQ];
+    const int w = threadIdx.x / PQ, l = threadIdx.x % PQ;
+    grid_wait();
+    red[w][l] = lane_squares<256>(V + (size_t)blockIdx.x * ld * PQ + l, PQ, 32 * w, N);
+    __syncthreads();
+    const int q = blockIdx.x * PQ + l;
+    if (w > 0 || q >= Q) return;
+    float s = 0.0f;
+    for (int i = 0; i < 8; ++i) s += red[i][l];
+    out[q] = fmaxf(0.0f, sf2 - s);
+}
+
 // L^-1 in the pieces of the backward product: block column cb holds rows
 // 128 cb .. npad - 1, 128 columns each, in chunks of 32 rows
 __global__ void k_pack_lb(const double* __restrict__ Linv, int N, int nb, float* __restrict__ out) {
@@ -305,6 +321,12 @@ int launch_rowsum(const float* V, int ld, int Q, int N, SumOrder order, float* o
     if (Np > 0 && Np < 64) Np = 64;
     auto kern = order == kSumPairs ? k_rowsum<kSumPairs> : k_rowsum<kSumLanes>;
     GPM_CUDA(launch_ex(kern, dim3((unsigned)((Q + PQ - 1) / PQ)), PQ, 0, st, true, V, ld, Q, Np, out));
+    return GPMPPI_OK;
+}
+
+int launch_block_variance(const float* V, int ld, int Q, int N, float sf2, float* out, cudaStream_t st) {
+    if (Q <= 0) return GPMPPI_OK;
+    GPM_CUDA(launch_ex(k_block_variance, dim3((unsigned)((Q + PQ - 1) / PQ)), 8 * PQ, 0, st, true, V, ld, Q, N, sf2, out));
     return GPMPPI_OK;
 }
 

@@ -1,9 +1,8 @@
 """The batched rollout's tile layouts (2, 4 and 8 threads a sample, scenes in and
 out of shared memory, two- and three-part formats) against the single step and the
-oracle.  Where both keep the small split products in their own column set (the
-three-part format, and any training set of more than 768 points) the single step
-adds its sums in the batched rollout's order: every cost, weight and control is the
-same bits."""
+oracle.  The single step adds its sums in the batched rollout's order, and every cost,
+weight and control is the same bits, but for training sets of up to 512 points in two
+parts (and there too where the environment asks for the batched order)."""
 import numpy as np
 import pytest
 
@@ -43,25 +42,27 @@ def _equal(one, many):
 # training sets on both sides of the 64-column steps, of an odd and an even count of
 # 128-column blocks and of the 256-column passes; ragged sample tiles
 @pytest.mark.parametrize("rps", [2, 4, 8])
-@pytest.mark.parametrize("precision,N", [(2, 769), (2, 897), (1, 1025), (2, 1200), (3, 1), (3, 65), (3, 129), (3, 333),
-                                         (3, 1025)])
+@pytest.mark.parametrize("precision,N", [(2, 1), (1, 65), (2, 129), (2, 333), (1, 512), (2, 513), (2, 640), (2, 641),
+                                         (1, 768), (2, 769), (2, 897), (1, 1025), (2, 1200), (3, 1), (3, 65), (3, 129),
+                                         (3, 333), (3, 1025)])
 def test_step_and_batch_are_the_same_bits(lib, precision, N, rps, monkeypatch):
+    monkeypatch.setenv("GPMPPI_NO_CLUSTER", "1")
     sc = S.scenario("small", K=301, T=5, N=N, O=5, precision=precision)
     one, many, _ = _both(lib, sc, rps, monkeypatch)
     _equal(one, many)
 
 
-@pytest.mark.parametrize("precision,N", [(3, 150), (2, 800)])
+@pytest.mark.parametrize("precision,N", [(3, 150), (2, 90), (1, 300), (2, 800)])
 def test_ensemble_step_and_batch_are_the_same_bits(lib, precision, N, monkeypatch):
     sc = S.terrain_scenario("small", M=2, N=N, K=213, T=4, precision=precision)
     one, many, _ = _both(lib, sc, 4, monkeypatch)
     _equal(one, many)
 
 
-@pytest.mark.parametrize("precision", [2, 3])
-def test_large_step_and_batch_are_the_same_bits(lib, precision, monkeypatch):
+@pytest.mark.parametrize("precision,N", [(2, 2048), (3, 2048), (2, 700)])
+def test_large_step_and_batch_are_the_same_bits(lib, precision, N, monkeypatch):
     """Every weight of a step whose queries fill the chip without a split of the passes."""
-    sc = S.scenario("small", K=16384, T=30, N=2048, O=20, path="eight", precision=precision)
+    sc = S.scenario("small", K=16384, T=30, N=N, O=20, path="eight", precision=precision)
     one, many, _ = _both(lib, sc, 2, monkeypatch)
     _equal(one, many)
 
@@ -69,8 +70,7 @@ def test_large_step_and_batch_are_the_same_bits(lib, precision, monkeypatch):
 @pytest.mark.parametrize("rps", [2, 4, 8])
 @pytest.mark.parametrize("precision,N", [(2, 333), (1, 700)])
 def test_batch_layouts_against_the_oracle(lib, precision, N, rps, monkeypatch):
-    """One column set for all products (up to 768 points): the oracle's step, and the
-    single step's within the two kernels' rounding."""
+    """The oracle's step, and the single step's within the two kernels' rounding."""
     sc = S.scenario("small", K=299, T=6, N=N, O=5, precision=precision)
     one, many, _ = _both(lib, sc, rps, monkeypatch)
     fits = O.gp_fit(sc.X, sc.Y, sc.hyper)
