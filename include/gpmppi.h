@@ -296,9 +296,9 @@ int terrain_weights(const double* Yv, const double* Yw, const double* Fv, const 
  * (GPMPPI_ERR_UNSUPPORTED beyond).
  * The first call, and the first call asking for dlengthscale, allocate
  * device scratch owned by the controller (freed by mppi_destroy) and may
- * synchronise: 2 T K N floats for as many samples at a time as fit 2 GB, fewer
- * on a full device (J and dU are the same bits, dlengthscale up to the order of
- * its sums).  A later call allocates nothing and may be captured.  Runs on the
+ * synchronise: 2 T K N floats for as many samples at a time as fit 2 GB (8 GB
+ * with dlengthscale), fewer on a full device (J and dU are the same bits,
+ * dlengthscale up to the order of its sums).  A later call allocates nothing and may be captured.  Runs on the
  * controller's FP32 path whatever its precision. */
 int mppi_grad(gpmppi_ctrl c, const float state[5], const float* U_nom, const float* sample_weights,
               float slope, float* J, float* dU, float* dlengthscale, void* stream);

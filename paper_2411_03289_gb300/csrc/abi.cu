@@ -967,11 +967,13 @@ int mppi_grad(gpmppi_ctrl c, const float state[5], const float* U_nom, const flo
     const GpSet gs = single_gp_set(g, 0);
     int nsm = 0;
     GPM_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device));
-    // Samples at a time: rows of v and b of up to 2 GB, fewer on a full device.  The
-    // count is kept with the scratch: every later call takes the same pieces.
-    size_t piece = ((size_t)1 << 29) / ((size_t)T * (g.npad + Np + 64));
+    // Samples at a time: rows of v and b of up to 2 GB, fewer on a full device; 8 GB
+    // with the lengthscales, whose Gram sums are grouped by the pieces.  The count is
+    // kept with the scratch: every later call takes the same pieces.
+    size_t piece = ((size_t)1 << (want_l ? 31 : 29)) / ((size_t)T * (g.npad + Np + 64));
     piece = piece < 8 ? 8 : piece / 8 * 8;
-    int Ks = c->grad_Ks > 0 ? c->grad_Ks : (piece < (size_t)K ? (int)piece : K);
+    const bool made = c->grad_scr && (c->grad_l || !want_l);
+    int Ks = made ? c->grad_Ks : (piece < (size_t)K ? (int)piece : K);
     auto kpad_of = [&](int s0) { return ((K - s0 < Ks ? K - s0 : Ks) + 7) / 8 * 8; };
     // scratch layout (bytes, each piece 256-aligned)
     size_t off = 0, o_ut = 0, o_zq = 0, o_st = 0, o_qq = 0, o_rec = 0, o_v = 0, o_S = 0, o_dU = 0, o_dl = 0, o_B = 0,
@@ -1003,11 +1005,9 @@ int mppi_grad(gpmppi_ctrl c, const float state[5], const float* U_nom, const flo
         }
     };
     layout();
-    if (off > c->grad_bytes) {
+    if (!made) {
         cudaFree(c->grad_scr);
         c->grad_scr = nullptr;
-        c->grad_bytes = 0;
-        c->grad_Ks = 0;
         cudaError_t e;
         while ((e = cudaMalloc(&c->grad_scr, off)) == cudaErrorMemoryAllocation && Ks > 8) {
             cudaGetLastError();
@@ -1018,8 +1018,8 @@ int mppi_grad(gpmppi_ctrl c, const float state[5], const float* U_nom, const flo
             c->grad_scr = nullptr;
             return cuda_fail(e, "mppi_grad: scratch");
         }
-        c->grad_bytes = off;
         c->grad_Ks = Ks;
+        c->grad_l = want_l;
     }
     char* base = static_cast<char*>(c->grad_scr);
     GradArgs ga;

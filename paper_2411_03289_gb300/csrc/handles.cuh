@@ -68,8 +68,8 @@ struct gpmppi_ctrl_s {
     float tw[gpm::kMaxTerrains] = {};
     // adjoint-rollout scratch (allocated by the first mppi_grad call)
     void* grad_scr = nullptr;
-    size_t grad_bytes = 0;
     int grad_Ks = 0;              // samples at a time that it was made for
+    bool grad_l = false;          // with room for the lengthscales' terms
     bool profiling = false;
     bool profiled = false;
     cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};

@@ -44,7 +44,7 @@ def _grad(lib, ctrl, sc, want_dl=True):
 
 @pytest.mark.parametrize("K,T,N,left", [
     (4001, 40, 500, 300 << 20),       # 0.7 GB of rows: one piece, and a few with a ragged last one
-    (6001, 60, 1000, 500 << 20)])     # 3 GB: two pieces, and more
+    (6001, 60, 1000, 500 << 20)])     # 3 GB: one piece, and more than four
 def test_gradient_on_a_full_device(lib, K, T, N, left):
     """Fewer samples at a time: J and dU are per-sample terms added in the samples'
     order, the same bits; the lengthscales' Gram sums are FP32 sums of thousands of
