@@ -283,8 +283,9 @@ def committed_traffic(kernel="tri", workload=WORKLOAD):
 
 def step_launches(P, sizes):
     """Kernels of one mppi_step over GPs of these sizes: the chain, the variances
-    (split precisions: one kernel; FP32: a product and its row sums for each GP and
-    each 256 MB of rows), the stage costs and the update."""
+    (split precisions: one kernel, a second where few queries split its passes;
+    FP32: a product and its row sums for each GP and each 256 MB of rows), the
+    stage costs and the update."""
     if P.precision != 0:
         return 4
     npad = max((n + 127) // 128 * 128 for n in sizes)

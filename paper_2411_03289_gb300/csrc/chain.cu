@@ -11,7 +11,7 @@
 // of the kernel rows (about 10 instructions for two points) once it does not.
 // With one sample per 16 lanes the shared-memory reads of the points bounded it
 // (12 KB per sample and step at N = 500): 112 us at K = 4096, T = 50, N = 500
-// against 87 us with four samples a warp.
+// against 71 us with four samples a warp (85 with the lanes' sums as a tree).
 #include "query.cuh"
 
 namespace gpm {
@@ -30,10 +30,10 @@ constexpr int CW = CT / 32;
 //   R = 1        kSumsShares: 16-point chunks; chains of the even and the odd chunks of
 //                each share, 257 to 512 points: 24-27, 12-23, then 28-31 with 0-11; 129
 //                to 256: 12-15, 0-11; fewer: 0-7
-// A lane forms the parts of its stages, and a lane a chain then adds them: a serial sum
-// of N / 32 terms a step that a tree would not have.  K = 16384 T = 100 N = 2048 (R =
-// 2): 1.64 ms (1.64 with the lanes' sums as a tree); K = 5000 T = 60 N = 1500 (R = 8):
-// 397 us (313); K = 1500 T = 37 N = 777 (R = 8): 77 us (55).
+// A lane forms the parts of its stages, and a lane a chain then adds them: for R > 1 a
+// serial sum of N / 32 terms a step that a tree would not have.  K = 16384 T = 100 N =
+// 2048 (R = 2): 1.62 ms (1.64 with the lanes' sums as a tree); K = 5000 T = 60 N = 1500
+// (R = 8): 380 us (313); K = 1500 T = 37 N = 777 (R = 8): 76 us (55).
 __host__ __device__ constexpr int part_pairs(int R) { return R == 1 ? 8 : 16 / R; }
 // R > 1: parts a lane forms before they are added, 16 or 32 stages (a batch's hand-over
 // costs as much as the sums of some 20 stages); R = 1: all of them
@@ -289,12 +289,12 @@ int launch_chain(const RolloutArgs& a, const GpSet& gs, const QueryWs& ws, cudaS
     for (int t = 0; t < gs.M; ++t) points += (size_t)gs.gp[t].npad;
     // two CTAs per SM keep their training sets in shared memory up to 4096 points
     const bool sm = points * 24 <= 100 * 1024;
-    // samples per warp: as many as leave every scheduler a warp and a half.
-    // Measured (us, 1 / 2 / 4 / 8 samples): K = 256 T = 20 N = 50: 14 / 16 / 16 /
-    // 20; K = 1000 T = 40 N = 300: 34 / 36 / 40 / 54; K = 4096 T = 50 N = 500:
-    // 114 / 98 / 87 / 87; K = 16384 T = 100 N = 2048: 2379 / 1683 / 1414 / 1509.
-    int sg = 1;
-    while (sg < 4 && a.K / (2 * sg) >= 900) sg *= 2;     // (a.K: the same in every piece of the samples)
+    // Samples per warp (the sums do not depend on them; a.K: the same in every piece of
+    // the samples).  Measured (us, 1 / 2 / 4 samples): K = 256 T = 20 N = 50: 14.3 /
+    // 16.9 / 22.6; K = 1000 T = 40 N = 300: 35.1 / 31.8 / 43.7, N = 1200: 85.9 / 77.8 /
+    // 118; K = 2000 T = 40 N = 1000: 110 / 78.9 / 95.1; K = 4096 T = 50 N = 500: 99.4 /
+    // 79.3 / 70.9, N = 1200: 294 / 201 / 199; K = 16384 T = 100 N = 2048: 2954 / 1954 / 1580.
+    const int sg = a.K >= 3600 ? 4 : a.K >= 900 ? 2 : 1;
 #define GPM_CHAIN(L, R)                                                                                         \
     do {                                                                                                        \
         const dim3 grid((unsigned)((ws.Ks + CW * L - 1) / (CW * L)));                                           \

@@ -1,6 +1,6 @@
 // Triangular products of the GP factor in FP32 on the CUDA cores, and the sums
 // of squares over their rows.
-//   forward   v_q = L^-1 k*_q   (query rollout, gp_predict, adjoint)
+//   forward   v_q = L^-1 k*_q   (query rollout, Alg. 1 Step 2, gp_predict, adjoint)
 //   backward  b_q = L^-T v_q = K^-1 k*_q   (adjoint)
 // An item is 128 queries x one 128-column block, reduced over the training points
 // of its triangle in chunks of 32: the factor piece (32 x 128 floats, contiguous)

@@ -3,9 +3,10 @@
 //
 // Operands are split into 16-bit parts (hi + lo in FP16 or BF16: three products
 // hi.hi, hi.lo, lo.hi; hi + mid + lo in BF16: six), accumulated in FP32 in
-// tensor memory.  hi.hi has its own column set and the small products a second
-// one, added when the squares are summed: the tensor core rounds its
-// accumulator at every MMA, so the large sum sees one addition per 16 points.
+// tensor memory.  The tensor core rounds its accumulator at every MMA, so that what
+// shares a column set and in which order is part of the result (VarSums): with the
+// small products in a set of their own, added when the squares are summed, the large
+// sum sees one addition per 16 points.
 //
 // A pair of CTAs (cluster of two, one pair per SM pair, persistent) takes 256
 // queries, 128 in each CTA, and the factor's columns in passes of 256.  The MMAs
@@ -29,8 +30,11 @@
 // triangle) at large N: K = 16384, T = 100, N = 2048 in FP16 11.0 ms, the measured BF16
 // peak of issued products (15.9 ms with 32-point stages and the stage's item divided
 // out by the loader each time; the step took 18.4 ms as one kernel over the horizon).
-// Up to N = 512 the roles' hand-offs per stage, the tensor pipe 65 % active: 123 us at
-// K = 4096, T = 50, N = 500 (the whole rollout as one kernel: 303 us).
+// Up to N = 512 the roles' hand-offs per stage, the tensor pipe 65 % active, and the
+// stages that come twice for the slices' orders (15 entries instead of 12): 159 us at
+// K = 4096, T = 50, N = 500, 125 us with one order for all columns, which an input in
+// six moved beyond rounding at K = 16000, T = 100 (the whole rollout as one kernel:
+// 303 us).
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
